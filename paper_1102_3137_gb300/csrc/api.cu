@@ -350,7 +350,7 @@ Bufs sub_bufs(const Geo& g, const Bufs& b, bool mixed, int k0) {
   if (k0 == 0) return b;
   Bufs s = b;
   const size_t K0 = (size_t)k0, S0 = K0 * g.nb, Ndd = g.Ndd, nsub = (size_t)g.Lx * g.W;
-  const size_t cs = mixed ? sizeof(cxf) : sizeof(cxd), Lx2 = (size_t)g.Lx * g.Lx;
+  const size_t cs = mixed ? sizeof(cxf) : sizeof(cxd);
   auto adv = [](auto* ptr, size_t bytes) {
     using T = std::remove_pointer_t<decltype(ptr)>;
     return ptr ? reinterpret_cast<T*>(reinterpret_cast<char*>(const_cast<std::remove_const_t<T>*>(ptr)) + bytes)
@@ -450,12 +450,12 @@ int enqueue_solve(dyson_plan p, int K, cudaStream_t s, bool cap) {
 // an interface, on the caller's staged inputs, run init, factorization and
 // preconditioner once, then time one X-matvec launch (after one untimed) for
 // each copy-ring configuration the geometry admits (ring slots; chunk height
-// for W > 64) and keep the fastest for every later launch and captured graph.
+// for W > 64; rows on chip or in scratch for the mixed form's strips) and keep the fastest for every later launch and captured graph.
 int autotune(dyson_plan p, int K, cudaStream_t s) {
   p->tuned = true;
   if (p->g.p < 2) return DYSON_OK;
-  int S[32], CR[32], NT[32];
-  const int n = dyson_internal_ring_candidates(p->g, p->mixed, S, CR, NT, 32);
+  int S[32], CR[32], ROWS[32];
+  const int n = dyson_internal_ring_candidates(p->g, p->mixed, S, CR, ROWS, 32);
   p->tune_candidates = n;
   if (n < 2) return DYSON_OK;
   Geo& g = p->g;
@@ -474,7 +474,7 @@ int autotune(dyson_plan p, int K, cudaStream_t s) {
   for (int c = 0; c < n && rc == DYSON_OK; ++c) {
     g.ring_S = S[c];
     g.ring_CR = CR[c];
-    g.xm_nt = NT[c];
+    g.xm_rows = ROWS[c];
     cudaError_t e = p->mixed ? launch_xmatvec<float>(g, p->b, K, 0, 1, g.nb, s)
                              : launch_xmatvec<double>(g, p->b, K, 0, 0, g.nb, s);
     if (e == cudaSuccess) e = cudaEventRecord(e0, s);
@@ -499,7 +499,7 @@ int autotune(dyson_plan p, int K, cudaStream_t s) {
   cudaEventDestroy(e1);
   g.ring_S = S[best];
   g.ring_CR = CR[best];
-  g.xm_nt = NT[best];
+  g.xm_rows = ROWS[best];
   p->tune_ms_best = best_ms;
   return rc;
 }
@@ -630,15 +630,6 @@ int dyson_plan_create(const dyson_geometry* geom, dyson_plan* out) {
   p->tune_candidates = 0;
   p->tune_ms_heuristic = p->tune_ms_best = 0.f;
   p->n_prof = 0;
-  // X-matvec CTA size (complex64 two-chain form): 128 threads, four CTAs per SM,
-  // when the solve's clusters would not all fit at two CTAs per SM; the
-  // autotuner may revise it at the first solve
-  if (p->mixed && p->g.W <= DY_MAXW_SMEM && p->g.p > 1) {
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
-    const long long ctas = (long long)p->g.p * p->Kcap * p->g.nb;
-    p->g.xm_nt = (sms > 0 && ctas > 2LL * sms) ? 128 : 256;
-  }
   // frequency groups: not with the shared wide-slice factor workspace
   p->ngroups = 1;
   if (p->g.p > 1 && !b.fwork) {

@@ -199,8 +199,8 @@ struct Geo {
   int ring_CR;         // rows per streamed chunk chosen by the autotuner (W > 64; 0: heuristic)
   int nb;              // Lanczos block size (1: the scalar recurrence of Sec. 2.1)
   int lpre;            // interface preconditioner: 1 exact layer blocks of S (2D strips), 0 banded
-  int xm_nt;           // threads per X-matvec CTA in the complex64 two-chain form (128: four CTAs
-                       // per SM; 0 or 256: two), chosen by the heuristic or the autotuner
+  int xm_rows;         // mixed form, W <= 64, ring_S > 0: sweep row buffers on chip (1) or in the
+                       // plan's scratch (0), chosen by the autotuner
   int qsplit;          // the Lanczos basis is stored as double-floats (cdfl; mixed form, nb = 1,
                        // k_max <= 64, where the double-float Lanczos step runs)
 };
@@ -220,7 +220,8 @@ struct Bufs {
   void* g;              // [K][p][Lx][W][W] slice factors g_s read by the sweeps (precision of the form)
   cxd* g64;             // [K][p][Lx][W][W] FP64 g_s kept for the mixed form's FP64 recursion
   cxd* diagB;           // [K][Ndd] diag(B^-1), zero on the interface
-  cxd* hdiag;           // [K][Ndd] H_ii (Eq. 1) in DD layout, zero on padding (mixed form), or null
+  cxd* hdiag;           // [K][Ndd] H_ii (Eq. 1) in DD layout, zero on padding (mixed form; double-floats
+                        // for W <= 64), or null
   cxd* offB;            // [K][p][Lx][W] diag of G_{s,s+1} (B_i^-1 between slices s, s+1), or null
   cxd* off2;            // [K][p][Lx][W] diag of G_{s,s+2} on the boundary rows (2D strips), or null
   cxd* Q;               // [K][k_max+nb][Ndd] Lanczos vectors (column j*nb + c of block j)
@@ -288,9 +289,9 @@ size_t dyson_internal_plan_bytes(dyson_plan_s* p);
 // the given form; 0 when the slice width and x extent do not fit on chip.
 size_t dyson_internal_sweep_smem(const Geo& g, bool mixed);
 // Copy-ring configurations the autotuner times for this geometry and form:
-// up to max pairs (slots, chunk rows), the shared-memory heuristic's first.
-int dyson_internal_ring_candidates(const Geo& g, bool mixed, int* S, int* CR, int* NT, int max);
-// The copy-ring configuration the kernels use for this geometry (slots, chunk rows).
+// up to max triples (slots, chunk rows, rows on chip), the shared-memory heuristic's first.
+int dyson_internal_ring_candidates(const Geo& g, bool mixed, int* S, int* CR, int* ROWS, int max);
+// The copy-ring configuration the kernels use for this geometry (slots, chunk rows, threads per CTA).
 void dyson_internal_ring_plan(const Geo& g, bool mixed, int* S, int* CR, int* NT);
 
 // ---------------------------------------------------------------- host launchers

@@ -464,14 +464,18 @@ __global__ void __launch_bounds__(DY_THREADS) k_precond(Geo g, Bufs b) {
 
 }  // namespace
 
-// H_ii (Eq. 1) of every DD slot, zero on padding: the mixed form's FP64
-// residuals read it coalesced instead of gathering V and Sigma in natural order.
+// H_ii (Eq. 1) of every DD slot, zero on padding: the mixed form's residuals
+// read it coalesced instead of gathering V and Sigma in natural order.  For
+// slices of up to 64 sites, whose residuals run in double-float arithmetic, an
+// entry is stored as a cdfl, else in binary64 (16 bytes either way).
 __global__ void __launch_bounds__(DY_THREADS) k_hdiag(Geo g, Bufs b) {
   const int kf = blockIdx.y;
   for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < (size_t)g.Ndd;
        k += (size_t)gridDim.x * blockDim.x) {
     const int nat = b.dd2nat[k];
-    b.hdiag[(size_t)kf * g.Ndd + k] = nat >= 0 ? dyson_diag(g, b, kf, nat) : cxd{0, 0};
+    const cxd d = nat >= 0 ? dyson_diag(g, b, kf, nat) : cxd{0, 0};
+    if (g.W <= DY_MAXW_SMEM) reinterpret_cast<cdfl*>(b.hdiag)[(size_t)kf * g.Ndd + k] = csplit(d);
+    else b.hdiag[(size_t)kf * g.Ndd + k] = d;
   }
 }
 

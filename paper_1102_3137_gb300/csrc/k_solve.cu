@@ -1,7 +1,7 @@
 // Lanczos step, start vector and the small per-frequency kernels (the
 // X-matvec and subdomain-solve kernels, which carry the block sweeps, are
 // compiled in k_xmatvec_c64.cu and k_xmatvec_c128.cu).
-#include "solve_device.cuh"
+#include "xmatvec_mixed.cuh"
 
 namespace {
 
@@ -217,21 +217,28 @@ cudaError_t launch_wait_selftest(unsigned long long limit_ns, int* out, cudaStre
 }
 
 size_t dyson_internal_sweep_smem(const Geo& g, bool mixed) {
+  if (mixed && g.W <= DY_MAXW_SMEM) return mix_plan(g).smem;
   return mixed ? sweep_smem<float>(g) : sweep_smem<double>(g);
 }
 
 void dyson_internal_ring_plan(const Geo& g, bool mixed, int* S, int* CR, int* NT) {
+  if (mixed && g.W <= DY_MAXW_SMEM) {
+    *S = 2 * mix_plan(g).S;
+    *CR = g.W;
+    *NT = mix_threads(g.W);
+    return;
+  }
   const RingPlan rp = mixed ? ring_plan<float>(g) : ring_plan<double>(g);
   *S = rp.S;
   *CR = rp.CR;
-  *NT = mixed ? xm_threads<float>(g) : xm_threads<double>(g);
+  *NT = DY_THREADS;
 }
 
-int dyson_internal_ring_candidates(const Geo& g, bool mixed, int* S, int* CR, int* NT, int max) {
-  return mixed ? ring_candidates<float>(g, S, CR, NT, max) : ring_candidates<double>(g, S, CR, NT, max);
+int dyson_internal_ring_candidates(const Geo& g, bool mixed, int* S, int* CR, int* ROWS, int max) {
+  if (mixed && g.W <= DY_MAXW_SMEM) return mix_candidates(g, S, CR, ROWS, max);
+  for (int k = 0; k < max; ++k) ROWS[k] = 0;
+  return mixed ? ring_candidates<float>(g, S, CR, max) : ring_candidates<double>(g, S, CR, max);
 }
-
-
 
 cudaError_t launch_lanczos(const Geo& g, const Bufs& b, int K, int j, cudaStream_t st) {
   if (g.k_max > KMAX_SMEM) return cudaErrorInvalidValue;

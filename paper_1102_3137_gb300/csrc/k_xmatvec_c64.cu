@@ -1,28 +1,24 @@
-// Mixed form (complex64 sweeps): the dispatch over sweep forms and the
-// W > 64 (row-chunked) and W <= 16 variants.  The W <= 32 and W <= 64
-// variants are compiled in k_xmatvec_c64_w32.cu and k_xmatvec_c64_w64.cu.
-#include "solve_device.cuh"
+// Mixed form (complex64 sweeps): the dispatch over sweep forms, the W > 64
+// (row-chunked) variant and the W <= 16 one.  The W <= 32 and W <= 64 variants
+// are compiled in k_xmatvec_c64_w32.cu and k_xmatvec_c64_w64.cu.
+#include "xmatvec_mixed.cuh"
 
 DY_SOLVE_VARIANT(float, 0)
-DY_SOLVE_VARIANT(float, 16)
+DY_MIXED_VARIANT(16)
 
 template <>
 cudaError_t launch_xmatvec<float>(const Geo& g, const Bufs& b, int K, int j, int mixed, int ncols, cudaStream_t st) {
-  switch (sweep_form<float>(g)) {
-    case 0: return run_xmatvec<float, 0>(g, b, K, j, mixed, ncols, st);
-    case 16: return run_xmatvec<float, 16>(g, b, K, j, mixed, ncols, st);
-    case 32: return run_xmatvec<float, 32>(g, b, K, j, mixed, ncols, st);
-    default: return run_xmatvec<float, 64>(g, b, K, j, mixed, ncols, st);
-  }
+  if (g.W > DY_MAXW_SMEM) return run_xmatvec<float, 0>(g, b, K, j, mixed, ncols, st);
+  if (g.W <= 16) return run_xmatvec_m<16>(g, b, K, j, ncols, st);
+  if (g.W <= 32) return run_xmatvec_m<32>(g, b, K, j, ncols, st);
+  return run_xmatvec_m<64>(g, b, K, j, ncols, st);
 }
 
 template <>
 cudaError_t launch_bsolve<float>(const Geo& g, const Bufs& b, int K, const cxd* q_dd, cxd* w_dd,
                                  cudaStream_t st) {
-  switch (sweep_form<float>(g)) {
-    case 0: return run_bsolve<float, 0>(g, b, K, q_dd, w_dd, st);
-    case 16: return run_bsolve<float, 16>(g, b, K, q_dd, w_dd, st);
-    case 32: return run_bsolve<float, 32>(g, b, K, q_dd, w_dd, st);
-    default: return run_bsolve<float, 64>(g, b, K, q_dd, w_dd, st);
-  }
+  if (g.W > DY_MAXW_SMEM) return run_bsolve<float, 0>(g, b, K, q_dd, w_dd, st);
+  if (g.W <= 16) return run_bsolve_m<16>(g, b, K, q_dd, w_dd, st);
+  if (g.W <= 32) return run_bsolve_m<32>(g, b, K, q_dd, w_dd, st);
+  return run_bsolve_m<64>(g, b, K, q_dd, w_dd, st);
 }

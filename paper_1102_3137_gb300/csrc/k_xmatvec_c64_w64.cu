@@ -1,4 +1,4 @@
-// Mixed form, slices of width 32 < W <= 64 (the two-chain sweep, two rows per lane).
-#include "solve_device.cuh"
+// Mixed form, slices of width 32 < W <= 64 (the two-chain sweep of xmatvec_mixed.cuh).
+#include "xmatvec_mixed.cuh"
 
-DY_SOLVE_VARIANT(float, 64)
+DY_MIXED_VARIANT(64)

@@ -45,8 +45,9 @@ __device__ __forceinline__ int own_count(const Geo& g, int i) {
 }
 
 // ---------------------------------------------------------------- reductions
+constexpr int RED_WARPS = 18;            // most warps of a CTA that reduces
 struct RedSmem {
-  cxd wred[DY_WARPS * 8];
+  cxd wred[RED_WARPS * 8];
   cxd slot[2 * 8];
   cxd res[8];
 };
@@ -185,8 +186,7 @@ struct Pipe {
   void* ybuf;      // forward intermediates in shared memory, or null (global scratch)
   int S;
   int CR;          // rows of a slice block per streamed chunk (= W unless W > 64)
-  unsigned seq;    // blocks issued (= consumed) so far by this CTA (left chain of the two-chain form)
-  unsigned seq2;   // the same for the right chain of the two-chain form
+  unsigned seq;    // blocks issued (= consumed) so far by this CTA
   int* err;        // shared flag: a bounded wait ran out
 };
 
@@ -255,47 +255,15 @@ __device__ void sweep_chunked(const Geo& g, int i, const SweepArgs<R>& a, cx<R>*
 
 // Pre-pass of a sweep (all threads): the right-hand side rows in precision R
 // into the row buffer yb [Lx][W] (zero on padding columns).
-// In complex64 the FP64 right-hand side is converted by integer operations
-// (d2f_bits) and scaled in FP32, so the pass issues nothing on the FP64 pipe;
-// the scale only keeps the values inside the FP32 range, so its product is
-// taken in FP32 whenever it is itself well inside that range.
 template <typename R>
 __device__ __forceinline__ void sweep_prepass(const Geo& g, int i, const SweepArgs<R>& a, cx<R>* yb) {
   const int W = g.W, Lx = g.Lx, T = g.T, w = T * g.h[i], nrow = Lx * W;
   const R t = (R)g.t;
-  const double as = fabs(a.in_scale);
-  const bool fast = sizeof(R) == 4 && as > 1e-30 && as < 1e30;
-  const R scf = (R)a.in_scale;
-  if constexpr (sizeof(R) == 4) {
-    if (a.src && fast) {                 // the common case: PU rows' loads in flight per thread
-      constexpr int PU = 4;
-      const int nt = (int)blockDim.x;
-      for (int e0 = threadIdx.x; e0 < nrow; e0 += PU * nt) {
-        cxd v[PU];
-        bool on[PU];
-#pragma unroll
-        for (int u = 0; u < PU; ++u) {
-          const int e = e0 + u * nt, j = e % W;
-          on[u] = e < nrow && j < w;
-          v[u] = on[u] ? a.src[e] : cxd{0, 0};
-        }
-#pragma unroll
-        for (int u = 0; u < PU; ++u) {
-          const int e = e0 + u * nt;
-          if (e < nrow) yb[e] = on[u] ? scf * c2f_bits(v[u]) : cx<R>{0, 0};
-        }
-      }
-      return;
-    }
-  }
   for (int e = threadIdx.x; e < nrow; e += (int)blockDim.x) {
     const int s = e / W, j = e - s * W;
     cxd v = {0, 0};
     if (j < w) {
-      if (a.src && fast) {
-        if constexpr (sizeof(R) == 4) yb[e] = scf * c2f_bits(a.src[e]);
-        continue;
-      } else if (a.src) {
+      if (a.src) {
         v = a.in_scale * a.src[e];
       } else {
         cx<R> u = {0, 0};
@@ -311,61 +279,16 @@ __device__ __forceinline__ void sweep_prepass(const Geo& g, int i, const SweepAr
 
 // Post-pass of a sweep (all threads): the solution rows x_s in yb to the FP64
 // outputs and the boundary-row copies.
-// In complex64 the scale is applied in FP32 and the value widened by integer
-// operations (f2d_bits); only the accumulating add/subtract into the FP64
-// output runs on the FP64 pipe.
 template <typename R>
 __device__ __forceinline__ void sweep_postpass(const Geo& g, int i, const SweepArgs<R>& a,
                                                const cx<R>* yb) {
   const int W = g.W, Lx = g.Lx, T = g.T, w = T * g.h[i], nrow = Lx * W;
-  const double os = fabs(a.out_scale);
-  const bool fast = sizeof(R) == 4 && os > 1e-30 && os < 1e30;
-  const R scf = (R)a.out_scale;
-  if constexpr (sizeof(R) == 4) {
-    if (a.dst && fast) {                 // the common case: PU rows' loads in flight per thread
-      constexpr int PU = 4;
-      const int nt = (int)blockDim.x;
-      const bool rd = a.dst_op == 1 || a.dst_op == 2;
-      for (int e0 = threadIdx.x; e0 < nrow; e0 += PU * nt) {
-        cx<R> xr[PU];
-        cxd dv[PU];
-        bool on[PU];
-#pragma unroll
-        for (int u = 0; u < PU; ++u) {
-          const int e = e0 + u * nt, j = e % W;
-          on[u] = e < nrow && j < w;
-          xr[u] = on[u] ? yb[e] : cx<R>{0, 0};
-          dv[u] = (on[u] && rd) ? a.dst[e] : cxd{0, 0};
-        }
-#pragma unroll
-        for (int u = 0; u < PU; ++u) {
-          if (!on[u]) continue;
-          const int e = e0 + u * nt, s = e / W, j = e - s * W;
-          const cxd xd = c2d_bits(scf * xr[u]);
-          cxd* d = a.dst + e;
-          if (a.dst_op == 0) *d = xd;
-          else if (a.dst_op == 1) *d = dv[u] + xd;
-          else if (a.dst_op == 2) *d = dv[u] - xd;
-          else *d = -xd;
-          if (a.bnd_lo && j < T) a.bnd_lo[s + Lx * j] = xr[u];
-          if (a.bnd_hi && j >= w - T) a.bnd_hi[s + Lx * (j - (w - T))] = xr[u];
-        }
-      }
-      return;
-    }
-  }
   for (int e = threadIdx.x; e < nrow; e += (int)blockDim.x) {
     const int s = e / W, j = e - s * W;
     if (j >= w) continue;
     const cx<R> xr = yb[e];
     if (a.dst) {
-      cxd xd;
-      if constexpr (sizeof(R) == 4) {
-        if (fast) xd = c2d_bits(scf * xr);
-        else xd = a.out_scale * cconv<double>(xr);
-      } else {
-        xd = a.out_scale * cconv<double>(xr);
-      }
+      const cxd xd = a.out_scale * cconv<double>(xr);
       cxd* d = a.dst + e;
       if (a.dst_op == 0) *d = xd;
       else if (a.dst_op == 1) *d = *d + xd;
@@ -377,324 +300,14 @@ __device__ __forceinline__ void sweep_postpass(const Geo& g, int i, const SweepA
   }
 }
 
-// y = g z for one slice block of the complex64 two-sided factors, by one warp:
-// lane r owns rows r (and r + 32 when WF = 64).  The block is stored with
-// column pairs interleaved, so row r's columns 2k, 2k+1 are one 16-byte load
-// at pair index k W + r (contiguous over the warp, conflict-free), against the
-// broadcast pair z[2k], z[2k+1].  Loads are plain (an inline-asm load with a
-// memory clobber ordered every load behind the previous one: 2.6x slower per
-// slice) and issued four pairs at a time, so a batch's loads are in flight
-// together; 8 (4 at WF = 64) accumulators per row keep the FMA chains short.
-template <int WF>
-__device__ __forceinline__ void pair_product(const cxf* blk, const cxf* z, int W, int lane, cxf& m0,
-                                             cxf& m1) {
-  const float4* g4 = reinterpret_cast<const float4*>(blk);
-  const float4* z4 = reinterpret_cast<const float4*>(z);
-  const int r0 = lane, r1 = lane + 32;
-  const bool v0 = r0 < W, v1 = WF > 32 && r1 < W;
-  constexpr int NA = WF <= 32 ? 8 : 4;
-  constexpr int NB = WF <= 32 ? WF / 8 : 1;        // batches unrolled (one at a time at WF = 64)
-  cxf a[NA], c[NA];
-#pragma unroll
-  for (int u = 0; u < NA; ++u) a[u] = c[u] = cxf{0.f, 0.f};
-  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll NB
-  for (int k0 = 0; k0 < WF / 2; k0 += 4) {
-    float4 zz[4], ga[4], gb[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      // pairs past W and rows past W read in-range entries (pair 0, row 0) and
-      // the z pair is zeroed, so they add nothing; such rows are not written
-      const int k = k0 + q;
-      const bool on = 2 * k < W;
-      const int kk = on ? k : 0;
-      zz[q] = on ? z4[kk] : zero;
-      ga[q] = g4[(size_t)kk * W + (v0 ? r0 : 0)];
-      if (WF > 32) gb[q] = g4[(size_t)kk * W + (v1 ? r1 : 0)];
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int u = (2 * q) & (NA - 1);
-      const cxf za = {zz[q].x, zz[q].y}, zb = {zz[q].z, zz[q].w};
-      a[u] = cfma(cxf{ga[q].x, ga[q].y}, za, a[u]);
-      a[u + 1] = cfma(cxf{ga[q].z, ga[q].w}, zb, a[u + 1]);
-      if (WF > 32) {
-        c[u] = cfma(cxf{gb[q].x, gb[q].y}, za, c[u]);
-        c[u + 1] = cfma(cxf{gb[q].z, gb[q].w}, zb, c[u + 1]);
-      }
-    }
-  }
-  if constexpr (NA == 8) {
-    m0 = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-    m1 = ((c[0] + c[1]) + (c[2] + c[3])) + ((c[4] + c[5]) + (c[6] + c[7]));
-  } else {
-    m0 = (a[0] + a[1]) + (a[2] + a[3]);
-    m1 = (c[0] + c[1]) + (c[2] + c[3]);
-  }
-}
-
-// complex64 sweep for W <= 64 on the two-sided factors (k_factor, mixed form),
-// with m = Lx / 2:
-//   left chain, warp 0:   y_s = g_s (rhs_s - t y_{s-1})        s = 0 .. m-1
-//   right chain, warp 1:  y_s = g_s (rhs_s - t y_{s+1})        s = Lx-1 .. m+1
-//   middle, warp 0:       x_m = G_mm (rhs_m - t y_{m-1} - t y_{m+1})
-//   back-substitution:    x_s = y_s - t g_s x_{s+1}  (warp 0, s = m-1 .. 0)
-//                         x_s = y_s - t g_s x_{s-1}  (warp 1, s = m+1 .. Lx-1)
-// so the dependent chain is ~Lx slices instead of 2 Lx - 1, and each slice
-// is one warp's work: in complex64 a W x W product is far cheaper than a CTA
-// barrier plus a cross-warp reduction, which is what a slice cost when eight
-// warps shared it.  Each chain streams its own blocks through its half of the
-// copy ring and its lane 0 refills a slot as soon as the warp has read it.
-// Rows of the right-hand side (forward) and of y (backward) are read two
-// slices ahead into registers, which hides the latency when the row buffer is
-// the global scratch.  The other warps join for the pre- and post-passes.
-template <int WF>
-__device__ void sweep_pair(const Geo& g, int i, const SweepArgs<float>& a, cxf* sm, Pipe& pp,
-                           unsigned long long* cnt) {
-  using C = cxf;
-  bool dead = *pp.err != 0;              // an earlier wait of this CTA ran out
-  const int W = g.W, Lx = g.Lx, m = Lx / 2, qR = Lx - 1 - m;
-  const int NLL = 2 * m + 1, NLR = 2 * qR;
-  C* zL = sm;                            // [2][W] left chain z
-  C* zR = sm + 2 * W;                    // [2][W] right chain z
-  C* zM = sm + 4 * W;                    // [2][W] partial middle z from the left / right chain
-  C* ring = reinterpret_cast<C*>(pp.ring);
-  C* yb = pp.ybuf ? reinterpret_cast<C*>(pp.ybuf) : a.y;   // [Lx][W] row buffer
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const float t = (float)g.t;
-  const int WW = W * W;
-  const uint32_t bytes = (uint32_t)(WW * sizeof(C));
-  const int SL = pp.S / 2, SR = pp.S - SL;
-  const int r0 = lane, r1 = lane + 32;
-  const bool v0 = r0 < W, v1 = WF > 32 && r1 < W;
-  auto sliceL = [&](int n) { return n <= m ? n : 2 * m - n; };
-  auto sliceR = [&](int n) { return n < qR ? Lx - 1 - n : m + 1 + (n - qR); };
-  // the chains consume their blocks in order: slot and phase parity advance
-  // by one step at a time (no division on the critical path); the block of
-  // step n + S_c reuses the slot of step n
-  int curL = (int)(pp.seq % (unsigned)SL), curR = SL + (int)(pp.seq2 % (unsigned)SR);
-  uint32_t phL = (pp.seq / (unsigned)SL) & 1u, phR = (pp.seq2 / (unsigned)SR) & 1u;
-  auto issue_at = [&](int slot, int slice) {
-    bulk_load(ring + (size_t)slot * WW, a.g + (size_t)slice * WW, bytes, pp.bar + slot);
-  };
-  // Wait for the block of step n, product with z, refill the slot.  The
-  // slot's loads have completed (their values are in p0, p1) before the warp
-  // barrier, so the copy that overwrites it needs no proxy fence.
-  auto stepL = [&](int n, const C* z, C& p0, C& p1) {
-    const int sl = curL;
-    ring_wait(pp.bar + sl, phL, dead, pp.err);
-    pair_product<WF>(ring + (size_t)sl * WW, z, W, lane, p0, p1);
-    __syncwarp();
-    if (lane == 0 && n + SL < NLL) issue_at(sl, sliceL(n + SL));
-    if (++curL == SL) {
-      curL = 0;
-      phL ^= 1u;
-    }
-  };
-  auto stepR = [&](int n, const C* z, C& p0, C& p1) {
-    const int sl = curR;
-    ring_wait(pp.bar + sl, phR, dead, pp.err);
-    pair_product<WF>(ring + (size_t)sl * WW, z, W, lane, p0, p1);
-    __syncwarp();
-    if (lane == 0 && n + SR < NLR) issue_at(sl, sliceR(n + SR));
-    if (++curR == SL + SR) {
-      curR = SL;
-      phR ^= 1u;
-    }
-  };
-  auto rd = [&](int s, int r) { return yb[(size_t)s * W + r]; };
-
-
-  __syncthreads();                       // previous users of ring, z buffers and yb are done
-  if (tid == 0) {
-    fence_proxy_async();
-    for (int n = 0; n < SL && n < NLL; ++n) issue_at((int)((pp.seq + n) % (unsigned)SL), sliceL(n));
-    for (int n = 0; n < SR && n < NLR; ++n) issue_at(SL + (int)((pp.seq2 + n) % (unsigned)SR), sliceR(n));
-  }
-  sweep_prepass<float>(g, i, a, yb);
-  __syncthreads();
-
-  // ---- forward chains
-  if (wid == 0) {
-    C fA0 = {0, 0}, fA1 = {0, 0}, fB0 = {0, 0}, fB1 = {0, 0};   // rhs_{s+1}, s even / odd
-    if (v0) zL[r0] = rd(0, r0);
-    if (v1) zL[r1] = rd(0, r1);
-    if (m >= 1) {
-      if (v0) fA0 = rd(1, r0);
-      if (v1) fA1 = rd(1, r1);
-    }
-    if (m >= 2) {
-      if (v0) fB0 = rd(2, r0);
-      if (v1) fB1 = rd(2, r1);
-    }
-    __syncwarp();
-    auto fwd = [&](int s, C& f0, C& f1) {
-      C y0, y1;
-      stepL(s, zL + (s & 1) * W, y0, y1);
-      C* zn = (s + 1 < m) ? zL + ((s + 1) & 1) * W : zM;   // z_{s+1}, or the middle partial
-      if (v0) {
-        yb[(size_t)s * W + r0] = y0;
-        zn[r0] = f0 - t * y0;
-        if (s + 3 <= m) f0 = rd(s + 3, r0);
-      }
-      if (v1) {
-        yb[(size_t)s * W + r1] = y1;
-        zn[r1] = f1 - t * y1;
-        if (s + 3 <= m) f1 = rd(s + 3, r1);
-      }
-      __syncwarp();
-    };
-    for (int s = 0; s < m; s += 2) {
-      fwd(s, fA0, fA1);
-      if (s + 1 < m) fwd(s + 1, fB0, fB1);
-    }
-    if (m == 0) {                        // no left chain: the middle starts from rhs_0
-      if (v0) zM[r0] = rd(0, r0);
-      if (v1) zM[r1] = rd(0, r1);
-    }
-  } else if (wid == 1 && qR > 0) {
-    C fA0 = {0, 0}, fA1 = {0, 0}, fB0 = {0, 0}, fB1 = {0, 0};   // rhs_{s-1}, step n even / odd
-    if (v0) zR[r0] = rd(Lx - 1, r0);
-    if (v1) zR[r1] = rd(Lx - 1, r1);
-    if (Lx - 2 > m) {
-      if (v0) fA0 = rd(Lx - 2, r0);
-      if (v1) fA1 = rd(Lx - 2, r1);
-    }
-    if (Lx - 3 > m) {
-      if (v0) fB0 = rd(Lx - 3, r0);
-      if (v1) fB1 = rd(Lx - 3, r1);
-    }
-    __syncwarp();
-    auto fwd = [&](int n, C& f0, C& f1) {
-      const int s = Lx - 1 - n;
-      C y0, y1;
-      stepR(n, zR + (n & 1) * W, y0, y1);
-      const bool inner = s - 1 > m;
-      C* zn = inner ? zR + ((n + 1) & 1) * W : zM + W;
-      if (v0) {
-        yb[(size_t)s * W + r0] = y0;
-        zn[r0] = inner ? f0 - t * y0 : -(t * y0);
-        if (s - 3 > m) f0 = rd(s - 3, r0);
-      }
-      if (v1) {
-        yb[(size_t)s * W + r1] = y1;
-        zn[r1] = inner ? f1 - t * y1 : -(t * y1);
-        if (s - 3 > m) f1 = rd(s - 3, r1);
-      }
-      __syncwarp();
-    };
-    for (int n = 0; n < qR; n += 2) {
-      fwd(n, fA0, fA1);
-      if (n + 1 < qR) fwd(n + 1, fB0, fB1);
-    }
-  }
-  __syncthreads();                       // both chains' partials of the middle z written
-
-  // ---- middle block
-  if (wid == 0) {
-    C* zc = zL + (m & 1) * W;
-    if (v0) zc[r0] = qR > 0 ? zM[r0] + zM[W + r0] : zM[r0];
-    if (v1) zc[r1] = qR > 0 ? zM[r1] + zM[W + r1] : zM[r1];
-    __syncwarp();
-    C x0, x1;
-    stepL(m, zc, x0, x1);
-    C* znL = zL + ((m + 1) & 1) * W;
-    C* znR = zR + (qR & 1) * W;
-    if (v0) {
-      yb[(size_t)m * W + r0] = x0;
-      znL[r0] = x0;
-      znR[r0] = x0;
-    }
-    if (v1) {
-      yb[(size_t)m * W + r1] = x1;
-      znL[r1] = x1;
-      znR[r1] = x1;
-    }
-  }
-  __syncthreads();                       // x_m visible to the right chain
-
-  // ---- back-substitution
-  if (wid == 0 && m > 0) {
-    C yA0 = {0, 0}, yA1 = {0, 0}, yB0 = {0, 0}, yB1 = {0, 0};   // y_s, step parity
-    if (v0) yA0 = rd(m - 1, r0);
-    if (v1) yA1 = rd(m - 1, r1);
-    if (m >= 2) {
-      if (v0) yB0 = rd(m - 2, r0);
-      if (v1) yB1 = rd(m - 2, r1);
-    }
-    auto bwd = [&](int n, C& y0v, C& y1v) {
-      const int s = 2 * m - n;
-      C p0, p1;
-      stepL(n, zL + (n & 1) * W, p0, p1);
-      C* zn = zL + ((n + 1) & 1) * W;
-      if (v0) {
-        const C xv = y0v - t * p0;
-        yb[(size_t)s * W + r0] = xv;
-        zn[r0] = xv;
-        if (s >= 2) y0v = rd(s - 2, r0);
-      }
-      if (v1) {
-        const C xv = y1v - t * p1;
-        yb[(size_t)s * W + r1] = xv;
-        zn[r1] = xv;
-        if (s >= 2) y1v = rd(s - 2, r1);
-      }
-      __syncwarp();
-    };
-    for (int n = m + 1; n < NLL; n += 2) {
-      bwd(n, yA0, yA1);
-      if (n + 1 < NLL) bwd(n + 1, yB0, yB1);
-    }
-  } else if (wid == 1 && qR > 0) {
-    C yA0 = {0, 0}, yA1 = {0, 0}, yB0 = {0, 0}, yB1 = {0, 0};
-    if (v0) yA0 = rd(m + 1, r0);
-    if (v1) yA1 = rd(m + 1, r1);
-    if (m + 2 < Lx) {
-      if (v0) yB0 = rd(m + 2, r0);
-      if (v1) yB1 = rd(m + 2, r1);
-    }
-    auto bwd = [&](int n, C& y0v, C& y1v) {
-      const int s = m + 1 + (n - qR);
-      C p0, p1;
-      stepR(n, zR + (n & 1) * W, p0, p1);
-      C* zn = zR + ((n + 1) & 1) * W;
-      if (v0) {
-        const C xv = y0v - t * p0;
-        yb[(size_t)s * W + r0] = xv;
-        zn[r0] = xv;
-        if (s + 2 < Lx) y0v = rd(s + 2, r0);
-      }
-      if (v1) {
-        const C xv = y1v - t * p1;
-        yb[(size_t)s * W + r1] = xv;
-        zn[r1] = xv;
-        if (s + 2 < Lx) y1v = rd(s + 2, r1);
-      }
-      __syncwarp();
-    };
-    for (int n = qR; n < NLR; n += 2) {
-      bwd(n, yA0, yA1);
-      if (n + 1 < NLR) bwd(n + 1, yB0, yB1);
-    }
-  }
-  __syncthreads();                       // yb complete for the post-pass
-  sweep_postpass<float>(g, i, a, yb);
-  pp.seq += NLL;
-  pp.seq2 += NLR;
-  if (tid == 0 && cnt) *cnt += 1;
-}
-
 // WF selects the sweep form at compile time, so each kernel carries only its
-// own: 0 = row-chunked (W > 64); otherwise W <= WF <= 64, the two-chain
-// single-warp form in complex64 and the 8-warp form in FP64.
+// own: 0 = row-chunked (W > 64, either precision); otherwise the 8-warp form of
+// the FP64 strips (W <= 64).  The mixed form's strips: xmatvec_mixed.cuh.
 template <typename R, int WF>
 __device__ void sweep(const Geo& g, int i, const SweepArgs<R>& a, cx<R>* sm, Pipe& pp,
                       unsigned long long* cnt) {
   if constexpr (WF == 0) {
     sweep_chunked<R>(g, i, a, sm, pp, cnt);
-    return;
-  } else if constexpr (sizeof(R) == 4) {
-    sweep_pair<WF>(g, i, a, sm, pp, cnt);
     return;
   }
   bool dead = *pp.err != 0;              // an earlier wait of this CTA ran out
@@ -822,7 +435,7 @@ template <typename R>
 __device__ void sweep_chunked(const Geo& g, int i, const SweepArgs<R>& a, cx<R>* sm, Pipe& pp,
                               unsigned long long* cnt) {
   bool dead = *pp.err != 0;              // an earlier wait of this CTA ran out
-  const int W = g.W, Lx = g.Lx, T = g.T, w = T * g.h[i];
+  const int W = g.W, Lx = g.Lx;
   const int CR = pp.CR, NC = W / CR;
   const SweepLayout L = sweep_layout(CR, W);
   cx<R>* zbuf = sm;
@@ -839,7 +452,6 @@ __device__ void sweep_chunked(const Geo& g, int i, const SweepArgs<R>& a, cx<R>*
   const uint32_t bytes = (uint32_t)(CW * sizeof(cx<R>));
   const int NL = 2 * Lx - 1, NQ = NL * NC;
   const int S = pp.S;
-  const int nrow = Lx * W;
   auto slice_of = [&](int n) { return n < Lx ? n : 2 * Lx - 2 - n; };
   auto issue = [&](int q) {
     const unsigned qq = pp.seq + q;
@@ -854,22 +466,7 @@ __device__ void sweep_chunked(const Geo& g, int i, const SweepArgs<R>& a, cx<R>*
     fence_proxy_async();
     for (int q = 0; q < S && q < NQ; ++q) issue(q);
   }
-  for (int e = tid; e < nrow; e += (int)blockDim.x) {
-    const int s = e / W, j = e - s * W;
-    cxd v = {0, 0};
-    if (j < w) {
-      if (a.src) {
-        v = a.in_scale * a.src[e];
-      } else {
-        cx<R> u = {0, 0};
-        if (a.lay_lo && j < T) u = u + t * a.lay_lo[s + Lx * j];
-        if (a.lay_hi && j >= w - T) u = u + t * a.lay_hi[s + Lx * (j - (w - T))];
-        yb[e] = u;
-        continue;
-      }
-    }
-    yb[e] = cconv<R>(v);
-  }
+  sweep_prepass<R>(g, i, a, yb);
   __syncthreads();
   for (int e = tid; e < W; e += (int)blockDim.x) zbuf[e] = yb[e];
   __syncthreads();
@@ -917,21 +514,7 @@ __device__ void sweep_chunked(const Geo& g, int i, const SweepArgs<R>& a, cx<R>*
       }
     }
   }
-  for (int e = tid; e < nrow; e += (int)blockDim.x) {
-    const int s = e / W, j = e - s * W;
-    if (j >= w) continue;
-    const cx<R> xr = yb[e];
-    if (a.dst) {
-      const cxd xd = a.out_scale * cconv<double>(xr);
-      cxd* d = a.dst + e;
-      if (a.dst_op == 0) *d = xd;
-      else if (a.dst_op == 1) *d = *d + xd;
-      else if (a.dst_op == 2) *d = *d - xd;
-      else *d = -xd;
-    }
-    if (a.bnd_lo && j < T) a.bnd_lo[s + Lx * j] = xr;
-    if (a.bnd_hi && j >= w - T) a.bnd_hi[s + Lx * (j - (w - T))] = xr;
-  }
+  sweep_postpass<R>(g, i, a, yb);
   pp.seq += NQ;
   if (tid == 0 && cnt) *cnt += 1;
 }
@@ -1468,37 +1051,27 @@ __device__ int solve_H(cg::cluster_group& cl, RedSmem& rs, int& phase, const Geo
 constexpr size_t YBUF_MAX = 64 * 1024;   // forward intermediates kept on chip up to this size
 
 // Shared-memory plan of a sweep: ring of S slots of CR x W entries (CR = W when
-// a whole slice block fits a slot, the W <= 64 strips; row chunks otherwise),
-// zw entries of z vectors (2 W; 6 W for the two-chain complex64 form, whose
-// ring is split evenly between its chains), and the on-chip row buffer when
-// it fits.  per_sm is the number of CTAs per SM the budget is shared by: 2
-// (256 threads, ~100 KB each) or, for the complex64 two-chain form, 4 (128
-// threads, ~52 KB each, the row buffer on chip only up to 16 KB).
+// a whole slice block fits a slot, the W <= 64 strips of the FP64 form; row
+// chunks otherwise), zw entries of z vectors, and the on-chip row buffer when
+// it fits.  W <= 64: 256 threads at two CTAs per SM, ~100 KB each.
 struct RingPlan {
   int CR, S, zw;
   size_t ybuf, smem;
 };
-constexpr size_t CTA4_BUDGET = 52 * 1024;   // dynamic shared memory per CTA at four CTAs per SM
-constexpr size_t CTA4_YBUF_MAX = 16 * 1024;
 template <typename R>
-__host__ __device__ inline RingPlan ring_plan(int W, int Lx, int per_sm = 2) {
+__host__ __device__ inline RingPlan ring_plan(int W, int Lx) {
   RingPlan rp;
   const size_t cs = sizeof(cx<R>);
   const size_t yb = (size_t)Lx * W * cs;
+  rp.zw = 2 * W;
   if (W <= DY_MAXW_SMEM) {
-    const bool pair = sizeof(R) == 4;
-    const bool four = pair && per_sm == 4;
-    rp.zw = pair ? 6 * W : 2 * W;
-    rp.ybuf = yb <= (four ? CTA4_YBUF_MAX : YBUF_MAX) ? yb : 0;
+    rp.ybuf = yb <= YBUF_MAX ? yb : 0;
     rp.CR = W;
-    const long budget = four ? (long)CTA4_BUDGET : (long)100 * 1024;
-    long S = (budget - (long)rp.ybuf - (long)(rp.zw * cs)) / (long)(W * W * cs);
+    long S = ((long)100 * 1024 - (long)rp.ybuf - (long)(rp.zw * cs)) / (long)(W * W * cs);
     if (S > MAX_STAGES) S = MAX_STAGES;
     if (S < 2) S = 2;
-    if (pair) S &= ~1L;
     rp.S = (int)S;
   } else {
-    rp.zw = 2 * W;
     rp.ybuf = yb;                                                       // one CTA per SM
     const long budget = (long)200 * 1024 - (long)yb - (long)(2 * W * cs);
     // largest divisor of W whose chunks leave >= 4 ring slots (>= 2 as a last
@@ -1520,18 +1093,12 @@ __host__ __device__ inline RingPlan ring_plan(int W, int Lx, int per_sm = 2) {
   rp.smem = rp.CR ? (size_t)rp.S * rp.CR * W * cs + (size_t)rp.zw * cs + rp.ybuf : 0;
   return rp;
 }
-// threads per CTA of the X-matvec of a geometry in precision R: 128 (four CTAs
-// per SM) for the complex64 two-chain form when the plan chose it, else 256
-template <typename R>
-__host__ __device__ inline int xm_threads(const Geo& g) {
-  return (sizeof(R) == 4 && g.W <= DY_MAXW_SMEM && g.xm_nt == 128) ? 128 : 256;
-}
 // The plan of a geometry: the heuristic above, or the autotuner's choice of
 // slots (and chunk rows for W > 64) with the same row buffer and z area.
-constexpr size_t SMEM_LIMIT = 225 * 1024;   // dynamic shared memory per CTA, below the 227 KB cap
+constexpr size_t SMEM_LIMIT = 223 * 1024;   // dynamic shared memory per CTA, below the 227 KB cap (static: ~3 KB)
 template <typename R>
 __host__ __device__ inline RingPlan ring_plan(const Geo& g) {
-  RingPlan rp = ring_plan<R>(g.W, g.Lx, xm_threads<R>(g) == 128 ? 4 : 2);
+  RingPlan rp = ring_plan<R>(g.W, g.Lx);
   if (g.ring_S > 0 && rp.CR > 0) {
     rp.S = g.ring_S;
     if (g.W > DY_MAXW_SMEM && g.ring_CR > 0) rp.CR = g.ring_CR;
@@ -1540,51 +1107,39 @@ __host__ __device__ inline RingPlan ring_plan(const Geo& g) {
   return rp;
 }
 // Configurations the autotuner times: the heuristic's first, then every slot
-// count 2..MAX_STAGES (even in the two-chain complex64 form) that fits, and
-// for W > 64 the chunk heights (divisors of W) with the most slots that fit;
-// the complex64 two-chain form adds the same slot counts at 128 threads per
-// CTA (four CTAs per SM).  NT[] receives each configuration's threads per CTA.
+// count 2..MAX_STAGES that fits, and for W > 64 the chunk heights (divisors of
+// W) with the most slots that fit.
 template <typename R>
-inline int ring_candidates(const Geo& g, int* S, int* CR, int* NT, int max) {
-  const int nt0 = xm_threads<R>(g);
-  const RingPlan h = ring_plan<R>(g.W, g.Lx, nt0 == 128 ? 4 : 2);
+inline int ring_candidates(const Geo& g, int* S, int* CR, int max) {
+  const RingPlan h = ring_plan<R>(g.W, g.Lx);
   if (h.CR == 0 || max < 1) return 0;
   int n = 0;
   S[n] = h.S;
   CR[n] = h.CR;
-  NT[n] = nt0;
   ++n;
-  const size_t cs = sizeof(cx<R>);
-  auto fits = [&](int s, int cr, int nt) {
-    const RingPlan b = ring_plan<R>(g.W, g.Lx, nt == 128 ? 4 : 2);
-    const size_t fixed = (size_t)b.zw * cs + b.ybuf;
-    return (size_t)s * cr * g.W * cs + fixed <= (nt == 128 ? CTA4_BUDGET : SMEM_LIMIT);
-  };
-  auto add = [&](int s, int cr, int nt) {
+  const size_t cs = sizeof(cx<R>), fixed = (size_t)h.zw * cs + h.ybuf;
+  auto fits = [&](int s, int cr) { return (size_t)s * cr * g.W * cs + fixed <= SMEM_LIMIT; };
+  auto add = [&](int s, int cr) {
     for (int k = 0; k < n; ++k)
-      if (S[k] == s && CR[k] == cr && NT[k] == nt) return;
-    if (n < max && fits(s, cr, nt)) {
+      if (S[k] == s && CR[k] == cr) return;
+    if (n < max && fits(s, cr)) {
       S[n] = s;
       CR[n] = cr;
-      NT[n] = nt;
       ++n;
     }
   };
   if (g.W <= DY_MAXW_SMEM) {
-    const int step = sizeof(R) == 4 ? 2 : 1;        // two chains split the ring evenly
-    for (int s = 2; s <= MAX_STAGES; s += step) add(s, g.W, 256);
-    if (sizeof(R) == 4)
-      for (int s = 2; s <= MAX_STAGES; s += step) add(s, g.W, 128);
+    for (int s = 2; s <= MAX_STAGES; ++s) add(s, g.W);
   } else {
     for (int cr = g.W; cr >= 1; --cr) {
       if (g.W % cr) continue;
       int best = 0;
       for (int s = MAX_STAGES; s >= 2; --s)
-        if (fits(s, cr, 256)) {
+        if (fits(s, cr)) {
           best = s;
           break;
         }
-      if (best >= 3) add(best, cr, 256);
+      if (best >= 3) add(best, cr);
       if (n >= max) break;
     }
   }
@@ -1599,8 +1154,8 @@ inline int ring_candidates(const Geo& g, int* S, int* CR, int* NT, int max) {
 //   mixed = 1: sweeps in complex64 (R = float).  w_B is refined against FP64
 //              residuals of B, u against FP64 residuals of H, each until the
 //              relative residual is below refine_tol.
-template <typename R, int WF, int NT>
-__global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2) k_xmatvec(Geo g, Bufs b, int j, int mixed, int ncols) {
+template <typename R, int WF>
+__global__ void __launch_bounds__(DY_THREADS, 2) k_xmatvec(Geo g, Bufs b, int j, int mixed, int ncols) {
   cg::cluster_group cl = cg::this_cluster();
   __shared__ RedSmem rs;
   __shared__ __align__(8) uint64_t bars[MAX_STAGES];
@@ -1619,7 +1174,6 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2) k_xmatvec(Geo g, Bufs b
   pp.CR = rp.CR;
   pp.ring = smem_raw;
   pp.seq = 0;
-  pp.seq2 = 0;
   pp.err = &err;
   pipe_init(pp);
   cx<R>* sm = reinterpret_cast<cx<R>*>(smem_raw + (size_t)rp.S * rp.CR * g.W * sizeof(cx<R>));
@@ -1797,7 +1351,6 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_bsolve(Geo g, Bufs b, const c
   pp.CR = rp.CR;
   pp.ring = smem_raw;
   pp.seq = 0;
-  pp.seq2 = 0;
   pp.err = &err;
   pipe_init(pp);
   cx<R>* sm = reinterpret_cast<cx<R>*>(smem_raw + (size_t)rp.S * rp.CR * g.W * sizeof(cx<R>));
@@ -1845,16 +1398,6 @@ cudaError_t launch_cluster(Kern kern, dim3 grid, int cx_, size_t smem, cudaStrea
 
 template <typename R>
 size_t sweep_smem(const Geo& g) { return ring_plan<R>(g).smem; }
-// the WF of the kernels for this geometry: every slice wider than 64 takes the
-// streamed form (CR may equal W there); the complex64 two-chain form is
-// compiled for W <= 16, 32 and 64 (fully unrolled block products); the FP64
-// 8-warp form needs no width class
-template <typename R>
-int sweep_form(const Geo& g) {
-  if (g.W > DY_MAXW_SMEM) return 0;
-  if (sizeof(R) == 8) return 64;
-  return g.W <= 16 ? 16 : (g.W <= 32 ? 32 : 64);
-}
 
 }  // namespace
 
@@ -1870,11 +1413,8 @@ cudaError_t run_bsolve(const Geo& g, const Bufs& b, int K, const cxd* q_dd, cxd*
   template <>                                                                                     \
   cudaError_t run_xmatvec<R, WF>(const Geo& g, const Bufs& b, int K, int j, int mixed, int ncols, \
                                  cudaStream_t st) {                                               \
-    if (sizeof(R) == 4 && xm_threads<R>(g) == 128)                                                \
-      return launch_cluster_nt(k_xmatvec<R, WF, (sizeof(R) == 4 ? 128 : 256)>, dim3(g.p, K * g.nb), \
-                               g.p, 128, sweep_smem<R>(g), st, g, b, j, mixed, ncols);           \
-    return launch_cluster_nt(k_xmatvec<R, WF, 256>, dim3(g.p, K * g.nb), g.p, 256,                \
-                             sweep_smem<R>(g), st, g, b, j, mixed, ncols);                        \
+    return launch_cluster(k_xmatvec<R, WF>, dim3(g.p, K * g.nb), g.p, sweep_smem<R>(g), st, g, b, j, mixed, \
+                          ncols);                                                                 \
   }                                                                                               \
   template <>                                                                                     \
   cudaError_t run_bsolve<R, WF>(const Geo& g, const Bufs& b, int K, const cxd* q_dd, cxd* w_dd,   \

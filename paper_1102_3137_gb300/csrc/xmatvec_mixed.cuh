@@ -1,0 +1,1071 @@
+// Mixed-form X-matvec for slices of up to 64 sites (W <= 64): complex64 block
+// sweeps on the two-sided factors, refined against double-float residuals.
+//
+// One cluster per (frequency, block column), one CTA per subdomain, as in
+// solve_device.cuh.  What is special here:
+//
+// 1. The sweep.  Each of the two chains of a subdomain (left to the middle
+//    slice, right to the middle slice, and back) is run by WF / 8 warps.  Four
+//    lanes share a row: lane (cg = lane / 8, rr = lane % 8) of warp w holds the
+//    column pairs cg, cg + 4, ... of row 8 w + rr, so a 32 x 32 block product is
+//    4 16-byte loads and 32 FMAs a lane plus two shuffles, and one barrier of
+//    the chain's warps a slice.  The block of the next step is read into
+//    registers before that barrier, which also frees its ring slot.  A producer
+//    warp per chain takes part in the same barrier: it waits for the copies (the
+//    chain's warps never touch an mbarrier) and refills the freed slots, and the
+//    copies run on from one sweep into the next, as every sweep reads the same
+//    sequence of blocks.
+// 2. Two right-hand sides in one sweep (NR = 2): the refinement's subdomain
+//    residual of w and that of u go through the factors together.
+// 3. No closing sweep: the interface solve's last product B^-1 E p is still in
+//    the row buffer when its step length alpha is known, and u_B is the sum of
+//    alpha B^-1 E p over the iterations, so B^-1 E y needs no sweep of its own.
+// 4. Residuals in double-float arithmetic: w and u are held as double-floats
+//    (47 bits; 16 bytes a complex entry like binary64) until the last pass
+//    widens u.  The part issues 2 binary64 operations per clock and SM, so the
+//    ~28 of a site's two binary64 residuals took ~14 clocks; ~280 binary32 ones
+//    take ~2.
+#pragma once
+#include "solve_device.cuh"
+
+namespace {
+
+constexpr int MIX_MAXS = 8;              // most ring slots of one chain
+constexpr size_t MIX_SMEM_2 = 112 * 1024;   // dynamic shared memory per CTA at two CTAs per SM
+constexpr size_t MIX_SMEM_1 = 226 * 1024;   // and at one
+
+template <int WF>
+struct Mix {
+  static constexpr int WARPS = WF / 8;   // compute warps of one chain
+  static constexpr int CT = 32 * WARPS;
+  static constexpr int KP = WF / 8;      // column pairs a lane holds
+  static constexpr int PROD = 2 * WARPS; // first of the two producer warps
+  static constexpr int NT = WF == 16 ? 256 : 32 * (2 * WARPS + 2);   // 256, 320, 576
+  static constexpr int PER_SM = WF <= 32 ? 2 : 1;
+};
+__host__ __device__ inline int mix_threads(int W) { return W <= 16 ? Mix<16>::NT : (W <= 32 ? Mix<32>::NT : Mix<64>::NT); }
+
+// Everything but the ring and the rows, at the start of the dynamic shared memory.
+template <int WF>
+struct MixSmem {
+  alignas(16) cxf z[2][2][2][WF];        // [chain][right-hand side][parity]: z of the current and next slice
+  alignas(16) cxf zm[2][2][WF];          // [chain][right-hand side]: the chain's part of the middle z
+  float wred[24 * 8];                    // per-warp partial sums
+  float slot[2][DY_MAXP * 8];            // [phase][rank]: the cluster's partial sums
+  alignas(8) uint64_t bars[2 * MIX_MAXS];
+  int err;
+};
+__host__ __device__ constexpr size_t mix_head(int W) {
+  return ((W <= 16 ? sizeof(MixSmem<16>) : (W <= 32 ? sizeof(MixSmem<32>) : sizeof(MixSmem<64>))) + 127) & ~(size_t)127;
+}
+
+// Shared-memory plan: S ring slots of one block for each chain, and both row
+// buffers on chip or in the plan's scratch.  g.ring_S (slots of both chains)
+// and g.xm_rows come from the autotuner; 0: the heuristic, which keeps the
+// rows on chip when four slots a chain fit beside them.
+struct MixPlan {
+  int S, rows;
+  size_t smem;
+};
+__host__ __device__ inline size_t mix_smem(int W, int Lx, int S, int rows) {
+  return mix_head(W) + ((size_t)2 * S * W * W + (rows ? 2 * (size_t)Lx * W : 0)) * sizeof(cxf);
+}
+__host__ __device__ inline MixPlan mix_plan(const Geo& g) {
+  MixPlan m;
+  if (g.ring_S > 0) {
+    m.S = g.ring_S / 2;
+    m.rows = g.xm_rows > 0 ? 1 : 0;
+  } else {
+    const size_t lim = g.W <= 32 ? MIX_SMEM_2 : MIX_SMEM_1;
+    m.rows = mix_smem(g.W, g.Lx, 4, 1) <= lim ? 1 : 0;
+    m.S = 4;
+    while (m.S > 2 && mix_smem(g.W, g.Lx, m.S, m.rows) > lim) --m.S;
+  }
+  m.smem = mix_smem(g.W, g.Lx, m.S, m.rows);
+  return m;
+}
+// Configurations the autotuner times: slots a chain, rows on chip or not.
+inline int mix_candidates(const Geo& g, int* S, int* CR, int* ROWS, int max) {
+  Geo h = g;
+  h.ring_S = 0;
+  const MixPlan d = mix_plan(h);
+  int n = 0;
+  auto add = [&](int s, int rows) {
+    for (int k = 0; k < n; ++k)
+      if (S[k] == 2 * s && ROWS[k] == rows) return;
+    if (n < max && mix_smem(g.W, g.Lx, s, rows) <= MIX_SMEM_1) {
+      S[n] = 2 * s;
+      CR[n] = g.W;
+      ROWS[n] = rows;
+      ++n;
+    }
+  };
+  add(d.S, d.rows);
+  for (int rows = 1; rows >= 0; --rows)
+    for (int s : {2, 3, 4, 6}) add(s, rows);
+  return n;
+}
+
+// The dynamic shared memory, named here so that every function (inlined or
+// not) addresses it as shared memory and not through generic pointers.
+extern __shared__ __align__(128) unsigned char mix_raw[];
+template <int WF>
+__device__ __forceinline__ MixSmem<WF>& mix_sm() {
+  return *reinterpret_cast<MixSmem<WF>*>(mix_raw);
+}
+template <int WF>
+__device__ __forceinline__ cxf* mix_ring() {
+  constexpr size_t head = (sizeof(MixSmem<WF>) + 127) & ~(size_t)127;
+  return reinterpret_cast<cxf*>(mix_raw + head);
+}
+
+__device__ __forceinline__ void named_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// What a thread keeps from sweep to sweep (compute warps: slot; producers: all).
+struct MixState {
+  int slot;                              // compute: slot of the next block to read; producer: next slot to fill
+  int pos;                               // producer: position of the next block to copy in the sweep's sequence
+  int wslot;                             // producer: slot of the next block to wait for
+  uint32_t wph;
+  bool dead;
+};
+
+// One CTA's constants and buffers.
+template <int WF, bool ROWS>
+struct MixCtx {
+  int W, Lx, S, m;
+  const cxf* src;                        // the subdomain's factors
+  cxf *g0, *g1;                          // row buffers in the scratch (ROWS = false)
+  unsigned long long* cnt;
+  float t;
+
+  __device__ __forceinline__ cxf* row(int k) const {
+    if constexpr (ROWS) return mix_ring<WF>() + 2 * S * W * W + (k ? Lx * W : 0);
+    else return k ? g1 : g0;
+  }
+  __device__ __forceinline__ int blocks(int chain) const { return chain == 0 ? 2 * m + 1 : 2 * (Lx - 1 - m); }
+  __device__ __forceinline__ int slice_at(int chain, int n) const {
+    if (chain == 0) return n <= m ? n : 2 * m - n;
+    const int qR = Lx - 1 - m;
+    return n < qR ? Lx - 1 - n : m + 1 + (n - qR);
+  }
+  __device__ __forceinline__ void issue(int chain, MixState& st) const {
+    MixSmem<WF>& sm = mix_sm<WF>();
+    bulk_load(mix_ring<WF>() + (chain * S + st.slot) * W * W, src + (size_t)slice_at(chain, st.pos) * W * W,
+              (uint32_t)(W * W * sizeof(cxf)), sm.bars + chain * MIX_MAXS + st.slot);
+    if (++st.slot == S) st.slot = 0;
+    if (++st.pos == blocks(chain)) st.pos = 0;
+  }
+  __device__ __forceinline__ void wait(int chain, MixState& st) const {
+    MixSmem<WF>& sm = mix_sm<WF>();
+    ring_wait(sm.bars + chain * MIX_MAXS + st.wslot, st.wph, st.dead, &sm.err);
+    if (++st.wslot == S) {
+      st.wslot = 0;
+      st.wph ^= 1u;
+    }
+  }
+};
+
+template <int WF, bool ROWS>
+__device__ void mix_init(const MixCtx<WF, ROWS>& cx, MixState& st) {
+  MixSmem<WF>& sm = mix_sm<WF>();
+  const int tid = threadIdx.x, wid = tid >> 5;
+  st.slot = st.pos = st.wslot = 0;
+  st.wph = 0;
+  st.dead = false;
+  for (int e = tid; e < 8 * WF; e += Mix<WF>::NT) (&sm.z[0][0][0][0])[e] = cxf{0.f, 0.f};
+  for (int e = tid; e < 4 * WF; e += Mix<WF>::NT) (&sm.zm[0][0][0])[e] = cxf{0.f, 0.f};
+  if (tid == 0) {
+    for (int k = 0; k < 2 * MIX_MAXS; ++k) mbar_init(sm.bars + k, 1);
+    sm.err = 0;
+    fence_mbar_init();
+  }
+  __syncthreads();
+  const int c = wid - Mix<WF>::PROD;
+  if ((c == 0 || c == 1) && (tid & 31) == 0 && cx.blocks(c) > 0)
+    for (int k = 0; k < cx.S; ++k) cx.issue(c, st);
+}
+// Before the kernel ends: the S copies of each chain issued beyond its last
+// step have landed (bounded waits, also after an earlier wait ran out; the
+// first that runs out ends it).
+template <int WF, bool ROWS>
+__device__ void mix_drain(const MixCtx<WF, ROWS>& cx, MixState& st) {
+  const int c = ((int)threadIdx.x >> 5) - Mix<WF>::PROD;
+  if ((c == 0 || c == 1) && (threadIdx.x & 31) == 0 && cx.blocks(c) > 0)
+    for (int k = 0; k < cx.S; ++k) {
+      if (!mbar_wait(mix_sm<WF>().bars + c * MIX_MAXS + st.wslot, st.wph)) {
+        mix_sm<WF>().err = 1;
+        break;
+      }
+      if (++st.wslot == cx.S) {
+        st.wslot = 0;
+        st.wph ^= 1u;
+      }
+    }
+}
+
+// B_i x = rhs for NR right-hand sides in place in the row buffers [Lx][W]
+// (complex64; padding columns zero; NR = 1: buffer k0; NR = 2: both), with
+// m = Lx / 2, qR = Lx - 1 - m:
+//   left   y_s = g_s (rhs_s - t y_{s-1})        s = 0 .. m-1
+//   right  y_s = g_s (rhs_s - t y_{s+1})        s = Lx-1 .. m+1
+//   middle x_m = G_mm (rhs_m - t y_{m-1} - t y_{m+1})        (left chain's warps)
+//   back   x_s = y_s - t g_s x_{s+1} (left, s = m-1 .. 0),  x_s = y_s - t g_s x_{s-1} (right)
+// Block n of a chain's sequence is in registers when its step begins; step n
+// reads block n + 1 after its products.  The producer has waited for block
+// n + 2 when it joins the barrier of step n, and refills block n + 1's slot
+// after it (block 0's after the first barrier, which starts the chain), so the
+// block it waits for is always in flight with two slots or more.  Rows are read PF slices ahead into registers (the latency of a row
+// buffer in the scratch), and a step's row is stored during the next step,
+// behind that step's loads of z.  Every warp of the CTA calls it; the rows are
+// complete and visible to the CTA on return.
+template <int WF, int NR, bool ROWS>
+__device__ __noinline__ void mix_sweep(const MixCtx<WF, ROWS>& ctx, MixState& state, int k0) {
+  constexpr int CT = Mix<WF>::CT, PF = NR == 1 ? 4 : 2, KP = Mix<WF>::KP, WARPS = Mix<WF>::WARPS;
+  constexpr int KH = KP < 4 ? KP : 4;    // column pairs handled at a time
+  MixSmem<WF>& sm = mix_sm<WF>();
+  const MixCtx<WF, ROWS> cx = ctx;
+  MixState st = state;
+  const int W = cx.W, Lx = cx.Lx, m = cx.m, qR = Lx - 1 - m;
+  const int wid = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+  const int role = wid < 2 * WARPS ? 0 : (wid < 2 * WARPS + 2 ? 1 : 2);
+  const int c = role == 0 ? wid / WARPS : (role == 1 ? wid - Mix<WF>::PROD : 0);
+  const int NL = cx.blocks(c), steps = c == 0 ? m : qR;
+  const float t = cx.t;
+  const int cg = lane >> 3, row = (wid % WARPS) * 8 + (lane & 7);
+  const bool own = role == 0 && cg == 0 && row < W;
+  const int off0 = cg * W + (row < W ? row : 0), W4 = 4 * W, WW2 = W * W / 2;
+  const int km = W / 2 > cg ? (W / 2 - cg + 3) / 4 : 0;
+  const float4* ring4 = reinterpret_cast<const float4*>(mix_ring<WF>()) + (size_t)c * cx.S * WW2 + off0;
+  cxf* yb[2] = {cx.row(NR == 1 ? k0 : 0), cx.row(1)};
+  float4 gb[KP];
+  auto load = [&]() {
+    const float4* p = ring4 + st.slot * WW2;
+#pragma unroll
+    for (int q = 0; q < KP; ++q) gb[q] = q < km ? p[q * W4] : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (++st.slot == cx.S) st.slot = 0;
+  };
+  auto load_z = [&](const cxf* z, int h, float4 (&zv)[KH]) {
+    const float4* z4 = reinterpret_cast<const float4*>(z) + cg + 16 * h;
+#pragma unroll
+    for (int q = 0; q < KH; ++q) zv[q] = z4[4 * q];
+  };
+  // this lane's part of (block row) . z, the first KH pairs of z already in zv
+  auto part = [&](const cxf* z, float4 (&zv)[KH]) -> cxf {
+    constexpr int NA = KP >= 4 ? 4 : 2;
+    cxf a[NA];
+#pragma unroll
+    for (int q = 0; q < NA; ++q) a[q] = cxf{0.f, 0.f};
+#pragma unroll
+    for (int h = 0; h < KP / KH; ++h) {
+      if (h > 0) load_z(z, h, zv);
+#pragma unroll
+      for (int q = 0; q < KH; ++q) {
+        const float4 gv = gb[h * KH + q];
+        a[(2 * q) % NA] = cfma(cxf{gv.x, gv.y}, cxf{zv[q].x, zv[q].y}, a[(2 * q) % NA]);
+        a[(2 * q + 1) % NA] = cfma(cxf{gv.z, gv.w}, cxf{zv[q].z, zv[q].w}, a[(2 * q + 1) % NA]);
+      }
+    }
+    cxf s = a[0] + a[1];
+    if constexpr (NA == 4) s = s + (a[2] + a[3]);
+    return s;
+  };
+  auto total = [&](cxf v) -> cxf {                       // over the row's four lanes
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, 8);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, 8);
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, 16);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, 16);
+    return v;
+  };
+  if (role == 1 && lane == 0) {
+    if (NL > 0) cx.wait(c, st);          // blocks 0 and 1
+    if (NL > 1) cx.wait(c, st);
+  }
+  __syncthreads();                       // the rows are written; earlier readers of z are done
+  if (role == 0) {
+    if (own) {
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        if (steps > 0) sm.z[c][r][0][row] = yb[r][(c == 0 ? 0 : Lx - 1) * W + row];
+        else sm.zm[c][r][row] = c == 0 ? yb[r][row] : cxf{0.f, 0.f};
+      }
+    }
+    if (NL > 0) load();
+    named_sync(3 + c, CT + 32);
+    // ---- towards the middle: step n is slice s0 + d n, its z needs row s0 + d (n + 1) next
+    const int d = c == 0 ? W : -W;       // row step
+    int o = (c == 0 ? 0 : (Lx - 1) * W) + row;           // this step's row entry
+    const int nf = c == 0 ? steps : steps - 1;           // steps whose next z has a right-hand side
+    cxf f[NR][PF], yp[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      yp[r] = cxf{0.f, 0.f};
+#pragma unroll
+      for (int u = 0; u < PF; ++u) f[r][u] = own && u < nf ? yb[r][o + d * (u + 1)] : cxf{0.f, 0.f};
+    }
+    for (int n0 = 0; n0 < steps; n0 += PF) {
+#pragma unroll
+      for (int u = 0; u < PF; ++u) {
+        const int n = n0 + u;
+        if (n < steps) {
+          cxf y[NR];
+          float4 zv[KH];
+          load_z(sm.z[c][0][u & 1], 0, zv);
+          if (own && n > 0) {            // row n - 1 out, its slot of f refilled
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+              yb[r][o - d] = yp[r];
+              f[r][(u + PF - 1) % PF] = n - 1 + PF < nf ? yb[r][o + d * PF] : cxf{0.f, 0.f};
+            }
+          }
+          y[0] = part(sm.z[c][0][u & 1], zv);
+          if constexpr (NR == 2) {
+            load_z(sm.z[c][1][u & 1], 0, zv);
+            y[1] = part(sm.z[c][1][u & 1], zv);
+          }
+          if (n + 1 < NL) load();
+#pragma unroll
+          for (int r = 0; r < NR; ++r) {
+            y[r] = total(y[r]);
+            if (own) {
+              cxf* zn = n + 1 < steps ? sm.z[c][r][(u + 1) & 1] : sm.zm[c][r];
+              zn[row] = f[r][u] - t * y[r];
+            }
+            yp[r] = y[r];
+          }
+          o += d;
+          named_sync(1 + c, CT + 32);
+        }
+      }
+    }
+    if (own && steps > 0) {
+#pragma unroll
+      for (int r = 0; r < NR; ++r) yb[r][o - d] = yp[r];
+    }
+  } else if (role == 1) {
+    named_sync(3 + c, CT + 32);          // block 0 has been read
+    if (lane == 0 && NL > 0) cx.issue(c, st);
+    for (int n = 0; n < steps; ++n) {
+      if (lane == 0 && n + 2 < NL) cx.wait(c, st);
+      __syncwarp();
+      named_sync(1 + c, CT + 32);        // block n + 1 has been read
+      if (lane == 0 && n + 1 < NL) cx.issue(c, st);
+    }
+  }
+  __syncthreads();                       // both parts of the middle z are written
+  if (c == 0 && role == 0) {
+    if (own) {
+#pragma unroll
+      for (int r = 0; r < NR; ++r) sm.z[0][r][1][row] = sm.zm[0][r][row] + sm.zm[1][r][row];
+    }
+    named_sync(3, CT);
+    cxf x[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      float4 zv[KH];
+      load_z(sm.z[0][r][1], 0, zv);
+      x[r] = part(sm.z[0][r][1], zv);
+    }
+    if (m + 1 < NL) load();
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      x[r] = total(x[r]);
+      if (own) {
+        yb[r][m * W + row] = x[r];
+        sm.z[0][r][0][row] = x[r];       // the first z of both ways back is z buffer 0
+        sm.z[1][r][0][row] = x[r];
+      }
+    }
+  } else if (c == 0 && role == 1 && lane == 0 && m + 2 < NL) {
+    cx.wait(c, st);
+  }
+  __syncthreads();                       // x_m is visible to both chains
+  if (c == 0 && role == 1 && lane == 0 && m + 1 < NL) cx.issue(c, st);
+  const int n1 = c == 0 ? m + 1 : qR;
+  if (role == 0) {
+    // ---- back from the middle: step k is slice m -+ (k + 1)
+    const int d = c == 0 ? -W : W;
+    int o = (c == 0 ? m - 1 : m + 1) * W + row;
+    cxf f[NR][PF], xp[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      xp[r] = cxf{0.f, 0.f};
+#pragma unroll
+      for (int u = 0; u < PF; ++u) f[r][u] = own && u < steps ? yb[r][o + d * u] : cxf{0.f, 0.f};
+    }
+    for (int kb = 0; kb < steps; kb += PF) {
+#pragma unroll
+      for (int u = 0; u < PF; ++u) {
+        const int k = kb + u;
+        if (k < steps) {
+          cxf y[NR];
+          float4 zv[KH];
+          load_z(sm.z[c][0][u & 1], 0, zv);
+          if (own && k > 0) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+              yb[r][o - d] = xp[r];
+              f[r][(u + PF - 1) % PF] = k - 1 + PF < steps ? yb[r][o + d * (PF - 1)] : cxf{0.f, 0.f};
+            }
+          }
+          y[0] = part(sm.z[c][0][u & 1], zv);
+          if constexpr (NR == 2) {
+            load_z(sm.z[c][1][u & 1], 0, zv);
+            y[1] = part(sm.z[c][1][u & 1], zv);
+          }
+          if (n1 + k + 1 < NL) load();
+#pragma unroll
+          for (int r = 0; r < NR; ++r) {
+            y[r] = total(y[r]);
+            xp[r] = f[r][u] - t * y[r];
+            if (own) sm.z[c][r][(u + 1) & 1][row] = xp[r];
+          }
+          o += d;
+          named_sync(1 + c, CT + 32);
+        }
+      }
+    }
+    if (own && steps > 0) {
+#pragma unroll
+      for (int r = 0; r < NR; ++r) yb[r][o - d] = xp[r];
+    }
+  } else if (role == 1) {
+    for (int k = 0; k < steps; ++k) {
+      const int n = n1 + k;
+      if (lane == 0 && n + 2 < NL) cx.wait(c, st);
+      __syncwarp();
+      named_sync(1 + c, CT + 32);
+      if (lane == 0 && n + 1 < NL) cx.issue(c, st);
+    }
+  }
+  __syncthreads();
+  state = st;
+  if (threadIdx.x == 0 && cx.cnt) *cx.cnt += 1;
+}
+
+// ---------------------------------------------------------------- reductions
+// Cluster-wide sums of NV binary32 values (every thread gets them), and this
+// CTA's own totals in loc if not null.  Warp totals, their sum by warp 0, which
+// puts it into every CTA's slot for this rank; after the cluster barrier each
+// warp adds the ranks' slots by the same tree, so all threads of the cluster
+// hold the same bits.  `phase` alternates two slot sets.
+template <int WF, int NV>
+__device__ __forceinline__ void mix_sum(cg::cluster_group& cl, int& phase, int p, float (&v)[NV], float* loc = nullptr) {
+  MixSmem<WF>& sm = mix_sm<WF>();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  constexpr int NW = Mix<WF>::NT / 32;
+  const int me = (int)cl.block_rank();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+  if (lane == 0) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) sm.wred[wid * 8 + k] = v[k];
+  }
+  __syncthreads();
+  if (wid == 0) {
+    float s[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) s[k] = lane < NW ? sm.wred[lane * 8 + k] : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < NV; ++k) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+    if (lane < p) {
+      float* rem = cl.map_shared_rank(&sm.slot[phase][me * 8], lane);
+#pragma unroll
+      for (int k = 0; k < NV; ++k) rem[k] = s[k];
+    }
+  }
+  cl.sync();
+#pragma unroll
+  for (int k = 0; k < NV; ++k) v[k] = lane < p ? sm.slot[phase][lane * 8 + k] : 0.f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+  if (loc) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) loc[k] = sm.slot[phase][me * 8 + k];
+  }
+  phase ^= 1;
+}
+
+// A sum of squares in binary32 without a known scale: three accumulators, of
+// which value() takes the one that neither under- nor overflowed.
+struct Norm3 {
+  float m = 0.f, s = 0.f, b = 0.f;
+  __device__ __forceinline__ void add(cxf v) {
+    constexpr float UP = 18446744073709551616.f, DN = 1.f / 18446744073709551616.f;   // 2^64, 2^-64
+    m += cabs2(v);
+    s += cabs2(UP * v);
+    b += cabs2(DN * v);
+  }
+  __device__ static __forceinline__ double value(float m, float s, float b) {
+    constexpr double UP2 = 340282366920938463463374607431768211456.0;                 // 2^128
+    if (m > 1e-28f && m < 1e28f) return (double)m;
+    return m >= 1e28f ? (double)b * UP2 : (double)s / UP2;
+  }
+};
+
+// ---------------------------------------------------------------- double-float pieces
+// a + b: the high words by TwoSum, the low words and the error added up (not renormalised)
+__device__ __forceinline__ void acc_add(dfl& a, dfl b) {
+  float s, e;
+  dfl_two_sum(a.hi, b.hi, s, e);
+  a.hi = s;
+  a.lo = __fadd_rn(__fadd_rn(a.lo, b.lo), e);
+}
+// a - b c
+__device__ __forceinline__ void acc_sub_mul(dfl& a, dfl b, dfl c) {
+  float p, e, s, t;
+  dfl_two_prod(-b.hi, c.hi, p, e);
+  e = __fmaf_rn(-b.hi, c.lo, e);
+  e = __fmaf_rn(-b.lo, c.hi, e);
+  dfl_two_sum(a.hi, p, s, t);
+  a.hi = s;
+  a.lo = __fadd_rn(a.lo, __fadd_rn(t, e));
+}
+__device__ __forceinline__ void acc_add(cdfl& a, const cdfl& b) {
+  acc_add(a.x, b.x);
+  acc_add(a.y, b.y);
+}
+// a - s b, s real
+__device__ __forceinline__ void acc_sub_scaled(cdfl& a, dfl s, const cdfl& b) {
+  acc_sub_mul(a.x, s, b.x);
+  acc_sub_mul(a.y, s, b.y);
+}
+// a - b c
+__device__ __forceinline__ void acc_sub_cmul(cdfl& a, const cdfl& b, const cdfl& c) {
+  acc_sub_mul(a.x, b.x, c.x);
+  acc_sub_mul(a.x, dfl(-b.y.hi, -b.y.lo), c.y);
+  acc_sub_mul(a.y, b.x, c.y);
+  acc_sub_mul(a.y, b.y, c.x);
+}
+__device__ __forceinline__ dfl renorm(dfl a) { return dfl_fast(a.hi, a.lo); }
+__device__ __forceinline__ cdfl renorm(const cdfl& a) { return {renorm(a.x), renorm(a.y)}; }
+// a + s c with a binary32 correction
+__device__ __forceinline__ dfl add_f(dfl a, float c) {
+  float s, e;
+  dfl_two_sum(a.hi, c, s, e);
+  return dfl_fast(s, __fadd_rn(a.lo, e));
+}
+__device__ __forceinline__ cdfl add_f(const cdfl& a, cxf c) { return {add_f(a.x, c.x), add_f(a.y, c.y)}; }
+__device__ __forceinline__ cdfl from_f(cxf v) { return {dfl(v.x, 0.f), dfl(v.y, 0.f)}; }
+__device__ __forceinline__ cxf scaled(float s, const cdfl& a) { return {s * (a.x.hi + a.x.lo), s * (a.y.hi + a.y.lo)}; }
+__device__ __forceinline__ dfl dfl_of(double v) { return d2dfl_bits(v); }
+
+// ---------------------------------------------------------------- interface solve
+// z = M_l^-1 r with the exact layer block (see lpre_apply), its columns split
+// over the warps: warp task (32 outputs, one of CS column ranges), the CS
+// partials added in a fixed order.  part: CS x A entries of scratch.
+__device__ __forceinline__ void mix_lpre(const Geo& g, const Bufs& b, int vs, int i, const cxf* r, cxf* z, cxf* part) {
+  const int A = g.A, nw = (int)blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nblk = (A + 31) / 32;
+  int CS = (2 * nw + nblk - 1) / nblk;
+  if (CS > g.W) CS = g.W;                // the scratch holds W entries per line site
+  const int per = (A + CS - 1) / CS;
+  const cxf* M = reinterpret_cast<const cxf*>(b.lpm) + ((size_t)slot_freq(g, vs) * (g.p - 1) + i) * (size_t)A * A;
+  constexpr int U = 8;
+  for (int task = wid; task < nblk * CS; task += nw) {
+    const int blk = task % nblk, ch = task / nblk, a = blk * 32 + lane;
+    const int c0 = ch * per, c1 = min(A, c0 + per);
+    if (a >= A) continue;
+    cxf acc[4] = {};
+    const cxf* col = M + a;
+    int c = c0;
+    for (; c + U <= c1; c += U) {
+      cxf mv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) mv[u] = col[(size_t)(c + u) * A];
+#pragma unroll
+      for (int u = 0; u < U; ++u) acc[u & 3] = cfma(mv[u], r[c + u], acc[u & 3]);
+    }
+    for (; c < c1; ++c) acc[0] = cfma(col[(size_t)c * A], r[c], acc[0]);
+    part[(size_t)ch * A + a] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  }
+  __syncthreads();
+  for (int a = threadIdx.x; a < A; a += (int)blockDim.x) {
+    cxf s = part[a];
+    for (int ch = 1; ch < CS; ++ch) s = s + part[(size_t)ch * A + a];
+    z[a] = s;
+  }
+}
+
+struct MixSolve {
+  bool useB0;                            // the subdomain part is B0 - alpha B1 (else - alpha B1)
+  cxf alpha;
+  int iters, conv;
+};
+
+// COCG on S y = IF_B (relative residual krylov_tol), S applied by one sweep in
+// row buffer 1 per iteration.  The solution's subdomain part -B^-1 E y is left
+// as B0 - alpha B1: each iteration but the last is folded into B0, the last one
+// is the caller's.  keep0: B0 holds a vector to add to (else it counts as zero).
+// IF_B is complete (a barrier after its writers) on entry.
+template <int WF, bool ROWS>
+__device__ __noinline__ MixSolve mix_cocg(const Geo& g, const Bufs& b, const MixCtx<WF, ROWS>& cx, MixState& st,
+                                          int& phase_, int vs, bool keep0) {
+  cg::cluster_group cl = cg::this_cluster();
+  int phase = phase_;
+  constexpr int nt = Mix<WF>::NT;
+  const int i = blockIdx.x, A = g.A, p = g.p, W = cx.W, Lx = cx.Lx, T = g.T, w = T * g.h[i], nsub = Lx * W;
+  const int ds = nt / W, dj = nt % W;
+  const bool has = i < p - 1;
+  cxf* B0 = cx.row(0);
+  cxf* B1 = cx.row(1);
+  const size_t o = (size_t)i * A;
+  cxf* X = ifv_ptr<float>(g, b, vs, IF_X) + o;
+  cxf* Rv = ifv_ptr<float>(g, b, vs, IF_R) + o;
+  cxf* Z = ifv_ptr<float>(g, b, vs, IF_Z) + o;
+  cxf* P = ifv_ptr<float>(g, b, vs, IF_P);
+  cxf* SP = ifv_ptr<float>(g, b, vs, IF_SP) + o;
+  const cxf* Bv = ifv_ptr<float>(g, b, vs, IF_B) + o;
+  const cxf* dC = ifv_ptr<float>(g, b, vs, IF_D) + o;
+  cxf* blo = bnd_ptr<float>(g, b, vs, i, 0);
+  cxf* bhi = bnd_ptr<float>(g, b, vs, i, 1);
+  const cxf* bnx = has ? bnd_ptr<float>(g, b, vs, i + 1, 0) : nullptr;
+  const cxf* plo = i > 0 ? P + o - A : nullptr;
+  cxf* phi = P + o;
+  const float t = cx.t;
+  auto precond = [&](const cxf* r, cxf* z) {
+    if (g.lpre) mix_lpre(g, b, vs, i, r, z, B1);
+    else precond_apply<float>(g, b, vs, i, r, z);
+  };
+  MixSolve out = {keep0, {0.f, 0.f}, 0, 1};
+  if (has) precond(Bv, Z);
+  __syncthreads();
+  float v3[3] = {0.f, 0.f, 0.f};
+  if (has) {
+    cxf rz = {0.f, 0.f};
+    for (int a = threadIdx.x; a < A; a += nt) {
+      const cxf zz = Z[a], r = Bv[a];
+      X[a] = cxf{0.f, 0.f};
+      Rv[a] = r;
+      phi[a] = zz;
+      rz = cfma(r, zz, rz);
+      v3[2] += cabs2(r);
+    }
+    v3[0] = rz.x;
+    v3[1] = rz.y;
+  }
+  mix_sum<WF, 3>(cl, phase, p, v3);      // also: P of the neighbour layers is final
+  cxf rho = {v3[0], v3[1]};
+  const float bn = v3[2];
+  const float tol2 = (float)(g.krylov_tol * g.krylov_tol);
+  if (bn > 0.f || bn != bn) {
+    for (;;) {
+      if (out.iters >= g.krylov_maxit) {
+        out.conv = 0;
+        break;
+      }
+      if (out.iters > 0) {
+        // fold the last product into B0, then the next direction
+        const bool z0 = !out.useB0;
+        for (int e = threadIdx.x; e < nsub; e += nt) {
+          const cxf q = out.alpha * B1[e];
+          B0[e] = z0 ? -q : B0[e] - q;
+        }
+        out.useB0 = true;
+        __syncthreads();                 // B1 is free (the preconditioner's scratch)
+        if (has) precond(Rv, Z);
+        __syncthreads();
+        float v2[2] = {0.f, 0.f};
+        if (has) {
+          cxf rz = {0.f, 0.f};
+          for (int a = threadIdx.x; a < A; a += nt) rz = cfma(Rv[a], Z[a], rz);
+          v2[0] = rz.x;
+          v2[1] = rz.y;
+        }
+        mix_sum<WF, 2>(cl, phase, p, v2);
+        const cxf rn = {v2[0], v2[1]}, beta = cdiv(rn, rho);
+        rho = rn;
+        if (has)
+          for (int a = threadIdx.x; a < A; a += nt) phi[a] = Z[a] + beta * phi[a];
+        cl.sync();                       // P of the neighbour layers is final
+      }
+      ++out.iters;
+      // B1 = E p
+      for (int e = threadIdx.x, s = e / W, j = e - s * W; e < nsub; e += nt) {
+        cxf u = {0.f, 0.f};
+        if (plo && j < T) u = u + t * plo[s + Lx * j];
+        if (has && j >= w - T && j < w) u = u + t * phi[s + Lx * (j - (w - T))];
+        B1[e] = u;
+        s += ds;
+        j += dj;
+        if (j >= W) {
+          j -= W;
+          ++s;
+        }
+      }
+      mix_sweep<WF, 1, ROWS>(cx, st, 1);
+      for (int e = threadIdx.x; e < A; e += nt) {
+        const int j = T == 1 ? 0 : e / Lx, s = e - j * Lx;
+        blo[e] = B1[s * W + j];
+        bhi[e] = B1[s * W + (w - T) + j];
+      }
+      cl.sync();                         // boundary rows of every subdomain written
+      float v2[2] = {0.f, 0.f};
+      if (has) {
+        cxf ps = {0.f, 0.f};
+        for (int a = threadIdx.x; a < A; a += nt) {
+          const cxf sp = layer_C_apply<float>(g, dC, phi, a) - t * (bhi[a] + bnx[a]);
+          SP[a] = sp;
+          ps = cfma(phi[a], sp, ps);
+        }
+        v2[0] = ps.x;
+        v2[1] = ps.y;
+      }
+      mix_sum<WF, 2>(cl, phase, p, v2);
+      out.alpha = cdiv(rho, cxf{v2[0], v2[1]});
+      float v1[1] = {0.f};
+      if (has) {
+        for (int a = threadIdx.x; a < A; a += nt) {
+          X[a] = X[a] + out.alpha * phi[a];
+          const cxf r = Rv[a] - out.alpha * SP[a];
+          Rv[a] = r;
+          v1[0] += cabs2(r);
+        }
+      }
+      mix_sum<WF, 1>(cl, phase, p, v1);
+      if (v1[0] <= tol2 * bn) break;
+    }
+  }
+  phase_ = phase;
+  return out;
+}
+
+// ---------------------------------------------------------------- the X-matvec
+// w = blkdiag(B^-1, 0) q and u = X q = H^-1 [0; q_C - E^T w_B] (Eqs. 6-8, no
+// cancellation) are found together:
+//   w  from one sweep on q_B, u from one interface solve on q_C - E^T w_B;
+//   then, until both relative residuals are below refine_tol, the residuals
+//     r_w = q_B - B w,   r_u = [0; q_C - E^T w] - H u       (double-float)
+//   and one correction: a sweep on both subdomain residuals gives d_w and
+//   z = B^-1 r_u, an interface solve on r_u,C - E^T (d_w + z) gives d_y, and
+//   w += d_w,  u_B += z - B^-1 E d_y,  u_C += d_y.
+// The residual pass writes its rows straight into the row buffers in complex64,
+// scaled by an estimate of their size (1e6 over the last residual's norm: about
+// what a complex64 correction leaves); the scale only keeps the values inside
+// the binary32 range, and the norms are measured on the scaled rows.
+template <int WF, bool ROWS>
+__global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
+    k_xmatvec_m(const __grid_constant__ Geo g, const __grid_constant__ Bufs b, int j, int ncols) {
+  cg::cluster_group cl = cg::this_cluster();
+  constexpr int nt = Mix<WF>::NT;
+  const int i = blockIdx.x, vs = blockIdx.y, p = g.p, A = g.A, W = g.W, Lx = g.Lx, T = g.T;
+  const int f = slot_freq(g, vs), c = vs - f * g.nb;
+  if (c >= ncols) return;                  // same values in every CTA of the cluster
+  int* st = b.st + (size_t)f * ST_N;
+  if (st[ST_DONE]) return;
+  const size_t Ndd = g.Ndd;
+  const int nsub = Lx * W, w = T * g.h[i], hh = g.h[i], tid = threadIdx.x;
+  const int ds = nt / W, dj = nt % W, s_0 = tid / W, j_0 = tid - s_0 * W;
+  MixCtx<WF, ROWS> cx;
+  cx.W = W;
+  cx.Lx = Lx;
+  cx.S = mix_plan(g).S;
+  cx.m = Lx / 2;
+  cx.src = reinterpret_cast<const cxf*>(b.g) + ((size_t)f * p + i) * (size_t)nsub * W;
+  cx.g0 = reinterpret_cast<cxf*>(b.yscr) + ((size_t)vs * p + i) * nsub;
+  cx.g1 = reinterpret_cast<cxf*>(b.v2 + (size_t)vs * Ndd + (size_t)i * nsub);
+  cx.cnt = sweep_cnt(g, b, vs, i);
+  cx.t = (float)g.t;
+  MixState ms;
+  mix_init<WF, ROWS>(cx, ms);
+  int phase = 0;
+  cxf* B0 = cx.row(0);
+  cxf* B1 = cx.row(1);
+  const bool has = i < p - 1;
+  const cxd* qd = b.Q + ((size_t)f * (g.k_max + g.nb) + (size_t)j * g.nb + c) * Ndd;
+  const cdfl* qs = reinterpret_cast<const cdfl*>(qd);
+  const bool split = g.qsplit != 0;
+  const size_t qo = (size_t)i * nsub, lo = (size_t)g.ifc_off + (size_t)i * A, o = (size_t)i * A;
+  cdfl* u = reinterpret_cast<cdfl*>(b.u + (size_t)vs * Ndd);       // double-floats until the last pass
+  cdfl* wv = reinterpret_cast<cdfl*>(b.v1 + (size_t)vs * Ndd);     // w_B
+  cdfl* rc = reinterpret_cast<cdfl*>(b.v2 + (size_t)vs * Ndd) + lo;   // interface residual
+  cdfl *us = u + qo, *ws = wv + qo;
+  const cdfl* hd = reinterpret_cast<const cdfl*>(b.hdiag + (size_t)f * Ndd);
+  const cdfl* hs = hd + qo;
+  const dfl td = dfl_of(g.t);
+  const float tf = cx.t;
+  cxf* Bv = ifv_ptr<float>(g, b, vs, IF_B) + o;
+  cxf* X = ifv_ptr<float>(g, b, vs, IF_X) + o;
+  cxf* dC = ifv_ptr<float>(g, b, vs, IF_D) + o;
+  cxf* blo = bnd_ptr<float>(g, b, vs, i, 0);
+  cxf* bhi = bnd_ptr<float>(g, b, vs, i, 1);
+  const cxf* bnx = has ? bnd_ptr<float>(g, b, vs, i + 1, 0) : nullptr;
+  auto ldq = [&](size_t k) -> cdfl { return split ? qs[k] : csplit(qd[k]); };
+
+  // ---- w_0 = B^-1 q_B
+  Norm3 qn;                                // ||q_B||^2 of this subdomain
+  for (int e = tid, jj = j_0; e < nsub; e += nt) {
+    cxf v = {0.f, 0.f};
+    if (jj < w) {
+      const cdfl q = ldq(qo + e);
+      v = cxf{q.x.hi, q.y.hi};
+      qn.add(v);
+    }
+    B0[e] = v;
+    jj += dj;
+    if (jj >= W) jj -= W;
+  }
+  if (has)
+    for (int a = tid; a < A; a += nt) {
+      const cdfl d = hd[lo + a];
+      dC[a] = cxf{d.x.hi, d.y.hi};
+    }
+  mix_sweep<WF, 1, ROWS>(cx, ms, 0);
+  for (int e = tid; e < nsub; e += nt) ws[e] = from_f(B0[e]);      // zero on the padding
+  for (int e = tid; e < A; e += nt) {
+    const int jj = T == 1 ? 0 : e / Lx, s = e - jj * Lx;
+    blo[e] = B0[s * W + jj];
+    bhi[e] = B0[s * W + (w - T) + jj];
+  }
+  cl.sync();                               // boundary rows (and w) of the neighbour subdomains are final
+  double hn2, qn2;
+  {
+    Norm3 h3;
+    if (has)
+      for (int a = tid; a < A; a += nt) {
+        cdfl h = ldq(lo + a);
+        acc_sub_scaled(h, td, from_f(bhi[a]));
+        acc_sub_scaled(h, td, from_f(bnx[a]));
+        h = renorm(h);
+        rc[a] = h;
+        h3.add(cxf{h.x.hi, h.y.hi});
+      }
+    float v[6] = {h3.m, h3.s, h3.b, qn.m, qn.s, qn.b}, own[6];
+    mix_sum<WF, 6>(cl, phase, p, v, own);
+    hn2 = Norm3::value(v[0], v[1], v[2]);
+    qn2 = Norm3::value(own[3], own[4], own[5]);
+  }
+  int iters = 0, solves = 0, refines = 0, conv_all = 1;
+  const double hn = sqrt(hn2), ihn = hn2 > 0.0 ? 1.0 / hn : 1.0;
+  const float ihf = (float)ihn;
+  // ---- u_0 = H^-1 [0; hr]
+  if (hn2 > 0.0) {
+    if (has)
+      for (int a = tid; a < A; a += nt) Bv[a] = scaled(ihf, rc[a]);
+    __syncthreads();
+    const MixSolve sv = mix_cocg<WF, ROWS>(g, b, cx, ms, phase, vs, false);
+    iters += sv.iters;
+    conv_all &= sv.conv;
+    ++solves;
+    const float hf = (float)hn;
+    for (int e = tid; e < nsub; e += nt) {   // zero on the padding, which the Lanczos step reads too
+      cxf v = sv.iters > 0 ? sv.alpha * B1[e] : cxf{0.f, 0.f};
+      if (sv.useB0) v = v - B0[e];
+      us[e] = from_f(-(hf * v));
+    }
+    if (has)
+      for (int a = tid; a < A; a += nt) u[lo + a] = from_f(hf * X[a]);
+  } else {
+    for (int e = tid; e < nsub; e += nt) us[e] = from_f(cxf{0.f, 0.f});
+    if (has)
+      for (int a = tid; a < A; a += nt) u[lo + a] = from_f(cxf{0.f, 0.f});
+  }
+  // ---- refinement of w and u together
+  const cdfl* xlo = i > 0 ? u + g.ifc_off + (size_t)(i - 1) * A : nullptr;
+  const cdfl* xhi = u + lo;
+  const double tol2 = g.refine_tol * g.refine_tol;
+  double su = 1e6 * ihn, sw = qn2 > 0.0 ? 1e6 / sqrt(qn2) : 1.0;   // row scales
+  double prev_u = INFINITY, prev_w = INFINITY;
+  bool wdone = qn2 == 0.0;
+  for (int pass = 0; pass < g.refine_max; ++pass) {
+    cl.sync();                             // u and w of the neighbours are final
+    const float suf = (float)su, swf = (float)sw;
+    float nu = 0.f, nw = 0.f;
+    for (int e = tid, s = s_0, jj = j_0; e < nsub; e += nt) {
+      cxf ru = {0.f, 0.f}, rw = {0.f, 0.f};
+      if (jj < w) {
+        const int tr = T == 1 ? 0 : jj % T, sl = T == 1 ? jj : jj / T;
+        const cdfl dv = hs[e];
+        const bool pl = s > 0, pr = s < Lx - 1, tl = tr > 0, trr = tr < T - 1, dl = sl > 0, dr = sl < hh - 1;
+        auto neighbours = [&](const cdfl* x) -> cdfl {
+          cdfl n = from_f(cxf{0.f, 0.f});
+          if (pl) n = x[e - W];
+          if (pr) acc_add(n, x[e + W]);
+          if (tl) acc_add(n, x[e - 1]);
+          if (trr) acc_add(n, x[e + 1]);
+          if (dl) acc_add(n, x[e - T]);
+          if (dr) acc_add(n, x[e + T]);
+          return n;
+        };
+        cdfl n = neighbours(us), r = from_f(cxf{0.f, 0.f});
+        if (sl == 0 && xlo) acc_add(n, xlo[s + Lx * tr]);
+        if (sl == hh - 1 && has) acc_add(n, xhi[s + Lx * tr]);
+        acc_sub_scaled(r, td, n);
+        acc_sub_cmul(r, dv, us[e]);
+        ru = scaled(suf, r);
+        nu += cabs2(ru);
+        if (!wdone) {
+          r = ldq(qo + e);
+          acc_sub_scaled(r, td, neighbours(ws));
+          acc_sub_cmul(r, dv, ws[e]);
+          rw = scaled(swf, r);
+          nw += cabs2(rw);
+        }
+      }
+      B0[e] = ru;
+      if (!wdone) B1[e] = rw;
+      s += ds;
+      jj += dj;
+      if (jj >= W) {
+        jj -= W;
+        ++s;
+      }
+    }
+    float v[3] = {nu, 0.f, nw}, own[3];      // ||su r_u||^2, ||hr / hn||^2, ||sw r_w||^2
+    if (has) {
+      const cdfl* xa = u + (size_t)(i + 1) * nsub;   // subdomain i + 1: its bottom row touches layer i
+      const cdfl* wa = wv + (size_t)(i + 1) * nsub;
+      const int hi = T * (hh - 1);
+      for (int a = tid; a < A; a += nt) {
+        const int tr = T == 1 ? 0 : a / Lx, xx = a - tr * Lx;
+        const int kb = xx * W + hi + tr, ka = xx * W + tr;
+        cdfl r = ldq(lo + a), n = ws[kb];
+        acc_add(n, wa[ka]);
+        acc_sub_scaled(r, td, n);              // hr = q_C - E^T w
+        const cxf hsc = scaled(ihf, r);
+        n = us[kb];
+        acc_add(n, xa[ka]);
+        if (xx > 0) acc_add(n, xhi[a - 1]);
+        if (xx < Lx - 1) acc_add(n, xhi[a + 1]);
+        if (tr > 0) acc_add(n, xhi[a - Lx]);
+        if (tr < T - 1) acc_add(n, xhi[a + Lx]);
+        acc_sub_scaled(r, td, n);
+        acc_sub_cmul(r, hd[lo + a], xhi[a]);
+        rc[a] = renorm(r);
+        v[0] += cabs2(scaled(suf, r));
+        v[1] += cabs2(hsc);
+      }
+    }
+    mix_sum<WF, 3>(cl, phase, p, v, own);
+    const double wn = (double)own[2] / (sw * sw);   // this subdomain's, which decides for its w alone
+    if (!wdone && (wn <= tol2 * qn2 || wn > REFINE_STALL * prev_w)) wdone = true;
+    if (!wdone) prev_w = wn;
+    const double rn = (double)v[0] / (su * su);
+    const bool udone = rn <= tol2 * ((double)v[1] * hn2) || rn > REFINE_STALL * prev_u;
+    if (udone) {
+      // u is done: go on only if some w of the cluster is not
+      float go[1] = {!wdone && tid == 0 ? 1.f : 0.f};
+      mix_sum<WF, 1>(cl, phase, p, go);
+      if (go[0] == 0.f) break;
+    }
+    prev_u = rn;
+    ++refines;
+    // ---- z = B^-1 r_u in B0, d_w = B^-1 r_w in B1
+    const bool wgo = !wdone;
+    if (wgo) mix_sweep<WF, 2, ROWS>(cx, ms, 0);
+    else mix_sweep<WF, 1, ROWS>(cx, ms, 0);
+    const double isu = 1.0 / su;
+    const float isuf = (float)isu, iswf = (float)(1.0 / sw), ratio = (float)(su / sw);
+    if (wgo)
+      for (int e = tid; e < nsub; e += nt) ws[e] = add_f(ws[e], iswf * B1[e]);
+    for (int e = tid; e < A; e += nt) {
+      const int jj = T == 1 ? 0 : e / Lx, s = e - jj * Lx;
+      const int k0 = s * W + jj, k1 = s * W + (w - T) + jj;
+      blo[e] = wgo ? B0[k0] + ratio * B1[k0] : B0[k0];
+      bhi[e] = wgo ? B0[k1] + ratio * B1[k1] : B0[k1];
+    }
+    cl.sync();                             // boundary rows of the neighbours
+    if (has)
+      for (int a = tid; a < A; a += nt) Bv[a] = scaled(suf, rc[a]) - tf * (bhi[a] + bnx[a]);
+    __syncthreads();
+    const MixSolve sv = mix_cocg<WF, ROWS>(g, b, cx, ms, phase, vs, true);
+    iters += sv.iters;
+    conv_all &= sv.conv;
+    ++solves;
+    for (int e = tid; e < nsub; e += nt) {
+      cxf v2 = B0[e];
+      if (sv.iters > 0) v2 = v2 - sv.alpha * B1[e];
+      us[e] = add_f(us[e], isuf * v2);
+    }
+    if (has)
+      for (int a = tid; a < A; a += nt) u[lo + a] = add_f(u[lo + a], isuf * X[a]);
+    if (rn > 0.0) su = 1e6 / sqrt(rn);
+    if (wgo && prev_w > 0.0) sw = 1e6 / sqrt(prev_w);
+  }
+  // ---- u to binary64 (in place: an entry is 16 bytes in both forms; the residuals that
+  // read this u were followed by a cluster barrier)
+  {
+    cxd* ud = b.u + (size_t)vs * Ndd;
+    for (int e = tid; e < nsub; e += nt) ud[qo + e] = cwiden(us[e]);
+    if (has)
+      for (int a = tid; a < A; a += nt) ud[lo + a] = cwiden(u[lo + a]);
+  }
+  mix_drain<WF, ROWS>(cx, ms);
+  __syncthreads();
+  if (tid == 0 && mix_sm<WF>().err) atomicOr(st + ST_STATUS, ST_WAIT_TIMEOUT);
+  if (i == 0 && tid == 0) {               // the nb clusters of a frequency share its counters
+    atomicAdd(st + ST_ITERS, iters);
+    atomicAdd(st + ST_SOLVES, solves);
+    atomicAdd(st + ST_REFINE, refines);
+    if (!conv_all) atomicOr(st + ST_STATUS, 4);
+  }
+  cl.sync();          // no CTA exits while a peer may still read its shared memory
+}
+
+// w = blkdiag(B^-1, 0) q for DD-layout vectors (Eq. 7), one CTA per subdomain.
+template <int WF, bool ROWS>
+__global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
+    k_bsolve_m(const __grid_constant__ Geo g, const __grid_constant__ Bufs b, const cxd* q, cxd* w) {
+  constexpr int nt = Mix<WF>::NT;
+  const int i = blockIdx.x, kf = blockIdx.y, vs = kf * g.nb, W = g.W, nsub = g.Lx * W, wd = g.T * g.h[i];
+  MixCtx<WF, ROWS> cx;
+  cx.W = W;
+  cx.Lx = g.Lx;
+  cx.S = mix_plan(g).S;
+  cx.m = g.Lx / 2;
+  cx.src = reinterpret_cast<const cxf*>(b.g) + ((size_t)kf * g.p + i) * (size_t)nsub * W;
+  cx.g0 = cx.g1 = reinterpret_cast<cxf*>(b.yscr) + ((size_t)vs * g.p + i) * nsub;
+  cx.cnt = sweep_cnt(g, b, vs, i);
+  cx.t = (float)g.t;
+  MixState ms;
+  mix_init<WF, ROWS>(cx, ms);
+  cxf* B0 = cx.row(0);
+  const cxd* qs = q + (size_t)kf * g.Ndd + (size_t)i * nsub;
+  cxd* ws = w + (size_t)kf * g.Ndd + (size_t)i * nsub;
+  for (int e = threadIdx.x; e < nsub; e += nt) B0[e] = e % W < wd ? c2f_bits(qs[e]) : cxf{0.f, 0.f};
+  mix_sweep<WF, 1, ROWS>(cx, ms, 0);
+  for (int e = threadIdx.x; e < nsub; e += nt)
+    if (e % W < wd) ws[e] = c2d_bits(B0[e]);
+  if (i < g.p - 1)
+    for (int a = threadIdx.x; a < g.A; a += nt)
+      w[(size_t)kf * g.Ndd + g.ifc_off + (size_t)i * g.A + a] = cxd{0, 0};
+  mix_drain<WF, ROWS>(cx, ms);
+  __syncthreads();
+  if (threadIdx.x == 0 && mix_sm<WF>().err) atomicOr(b.st + (size_t)kf * ST_N + ST_STATUS, ST_WAIT_TIMEOUT);
+}
+
+}  // namespace
+
+template <int WF>
+cudaError_t run_xmatvec_m(const Geo& g, const Bufs& b, int K, int j, int ncols, cudaStream_t st);
+template <int WF>
+cudaError_t run_bsolve_m(const Geo& g, const Bufs& b, int K, const cxd* q_dd, cxd* w_dd, cudaStream_t st);
+
+#define DY_MIXED_VARIANT(WF)                                                                               \
+  template <>                                                                                              \
+  cudaError_t run_xmatvec_m<WF>(const Geo& g, const Bufs& b, int K, int j, int ncols, cudaStream_t st) {   \
+    const MixPlan mp = mix_plan(g);                                                                        \
+    if (mp.rows)                                                                                           \
+      return launch_cluster_nt(k_xmatvec_m<WF, true>, dim3(g.p, K * g.nb), g.p, Mix<WF>::NT, mp.smem, st,  \
+                               g, b, j, ncols);                                                            \
+    return launch_cluster_nt(k_xmatvec_m<WF, false>, dim3(g.p, K * g.nb), g.p, Mix<WF>::NT, mp.smem, st,   \
+                             g, b, j, ncols);                                                              \
+  }                                                                                                        \
+  template <>                                                                                              \
+  cudaError_t run_bsolve_m<WF>(const Geo& g, const Bufs& b, int K, const cxd* q_dd, cxd* w_dd,             \
+                               cudaStream_t st) {                                                          \
+    const MixPlan mp = mix_plan(g);                                                                        \
+    auto kern = mp.rows ? k_bsolve_m<WF, true> : k_bsolve_m<WF, false>;                                    \
+    cudaError_t e = raise_smem_limit((const void*)kern, mp.smem);                                          \
+    if (e != cudaSuccess) return e;                                                                        \
+    kern<<<dim3(g.p, K), Mix<WF>::NT, mp.smem, st>>>(g, b, q_dd, w_dd);                                    \
+    return cudaGetLastError();                                                                             \
+  }
