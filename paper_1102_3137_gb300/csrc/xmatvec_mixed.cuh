@@ -123,11 +123,15 @@ __device__ __forceinline__ void named_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
-// What a thread keeps from sweep to sweep (compute warps: slot; producers: all).
+// What a thread keeps from sweep to sweep (compute warps: slot; producers: the
+// rest).  The addresses of the next copy and of the next wait are computed when
+// the previous one is done, off the chain's critical path: after a barrier the
+// producer only issues.
 struct MixState {
   int slot;                              // compute: slot of the next block to read; producer: next slot to fill
-  int pos;                               // producer: position of the next block to copy in the sweep's sequence
-  int wslot;                             // producer: slot of the next block to wait for
+  int pos;                               // position of the next block to copy in the sweep's sequence
+  const cxf* src;                        // its address
+  int wslot;                             // slot of the next block to wait for
   uint32_t wph;
   bool dead;
 };
@@ -146,17 +150,20 @@ struct MixCtx {
     else return k ? g1 : g0;
   }
   __device__ __forceinline__ int blocks(int chain) const { return chain == 0 ? 2 * m + 1 : 2 * (Lx - 1 - m); }
-  __device__ __forceinline__ int slice_at(int chain, int n) const {
-    if (chain == 0) return n <= m ? n : 2 * m - n;
-    const int qR = Lx - 1 - m;
-    return n < qR ? Lx - 1 - n : m + 1 + (n - qR);
-  }
+  // The sequence of a chain's slices over one sweep: left 0 .. m, m-1 .. 0, right
+  // Lx-1 .. m+1, m+1 .. Lx-1; the next sweep starts with the last one's last slice.
+  __device__ __forceinline__ const cxf* first(int chain) const { return src + (chain == 0 ? 0 : (size_t)(Lx - 1) * W * W); }
   __device__ __forceinline__ void issue(int chain, MixState& st) const {
     MixSmem<WF>& sm = mix_sm<WF>();
-    bulk_load(mix_ring<WF>() + (chain * S + st.slot) * W * W, src + (size_t)slice_at(chain, st.pos) * W * W,
-              (uint32_t)(W * W * sizeof(cxf)), sm.bars + chain * MIX_MAXS + st.slot);
+    const int n = W * W;
+    bulk_load(mix_ring<WF>() + (chain * S + st.slot) * n, st.src, (uint32_t)(n * sizeof(cxf)),
+              sm.bars + chain * MIX_MAXS + st.slot);
     if (++st.slot == S) st.slot = 0;
-    if (++st.pos == blocks(chain)) st.pos = 0;
+    const int up = chain == 0 ? m : Lx - 2 - m, last = blocks(chain) - 1;   // the turn: left at m, right repeats m+1
+    const int dn = chain == 0 ? n : -n;
+    const int turn = chain == 0 ? 0 : 1;
+    st.src += st.pos < up ? dn : (st.pos < up + turn || st.pos == last ? 0 : -dn);
+    st.pos = st.pos == last ? 0 : st.pos + 1;
   }
   __device__ __forceinline__ void wait(int chain, MixState& st) const {
     MixSmem<WF>& sm = mix_sm<WF>();
@@ -173,6 +180,7 @@ __device__ void mix_init(const MixCtx<WF, ROWS>& cx, MixState& st) {
   MixSmem<WF>& sm = mix_sm<WF>();
   const int tid = threadIdx.x, wid = tid >> 5;
   st.slot = st.pos = st.wslot = 0;
+  st.src = cx.first(wid == Mix<WF>::PROD + 1 ? 1 : 0);
   st.wph = 0;
   st.dead = false;
   for (int e = tid; e < 8 * WF; e += Mix<WF>::NT) (&sm.z[0][0][0][0])[e] = cxf{0.f, 0.f};
@@ -560,37 +568,68 @@ __device__ __forceinline__ dfl dfl_of(double v) { return d2dfl_bits(v); }
 
 // ---------------------------------------------------------------- interface solve
 // z = M_l^-1 r with the exact layer block (see lpre_apply), its columns split
-// over the warps: warp task (32 outputs, one of CS column ranges), the CS
-// partials added in a fixed order.  part: CS x A entries of scratch.
+// over the warps: warp task (32 V outputs, one of CS column ranges), the CS
+// partials added in a fixed order.  The block (2 MB at A = 512) comes from HBM on
+// every application, so what counts is the bytes in flight: V = 2 outputs a lane
+// by 16-byte loads where a row's length keeps them aligned, eight columns at a time.
+// part: CS x A entries of scratch.
+template <int V>
 __device__ __forceinline__ void mix_lpre(const Geo& g, const Bufs& b, int vs, int i, const cxf* r, cxf* z, cxf* part) {
   const int A = g.A, nw = (int)blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nblk = (A + 31) / 32;
-  int CS = (2 * nw + nblk - 1) / nblk;
+  const int nblk = (A + 32 * V - 1) / (32 * V);
+  int CS = (3 * nw + nblk - 1) / nblk;
   if (CS > g.W) CS = g.W;                // the scratch holds W entries per line site
   const int per = (A + CS - 1) / CS;
   const cxf* M = reinterpret_cast<const cxf*>(b.lpm) + ((size_t)slot_freq(g, vs) * (g.p - 1) + i) * (size_t)A * A;
   constexpr int U = 8;
   for (int task = wid; task < nblk * CS; task += nw) {
-    const int blk = task % nblk, ch = task / nblk, a = blk * 32 + lane;
+    const int blk = task % nblk, ch = task / nblk, a = (blk * 32 + lane) * V;
     const int c0 = ch * per, c1 = min(A, c0 + per);
     if (a >= A) continue;
-    cxf acc[4] = {};
+    cxf acc[2][V] = {};
     const cxf* col = M + a;
+    auto mul = [&](int c, int k) {
+      if constexpr (V == 2) {
+        const float4 m = *reinterpret_cast<const float4*>(col + (size_t)c * A);
+        const cxf rv = r[c];
+        acc[k][0] = cfma(cxf{m.x, m.y}, rv, acc[k][0]);
+        acc[k][1] = cfma(cxf{m.z, m.w}, rv, acc[k][1]);
+      } else {
+        acc[k][0] = cfma(col[(size_t)c * A], r[c], acc[k][0]);
+      }
+    };
     int c = c0;
     for (; c + U <= c1; c += U) {
-      cxf mv[U];
+      if constexpr (V == 2) {
+        float4 m[U];
+        cxf rv[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) mv[u] = col[(size_t)(c + u) * A];
+        for (int u = 0; u < U; ++u) m[u] = *reinterpret_cast<const float4*>(col + (size_t)(c + u) * A);
 #pragma unroll
-      for (int u = 0; u < U; ++u) acc[u & 3] = cfma(mv[u], r[c + u], acc[u & 3]);
+        for (int u = 0; u < U; ++u) rv[u] = r[c + u];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          acc[u & 1][0] = cfma(cxf{m[u].x, m[u].y}, rv[u], acc[u & 1][0]);
+          acc[u & 1][1] = cfma(cxf{m[u].z, m[u].w}, rv[u], acc[u & 1][1]);
+        }
+      } else {
+        cxf m[U], rv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) m[u] = col[(size_t)(c + u) * A];
+#pragma unroll
+        for (int u = 0; u < U; ++u) rv[u] = r[c + u];
+#pragma unroll
+        for (int u = 0; u < U; ++u) acc[u & 1][0] = cfma(m[u], rv[u], acc[u & 1][0]);
+      }
     }
-    for (; c < c1; ++c) acc[0] = cfma(col[(size_t)c * A], r[c], acc[0]);
-    part[(size_t)ch * A + a] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    for (; c < c1; ++c) mul(c, 0);
+#pragma unroll
+    for (int v = 0; v < V; ++v) part[ch * A + a + v] = acc[0][v] + acc[1][v];
   }
   __syncthreads();
   for (int a = threadIdx.x; a < A; a += (int)blockDim.x) {
     cxf s = part[a];
-    for (int ch = 1; ch < CS; ++ch) s = s + part[(size_t)ch * A + a];
+    for (int ch = 1; ch < CS; ++ch) s = s + part[ch * A + a];
     z[a] = s;
   }
 }
@@ -632,7 +671,8 @@ __device__ __noinline__ MixSolve mix_cocg(const Geo& g, const Bufs& b, const Mix
   cxf* phi = P + o;
   const float t = cx.t;
   auto precond = [&](const cxf* r, cxf* z) {
-    if (g.lpre) mix_lpre(g, b, vs, i, r, z, B1);
+    if (g.lpre && A % 2 == 0) mix_lpre<2>(g, b, vs, i, r, z, B1);
+    else if (g.lpre) mix_lpre<1>(g, b, vs, i, r, z, B1);
     else precond_apply<float>(g, b, vs, i, r, z);
   };
   MixSolve out = {keep0, {0.f, 0.f}, 0, 1};
@@ -884,28 +924,40 @@ __global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
       if (jj < w) {
         const int tr = T == 1 ? 0 : jj % T, sl = T == 1 ? jj : jj / T;
         const cdfl dv = hs[e];
-        const bool pl = s > 0, pr = s < Lx - 1, tl = tr > 0, trr = tr < T - 1, dl = sl > 0, dr = sl < hh - 1;
-        auto neighbours = [&](const cdfl* x) -> cdfl {
-          cdfl n = from_f(cxf{0.f, 0.f});
-          if (pl) n = x[e - W];
-          if (pr) acc_add(n, x[e + W]);
-          if (tl) acc_add(n, x[e - 1]);
-          if (trr) acc_add(n, x[e + 1]);
-          if (dl) acc_add(n, x[e - T]);
-          if (dr) acc_add(n, x[e + T]);
+        const bool pl = s > 0, pr = s < Lx - 1, dl = sl > 0, dr = sl < hh - 1;
+        const cdfl zero = from_f(cxf{0.f, 0.f});
+        // the sum of x over the neighbours inside the subdomain; every load is issued
+        // before the first sum
+        auto neighbours = [&](const cdfl* x, const cdfl& lo_, const cdfl& hi_) -> cdfl {
+          cdfl n = pl ? x[e - W] : zero;
+          const cdfl n1 = pr ? x[e + W] : zero, n2 = dl ? x[e - T] : lo_, n3 = dr ? x[e + T] : hi_;
+          cdfl n4 = zero, n5 = zero;
+          if (T > 1) {
+            n4 = tr > 0 ? x[e - 1] : zero;
+            n5 = tr < T - 1 ? x[e + 1] : zero;
+          }
+          acc_add(n, n1);
+          acc_add(n, n2);
+          acc_add(n, n3);
+          if (T > 1) {
+            acc_add(n, n4);
+            acc_add(n, n5);
+          }
           return n;
         };
-        cdfl n = neighbours(us), r = from_f(cxf{0.f, 0.f});
-        if (sl == 0 && xlo) acc_add(n, xlo[s + Lx * tr]);
-        if (sl == hh - 1 && has) acc_add(n, xhi[s + Lx * tr]);
-        acc_sub_scaled(r, td, n);
-        acc_sub_cmul(r, dv, us[e]);
+        // the interface layers' u stands in for the neighbour outside the subdomain
+        const cdfl ul = !dl && xlo ? xlo[s + Lx * tr] : zero, uh = !dr && has ? xhi[s + Lx * tr] : zero;
+        const cdfl uc = us[e];
+        cdfl r = zero;
+        acc_sub_scaled(r, td, neighbours(us, ul, uh));
+        acc_sub_cmul(r, dv, uc);
         ru = scaled(suf, r);
         nu += cabs2(ru);
         if (!wdone) {
+          const cdfl wc = ws[e];
           r = ldq(qo + e);
-          acc_sub_scaled(r, td, neighbours(ws));
-          acc_sub_cmul(r, dv, ws[e]);
+          acc_sub_scaled(r, td, neighbours(ws, zero, zero));
+          acc_sub_cmul(r, dv, wc);
           rw = scaled(swf, r);
           nw += cabs2(rw);
         }
