@@ -73,6 +73,21 @@ __device__ __forceinline__ dfl fma(dfl a, dfl b, dfl c) {
   return dfl_fast(s, e2);
 }
 
+// acc + a*b without renormalisation: the product's hi part and its exact error
+// (TwoProduct) plus the cross terms; hi added to acc.hi by TwoSum; every error
+// term lands in acc.lo, which is not renormalised (it stays within a few ulp of
+// acc.hi, so TwoSum stays exact and acc.lo's own rounding is of the order
+// 2^-48 |acc|).  dfl_fast(acc.hi, acc.lo) at the end of a sum.
+__device__ __forceinline__ void dfl_mac(dfl& acc, dfl a, dfl b) {
+  float p, e, s, t;
+  dfl_two_prod(a.hi, b.hi, p, e);
+  e = __fmaf_rn(a.hi, b.lo, e);
+  e = __fmaf_rn(a.lo, b.hi, e);
+  dfl_two_sum(acc.hi, p, s, t);
+  acc.hi = s;
+  acc.lo = __fadd_rn(acc.lo, __fadd_rn(t, e));
+}
+
 // a / b: the float quotient, corrected once by the remainder a - q b
 __device__ __forceinline__ dfl operator/(dfl a, dfl b) {
   const float q1 = __fdiv_rn(a.hi, b.hi);

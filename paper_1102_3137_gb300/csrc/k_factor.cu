@@ -12,7 +12,13 @@
 // because every pivot block has a positive-definite imaginary part
 // (Im H_jj >= w_0 > 0 and -t^2 Im g_{s-1} is positive semi-definite), so
 // all Schur complements stay non-singular.
+#include <cooperative_groups.h>
+
+#include <type_traits>
+
 #include "dyson_common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -245,118 +251,140 @@ __global__ void __launch_bounds__(DY_THREADS) k_factor(Geo g, Bufs b) {
 }
 
 // ---------------------------------------------------------------- wide slices
-// 64 < W <= 256 (3D slabs): a W x W block no longer fits shared memory.  The
-// same recursion runs on global memory, which at these sizes stays in L2: the
-// forward g_s is formed and inverted in place in its final slot of b.g (or
-// b.g64), and the backward pass keeps G_{s+1,s+1} and the product g_s G_{s+1}
-// in two W x W matrices of a per-CTA workspace.  A persistent grid of
-// DY_FACTOR_CTAS CTAs walks the (subdomain, frequency) units, so the workspace
-// is bounded by the grid, not by K.
+// W > 64 (3D slabs, wide strips, one subdomain): a W x W block no longer fits
+// shared memory.  The same recursion runs on global memory, which at these sizes
+// stays in L2, as products of 32 x 32 tiles: the inverse g_s by the block form of
+// the symmetric sweep operator (gj_invert with 32 x 32 pivots: the pivot block
+// inverted in shared memory, the row panel, a rank-32 update of the upper tiles),
+// the backward pass as two W x W products.
+//
+// A (subdomain, frequency) unit is worked on by a cluster of C CTAs that share the
+// tiles of every phase, C the largest of 8, 4, 2, 1 that keeps the units within the
+// DY_FACTOR_CTAS CTAs of the persistent grid: 32 units of 128 x 128 blocks
+// (128 x 128 sites, p = 1) left 120 of the 152 SMs idle with one CTA each.
+constexpr int TB = 32, TP = 33;          // tile edge and padded row length in shared memory
 
-// In-place inverse of a complex symmetric global W x W matrix by the
-// symmetric sweep operator (see gj_invert): the upper triangle only, then
-// negation and mirror.  Step k caches column k (unscaled in prow, scaled by
-// the pivot inverse in fcol, -1/a_kk at fcol[k]) on chip.
 template <typename R>
-__device__ void gj_invert_global(cx<R>* A, int W, cx<R>* prow, cx<R>* fcol) {
-  using C = cx<R>;
-  const int n = W * W;
-  for (int k = 0; k < W; ++k) {
-    __syncthreads();                         // step k-1 finished by every thread
-    for (int e = threadIdx.x; e < W; e += DY_THREADS) {
-      const C piv = cinv(A[(size_t)k * W + k]);
-      const C a = (e < k) ? A[(size_t)e * W + k] : A[(size_t)k * W + e];
-      prow[e] = a;
-      fcol[e] = (e == k) ? -piv : a * piv;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < n; e += DY_THREADS) {
-      const int r = e / W, c = e - r * W;
-      if (c < r) continue;
-      if (r == k || c == k) A[e] = fcol[r == k ? c : r];
-      else A[e] = cfma(-fcol[r], prow[c], A[e]);
-    }
+__device__ __forceinline__ cx<R> mac(cx<R> a, cx<R> b, cx<R> acc) {
+  if constexpr (sizeof(R) == sizeof(double) && !std::is_same<R, dfl>::value) {
+    return cfma(a, b, acc);
+  } else {
+    // products by TwoProduct, sums by TwoSum, the low words not renormalised (see tile_done)
+    dfl_mac(acc.x, a.x, b.x);
+    dfl_mac(acc.x, dfl(-a.y.hi, -a.y.lo), b.y);
+    dfl_mac(acc.y, a.x, b.y);
+    dfl_mac(acc.y, a.y, b.x);
+    return acc;
   }
-  __syncthreads();
-  for (int e = threadIdx.x; e < n; e += DY_THREADS) {
-    const int r = e / W, c = e - r * W;
-    if (c >= r) A[e] = -A[e];
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < n; e += DY_THREADS) {
-    const int r = e / W, c = e - r * W;
-    if (c < r) A[e] = A[(size_t)c * W + r];
-  }
-  __syncthreads();
+}
+template <typename R>
+__device__ __forceinline__ cx<R> tile_done(cx<R> v) {
+  if constexpr (std::is_same<R, dfl>::value) return {dfl_fast(v.x.hi, v.x.lo), dfl_fast(v.y.hi, v.y.lo)};
+  else return v;
 }
 
-// C = base + scale * X Y for global W x W matrices (base may be null: C = X Y),
-// in 32 x 32 output tiles staged through shared memory; W need not be a
-// multiple of 32.  C must not alias X or Y.
 template <typename R>
-__device__ void gmem_matmul(cx<R>* C, const cx<R>* X, const cx<R>* Y, const cx<R>* base, R scale,
-                            int W, cx<R> (*tx)[32], cx<R> (*ty)[32]) {
-  using CC = cx<R>;
-  const int tid = threadIdx.x, lc = tid & 31, lr = tid >> 5;   // 8 row groups x 32 columns
-  const int nt = (W + 31) / 32;
-  for (int tile = 0; tile < nt * nt; ++tile) {
-    const int r0 = (tile / nt) * 32, c0 = (tile % nt) * 32;
-    CC acc[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-    for (int k0 = 0; k0 < W; k0 += 32) {
-      __syncthreads();                       // previous tiles fully read
+struct TileSmem {
+  cx<R> tx[TB][TP], ty[TB][TP], tp[TB][TP];
+  cx<R> prow[TB], fcol[TB];
+};
+
+// tile (r0, c0) of the row-major ld-wide matrix M (n x n; identity outside) to t, or
+// its transpose
+template <typename R, bool TR>
+__device__ __forceinline__ void tile_in(cx<R> (*t)[TP], const cx<R>* M, int n, int ld, int r0, int c0) {
+  const int lc = threadIdx.x & 31, lr = threadIdx.x >> 5;
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        const int r = lr + 8 * m;
-        tx[r][lc] = (r0 + r < W && k0 + lc < W) ? X[(size_t)(r0 + r) * W + k0 + lc] : CC{0, 0};
-        ty[r][lc] = (k0 + r < W && c0 + lc < W) ? Y[(size_t)(k0 + r) * W + c0 + lc] : CC{0, 0};
-      }
-      __syncthreads();
-#pragma unroll 8
-      for (int k = 0; k < 32; ++k) {
-        const CC yv = ty[k][lc];
+  for (int m = 0; m < 4; ++m) {
+    const int r = lr + 8 * m, gr = r0 + r, gc = c0 + lc;
+    const cx<R> v = gr < n && gc < n ? M[(size_t)gr * ld + gc] : (gr == gc ? cx<R>{1, 0} : cx<R>{0, 0});
+    if (TR) t[lc][r] = v;
+    else t[r][lc] = v;
+  }
+}
+// acc[m] += sum_k tx[lr + 8 m][k] ty[k][lc], renormalised every KR terms (the low
+// words stay small: without it the diagonal of 128 x 128 blocks lost a bit)
+template <typename R>
+__device__ __forceinline__ void tile_mac(const cx<R> (*tx)[TP], const cx<R> (*ty)[TP], cx<R> (&acc)[4]) {
+  const int lc = threadIdx.x & 31, lr = threadIdx.x >> 5;
+  constexpr int KR = 4;
+#pragma unroll 1
+  for (int k0 = 0; k0 < TB; k0 += KR) {
 #pragma unroll
-        for (int m = 0; m < 4; ++m) acc[m] = cfma(tx[lr + 8 * m][k], yv, acc[m]);
-      }
+    for (int k = k0; k < k0 + KR; ++k) {
+      const cx<R> y = ty[k][lc];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) acc[m] = mac<R>(tx[lr + 8 * m][k], y, acc[m]);
     }
+#pragma unroll
+    for (int m = 0; m < 4; ++m) acc[m] = tile_done<R>(acc[m]);
+  }
+}
+
+// tp <- inverse of the complex symmetric 32 x 32 tile tp (the sweep operator of
+// gj_invert, full tile)
+template <typename R>
+__device__ void tile_invert(TileSmem<R>& sm) {
+  const int lc = threadIdx.x & 31, lr = threadIdx.x >> 5;
+  for (int k = 0; k < TB; ++k) {
+    __syncthreads();
+    if (threadIdx.x < TB) {
+      const cx<R> piv = cinv(sm.tp[k][k]);
+      const cx<R> a = sm.tp[k][threadIdx.x];
+      sm.prow[threadIdx.x] = a;
+      sm.fcol[threadIdx.x] = (int)threadIdx.x == k ? -piv : a * piv;
+    }
+    __syncthreads();
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-      const int r = r0 + lr + 8 * m, c = c0 + lc;
-      if (r < W && c < W) {
-        const size_t e = (size_t)r * W + c;
-        C[e] = base ? base[e] + scale * acc[m] : acc[m];
-      }
+      const int r = lr + 8 * m;
+      if (r == k || lc == k) sm.tp[r][lc] = sm.fcol[r == k ? lc : r];
+      else sm.tp[r][lc] = cfma(-sm.fcol[r], sm.prow[lc], sm.tp[r][lc]);
     }
   }
+  __syncthreads();
+#pragma unroll
+  for (int m = 0; m < 4; ++m) sm.tp[lr + 8 * m][lc] = -sm.tp[lr + 8 * m][lc];
   __syncthreads();
 }
 
 // R: the recursion's arithmetic, binary64 (FP64 form) or double-float (mixed
-// form, R12: on the FP32 pipe), stored in b.g (FP64 form) or b.g64 (mixed: the
+// form, on the FP32 pipe), stored in b.g (FP64 form) or b.g64 (mixed: the
 // double-float factors, beside their complex64 copy in b.g for the sweeps).
 template <typename R, typename S>
-__global__ void __launch_bounds__(DY_THREADS) k_factor_big(Geo g, Bufs b, int K) {
+__global__ void __launch_bounds__(DY_THREADS, 2) k_factor_wide(Geo g, Bufs b, int K) {
   using C = cx<R>;
-  __shared__ C prow[DY_MAXW], fcol[DY_MAXW];
-  __shared__ C tx[32][32], ty[32][32];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  TileSmem<R>& sm = *reinterpret_cast<TileSmem<R>*>(smem_raw);
+  cg::cluster_group cl = cg::this_cluster();
   constexpr bool two = sizeof(S) != sizeof(double);
   static_assert(sizeof(C) == sizeof(cxd), "factor storage holds 16 bytes per entry");
-  const int W = g.W, Lx = g.Lx, T = g.T;
+  const int CN = (int)cl.num_blocks(), ci = (int)cl.block_rank();
+  const int clu = blockIdx.x / CN, nclu = gridDim.x / CN;
+  const int W = g.W, Lx = g.Lx, T = g.T, nt = (W + TB - 1) / TB;
   const size_t n = (size_t)W * W;
   const R t = (R)g.t, t2 = (R)(g.t * g.t);
-  C* Gw = reinterpret_cast<C*>(b.fwork) + (size_t)blockIdx.x * 2 * n;   // G_{s+1,s+1}
-  C* Pw = Gw + n;                                                    // g_s G_{s+1,s+1}
-  for (int unit = blockIdx.x; unit < g.p * K; unit += gridDim.x) {
+  C* Gw = reinterpret_cast<C*>(b.fwork) + (size_t)clu * CN * 2 * n;     // G_{s+1,s+1}
+  C* Pw = Gw + n;                        // g_s G_{s+1,s+1}; during the inversion the panels F and O
+  C* Fb = Pw;                            // [nt][32][32] F_i = A_ik A_kk^-1
+  C* Ob = Pw + (size_t)nt * TB * TB;     // [nt][32][32] A_ik before
+  const int lc = threadIdx.x & 31, lr = threadIdx.x >> 5;
+  const int gt = ci * DY_THREADS + threadIdx.x, gn = CN * DY_THREADS;
+  auto sync = [&]() {
+    if (CN > 1) cl.sync();
+    else __syncthreads();
+  };
+  for (int unit = clu; unit < g.p * K; unit += nclu) {
     const int i = unit % g.p, kf = unit / g.p, w = T * g.h[i];
     const size_t uoff = ((size_t)kf * g.p + i) * (size_t)Lx * n;
     C* gout = reinterpret_cast<C*>(two ? b.g64 : b.g) + uoff;
     cx<S>* gsw = reinterpret_cast<cx<S>*>(b.g) + uoff;
     cxd* dB = b.diagB + (size_t)kf * g.Ndd + (size_t)i * Lx * W;
-    // forward: g_s = (D_s - t^2 g_{s-1})^-1, formed and inverted in place
+    // ---- forward: g_s = (D_s - t^2 g_{s-1})^-1, formed and inverted in place
     for (int s = 0; s < Lx; ++s) {
       C* A = gout + (size_t)s * n;
       const C* Ap = A - n;
-      __syncthreads();                       // g_{s-1} complete
-      for (int e = threadIdx.x; e < (int)n; e += DY_THREADS) {
+      for (int e = gt; e < (int)n; e += gn) {
         const int r = e / W, c = e - r * W;
         C v = {0, 0};
         if (r < w && c < w) {
@@ -367,45 +395,171 @@ __global__ void __launch_bounds__(DY_THREADS) k_factor_big(Geo g, Bufs b, int K)
             v.x += t;
           }
         } else if (r == c) {
-          v = C{1, 0};                       // padding: identity, inverted to itself
+          v = C{1, 0};                   // padding: identity, inverted to itself
         }
         A[e] = v;
       }
-      gj_invert_global<R>(A, W, prow, fcol);
-      for (int e = threadIdx.x; e < (int)n; e += DY_THREADS) {
-        const int r = e / W, c = e - r * W;
-        C v = A[e];
-        if (r >= w || c >= w) {
-          v = C{0, 0};
-          A[e] = v;
+      sync();
+      for (int k = 0; k < nt; ++k) {
+        // pivot block, by every CTA for itself
+        tile_in<R, false>(sm.tp, A, W, W, k * TB, k * TB);
+        tile_invert<R>(sm);
+        // panel F_i = A_ik A_kk^-1 (kept beside the old A_ik for the update)
+        for (int q = ci; q < nt - 1; q += CN) {
+          const int ii = q < k ? q : q + 1;
+          if (ii < k) tile_in<R, false>(sm.tx, A, W, W, ii * TB, k * TB);
+          else tile_in<R, true>(sm.tx, A, W, W, k * TB, ii * TB);
+          __syncthreads();
+          C acc[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+          tile_mac<R>(sm.tx, sm.tp, acc);
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            const int r = lr + 8 * m;
+            const C v = tile_done<R>(acc[m]);
+            Fb[((size_t)ii * TB + r) * TB + lc] = v;
+            Ob[((size_t)ii * TB + r) * TB + lc] = sm.tx[r][lc];
+          }
+          __syncthreads();
         }
-        if (two) gsw[(size_t)s * n + e] = cconv<S>(v);
+        sync();                          // panels complete, nobody reads A_.k any more
+        // A_ij -= F_i A_kj on the upper tiles, and the new row and column k
+        int tile = 0;
+        for (int ii = 0; ii < nt; ++ii) {
+          for (int jj = ii; jj < nt; ++jj, ++tile) {
+            if (tile % CN != ci) continue;
+            const int r0 = ii * TB, c0 = jj * TB;
+            if (ii == k || jj == k) {
+              const int o = ii == k ? jj : ii;
+#pragma unroll
+              for (int m = 0; m < 4; ++m) {
+                const int r = lr + 8 * m;
+                if (r0 + r < W && c0 + lc < W) {
+                  C v;
+                  if (ii == jj) v = -sm.tp[r][lc];
+                  else if (jj == k) v = Fb[((size_t)o * TB + r) * TB + lc];
+                  else v = Fb[((size_t)o * TB + lc) * TB + r];      // row k: F_j transposed
+                  A[(size_t)(r0 + r) * W + c0 + lc] = v;
+                }
+              }
+              continue;
+            }
+            tile_in<R, false>(sm.tx, Fb + (size_t)ii * TB * TB, TB, TB, 0, 0);
+            tile_in<R, true>(sm.ty, Ob + (size_t)jj * TB * TB, TB, TB, 0, 0);
+            __syncthreads();
+            C acc[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+              const int r = r0 + lr + 8 * m, c = c0 + lc;
+              // double-float: the products summed first (the smaller error), binary64: from A_ij
+              const bool from = !std::is_same<R, dfl>::value && r < W && c < W;
+              acc[m] = from ? -A[(size_t)r * W + c] : C{0, 0};
+            }
+            tile_mac<R>(sm.tx, sm.ty, acc);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+              const int r = r0 + lr + 8 * m, c = c0 + lc;
+              if (r < W && c < W) {
+                C* d = A + (size_t)r * W + c;
+                *d = std::is_same<R, dfl>::value ? *d - acc[m] : -acc[m];
+              }
+            }
+            __syncthreads();
+          }
+        }
+        sync();
       }
+      // -(-A^-1), mirrored from the upper triangle, zero on the padding
+      for (int e = gt; e < (int)n; e += gn) {
+        const int r = e / W, c = e - r * W;
+        if (c < r) continue;
+        C v = -A[e];
+        if (r >= w || c >= w) v = C{0, 0};
+        const size_t e2 = (size_t)c * W + r;
+        A[e] = v;
+        A[e2] = v;
+        if (two) {
+          const cx<S> vs = cconv<S>(v);
+          gsw[(size_t)s * n + e] = vs;
+          gsw[(size_t)s * n + e2] = vs;
+        }
+      }
+      sync();
     }
-    __syncthreads();
-    // backward: Gw holds G_{s+1,s+1}
+    // ---- backward: Gw holds G_{s+1,s+1}
     const C* glast = gout + (size_t)(Lx - 1) * n;
-    for (int e = threadIdx.x; e < (int)n; e += DY_THREADS) Gw[e] = glast[e];
-    for (int r = threadIdx.x; r < W; r += DY_THREADS)
+    for (int e = gt; e < (int)n; e += gn) Gw[e] = glast[e];
+    for (int r = gt; r < W; r += gn)
       dB[(size_t)(Lx - 1) * W + r] = (r < w) ? cconv<double>(glast[(size_t)r * W + r]) : cxd{0, 0};
+    sync();
+    // out = X Y on this CTA's tiles, the tiles' k range staged one 32-block at a time with
+    // the next block's loads in flight
+    auto product = [&](const C* X, const C* Y, int r0, int c0, C (&acc)[4]) {
+      C px[4], py[4];
+      auto fetch = [&](int k0) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const int r = lr + 8 * m;
+          px[m] = (r0 + r < W && k0 + lc < W) ? X[(size_t)(r0 + r) * W + k0 + lc] : C{0, 0};
+          py[m] = (k0 + r < W && c0 + lc < W) ? Y[(size_t)(k0 + r) * W + c0 + lc] : C{0, 0};
+        }
+      };
+      fetch(0);
+      for (int k0 = 0; k0 < W; k0 += TB) {
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          sm.tx[lr + 8 * m][lc] = px[m];
+          sm.ty[lr + 8 * m][lc] = py[m];
+        }
+        __syncthreads();
+        if (k0 + TB < W) fetch(k0 + TB);
+        tile_mac<R>(sm.tx, sm.ty, acc);
+      }
+    };
     for (int s = Lx - 2; s >= 0; --s) {
       const C* gs = gout + (size_t)s * n;
-      gmem_matmul<R>(Pw, gs, Gw, nullptr, R(0), W, tx, ty);   // g_s G_{s+1}
-      if (b.offB) {                                           // diag of G_{s,s+1} = -t g_s G_{s+1}
-        cxd* oB = b.offB + ((size_t)kf * g.p + i) * (size_t)Lx * W + (size_t)s * W;
-        for (int r = threadIdx.x; r < W; r += DY_THREADS)
-          oB[r] = (r < w) ? cconv<double>((-t) * Pw[(size_t)r * W + r]) : cxd{0, 0};
+      for (int tile = ci; tile < nt * nt; tile += CN) {       // P = g_s G_{s+1}
+        const int r0 = (tile / nt) * TB, c0 = (tile % nt) * TB;
+        C acc[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+        product(gs, Gw, r0, c0, acc);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const int r = r0 + lr + 8 * m, c = c0 + lc;
+          if (r >= W || c >= W) continue;
+          const C v = tile_done<R>(acc[m]);
+          Pw[(size_t)r * W + c] = v;
+          if (r == c && b.offB)                               // diag of G_{s,s+1} = -t g_s G_{s+1}
+            b.offB[((size_t)kf * g.p + i) * (size_t)Lx * W + (size_t)s * W + r] =
+                (r < w) ? cconv<double>((-t) * v) : cxd{0, 0};
+        }
       }
-      gmem_matmul<R>(Gw, Pw, gs, gs, t2, W, tx, ty);          // g_s + t^2 g_s G_{s+1} g_s
-      for (int r = threadIdx.x; r < W; r += DY_THREADS)
-        dB[(size_t)s * W + r] = (r < w) ? cconv<double>(Gw[(size_t)r * W + r]) : cxd{0, 0};
+      sync();
+      int tile = 0;
+      for (int ii = 0; ii < nt; ++ii) {                       // G_ss = g_s + t^2 P g_s, upper tiles
+        for (int jj = ii; jj < nt; ++jj, ++tile) {
+          if (tile % CN != ci) continue;
+          const int r0 = ii * TB, c0 = jj * TB;
+          C acc[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+          product(Pw, gs, r0, c0, acc);
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            const int r = r0 + lr + 8 * m, c = c0 + lc;
+            if (r >= W || c >= W) continue;
+            const C v = gs[(size_t)r * W + c] + t2 * tile_done<R>(acc[m]);
+            Gw[(size_t)r * W + c] = v;
+            if (ii != jj) Gw[(size_t)c * W + r] = v;
+            if (r == c) dB[(size_t)s * W + r] = (r < w) ? cconv<double>(v) : cxd{0, 0};
+          }
+        }
+      }
+      sync();
     }
     if (i == g.p - 1) {
       cxd* dI = b.diagB + (size_t)kf * g.Ndd + g.ifc_off;
       const size_t m = (size_t)(g.p - 1) * g.A;
-      for (size_t e = threadIdx.x; e < m; e += DY_THREADS) dI[e] = cxd{0, 0};
+      for (size_t e = gt; e < m; e += gn) dI[e] = cxd{0, 0};
     }
-    __syncthreads();                         // workspace reads done before the next unit
+    sync();                              // workspace reads done before the next unit
   }
 }
 
@@ -489,12 +643,28 @@ cudaError_t launch_factor(const Geo& g, const Bufs& b, int K, cudaStream_t st) {
   }
   if (g.W > DY_MAXW_SMEM) {
     // wide slices: the recursion in global memory (binary64, or double-float in the
-    // mixed form)
+    // mixed form), a cluster of CTAs per unit where there are few units
     if constexpr (sizeof(cx<R>) == sizeof(cxd)) {
       if (g.W > DY_MAXW || !b.fwork) return cudaErrorInvalidValue;
-      int units = g.p * K;
-      k_factor_big<R, S><<<units < DY_FACTOR_CTAS ? units : DY_FACTOR_CTAS, DY_THREADS, 0, st>>>(g, b, K);
-      return cudaGetLastError();
+      const int units = g.p * K;
+      int C = 8;
+      while (C > 1 && units * C > DY_FACTOR_CTAS) C /= 2;
+      const int clusters = units < DY_FACTOR_CTAS / C ? units : DY_FACTOR_CTAS / C;
+      const size_t smem = sizeof(TileSmem<R>);
+      cudaError_t e = raise_smem_limit((const void*)k_factor_wide<R, S>, smem);
+      if (e != cudaSuccess) return e;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(clusters * C);
+      cfg.blockDim = dim3(DY_THREADS);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = st;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = C;
+      attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      return cudaLaunchKernelEx(&cfg, k_factor_wide<R, S>, g, b, K);
     } else {
       return cudaErrorInvalidValue;
     }

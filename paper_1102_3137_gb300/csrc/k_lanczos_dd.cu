@@ -55,25 +55,11 @@ constexpr double REORTH_ETA = 0.05;
 
 __device__ __forceinline__ cdfl czero() { return {dfl(0.f, 0.f), dfl(0.f, 0.f)}; }
 
-// acc + a*b for double-floats: the product's hi part and its exact error
-// (TwoProduct) plus the cross terms; hi added to acc.hi by TwoSum; every
-// error term lands in acc.lo, which is not renormalised (it stays within a
-// few ulp of acc.hi, so TwoSum stays exact and acc.lo's own rounding is of
-// the order 2^-48 |acc|).
-__device__ __forceinline__ void dmac(dfl& acc, dfl a, dfl b) {
-  float p, e, s, t;
-  dfl_two_prod(a.hi, b.hi, p, e);
-  e = __fmaf_rn(a.hi, b.lo, e);
-  e = __fmaf_rn(a.lo, b.hi, e);
-  dfl_two_sum(acc.hi, p, s, t);
-  acc.hi = s;
-  acc.lo = __fadd_rn(acc.lo, __fadd_rn(t, e));
-}
 __device__ __forceinline__ void cmac(cdfl& acc, const cdfl& a, const cdfl& b) {
-  dmac(acc.x, a.x, b.x);
-  dmac(acc.x, dfl(-a.y.hi, -a.y.lo), b.y);
-  dmac(acc.y, a.x, b.y);
-  dmac(acc.y, a.y, b.x);
+  dfl_mac(acc.x, a.x, b.x);
+  dfl_mac(acc.x, dfl(-a.y.hi, -a.y.lo), b.y);
+  dfl_mac(acc.y, a.x, b.y);
+  dfl_mac(acc.y, a.y, b.x);
 }
 // renormalised sum / difference of two double-floats
 __device__ __forceinline__ cdfl cadd(const cdfl& a, const cdfl& b) { return {a.x + b.x, a.y + b.y}; }
