@@ -277,6 +277,32 @@ __device__ __forceinline__ int sub_nat(const Geo& g, int i, int s, int j) {
 // for a large plan may be replayed after a small plan ran, so the limit only grows.
 cudaError_t raise_smem_limit(const void* func, size_t bytes);
 
+// CTAs that share one unit of a tiled factorization kernel: the largest of 8, 4, 2,
+// 1 that keeps the units within the DY_FACTOR_CTAS CTAs of one wave.
+inline int unit_cluster(int units) {
+  int C = 8;
+  while (C > 1 && (long long)units * C > DY_FACTOR_CTAS) C /= 2;
+  return C;
+}
+// Launch with clusters of C CTAs of DY_THREADS threads along x.
+template <typename Kern, typename... Args>
+cudaError_t launch_clustered(Kern kern, dim3 grid, int C, size_t smem, cudaStream_t st, Args... args) {
+  cudaError_t e = raise_smem_limit((const void*)kern, smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(DY_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = C;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // Record msg as this thread's dyson_last_error() and return code.
 int dyson_internal_fail(int code, const std::string& msg);
 struct dyson_plan_s;

@@ -647,24 +647,9 @@ cudaError_t launch_factor(const Geo& g, const Bufs& b, int K, cudaStream_t st) {
     if constexpr (sizeof(cx<R>) == sizeof(cxd)) {
       if (g.W > DY_MAXW || !b.fwork) return cudaErrorInvalidValue;
       const int units = g.p * K;
-      int C = 8;
-      while (C > 1 && units * C > DY_FACTOR_CTAS) C /= 2;
+      const int C = unit_cluster(units);
       const int clusters = units < DY_FACTOR_CTAS / C ? units : DY_FACTOR_CTAS / C;
-      const size_t smem = sizeof(TileSmem<R>);
-      cudaError_t e = raise_smem_limit((const void*)k_factor_wide<R, S>, smem);
-      if (e != cudaSuccess) return e;
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(clusters * C);
-      cfg.blockDim = dim3(DY_THREADS);
-      cfg.dynamicSmemBytes = smem;
-      cfg.stream = st;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = C;
-      attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      return cudaLaunchKernelEx(&cfg, k_factor_wide<R, S>, g, b, K);
+      return launch_clustered(k_factor_wide<R, S>, dim3(clusters * C), C, sizeof(TileSmem<R>), st, g, b, K);
     } else {
       return cudaErrorInvalidValue;
     }

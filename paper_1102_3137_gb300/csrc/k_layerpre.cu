@@ -25,10 +25,9 @@
 //   k_surface_g  keeps the boundary columns of G_{s,s'} in global memory
 //                (one warp per column, the column broadcast through shared
 //                memory), and
-//   k_layer_inv_g forms S_ll in place of P_top(l) and inverts it there by
-//                block Gauss-Jordan on 32 x 32 blocks (pivot block by the sweep
-//                operator in shared memory, row panel, rank-32 update of the
-//                rest, column panel), then writes the symmetrised inverse.
+//   k_layer_inv_g forms S_ll in place of P_top(l) and inverts it there by the
+//                block sweep operator (32 x 32 pivots, rank-32 updates of the
+//                upper 64 x 64 tiles), then writes the mirrored inverse.
 // 3D slabs (slice width W = T h, T = Ly > 1) have interface layers of
 // A = Lx T sites, S_ll is A x A (in-plane hopping along x and y), and
 //   k_surface_3d forms P_bot(i), P_top(i) from the factorization's
@@ -38,7 +37,7 @@
 //                of each slice c, with 32 x 32 tiles through shared memory
 //                multiplied on the tensor cores (3xTF32; persistent grid, one
 //                (slab, frequency) at a time per CTA);
-//   k_layer_inv_g  inverts the A x A blocks as above (A <= 1024).
+//   k_layer_inv_g  inverts the A x A blocks (A <= 1024).
 #include <type_traits>
 
 #include "solve_device.cuh"
@@ -339,21 +338,16 @@ __global__ void __launch_bounds__(DY_THREADS) k_surface_g(Geo g, Bufs b) {
   }
 }
 
-// S_ll and its inverse for lines longer than the shared-memory form takes, in
-// place of P_top(l) (only line l reads it): A = S_ll, then block Gauss-Jordan
-// with NB x NB blocks,
-//   P = A_kk^-1;  A_kj <- P A_kj;  A_ij <- A_ij - A_ik A_kj;  A_ik <- -A_ik P;  A_kk <- P
-// (i, j != k), which leaves A^-1; pivots come from the sweep operator on the
-// diagonal block (Im S_ll > 0 keeps them away from zero).  The symmetrised
-// inverse is written in the form's precision.
 // C (M x N, row stride ldc) = alpha X Y (+ D), X: M x K, Y: K x N, D: M x N, all in
 // global memory in any of binary64 / complex64 (converted to complex64 on load),
 // 32 x 32 tiles staged through shared memory and multiplied on the tensor cores
 // (3xTF32, binary32 accuracy): warp w forms the 16 x 8 sub-tile at rows 16 (w / 4),
-// columns 8 (w % 4) of each output tile.  Callers keep C apart from X, Y.
+// columns 8 (w % 4) of each output tile.  Callers keep C apart from X, Y.  The
+// output tiles are shared out over CN CTAs (this one is ci); the next k block's
+// loads are in flight during a block's products.
 template <typename TX, typename TY, typename TD>
 __device__ void gmm_c64(cxf_* C, int ldc, const TX* X, int ldx, const TY* Y, int ldy, const TD* D, int ldd,
-                        int M, int N, int K, float alpha, cxf_ (&tx)[32][32], cxf_ (&ty)[32][32]) {
+                        int M, int N, int K, float alpha, cxf_ (&tx)[32][32], cxf_ (&ty)[32][32], int ci, int CN) {
   auto f32 = [](auto v) -> cxf_ {
     using V = decltype(v);
     if constexpr (std::is_same_v<V, cxd>) return cxf_{d2f_bits(v.x), d2f_bits(v.y)};
@@ -363,51 +357,71 @@ __device__ void gmm_c64(cxf_* C, int ldc, const TX* X, int ldx, const TY* Y, int
   static_assert(DY_THREADS == 256, "eight 16 x 8 tensor-core tiles per 32 x 32 output tile");
   const int lr = threadIdx.x >> 5, lc = threadIdx.x & 31;
   const int tm = 16 * (lr >> 2), tn = 8 * (lr & 3);
-  for (int r0 = 0; r0 < M; r0 += 32)
-    for (int c0 = 0; c0 < N; c0 += 32) {
-      tc::CTile acc = {};
-      for (int k0 = 0; k0 < K; k0 += 32) {
-        __syncthreads();                     // previous tiles fully read
+  const int nr = (M + 31) / 32, ncol = (N + 31) / 32;
+  for (int tile = ci; tile < nr * ncol; tile += CN) {
+    const int r0 = (tile / ncol) * 32, c0 = (tile % ncol) * 32;
+    tc::CTile acc = {};
+    cxf_ px[4], py[4];
+    auto fetch = [&](int k0) {
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          const int r = lr + 8 * m;
-          tx[r][lc] = (r0 + r < M && k0 + lc < K) ? f32(X[(size_t)(r0 + r) * ldx + k0 + lc]) : cxf_{0.f, 0.f};
-          ty[r][lc] = (k0 + r < K && c0 + lc < N) ? f32(Y[(size_t)(k0 + r) * ldy + c0 + lc]) : cxf_{0.f, 0.f};
-        }
-        __syncthreads();
-        tc::cgemm_tile_3xtf32(acc, &tx[0][0], &ty[0][0], 32, tm, tn);
+      for (int m = 0; m < 4; ++m) {
+        const int r = lr + 8 * m;
+        px[m] = (r0 + r < M && k0 + lc < K) ? f32(X[(size_t)(r0 + r) * ldx + k0 + lc]) : cxf_{0.f, 0.f};
+        py[m] = (k0 + r < K && c0 + lc < N) ? f32(Y[(size_t)(k0 + r) * ldy + c0 + lc]) : cxf_{0.f, 0.f};
       }
+    };
+    fetch(0);
+    for (int k0 = 0; k0 < K; k0 += 32) {
+      __syncthreads();                     // previous tiles fully read
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        int r, c;
-        tc::tile_pos(e, tm, tn, r, c);
-        if (r0 + r < M && c0 + c < N) {
-          cxf_ v = {alpha * acc.re[e], alpha * acc.im[e]};
-          if (D) v = v + f32(D[(size_t)(r0 + r) * ldd + c0 + c]);
-          C[(size_t)(r0 + r) * ldc + c0 + c] = v;
-        }
+      for (int m = 0; m < 4; ++m) {
+        tx[lr + 8 * m][lc] = px[m];
+        ty[lr + 8 * m][lc] = py[m];
+      }
+      __syncthreads();
+      if (k0 + 32 < K) fetch(k0 + 32);
+      tc::cgemm_tile_3xtf32(acc, &tx[0][0], &ty[0][0], 32, tm, tn);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      int r, c;
+      tc::tile_pos(e, tm, tn, r, c);
+      if (r0 + r < M && c0 + c < N) {
+        cxf_ v = {alpha * acc.re[e], alpha * acc.im[e]};
+        if (D) v = v + f32(D[(size_t)(r0 + r) * ldd + c0 + c]);
+        C[(size_t)(r0 + r) * ldc + c0 + c] = v;
       }
     }
-  __syncthreads();
+  }
 }
 
 // Surface Green's functions of 3D slabs (see the top of the file).  Chains are kept
 // as one W x NV matrix per CTA, NV = 2 Lx T columns: [side][slice c][boundary column b]
 // (side 0 top, 1 bottom), updated by one product per step into the other half of
 // the ping-pong pair.  G_{s+1,s+1} and the product g_s G_{s+1,s+1} (complex64) use
-// the factor's per-CTA workspace, free once the factorization has run.
+// the factor's workspace, free once the factorization has run.  A unit's products
+// are shared by a cluster of CTAs (as in k_factor_wide): with one CTA a unit the 64
+// units of 24^3 x 16 kept 64 SMs waiting on their tiles' loads.
 template <typename FT>   // the factors' element: binary64 (FP64 form) or double-float (mixed)
-__global__ void __launch_bounds__(DY_THREADS) k_surface_3d(Geo g, Bufs b, int K) {
+__global__ void __launch_bounds__(DY_THREADS, 2) k_surface_3d(Geo g, Bufs b, int K) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int CN = (int)cl.num_blocks(), ci = (int)cl.block_rank();
+  const int clu = blockIdx.x / CN, nclu = gridDim.x / CN;
+  const int gt = ci * DY_THREADS + threadIdx.x, gn = CN * DY_THREADS;
+  auto sync = [&]() {
+    if (CN > 1) cl.sync();
+    else __syncthreads();
+  };
   __shared__ __align__(16) cxf_ tx[32][32];
   __shared__ __align__(16) cxf_ ty[32][32];
   const int W = g.W, Lx = g.Lx, T = g.T, A = g.A;
   const size_t n = (size_t)W * W, NV = (size_t)2 * Lx * T;
-  cxf_* Gd = reinterpret_cast<cxf_*>(b.fwork + (size_t)blockIdx.x * 2 * n);   // G_{s+1,s+1}
+  cxf_* Gd = reinterpret_cast<cxf_*>(b.fwork + (size_t)clu * 2 * n);   // G_{s+1,s+1}
   cxf_* Tm = Gd + n;
-  cxf_* Va = b.lpw + (size_t)blockIdx.x * 2 * W * NV;
+  cxf_* Va = b.lpw + (size_t)clu * 2 * W * NV;
   cxf_* Vb = Va + (size_t)W * NV;
   const float t = d2f_bits(g.t), t2 = t * t;
-  for (int unit = blockIdx.x; unit < g.p * K; unit += gridDim.x) {
+  for (int unit = clu; unit < g.p * K; unit += nclu) {
     const int i = unit % g.p, f = unit / g.p, w = T * g.h[i];
     const FT* gs = reinterpret_cast<const FT*>(b.g64 ? (const void*)b.g64 : b.g) + ((size_t)f * g.p + i) * (size_t)Lx * n;
     cxf_* P[2] = {b.lpt + (((size_t)f * g.p + i) * 2 + 0) * (size_t)A * A,
@@ -426,15 +440,16 @@ __global__ void __launch_bounds__(DY_THREADS) k_surface_3d(Geo g, Bufs b, int K)
         for (int sd = 0; sd < 2; ++sd) {
           if (!need[sd]) continue;
           const size_t off = (size_t)sd * Lx * T + c0;
-          gmm_c64(Vn + off, (int)NV, g_s, W, V + off, (int)NV, (const cxf_*)nullptr, 0, W, nc, W, -t, tx, ty);
+          gmm_c64(Vn + off, (int)NV, g_s, W, V + off, (int)NV, (const cxf_*)nullptr, 0, W, nc, W, -t, tx, ty, ci, CN);
         }
+        sync();
         cxf_* tmp = V;
         V = Vn;
         Vn = tmp;
         // P[s][c] = rows bnd(s) of the chains, and its mirror (G is complex symmetric)
         for (int sd = 0; sd < 2; ++sd) {
           if (!need[sd]) continue;
-          for (int e = threadIdx.x; e < T * nc; e += DY_THREADS) {
+          for (int e = gt; e < T * nc; e += gn) {
             const int ra = e / nc, q = e - ra * nc;            // row b_s, chain column (c, b_c)
             const int c = s + 1 + q / T, bc = q % T;
             const cxf_ v = V[(size_t)bj(sd, ra) * NV + (size_t)sd * Lx * T + c0 + q];
@@ -446,49 +461,70 @@ __global__ void __launch_bounds__(DY_THREADS) k_surface_3d(Geo g, Bufs b, int K)
       }
       // G_ss = g_s + t^2 g_s G_{s+1,s+1} g_s  (g_{Lx-1} itself at the end of the slab)
       if (s == Lx - 1) {
-        for (size_t e = threadIdx.x; e < n; e += DY_THREADS) {
+        for (size_t e = gt; e < n; e += gn) {
           if constexpr (std::is_same_v<FT, cxd>) Gd[e] = cxf_{d2f_bits(g_s[e].x), d2f_bits(g_s[e].y)};
           else Gd[e] = cxf_{g_s[e].x.hi + g_s[e].x.lo, g_s[e].y.hi + g_s[e].y.lo};
         }
-        __syncthreads();
       } else {
-        gmm_c64(Tm, W, g_s, W, Gd, W, (const cxf_*)nullptr, 0, W, W, W, 1.f, tx, ty);
-        gmm_c64(Gd, W, Tm, W, g_s, W, g_s, W, W, W, W, t2, tx, ty);
+        gmm_c64(Tm, W, g_s, W, Gd, W, (const cxf_*)nullptr, 0, W, W, W, 1.f, tx, ty, ci, CN);
+        sync();
+        gmm_c64(Gd, W, Tm, W, g_s, W, g_s, W, W, W, W, t2, tx, ty, ci, CN);
       }
+      sync();
       // start the chains of column c = s, and the diagonal block P[s][s]
       for (int sd = 0; sd < 2; ++sd) {
         if (!need[sd]) continue;
-        for (int e = threadIdx.x; e < W * T; e += DY_THREADS) {
+        for (int e = gt; e < W * T; e += gn) {
           const int r = e / T, bc = e - r * T;
           V[(size_t)r * NV + (size_t)sd * Lx * T + (size_t)s * T + bc] = Gd[(size_t)r * W + bj(sd, bc)];
         }
-        for (int e = threadIdx.x; e < T * T; e += DY_THREADS) {
+        for (int e = gt; e < T * T; e += gn) {
           const int ra = e / T, bc = e - ra * T;
           P[sd][((size_t)s + (size_t)Lx * ra) * A + (size_t)s + (size_t)Lx * bc] = Gd[(size_t)bj(sd, ra) * W + bj(sd, bc)];
         }
       }
-      __syncthreads();
+      sync();
     }
   }
 }
 
+// S_ll and its inverse for layers larger than the shared-memory form takes, in
+// place of P_top(l) (only line l reads it): A = S_ll, then the block form of the
+// symmetric sweep operator with NB x NB pivots on the upper 64 x 64 tiles,
+//   P = A_kk^-1;  F_i = A_ik P;  A_ij -= F_i A_kj;  A_ik <- F_i;  A_kk <- -P   (i, j != k),
+// which leaves -A^-1 (pivots by the sweep operator on the diagonal block; Im S_ll > 0
+// keeps them away from zero), and is written mirrored in the form's precision.
+// F_i and the old A_ik go through P_bot(l+1)'s space (read once, while A is formed),
+// k-major, so that a tile's update reads 64 consecutive entries of each.
+// A rank-32 update of a 64 x 64 tile is 2 x 2 KB in and 32 KB out and back for 524 k
+// FMAs: 16 bytes a clock and SM, below the HBM share, so the matrix may stream.  Each
+// thread holds 4 x 4 complex accumulators in binary32 (64 FMAs for four 16-byte
+// shared loads).  The CTAs of a cluster share the tiles of one matrix (as many as keep
+// the grid within DY_FACTOR_CTAS): 7 x 16 matrices of 1024 x 1024 had one SM each.
 constexpr int LINV_NB = 32;
 template <typename R>
-__global__ void __launch_bounds__(DY_THREADS) k_layer_inv_g(Geo g, Bufs b) {
-  __shared__ __align__(16) cxf_ Pk[LINV_NB * LINV_NB];
-  __shared__ __align__(16) cxf_ X[LINV_NB * LINV_NB];
-  __shared__ __align__(16) cxf_ Y[LINV_NB * LINV_NB];
-  __shared__ cxf_ prow[LINV_NB], fcol[LINV_NB];
-  constexpr int NB = LINV_NB;
-  // the layer has A = Lx T sites (T = 1 in 2D), layer index a = x + Lx y; below,
-  // "Lx" is the matrix dimension A
-  const int l = blockIdx.x, f = blockIdx.y, Lx = g.A, lx = g.Lx;
-  const size_t n2 = (size_t)Lx * Lx;
+__global__ void __launch_bounds__(DY_THREADS, 2) k_layer_inv_g(Geo g, Bufs b) {
+  constexpr int NB = LINV_NB, TU = 64;
+  __shared__ __align__(16) cxf_ Pk[NB * NB];
+  __shared__ __align__(16) cxf_ FO[2][NB][TU];               // F and O of a tile, k-major
+  __shared__ cxf_ prow[NB], fcol[NB];
+  cxf_ (*tx)[NB + 1] = reinterpret_cast<cxf_ (*)[NB + 1]>(&FO[0][0][0]);   // panel tile (before the update)
+  static_assert(sizeof(cxf_) * NB * (NB + 1) <= sizeof(FO), "the panel tile shares the update tiles' space");
+  cg::cluster_group cl = cg::this_cluster();
+  const int CN = (int)cl.num_blocks(), ci = (int)cl.block_rank();
+  auto sync = [&]() {
+    if (CN > 1) cl.sync();
+    else __syncthreads();
+  };
+  const int l = blockIdx.x / CN, f = blockIdx.y, n = g.A, lx = g.Lx;   // layer index a = x + Lx y
+  const size_t n2 = (size_t)n * n;
   cxf_* A = b.lpt + (((size_t)f * g.p + l) * 2 + 0) * n2;          // P_top(l), overwritten
-  const cxf_* Pb = b.lpt + (((size_t)f * g.p + l + 1) * 2 + 1) * n2;
+  cxf_* Pb = b.lpt + (((size_t)f * g.p + l + 1) * 2 + 1) * n2;     // P_bot(l+1), then F and O
+  cxf_ *Ft = Pb, *Ot = Pb + (size_t)NB * n;                        // [NB][n] each
   const float t = d2f_bits(g.t), t2 = t * t;
-  for (size_t e = threadIdx.x; e < n2; e += DY_THREADS) {
-    const int r = (int)(e / Lx), c = (int)(e - (size_t)r * Lx);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  for (size_t e = (size_t)ci * DY_THREADS + tid; e < n2; e += (size_t)CN * DY_THREADS) {
+    const int r = (int)(e / n), c = (int)(e - (size_t)r * n);
     cxf_ v = {0.f, 0.f};
     if (r == c) {
       const cxd d = dyson_diag(g, b, f, r + g.A * g.ylayer[l]);
@@ -498,80 +534,96 @@ __global__ void __launch_bounds__(DY_THREADS) k_layer_inv_g(Geo g, Bufs b) {
     }
     A[e] = cfma(cxf_{-t2, 0.f}, A[e] + Pb[e], v);
   }
-  const int nbk = (Lx + NB - 1) / NB;
-  // load / store a block (rows r0.., cols c0..), zero-padded past Lx (identity on the diagonal pad)
-  auto ld = [&](cxf_* T, int r0, int c0, bool diag) {
-    for (int e = threadIdx.x; e < NB * NB; e += DY_THREADS) {
-      const int r = e / NB, c = e - r * NB;
-      cxf_ v = {0.f, 0.f};
-      if (r0 + r < Lx && c0 + c < Lx) v = A[(size_t)(r0 + r) * Lx + c0 + c];
-      else if (diag && r == c) v = cxf_{1.f, 0.f};
-      T[e] = v;
-    }
-  };
-  auto st = [&](const cxf_* T, int r0, int c0) {
-    for (int e = threadIdx.x; e < NB * NB; e += DY_THREADS) {
-      const int r = e / NB, c = e - r * NB;
-      if (r0 + r < Lx && c0 + c < Lx) A[(size_t)(r0 + r) * Lx + c0 + c] = T[e];
-    }
-  };
-  // C(r0, c0) <- C + alpha * (Xm Ym) or alpha * (Xm Ym) (overwrite), 32 x 32 x 32 on
-  // the tensor cores (3xTF32, binary32 accuracy): warp w computes the 16 x 8 tile
-  // at rows 16 (w / 4), columns 8 (w % 4)
-  auto mm = [&](const cxf_* Xm, const cxf_* Ym, int r0, int c0, float alpha, bool accumulate) {
-    const int wq = threadIdx.x >> 5, tm = 16 * (wq >> 2), tn = 8 * (wq & 3);
-    tc::CTile acc = {};
-    tc::cgemm_tile_3xtf32(acc, Xm, Ym, NB, tm, tn);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      int r, c;
-      tc::tile_pos(e, tm, tn, r, c);
-      if (r0 + r < Lx && c0 + c < Lx) {
-        cxf_& o = A[(size_t)(r0 + r) * Lx + c0 + c];
-        const cxf_ v = {alpha * acc.re[e], alpha * acc.im[e]};
-        o = accumulate ? o + v : v;
-      }
-    }
-  };
-  static_assert(LINV_NB == 32 && DY_THREADS == 256, "eight 16 x 8 tensor-core tiles per 32 x 32 block");
+  sync();
+  const int nbk = (n + NB - 1) / NB, ntu = (n + TU - 1) / TU;
+  const int ty = tid >> 4, txi = tid & 15;                          // 16 x 16 threads of a tile, 4 x 4 entries each
   for (int kb = 0; kb < nbk; ++kb) {
     const int k0 = kb * NB;
-    __syncthreads();
-    ld(Pk, k0, k0, true);
-    sweep_invert_f(Pk, NB, prow, fcol);                   // Pk = A_kk^-1
-    // row panel A_kj <- Pk A_kj
-    for (int jb = 0; jb < nbk; ++jb) {
-      if (jb == kb) continue;
-      __syncthreads();
-      ld(Y, k0, jb * NB, false);
-      __syncthreads();
-      mm(Pk, Y, k0, jb * NB, 1.f, false);
+    for (int e = tid; e < NB * NB; e += DY_THREADS) {
+      const int r = e / NB, c = e - r * NB;
+      Pk[e] = k0 + r < n && k0 + c < n ? A[(size_t)(k0 + r) * n + k0 + c] : (r == c ? cxf_{1.f, 0.f} : cxf_{0.f, 0.f});
     }
-    // rank-NB update of the rest with the old column panel
-    for (int ib = 0; ib < nbk; ++ib) {
-      if (ib == kb) continue;
+    sweep_invert_f(Pk, NB, prow, fcol);                   // every CTA for itself
+    // panel: O = A_ik (from the upper triangle), F_i = O P
+    for (int q = ci; q < nbk - 1; q += CN) {
+      const int ib = q < kb ? q : q + 1, i0 = ib * NB;
       __syncthreads();
-      ld(X, ib * NB, k0, false);
-      for (int jb = 0; jb < nbk; ++jb) {
-        if (jb == kb) continue;
-        __syncthreads();
-        ld(Y, k0, jb * NB, false);
-        __syncthreads();
-        mm(X, Y, ib * NB, jb * NB, -1.f, true);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int rr = wid + 8 * m;
+        if (ib < kb) tx[rr][lane] = i0 + rr < n && k0 + lane < n ? A[(size_t)(i0 + rr) * n + k0 + lane] : cxf_{0.f, 0.f};
+        else tx[lane][rr] = k0 + rr < n && i0 + lane < n ? A[(size_t)(k0 + rr) * n + i0 + lane] : cxf_{0.f, 0.f};
       }
-      // column panel of this block row: A_ik <- -A_ik Pk (X still holds the old A_ik)
       __syncthreads();
-      mm(X, Pk, ib * NB, k0, -1.f, false);
+      cxf_ acc[4] = {};
+#pragma unroll 8
+      for (int k = 0; k < NB; ++k) {
+        const cxf_ x = tx[lane][k];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) acc[m] = cfma(x, Pk[k * NB + wid * 4 + m], acc[m]);
+      }
+      if (i0 + lane < n) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          Ft[(size_t)(wid * 4 + m) * n + i0 + lane] = acc[m];
+          Ot[(size_t)(wid * 4 + m) * n + i0 + lane] = tx[lane][wid * 4 + m];
+        }
+      }
     }
-    __syncthreads();
-    st(Pk, k0, k0);
+    sync();                                               // F and O complete, the old panel is not read any more
+    int tile = 0;
+    for (int ti = 0; ti < ntu; ++ti)
+      for (int tj = ti; tj < ntu; ++tj, ++tile) {
+        if (tile % CN != ci) continue;
+        const int r0 = ti * TU, c0 = tj * TU, rt = r0 + ty * 4, ct = c0 + txi * 4;
+        cxf_ acc[4][4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            acc[a][c] = rt + a < n && ct + c < n ? A[(size_t)(rt + a) * n + ct + c] : cxf_{0.f, 0.f};
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+          const int e = tid + DY_THREADS * m, k = e / TU, x = e % TU;
+          FO[0][k][x] = r0 + x < n ? -Ft[(size_t)k * n + r0 + x] : cxf_{0.f, 0.f};
+          FO[1][k][x] = c0 + x < n ? Ot[(size_t)k * n + c0 + x] : cxf_{0.f, 0.f};
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int k = 0; k < NB; ++k) {
+          const float4* fp = reinterpret_cast<const float4*>(&FO[0][k][ty * 4]);
+          const float4* op = reinterpret_cast<const float4*>(&FO[1][k][txi * 4]);
+          const float4 f0 = fp[0], f1 = fp[1], o0 = op[0], o1 = op[1];
+          const cxf_ fv[4] = {{f0.x, f0.y}, {f0.z, f0.w}, {f1.x, f1.y}, {f1.z, f1.w}};
+          const cxf_ ov[4] = {{o0.x, o0.y}, {o0.z, o0.w}, {o1.x, o1.y}, {o1.z, o1.w}};
+#pragma unroll
+          for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[a][c] = cfma(fv[a], ov[c], acc[a][c]);
+        }
+        // a thread's four rows (columns) lie in one pivot block
+        const bool rk = rt / NB == kb, ck = ct / NB == kb;
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const int r = rt + a, cc = ct + c;
+            if (r >= n || cc >= n) continue;
+            cxf_ v = acc[a][c];
+            if (rk && ck) v = -Pk[(r - k0) * NB + cc - k0];
+            else if (ck) v = Ft[(size_t)(cc - k0) * n + r];
+            else if (rk) v = Ft[(size_t)(r - k0) * n + cc];
+            A[(size_t)r * n + cc] = v;
+          }
+      }
+    sync();
   }
-  __syncthreads();
   cx<R>* M = reinterpret_cast<cx<R>*>(b.lpm) + ((size_t)f * (g.p - 1) + l) * n2;
-  for (size_t e = threadIdx.x; e < n2; e += DY_THREADS) {
-    const int r = (int)(e / Lx), c = (int)(e - (size_t)r * Lx);
-    const cxf_ a = A[e], at = A[(size_t)c * Lx + r];
-    M[e] = cx<R>{(R)(0.5f * (a.x + at.x)), (R)(0.5f * (a.y + at.y))};
+  for (size_t e = (size_t)ci * DY_THREADS + tid; e < n2; e += (size_t)CN * DY_THREADS) {
+    const int r = (int)(e / n), c = (int)(e - (size_t)r * n);
+    const cxf_ a = r <= c ? A[e] : A[(size_t)c * n + r];
+    M[e] = cx<R>{(R)-a.x, (R)-a.y};
   }
 }
 
@@ -579,7 +631,7 @@ __global__ void __launch_bounds__(DY_THREADS) k_layer_inv_g(Geo g, Bufs b) {
 template <typename R>
 __global__ void __launch_bounds__(DY_THREADS) k_layer_inv(Geo g, Bufs b) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int l = blockIdx.x, f = blockIdx.y, Lx = g.Lx, n = Lx * Lx;
+  const int l = blockIdx.x, f = blockIdx.y, Lx = g.A, lx = g.Lx, n = Lx * Lx;   // layer index a = x + lx y
   cxf_* S = reinterpret_cast<cxf_*>(smem_raw);
   cxf_* prow = S + n;
   cxf_* fcol = prow + Lx;
@@ -592,8 +644,8 @@ __global__ void __launch_bounds__(DY_THREADS) k_layer_inv(Geo g, Bufs b) {
     if (r == c) {
       const cxd d = dyson_diag(g, b, f, r + g.A * g.ylayer[l]);
       v = cxf_{d2f_bits(d.x), d2f_bits(d.y)};
-    } else if (r == c + 1 || c == r + 1) {
-      v = cxf_{t, 0.f};
+    } else if (((r == c + 1 || c == r + 1) && r / lx == c / lx) || r == c + lx || c == r + lx) {
+      v = cxf_{t, 0.f};                                             // in-plane neighbours along x and y
     }
     S[e] = cfma(cxf_{-t2, 0.f}, Pt[e] + Pb[e], v);
   }
@@ -614,8 +666,8 @@ size_t dyson_internal_surface_smem(const Geo& g) {
 }
 
 size_t dyson_internal_layer_inv_smem(const Geo& g) {
-  if (g.Lx > DY_LPRE_MAXLX) return 0;                      // global-memory form
-  return ((size_t)g.Lx * g.Lx + 2 * (size_t)g.Lx) * sizeof(cxf_);
+  if (g.A > DY_LPRE_MAXLX) return 0;                       // global-memory form
+  return ((size_t)g.A * g.A + 2 * (size_t)g.A) * sizeof(cxf_);
 }
 
 static size_t surface_g_smem() { return (3 * 32 * 32 + 2 * 32 + DY_WARPS * 32) * sizeof(cxf_); }
@@ -625,10 +677,10 @@ cudaError_t launch_surface(const Geo& g, const Bufs& b, int K, cudaStream_t st) 
   if (g.T > 1) {                           // 3D slabs: persistent grid over (slab, frequency)
     if (!b.lpw || !b.fwork || g.W <= DY_MAXW_SMEM || g.A > DY_LPRE_MAXLX_G) return cudaErrorInvalidValue;
     const int units = g.p * K;
-    const int grid = units < DY_FACTOR_CTAS ? units : DY_FACTOR_CTAS;
-    if (b.g64) k_surface_3d<cx<dfl>><<<grid, DY_THREADS, 0, st>>>(g, b, K);   // mixed: double-float factors
-    else k_surface_3d<cxd><<<grid, DY_THREADS, 0, st>>>(g, b, K);
-    return cudaGetLastError();
+    const int C = unit_cluster(units);
+    const int grid = C * (units < DY_FACTOR_CTAS / C ? units : DY_FACTOR_CTAS / C);
+    if (b.g64) return launch_clustered(k_surface_3d<cx<dfl>>, dim3(grid), C, 0, st, g, b, K);   // mixed: double-float factors
+    return launch_clustered(k_surface_3d<cxd>, dim3(grid), C, 0, st, g, b, K);
   }
   if (g.W > SURF_MAXW || g.Lx > DY_LPRE_MAXLX_G) return cudaErrorInvalidValue;
   if (g.Lx > DY_LPRE_MAXLX) {
@@ -652,9 +704,9 @@ cudaError_t launch_surface(const Geo& g, const Bufs& b, int K, cudaStream_t st) 
 template <typename R>
 cudaError_t launch_layer_inv(const Geo& g, const Bufs& b, int K, cudaStream_t st) {
   if (!g.lpre) return cudaSuccess;
-  if (g.T > 1 || g.Lx > DY_LPRE_MAXLX) {
-    k_layer_inv_g<R><<<dim3(g.p - 1, K), DY_THREADS, 0, st>>>(g, b);
-    return cudaGetLastError();
+  if (g.A > DY_LPRE_MAXLX) {               // also: k_layer_inv_g keeps its panels in 64 A <= A^2 entries
+    const int C = unit_cluster((g.p - 1) * K);
+    return launch_clustered(k_layer_inv_g<R>, dim3((g.p - 1) * C, K), C, 0, st, g, b);
   }
   const size_t smem = dyson_internal_layer_inv_smem(g);
   cudaError_t e = raise_smem_limit((const void*)k_layer_inv<R>, smem);
