@@ -84,22 +84,10 @@ __device__ __forceinline__ void smem_matmul(cx<R>* C, const cx<R>* X, const cx<R
   }
 }
 
-// R: arithmetic of the recursion; S: storage of the g_s handed to the sweeps.
-//
-// FP64 form (S == R): one-sided recursion, g_s left-connected for every s,
-// stored row-major for the 8-warp sweeps.
-//
-// Mixed form (S != R): two-sided recursion, so that the complex64 sweeps can
-// run two chains at once (one from each end).  With m = Lx / 2:
-//   left   g_s = (D_s - t^2 g_{s-1})^-1            s < m
-//   right  g_s = (D_s - t^2 g_{s+1})^-1            s > m
-//   middle G_mm = (D_m - t^2 g_{m-1} - t^2 g_{m+1})^-1
-//   G_ss = g_s + t^2 g_s G_{s+1,s+1} g_s  (s < m),  g_s + t^2 g_s G_{s-1,s-1} g_s  (s > m)
-// Slot s holds g_s, or G_mm for s = m.  The recursion runs in R (FP64) with
-// the factors kept in b.g64; the complex64 copy in b.g is written with column
-// pairs interleaved: entry (r, c) of a block at ((c / 2) W + r) 2 + c % 2, so
-// that the lane owning row r reads columns 2k, 2k+1 as one 16-byte word.
-template <typename R, typename S>
+// One CTA per (subdomain, frequency), W <= 64, binary64 (the FP64 form; the mixed
+// form runs k_factor_two): g_s left-connected for every s, stored row-major for the
+// 8-warp sweeps.
+template <typename R>
 __global__ void __launch_bounds__(DY_THREADS) k_factor(Geo g, Bufs b) {
   using C = cx<R>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -112,22 +100,18 @@ __global__ void __launch_bounds__(DY_THREADS) k_factor(Geo g, Bufs b) {
   C* prow = Cm + n;                          // Gauss-Jordan pivot row / column caches
   C* fcol = prow + W;
   C* Gprev = fcol + W;                       // [2][W] columns of the last off-diagonal block at the boundary rows
-  C* Gmid = Gprev + 2 * W;                   // [2][W] rows of G_{m+1,m} at the boundary rows (two-sided)
-  constexpr bool two = sizeof(S) != sizeof(R);
   const size_t uoff = ((size_t)kf * g.p + i) * (size_t)Lx * n;
-  C* gout = reinterpret_cast<C*>(two ? b.g64 : b.g) + uoff;
-  cx<S>* gsw = reinterpret_cast<cx<S>*>(b.g) + uoff;
+  C* gout = reinterpret_cast<C*>(b.g) + uoff;
   cxd* dB = b.diagB + (size_t)kf * g.Ndd + (size_t)i * Lx * W;
   const R t = (R)g.t, t2 = (R)(g.t * g.t);
 
-  // A = D_s - t^2 (pa + pb); pa may be A itself (each entry is read and
-  // written by the same thread), either may be null
-  auto form = [&](int s, const C* pa, const C* pb) {
+  // A = D_s - t^2 pa; pa may be A itself (each entry is read and written by the
+  // same thread) or null
+  auto form = [&](int s, const C* pa) {
     for (int e = threadIdx.x; e < n; e += DY_THREADS) {
       int r = e / W, c = e - r * W;
       C v = {0, 0};
       if (pa) v = v - t2 * pa[e];
-      if (pb) v = v - t2 * pb[e];
       if (r < w && c < w) {
         if (r == c) {
           cxd d = dyson_diag(g, b, kf, sub_nat(g, i, s, r));
@@ -150,7 +134,6 @@ __global__ void __launch_bounds__(DY_THREADS) k_factor(Geo g, Bufs b) {
       if (r >= w || c >= w) v = C{0, 0};
       A[e] = v;
       gout[(size_t)s * n + e] = v;
-      if (two) gsw[(size_t)s * n + ((size_t)(c >> 1) * W + r) * 2 + (c & 1)] = cconv<S>(v);
     }
     __syncthreads();
   };
@@ -167,9 +150,8 @@ __global__ void __launch_bounds__(DY_THREADS) k_factor(Geo g, Bufs b) {
   // A <- g_s + t^2 g_s A g_s with g_s from slot s (A = G of the neighbour toward
   // the start, slice sn); -t g_s A is the off-diagonal block G_{s,sn}, whose
   // diagonal the interface preconditioner uses (stored at min(s, sn)).
-  // prevc: boundary columns of G_{sn,s2} (null if s2 is outside the strip);
-  // mid: also keep the boundary rows of G_{s,sn} in Gmid
-  auto grow_G = [&](int s, int sn, const C* prevc, bool mid) {
+  // prevc: boundary columns of G_{sn,s2} (null if s2 is outside the strip)
+  auto grow_G = [&](int s, int sn, const C* prevc) {
     for (int e = threadIdx.x; e < n; e += DY_THREADS) Bm[e] = gout[(size_t)s * n + e];
     __syncthreads();
     smem_matmul<R>(Cm, Bm, A, W);
@@ -193,7 +175,6 @@ __global__ void __launch_bounds__(DY_THREADS) k_factor(Geo g, Bufs b) {
       for (int e = threadIdx.x; e < 2 * W; e += DY_THREADS) {
         const int jj = e / W, c = e - jj * W, j = jj ? w - 1 : 0;
         Gprev[e] = (-t) * Cm[c * W + j];
-        if (mid) Gmid[e] = (-t) * Cm[j * W + c];
       }
     }
     // g_s + t^2 (g_s A) g_s is complex symmetric: the upper triangle, then the mirror
@@ -214,39 +195,258 @@ __global__ void __launch_bounds__(DY_THREADS) k_factor(Geo g, Bufs b) {
     diag_out(s);
   };
 
-  if constexpr (!two) {
-    for (int s = 0; s < Lx; ++s) {          // forward: A holds g_{s-1} on entry
-      form(s, s > 0 ? A : nullptr, nullptr);
-      invert_store(s);
-    }
-    diag_out(Lx - 1);                        // backward: A holds G_{s+1,s+1}
-    for (int s = Lx - 2; s >= 0; --s) grow_G(s, s + 1, s < Lx - 2 ? Gprev : nullptr, false);
-  } else {
-    const int m = Lx / 2;
-    for (int s = 0; s < m; ++s) {           // left chain
-      form(s, s > 0 ? A : nullptr, nullptr);
-      invert_store(s);
-    }
-    for (int s = Lx - 1; s > m; --s) {      // right chain
-      form(s, s < Lx - 1 ? A : nullptr, nullptr);
-      invert_store(s);
-    }
-    form(m, m > 0 ? gout + (size_t)(m - 1) * n : nullptr,
-         m < Lx - 1 ? gout + (size_t)(m + 1) * n : nullptr);
-    invert_store(m);                         // G_mm
-    diag_out(m);
-    // right side first, so that the left side's first step finds G_{m,m+1}
-    for (int s = m + 1; s < Lx; ++s) grow_G(s, s - 1, s > m + 1 ? Gprev : nullptr, s == m + 1);
-    for (int e = threadIdx.x; e < n; e += DY_THREADS) A[e] = gout[(size_t)m * n + e];
-    __syncthreads();
-    for (int s = m - 1; s >= 0; --s)
-      grow_G(s, s + 1, s < m - 1 ? Gprev : (m + 1 < Lx ? Gmid : nullptr), false);
+  for (int s = 0; s < Lx; ++s) {            // forward: A holds g_{s-1} on entry
+    form(s, s > 0 ? A : nullptr);
+    invert_store(s);
   }
+  diag_out(Lx - 1);                          // backward: A holds G_{s+1,s+1}
+  for (int s = Lx - 2; s >= 0; --s) grow_G(s, s + 1, s < Lx - 2 ? Gprev : nullptr);
   // interface part of diag(B^-1) is zero (blkdiag(B^-1, 0), Eq. 9)
   if (i == g.p - 1) {
     cxd* dI = b.diagB + (size_t)kf * g.Ndd + g.ifc_off;
     size_t m = (size_t)(g.p - 1) * g.A;
     for (size_t e = threadIdx.x; e < m; e += DY_THREADS) dI[e] = cxd{0, 0};
+  }
+}
+
+// ---------------------------------------------------------------- two-sided, double-float
+// The mixed form's recursion for W <= 64, from both ends, so that the complex64
+// sweeps can run two chains at once.  With m = Lx / 2:
+//   left   g_s = (D_s - t^2 g_{s-1})^-1            s < m
+//   right  g_s = (D_s - t^2 g_{s+1})^-1            s > m
+//   middle G_mm = (D_m - t^2 g_{m-1} - t^2 g_{m+1})^-1
+//   G_ss = g_s + t^2 g_s G_{s+1,s+1} g_s  (s < m),  g_s + t^2 g_s G_{s-1,s-1} g_s  (s > m)
+// Slot s holds g_s, or G_mm for s = m: in double-float in b.g64, and in complex64 in
+// b.g with column pairs interleaved (entry (r, c) at ((c / 2) W + r) 2 + c % 2, so
+// that a lane reads columns 2k, 2k+1 of its row as one 16-byte word).
+// One cluster of two CTAs per (subdomain, frequency): CTA 0 the left chain, CTA 1 the
+// right one, which meet at the middle block (each inverts it for itself) and go back
+// separately.  One CTA running both chains in turn took 65 us a slice at W = 28 with
+// 21 x 4 units on 152 SMs.
+//
+// Inversion: the sweep operator on the upper triangle, whose entries stay in the
+// threads' registers (thread t owns triangle entries t, t + 256, ...); a pivot's
+// column goes through shared memory, one warp scales it by the inverse pivot.
+// Entries are renormalised every fourth pivot.
+template <int WF>
+struct TwoCfg {
+  static constexpr int NE = (WF * (WF + 1) / 2 + DY_THREADS - 1) / DY_THREADS;   // triangle entries a thread owns
+};
+using cxl = cx<dfl>;
+
+__device__ __forceinline__ cxl mac_l(const cxl& a, const cxl& b, cxl acc) {
+  dfl_mac(acc.x, a.x, b.x);
+  dfl_mac(acc.x, dfl(-a.y.hi, -a.y.lo), b.y);
+  dfl_mac(acc.y, a.x, b.y);
+  dfl_mac(acc.y, a.y, b.x);
+  return acc;
+}
+__device__ __forceinline__ cxl norm_l(const cxl& v) { return {dfl_fast(v.x.hi, v.x.lo), dfl_fast(v.y.hi, v.y.lo)}; }
+
+template <int WF>
+__global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 3 : 1) k_factor_two(Geo g, Bufs b) {
+  constexpr int NE = TwoCfg<WF>::NE;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cg::cluster_group cl = cg::this_cluster();
+  const int side = (int)cl.block_rank(), i = blockIdx.x / 2, kf = blockIdx.y;
+  const int W = g.W, Lx = g.Lx, T = g.T, w = T * g.h[i], n = W * W, m = Lx / 2;
+  cxl* A = reinterpret_cast<cxl*>(smem_raw);
+  cxl* Bm = A + n;
+  cxl* Cm = Bm + n;
+  cxl* prow = Cm + n;                        // [2][W] the pivot's column, by step parity
+  cxl* fcol = prow + 2 * W;                  // [W] the column scaled by the inverse pivot
+  cxl* Gprev = fcol + W;                     // [2][W] columns of the last off-diagonal block at the boundary rows
+  cxl* Gmid = Gprev + 2 * W;                 // [2][W] rows of G_{m+1,m} at the boundary rows (left CTA's copy is used)
+  const size_t uoff = ((size_t)kf * g.p + i) * (size_t)Lx * n;
+  cxl* gout = reinterpret_cast<cxl*>(b.g64) + uoff;
+  cxf* gsw = reinterpret_cast<cxf*>(b.g) + uoff;
+  cxd* dB = b.diagB + (size_t)kf * g.Ndd + (size_t)i * Lx * W;
+  const bool band = !g.lpre;                 // the banded preconditioner reads the off-diagonal blocks
+  cxd* oB = band && b.offB ? b.offB + ((size_t)kf * g.p + i) * (size_t)Lx * W : nullptr;
+  cxd* o2 = band && b.off2 && T == 1 ? b.off2 + ((size_t)kf * g.p + i) * (size_t)Lx * W : nullptr;
+  const dfl t = (dfl)g.t, t2 = (dfl)(g.t * g.t);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+
+  // the triangle entries (r <= c) this thread owns: rows of length W, W - 1, ...
+  int er[NE], ec[NE];
+  bool on[NE];
+#pragma unroll
+  for (int q = 0; q < NE; ++q) {
+    int e = tid + DY_THREADS * q, r = 0;
+    on[q] = e < W * (W + 1) / 2;
+    while (on[q] && e >= W - r) {
+      e -= W - r;
+      ++r;
+    }
+    er[q] = r;
+    ec[q] = r + e;
+  }
+
+  // A <- (D_s - t^2 (pa + pb))^-1, zero on the padding; pa, pb (full W x W, either may be
+  // null) may be A itself; stored in slot s when keep
+  auto invert = [&](int s, const cxl* pa, const cxl* pb, bool keep) {
+    cxl v[NE];
+#pragma unroll
+    for (int q = 0; q < NE; ++q) {
+      if (!on[q]) continue;
+      const int r = er[q], c = ec[q], e = r * W + c;
+      cxl x = {0, 0};
+      if (pa) x = x - t2 * pa[e];
+      if (pb) x = x - t2 * pb[e];
+      if (c < w) {
+        if (r == c) x = x + cconv<dfl>(dyson_diag(g, b, kf, sub_nat(g, i, s, r)));
+        else if (slice_adjacent<dfl>(r, c, T)) x.x += t;
+      } else {
+        x = r == c ? cxl{1, 0} : cxl{0, 0};
+      }
+      v[q] = x;
+      if (r == 0) prow[c] = x;               // the first pivot's column
+    }
+    for (int k = 0; k < W; ++k) {
+      cxl* pk = prow + (k & 1) * W;
+      cxl* pn = prow + ((k + 1) & 1) * W;
+      __syncthreads();                       // column k published; A, fcol free
+      if (wid == 0) {
+        const cxl piv = cinv(pk[k]);
+        for (int e = lane; e < W; e += 32) fcol[e] = e == k ? -piv : pk[e] * piv;
+      }
+      __syncthreads();
+      const bool rn = (k & 3) == 3 || k == W - 1;
+#pragma unroll
+      for (int q = 0; q < NE; ++q) {
+        if (!on[q]) continue;
+        const int r = er[q], c = ec[q];
+        if (r == k || c == k) {
+          v[q] = fcol[r == k ? c : r];
+        } else {
+          const cxl f = fcol[r];
+          v[q] = mac_l(cxl{-f.x, -f.y}, pk[c], v[q]);
+          if (rn) v[q] = norm_l(v[q]);
+        }
+        if (r == k + 1) pn[c] = v[q];
+        else if (c == k + 1) pn[r] = v[q];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NE; ++q) {           // -(-A^-1), both triangles
+      if (!on[q]) continue;
+      const int r = er[q], c = ec[q];
+      cxl x = norm_l(v[q]);
+      x = c < w ? cxl{-x.x, -x.y} : cxl{0, 0};
+      A[r * W + c] = x;
+      A[c * W + r] = x;
+    }
+    __syncthreads();
+    if (keep)
+      for (int e = tid; e < n; e += DY_THREADS) {
+        const int r = e / W, c = e - r * W;
+        const cxl x = A[e];
+        gout[(size_t)s * n + e] = x;
+        gsw[(size_t)s * n + ((size_t)(c >> 1) * W + r) * 2 + (c & 1)] = cconv<float>(x);
+      }
+    __syncthreads();
+  };
+  auto diag_out = [&](int s) {
+    for (int r = tid; r < W; r += DY_THREADS) dB[(size_t)s * W + r] = (r < w) ? cconv<double>(A[r * W + r]) : cxd{0, 0};
+  };
+  // A <- g_s + t^2 g_s A g_s with g_s from slot s, A = G of the neighbour towards the
+  // middle, slice sn (see k_factor for the off-diagonal by-products)
+  auto grow = [&](int s, int sn, const cxl* prevc, bool mid) {
+    for (int e = tid; e < n; e += DY_THREADS) Bm[e] = gout[(size_t)s * n + e];
+    __syncthreads();
+    // Cm = g_s A: lane = column (WF >= 32), 8 warps' rows; the row of g_s is a broadcast
+    for (int e0 = tid; e0 < n; e0 += 4 * DY_THREADS) {
+      cxl acc[4];
+      int rr[4], cc[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = e0 + u * DY_THREADS;
+        rr[u] = e < n ? e / W : 0;
+        cc[u] = e < n ? e - rr[u] * W : 0;
+        acc[u] = cxl{0, 0};
+      }
+      for (int k0 = 0; k0 < W; k0 += 4) {    // W is a multiple of 4
+#pragma unroll
+        for (int k = k0; k < k0 + 4; ++k)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) acc[u] = mac_l(Bm[rr[u] * W + k], A[k * W + cc[u]], acc[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] = norm_l(acc[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (e0 + u * DY_THREADS < n) Cm[e0 + u * DY_THREADS] = acc[u];
+    }
+    __syncthreads();
+    if (oB)
+      for (int r = tid; r < W; r += DY_THREADS)
+        oB[(size_t)(s < sn ? s : sn) * W + r] = (r < w) ? cconv<double>((-t) * Cm[r * W + r]) : cxd{0, 0};
+    if (o2) {
+      const int s2 = 2 * sn - s;
+      if (prevc && wid < 2) {                // warp jj: boundary row jj ? w-1 : 0
+        const int j = wid ? w - 1 : 0;
+        cxl acc = {0, 0};
+        for (int c = lane; c < W; c += 32) acc = cfma(Bm[j * W + c], prevc[wid * W + c], acc);
+        for (int off = 16; off > 0; off >>= 1) {
+          acc.x += shfl_xor_any(acc.x, off);
+          acc.y += shfl_xor_any(acc.y, off);
+        }
+        if (lane == 0) o2[(size_t)(s < s2 ? s : s2) * W + j] = cconv<double>((-t) * acc);
+      }
+      __syncthreads();                       // prevc read before Gprev is rewritten
+      cxl* other = cl.map_shared_rank(Gmid, 0);
+      for (int e = tid; e < 2 * W; e += DY_THREADS) {
+        const int jj = e / W, c = e - jj * W, j = jj ? w - 1 : 0;
+        Gprev[e] = (-t) * Cm[c * W + j];
+        if (mid) other[e] = (-t) * Cm[j * W + c];
+      }
+    }
+    // g_s + t^2 (g_s A) g_s on the upper triangle, mirrored
+    cxl v[NE];
+#pragma unroll
+    for (int q = 0; q < NE; ++q) v[q] = cxl{0, 0};
+    for (int k0 = 0; k0 < W; k0 += 4) {
+#pragma unroll
+      for (int q = 0; q < NE; ++q) {
+        if (!on[q]) continue;
+#pragma unroll
+        for (int k = k0; k < k0 + 4; ++k) v[q] = mac_l(Cm[er[q] * W + k], Bm[k * W + ec[q]], v[q]);
+        v[q] = norm_l(v[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NE; ++q) {
+      if (!on[q]) continue;
+      const int r = er[q], c = ec[q];
+      const cxl x = Bm[r * W + c] + t2 * v[q];
+      A[r * W + c] = x;
+      A[c * W + r] = x;
+    }
+    __syncthreads();
+    diag_out(s);
+    __syncthreads();
+  };
+
+  if (side == 0) {
+    for (int s = 0; s < m; ++s) invert(s, s > 0 ? A : nullptr, nullptr, true);
+  } else {
+    for (int s = Lx - 1; s > m; --s) invert(s, s < Lx - 1 ? A : nullptr, nullptr, true);
+  }
+  cl.sync();                                 // both neighbours of the middle slice are stored
+  invert(m, m > 0 ? gout + (size_t)(m - 1) * n : nullptr, m < Lx - 1 ? gout + (size_t)(m + 1) * n : nullptr, side == 0);
+  if (side == 0) diag_out(m);
+  if (side == 1 && m + 1 < Lx) grow(m + 1, m, nullptr, true);
+  cl.sync();                                 // Gmid is in the left CTA's shared memory
+  if (side == 1) {
+    for (int s = m + 2; s < Lx; ++s) grow(s, s - 1, Gprev, false);
+  } else {
+    for (int s = m - 1; s >= 0; --s) grow(s, s + 1, s < m - 1 ? Gprev : (m + 1 < Lx ? Gmid : nullptr), false);
+  }
+  // interface part of diag(B^-1) is zero (blkdiag(B^-1, 0), Eq. 9)
+  if (i == g.p - 1 && side == 0) {
+    cxd* dI = b.diagB + (size_t)kf * g.Ndd + g.ifc_off;
+    const size_t mi = (size_t)(g.p - 1) * g.A;
+    for (size_t e = tid; e < mi; e += DY_THREADS) dI[e] = cxd{0, 0};
   }
 }
 
@@ -654,15 +854,20 @@ cudaError_t launch_factor(const Geo& g, const Bufs& b, int K, cudaStream_t st) {
       return cudaErrorInvalidValue;
     }
   }
-  size_t smem = (3 * (size_t)g.W * g.W + 6 * (size_t)g.W) * sizeof(cx<R>);
-  cudaError_t e = raise_smem_limit((const void*)k_factor<R, S>, smem);
-  if (e != cudaSuccess) return e;
-  k_factor<R, S><<<dim3(g.p, K), DY_THREADS, smem, st>>>(g, b);
-  return cudaGetLastError();
+  if constexpr (std::is_same<R, dfl>::value) {
+    const size_t smem = (3 * (size_t)g.W * g.W + 7 * (size_t)g.W) * sizeof(cxl);
+    auto kern = g.W <= 16 ? k_factor_two<16> : (g.W <= 32 ? k_factor_two<32> : k_factor_two<64>);
+    return launch_clustered(kern, dim3(2 * g.p, K), 2, smem, st, g, b);
+  } else {
+    const size_t smem = (3 * (size_t)g.W * g.W + 4 * (size_t)g.W) * sizeof(cx<R>);
+    cudaError_t e = raise_smem_limit((const void*)k_factor<R>, smem);
+    if (e != cudaSuccess) return e;
+    k_factor<R><<<dim3(g.p, K), DY_THREADS, smem, st>>>(g, b);
+    return cudaGetLastError();
+  }
 }
 template cudaError_t launch_factor<double, double>(const Geo&, const Bufs&, int, cudaStream_t);
 template cudaError_t launch_factor<dfl, float>(const Geo&, const Bufs&, int, cudaStream_t);
-template cudaError_t launch_factor<float, float>(const Geo&, const Bufs&, int, cudaStream_t);
 
 template <typename R>
 cudaError_t launch_precond(const Geo& g, const Bufs& b, int K, cudaStream_t st) {
