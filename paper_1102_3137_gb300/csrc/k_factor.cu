@@ -225,117 +225,166 @@ __global__ void __launch_bounds__(DY_THREADS) k_factor(Geo g, Bufs b) {
 // 21 x 4 units on 152 SMs.
 //
 // Inversion: the sweep operator on the upper triangle, whose entries stay in the
-// threads' registers (thread t owns triangle entries t, t + 256, ...); a pivot's
-// column goes through shared memory, one warp scales it by the inverse pivot.
-// Entries are renormalised every fourth pivot.
+// registers of warps 1..7 (thread t of them owns triangle entries t, t + 224, ...).
+// Warp 0 runs one pivot ahead: while the others apply pivot k it brings column k + 1
+// up to date itself, inverts pivot k + 1 and scales the column, so a pivot costs one
+// barrier and the longer of the two (~650 cycles at W = 32) instead of their sum
+// (2250).  Every product is renormalised as it is added: sums without it, 48
+// operations a term instead of 60, made the diagonal's error 1.2 to 1.4 times as large.
 template <int WF>
 struct TwoCfg {
-  static constexpr int NE = (WF * (WF + 1) / 2 + DY_THREADS - 1) / DY_THREADS;   // triangle entries a thread owns
+  static constexpr int OWN = DY_THREADS - 32;
+  static constexpr int NE = (WF * (WF + 1) / 2 + OWN - 1) / OWN;                 // triangle entries an owner holds
+  static constexpr int NP = (WF * (WF + 1) / 2 + DY_THREADS - 1) / DY_THREADS;   // and a thread of the last product
 };
 using cxl = cx<dfl>;
 
-__device__ __forceinline__ cxl mac_l(const cxl& a, const cxl& b, cxl acc) {
-  dfl_mac(acc.x, a.x, b.x);
-  dfl_mac(acc.x, dfl(-a.y.hi, -a.y.lo), b.y);
-  dfl_mac(acc.y, a.x, b.y);
-  dfl_mac(acc.y, a.y, b.x);
-  return acc;
+// 1 / z: one Newton step from the binary32 reciprocal of |z|^2, with its square term
+// (the start is off by at most 2^-24, so the result by ~2^-70 before rounding)
+__device__ __forceinline__ cxl inv_l(const cxl& z) {
+  dfl d = dfl(0.f, 0.f);
+  dfl_mac(d, z.x, z.x);
+  dfl_mac(d, z.y, z.y);
+  d = dfl_fast(d.hi, d.lo);
+  const float r0 = __frcp_rn(d.hi);
+  const float e = __fmaf_rn(-d.lo, r0, __fmaf_rn(-d.hi, r0, 1.f));
+  const dfl r = dfl_fast(r0, r0 * __fmaf_rn(e, e, e));
+  const dfl im = z.y * r;
+  return {z.x * r, dfl(-im.hi, -im.lo)};
 }
-__device__ __forceinline__ cxl norm_l(const cxl& v) { return {dfl_fast(v.x.hi, v.x.lo), dfl_fast(v.y.hi, v.y.lo)}; }
 
 template <int WF>
-__global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 3 : 1) k_factor_two(Geo g, Bufs b) {
-  constexpr int NE = TwoCfg<WF>::NE;
+__global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo g, Bufs b) {
+  constexpr int NE = TwoCfg<WF>::NE, NP = TwoCfg<WF>::NP, OWN = TwoCfg<WF>::OWN;
+  constexpr int NB = (WF * WF + DY_THREADS - 1) / DY_THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cg::cluster_group cl = cg::this_cluster();
   const int side = (int)cl.block_rank(), i = blockIdx.x / 2, kf = blockIdx.y;
-  const int W = g.W, Lx = g.Lx, T = g.T, w = T * g.h[i], n = W * W, m = Lx / 2;
+  const int W = g.W, Lx = g.Lx, T = g.T, w = T * g.h[i], n = W * W, m = Lx / 2, ntri = W * (W + 1) / 2;
   cxl* A = reinterpret_cast<cxl*>(smem_raw);
   cxl* Bm = A + n;
   cxl* Cm = Bm + n;
-  cxl* prow = Cm + n;                        // [2][W] the pivot's column, by step parity
-  cxl* fcol = prow + 2 * W;                  // [W] the column scaled by the inverse pivot
-  cxl* Gprev = fcol + W;                     // [2][W] columns of the last off-diagonal block at the boundary rows
+  cxl* prow = Cm + n;                        // [2][W] the pivot's column, by pivot parity
+  cxl* fcol = prow + 2 * W;                  // [2][W] the column scaled by the inverse pivot
+  cxl* craw = fcol + 2 * W;                  // [2][W] the column after it, one pivot behind
+  cxl* dg = craw + 2 * W;                    // [W] H_ii of the slice being formed
+  cxl* Gprev = dg + W;                       // [2][W] columns of the last off-diagonal block at the boundary rows
   cxl* Gmid = Gprev + 2 * W;                 // [2][W] rows of G_{m+1,m} at the boundary rows (left CTA's copy is used)
   const size_t uoff = ((size_t)kf * g.p + i) * (size_t)Lx * n;
   cxl* gout = reinterpret_cast<cxl*>(b.g64) + uoff;
   cxf* gsw = reinterpret_cast<cxf*>(b.g) + uoff;
   cxd* dB = b.diagB + (size_t)kf * g.Ndd + (size_t)i * Lx * W;
+  const cdfl* hd = reinterpret_cast<const cdfl*>(b.hdiag) + (size_t)kf * g.Ndd + (size_t)i * Lx * W;
   const bool band = !g.lpre;                 // the banded preconditioner reads the off-diagonal blocks
   cxd* oB = band && b.offB ? b.offB + ((size_t)kf * g.p + i) * (size_t)Lx * W : nullptr;
   cxd* o2 = band && b.off2 && T == 1 ? b.off2 + ((size_t)kf * g.p + i) * (size_t)Lx * W : nullptr;
   const dfl t = (dfl)g.t, t2 = (dfl)(g.t * g.t);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
-  // the triangle entries (r <= c) this thread owns: rows of length W, W - 1, ...
-  int er[NE], ec[NE];
-  bool on[NE];
-#pragma unroll
-  for (int q = 0; q < NE; ++q) {
-    int e = tid + DY_THREADS * q, r = 0;
-    on[q] = e < W * (W + 1) / 2;
-    while (on[q] && e >= W - r) {
+  // triangle entry number e (rows of length W, W - 1, ...) as (r, c), r <= c; (0, 0) past the end
+  auto tri = [&](int e, int& r, int& c) {
+    r = 0;
+    const bool on = e < ntri;
+    while (on && e >= W - r) {
       e -= W - r;
       ++r;
     }
-    er[q] = r;
-    ec[q] = r + e;
-  }
-
-  // A <- (D_s - t^2 (pa + pb))^-1, zero on the padding; pa, pb (full W x W, either may be
-  // null) may be A itself; stored in slot s when keep
-  auto invert = [&](int s, const cxl* pa, const cxl* pb, bool keep) {
-    cxl v[NE];
+    c = on ? r + e : 0;
+    return on;
+  };
+  int er[NE], ec[NE], pr[NP], pc[NP];
+  unsigned eon = 0, pon = 0;                 // bit q: entry q exists
 #pragma unroll
-    for (int q = 0; q < NE; ++q) {
-      if (!on[q]) continue;
-      const int r = er[q], c = ec[q], e = r * W + c;
+  for (int q = 0; q < NE; ++q)
+    if (tri(wid > 0 ? tid - 32 + OWN * q : ntri, er[q], ec[q])) eon |= 1u << q;
+#pragma unroll
+  for (int q = 0; q < NP; ++q)
+    if (tri(tid + DY_THREADS * q, pr[q], pc[q])) pon |= 1u << q;
+
+  auto load_h = [&](int s) {
+    if (tid < W) {
+      const cdfl d = hd[(size_t)s * W + tid];
+      dg[tid] = cxl{d.x, d.y};
+    }
+  };
+  // A <- (D_s - t^2 (pa + pb))^-1, zero on the padding; pa, pb (full W x W, either may be
+  // null) may be A itself; stored in slot s when keep.  dg holds slice s's diagonal;
+  // slice sn's (if >= 0) is fetched for the next call.
+  auto invert = [&](int s, const cxl* pa, const cxl* pb, bool keep, int sn) {
+    cxl v[NE];
+    cdfl hn = {dfl(0.f, 0.f), dfl(0.f, 0.f)};
+    if (sn >= 0 && tid < W) hn = hd[(size_t)sn * W + tid];
+    auto formed = [&](int r, int c) -> cxl {
+      const int e = r * W + c;
       cxl x = {0, 0};
       if (pa) x = x - t2 * pa[e];
       if (pb) x = x - t2 * pb[e];
-      if (c < w) {
-        if (r == c) x = x + cconv<dfl>(dyson_diag(g, b, kf, sub_nat(g, i, s, r)));
+      if (r < w && c < w) {
+        if (r == c) x = x + dg[r];
         else if (slice_adjacent<dfl>(r, c, T)) x.x += t;
       } else {
         x = r == c ? cxl{1, 0} : cxl{0, 0};
       }
-      v[q] = x;
-      if (r == 0) prow[c] = x;               // the first pivot's column
+      return x;
+    };
+#pragma unroll
+    for (int q = 0; q < NE; ++q) v[q] = wid > 0 ? formed(er[q], ec[q]) : cxl{0, 0};
+    if (wid == 0) {
+      for (int e = lane; e < W; e += 32) {
+        prow[e] = formed(0, e);
+        craw[W + e] = formed(e < 1 ? e : 1, e < 1 ? 1 : e);       // column 1
+      }
+      __syncwarp();
+      const cxl piv = inv_l(prow[0]);
+      for (int e = lane; e < W; e += 32) fcol[e] = e == 0 ? -piv : prow[e] * piv;
     }
     for (int k = 0; k < W; ++k) {
-      cxl* pk = prow + (k & 1) * W;
-      cxl* pn = prow + ((k + 1) & 1) * W;
-      __syncthreads();                       // column k published; A, fcol free
+      const cxl *pk = prow + (k & 1) * W, *fk = fcol + (k & 1) * W, *cr = craw + ((k + 1) & 1) * W;
+      cxl *pn = prow + ((k + 1) & 1) * W, *fn = fcol + ((k + 1) & 1) * W, *cn = craw + (k & 1) * W;
+      __syncthreads();                       // pk, fk and column k + 1 as of pivot k - 1 are complete
       if (wid == 0) {
-        const cxl piv = cinv(pk[k]);
-        for (int e = lane; e < W; e += 32) fcol[e] = e == k ? -piv : pk[e] * piv;
-      }
-      __syncthreads();
-      const bool rn = (k & 3) == 3 || k == W - 1;
-#pragma unroll
-      for (int q = 0; q < NE; ++q) {
-        if (!on[q]) continue;
-        const int r = er[q], c = ec[q];
-        if (r == k || c == k) {
-          v[q] = fcol[r == k ? c : r];
-        } else {
-          const cxl f = fcol[r];
-          v[q] = mac_l(cxl{-f.x, -f.y}, pk[c], v[q]);
-          if (rn) v[q] = norm_l(v[q]);
+        if (k + 1 < W) {
+          const cxl p1 = pk[k + 1], f1 = fk[k + 1];
+          for (int e = lane; e < W; e += 32) {
+            // the same product the entry's owner forms (f of the row, p of the column)
+            const bool up = e <= k + 1;
+            cxl x = cfma(up ? -fk[e] : -f1, up ? p1 : pk[e], cr[e]);
+            if (e == k) x = f1;
+            pn[e] = x;
+          }
+          __syncwarp();
+          const cxl piv = inv_l(pn[k + 1]);
+          for (int e = lane; e < W; e += 32) {
+            const cxl x = pn[e] * piv;
+            fn[e] = e == k + 1 ? -piv : x;
+          }
         }
-        if (r == k + 1) pn[c] = v[q];
-        else if (c == k + 1) pn[r] = v[q];
+      } else {
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {
+          const int r = er[q], c = ec[q];
+          const cxl f = fk[r], x = fk[r == k ? c : r];
+          const cxl u = cfma(-f, pk[c], v[q]);
+          v[q] = r == k || c == k ? x : u;
+        }
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {       // column k + 2 for the pivot warp
+          if (!(eon >> q & 1)) continue;
+          if (er[q] == k + 2) cn[ec[q]] = v[q];
+          else if (ec[q] == k + 2) cn[er[q]] = v[q];
+        }
       }
     }
+    __syncthreads();                         // every read of A (pa) is long past; fcol free
 #pragma unroll
     for (int q = 0; q < NE; ++q) {           // -(-A^-1), both triangles
-      if (!on[q]) continue;
+      if (!(eon >> q & 1)) continue;
       const int r = er[q], c = ec[q];
-      cxl x = norm_l(v[q]);
-      x = c < w ? cxl{-x.x, -x.y} : cxl{0, 0};
+      const cxl x = c < w ? -v[q] : cxl{0, 0};
       A[r * W + c] = x;
       A[c * W + r] = x;
     }
+    if (sn >= 0 && tid < W) dg[tid] = cxl{hn.x, hn.y};
     __syncthreads();
     if (keep)
       for (int e = tid; e < n; e += DY_THREADS) {
@@ -344,38 +393,58 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 3 : 1) k_factor_two(Geo
         gout[(size_t)s * n + e] = x;
         gsw[(size_t)s * n + ((size_t)(c >> 1) * W + r) * 2 + (c & 1)] = cconv<float>(x);
       }
-    __syncthreads();
   };
+  // the layer preconditioner's input: columns w - 1 and 0 of G_ss (k_surface_two)
+  cxf* bc = g.lpre ? b.lpg + uoff : nullptr;
   auto diag_out = [&](int s) {
     for (int r = tid; r < W; r += DY_THREADS) dB[(size_t)s * W + r] = (r < w) ? cconv<double>(A[r * W + r]) : cxd{0, 0};
+    if (bc)
+      for (int e = tid; e < 2 * W; e += DY_THREADS) {
+        const int sd = e / W, r = e - sd * W;
+        bc[((size_t)s * 2 + sd) * W + r] = cconv<float>(A[r * W + (sd == 0 ? w - 1 : 0)]);
+      }
   };
-  // A <- g_s + t^2 g_s A g_s with g_s from slot s, A = G of the neighbour towards the
-  // middle, slice sn (see k_factor for the off-diagonal by-products)
-  auto grow = [&](int s, int sn, const cxl* prevc, bool mid) {
-    for (int e = tid; e < n; e += DY_THREADS) Bm[e] = gout[(size_t)s * n + e];
+  cxl nb[NB];                                // the next slice's factor on its way to Bm
+  auto fetch = [&](int s) {
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int e = tid + DY_THREADS * q;
+      nb[q] = e < n ? gout[(size_t)s * n + e] : cxl{0, 0};
+    }
+  };
+  // A <- g_s + t^2 g_s A g_s with g_s from nb, A = G of the neighbour towards the
+  // middle, slice sn; -t g_s A is the off-diagonal block G_{s,sn}, whose diagonal (and,
+  // through the boundary columns prevc of G_{sn,s2}, s2 = 2 sn - s, the distance-2
+  // couplings on the two boundary rows) the banded preconditioner uses.  mid: also put
+  // the boundary rows of G_{s,sn} into the left CTA's Gmid.  nx: the next slice (or -1).
+  auto grow = [&](int s, int sn, const cxl* prevc, bool mid, int nx) {
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int e = tid + DY_THREADS * q;
+      if (e < n) Bm[e] = nb[q];
+    }
     __syncthreads();
-    // Cm = g_s A: lane = column (WF >= 32), 8 warps' rows; the row of g_s is a broadcast
-    for (int e0 = tid; e0 < n; e0 += 4 * DY_THREADS) {
-      cxl acc[4];
-      int rr[4], cc[4];
+    if (nx >= 0) fetch(nx);
+    // Cm = g_s A, 2 x 2 entries a thread: rows r, r + W/2, columns c, c + W/2
+    const int h = W / 2;
+    for (int e = tid; e < h * h; e += DY_THREADS) {
+      const int r = e / h, c = e - r * h;
+      const cxl *x0 = Bm + r * W, *x1 = x0 + h * W, *y = A + c;
+      cxl a00 = {0, 0}, a01 = {0, 0}, a10 = {0, 0}, a11 = {0, 0};
+      for (int k0 = 0; k0 < W; k0 += 2) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int e = e0 + u * DY_THREADS;
-        rr[u] = e < n ? e / W : 0;
-        cc[u] = e < n ? e - rr[u] * W : 0;
-        acc[u] = cxl{0, 0};
+        for (int k = k0; k < k0 + 2; ++k) {
+          const cxl xa = x0[k], xb = x1[k], ya = y[k * W], yb = y[k * W + h];
+          a00 = cfma(xa, ya, a00);
+          a01 = cfma(xa, yb, a01);
+          a10 = cfma(xb, ya, a10);
+          a11 = cfma(xb, yb, a11);
+        }
       }
-      for (int k0 = 0; k0 < W; k0 += 4) {    // W is a multiple of 4
-#pragma unroll
-        for (int k = k0; k < k0 + 4; ++k)
-#pragma unroll
-          for (int u = 0; u < 4; ++u) acc[u] = mac_l(Bm[rr[u] * W + k], A[k * W + cc[u]], acc[u]);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u] = norm_l(acc[u]);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (e0 + u * DY_THREADS < n) Cm[e0 + u * DY_THREADS] = acc[u];
+      Cm[r * W + c] = a00;
+      Cm[r * W + c + h] = a01;
+      Cm[(r + h) * W + c] = a10;
+      Cm[(r + h) * W + c + h] = a11;
     }
     __syncthreads();
     if (oB)
@@ -401,46 +470,56 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 3 : 1) k_factor_two(Geo
         if (mid) other[e] = (-t) * Cm[j * W + c];
       }
     }
-    // g_s + t^2 (g_s A) g_s on the upper triangle, mirrored
-    cxl v[NE];
+    // g_s + t^2 (g_s A) g_s on the upper triangle, mirrored; a warp without a last entry
+    // leaves it out
+    auto last = [&](auto nq) {
+      constexpr int NQ = decltype(nq)::value;
+      cxl v[NQ > 0 ? NQ : 1];
 #pragma unroll
-    for (int q = 0; q < NE; ++q) v[q] = cxl{0, 0};
-    for (int k0 = 0; k0 < W; k0 += 4) {
+      for (int q = 0; q < NQ; ++q) v[q] = cxl{0, 0};
+      for (int k0 = 0; k0 < W; k0 += 2) {
 #pragma unroll
-      for (int q = 0; q < NE; ++q) {
-        if (!on[q]) continue;
+        for (int k = k0; k < k0 + 2; ++k)
 #pragma unroll
-        for (int k = k0; k < k0 + 4; ++k) v[q] = mac_l(Cm[er[q] * W + k], Bm[k * W + ec[q]], v[q]);
-        v[q] = norm_l(v[q]);
+          for (int q = 0; q < NQ; ++q) v[q] = cfma(Cm[pr[q] * W + k], Bm[k * W + pc[q]], v[q]);
       }
-    }
 #pragma unroll
-    for (int q = 0; q < NE; ++q) {
-      if (!on[q]) continue;
-      const int r = er[q], c = ec[q];
-      const cxl x = Bm[r * W + c] + t2 * v[q];
-      A[r * W + c] = x;
-      A[c * W + r] = x;
-    }
+      for (int q = 0; q < NQ; ++q) {
+        if (!(pon >> q & 1)) continue;
+        const int r = pr[q], c = pc[q];
+        const cxl x = Bm[r * W + c] + t2 * v[q];
+        A[r * W + c] = x;
+        A[c * W + r] = x;
+      }
+    };
+    if (NP > 1 && wid * 32 + DY_THREADS * (NP - 1) >= ntri) last(std::integral_constant<int, NP - 1>{});
+    else last(std::integral_constant<int, NP>{});
     __syncthreads();
     diag_out(s);
-    __syncthreads();
   };
 
+  load_h(side == 0 ? 0 : Lx - 1);
+  __syncthreads();
   if (side == 0) {
-    for (int s = 0; s < m; ++s) invert(s, s > 0 ? A : nullptr, nullptr, true);
+    for (int s = 0; s < m; ++s) invert(s, s > 0 ? A : nullptr, nullptr, true, s + 1);
   } else {
-    for (int s = Lx - 1; s > m; --s) invert(s, s < Lx - 1 ? A : nullptr, nullptr, true);
+    for (int s = Lx - 1; s > m; --s) invert(s, s < Lx - 1 ? A : nullptr, nullptr, true, s - 1);
   }
   cl.sync();                                 // both neighbours of the middle slice are stored
-  invert(m, m > 0 ? gout + (size_t)(m - 1) * n : nullptr, m < Lx - 1 ? gout + (size_t)(m + 1) * n : nullptr, side == 0);
+  invert(m, m > 0 ? gout + (size_t)(m - 1) * n : nullptr, m < Lx - 1 ? gout + (size_t)(m + 1) * n : nullptr,
+         side == 0, -1);
   if (side == 0) diag_out(m);
-  if (side == 1 && m + 1 < Lx) grow(m + 1, m, nullptr, true);
+  if (side == 1 && m + 1 < Lx) {
+    fetch(m + 1);
+    __syncthreads();
+    grow(m + 1, m, nullptr, true, m + 2 < Lx ? m + 2 : -1);
+  }
   cl.sync();                                 // Gmid is in the left CTA's shared memory
   if (side == 1) {
-    for (int s = m + 2; s < Lx; ++s) grow(s, s - 1, Gprev, false);
-  } else {
-    for (int s = m - 1; s >= 0; --s) grow(s, s + 1, s < m - 1 ? Gprev : (m + 1 < Lx ? Gmid : nullptr), false);
+    for (int s = m + 2; s < Lx; ++s) grow(s, s - 1, Gprev, false, s + 1 < Lx ? s + 1 : -1);
+  } else if (m > 0) {
+    fetch(m - 1);
+    for (int s = m - 1; s >= 0; --s) grow(s, s + 1, s < m - 1 ? Gprev : (m + 1 < Lx ? Gmid : nullptr), false, s - 1);
   }
   // interface part of diag(B^-1) is zero (blkdiag(B^-1, 0), Eq. 9)
   if (i == g.p - 1 && side == 0) {
@@ -828,7 +907,7 @@ __global__ void __launch_bounds__(DY_THREADS) k_hdiag(Geo g, Bufs b) {
        k += (size_t)gridDim.x * blockDim.x) {
     const int nat = b.dd2nat[k];
     const cxd d = nat >= 0 ? dyson_diag(g, b, kf, nat) : cxd{0, 0};
-    if (g.W <= DY_MAXW_SMEM) reinterpret_cast<cdfl*>(b.hdiag)[(size_t)kf * g.Ndd + k] = csplit(d);
+    if (g.W <= DY_MAXW_SMEM) reinterpret_cast<cdfl*>(b.hdiag)[(size_t)kf * g.Ndd + k] = cdfl{dfl(d.x), dfl(d.y)};   // 48 bits
     else b.hdiag[(size_t)kf * g.Ndd + k] = d;
   }
 }
@@ -855,7 +934,7 @@ cudaError_t launch_factor(const Geo& g, const Bufs& b, int K, cudaStream_t st) {
     }
   }
   if constexpr (std::is_same<R, dfl>::value) {
-    const size_t smem = (3 * (size_t)g.W * g.W + 7 * (size_t)g.W) * sizeof(cxl);
+    const size_t smem = (3 * (size_t)g.W * g.W + 11 * (size_t)g.W) * sizeof(cxl);
     auto kern = g.W <= 16 ? k_factor_two<16> : (g.W <= 32 ? k_factor_two<32> : k_factor_two<64>);
     return launch_clustered(kern, dim3(2 * g.p, K), 2, smem, st, g, b);
   } else {

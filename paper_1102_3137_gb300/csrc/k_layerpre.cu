@@ -338,6 +338,145 @@ __global__ void __launch_bounds__(DY_THREADS) k_surface_g(Geo g, Bufs b) {
   }
 }
 
+// The surface Green's functions of the mixed form's strips, from the two-sided
+// factors g_s and the boundary columns of G_ss that the factorization leaves (in
+// complex64, the latter in b.lpg): no recursion of its own.  With m the middle slice
+// and rb the boundary row, per side:
+//   pairs of one half:  G_{s,c} e_rb = -t g_s G_{s+-1,c} e_rb   (towards the ends, all c at once)
+//   pairs across:       G_{s,c} = G_{s,m} N_c^T,  G_{s,m} = -t g_s G_{s+1,m} (s < m),
+//                       N_c = -t g_c N_{c-1}, N_m = 1 (c > m)
+// so a half is one chain of products of the 32 x 32 block -t g_s with its boundary
+// columns plus W columns of G_{.,m} or N, and the across pairs are dot products of the
+// rows rb of the two.  A cluster of two CTAs (left, right) per (side, strip, frequency),
+// lane = row with its row of g_s in registers, a warp's columns two at a time by 16-byte
+// broadcasts from shared memory.  The one-CTA form ran its own complex64 recursion and a
+// chain of Lx slices: 4.0 ms at 128^2 x 32 with 128 CTAs.
+template <int WT>
+__global__ void __launch_bounds__(DY_THREADS, 2) k_surface_two(Geo g, Bufs b) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cg::cluster_group cl = cg::this_cluster();
+  const int half = (int)cl.block_rank(), u = blockIdx.x / 2, i = u / 2, sd = u - 2 * i, f = blockIdx.y;
+  const int W = WT ? WT : g.W, Lx = g.Lx, w = g.h[i], n = W * W, m = Lx / 2;
+  if (sd == 0 ? i == g.p - 1 : i == 0) return;                  // no layer on that side (the whole cluster)
+  const int steps = half == 0 ? m : Lx - 1 - m, rb = sd == 0 ? w - 1 : 0;
+  cxf_* gb[2] = {reinterpret_cast<cxf_*>(smem_raw), reinterpret_cast<cxf_*>(smem_raw) + n};
+  cxf_* M = gb[1] + n;                            // [W columns][W]: G_{s,m} or N_s
+  cxf_* V = M + n;                                // [steps][W]: the boundary columns, by distance from the middle
+  const size_t unit = (size_t)f * g.p + i;
+  const cxf_* gsrc = reinterpret_cast<const cxf_*>(b.g) + unit * (size_t)Lx * n;   // column pairs interleaved
+  const cxf_* bc = b.lpg + unit * (size_t)Lx * n;
+  cxf_* Rr = b.lpg + unit * (size_t)Lx * n + (size_t)2 * Lx * W + (size_t)sd * Lx * W;   // [Lx][W] rows rb of G_{s,m} / N_s
+  cxf_* P = b.lpt + (unit * 2 + sd) * (size_t)Lx * Lx;
+  const float t = d2f_bits(g.t);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int n4 = n / 2;                           // 16-byte words of a block
+  auto slice = [&](int k) { return half == 0 ? m - 1 - k : m + 1 + k; };     // k-th step's slice
+  constexpr int NF = (SURF_MAXW * SURF_MAXW / 2 + DY_THREADS - 1) / DY_THREADS;
+  float4 nx[NF];
+  auto fetch = [&](int s) {
+#pragma unroll
+    for (int q = 0; q < NF; ++q)
+      if (tid + DY_THREADS * q < n4) nx[q] = reinterpret_cast<const float4*>(gsrc + (size_t)s * n)[tid + DY_THREADS * q];
+  };
+  auto put = [&](cxf_* d) {
+#pragma unroll
+    for (int q = 0; q < NF; ++q)
+      if (tid + DY_THREADS * q < n4) reinterpret_cast<float4*>(d)[tid + DY_THREADS * q] = nx[q];
+  };
+  // M: G_mm (slot m; symmetric, so its rows are its columns) or 1
+  for (int e = tid; e < n; e += DY_THREADS) {
+    const int c = e / W, r = e - c * W;
+    M[e] = half == 0 ? gsrc[(size_t)m * n + ((size_t)(c >> 1) * W + r) * 2 + (c & 1)] : cxf_{r == c ? 1.f : 0.f, 0.f};
+  }
+  if (steps > 0) {
+    fetch(slice(0));
+    put(gb[0]);
+  }
+  __syncthreads();
+  if (half == 0) {                                // s = m: row rb of G_mm, and P[m][m]
+    for (int c = tid; c < W; c += DY_THREADS) Rr[(size_t)m * W + c] = M[c * W + rb];
+    if (tid == 0) P[(size_t)m * Lx + m] = M[rb * W + rb];
+  }
+  for (int k = 0; k < steps; ++k) {
+    const int s = slice(k);
+    const cxf_* G = gb[k & 1];
+    if (k + 1 < steps) fetch(slice(k + 1));
+    cxf_ gr[SURF_MAXW];                           // row `lane` of -t g_s
+#pragma unroll
+    for (int q = 0; q < SURF_MAXW / 2; ++q) {
+      const float4 v = lane < W && 2 * q < W ? reinterpret_cast<const float4*>(G)[q * W + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+      gr[2 * q] = cxf_{-t * v.x, -t * v.y};
+      gr[2 * q + 1] = cxf_{-t * v.z, -t * v.w};
+    }
+    // this step's columns: W of M, then the boundary columns of the k slices nearer the middle
+    const int nc = W + k;
+    for (int c0 = 2 * wid; c0 < nc; c0 += 2 * DY_WARPS) {
+      const bool b2 = c0 + 1 < nc;
+      cxf_* x0 = M + (size_t)c0 * W;              // M and V are contiguous: column c at M + c W
+      cxf_* x1 = b2 ? x0 + W : x0;
+      cxf_ a0 = {0.f, 0.f}, a1 = {0.f, 0.f}, d0 = {0.f, 0.f}, d1 = {0.f, 0.f};
+#pragma unroll
+      for (int q = 0; q < SURF_MAXW / 2; ++q) {
+        if (2 * q < W) {
+          const float4 v = reinterpret_cast<const float4*>(x0)[q], y = reinterpret_cast<const float4*>(x1)[q];
+          a0 = cfma(gr[2 * q], cxf_{v.x, v.y}, a0);
+          d0 = cfma(gr[2 * q], cxf_{y.x, y.y}, d0);
+          a1 = cfma(gr[2 * q + 1], cxf_{v.z, v.w}, a1);
+          d1 = cfma(gr[2 * q + 1], cxf_{y.z, y.w}, d1);
+        }
+      }
+      a0 = a0 + a1;
+      d0 = d0 + d1;
+      __syncwarp();                               // both columns are read before they are rewritten
+      auto out = [&](int c, cxf_* x, cxf_ v) {
+        if (lane >= W) return;
+        x[lane] = v;
+        if (lane != rb) return;
+        if (c < W) {
+          Rr[(size_t)s * W + c] = v;
+          if (half == 0 && c == rb) P[(size_t)s * Lx + m] = P[(size_t)m * Lx + s] = v;
+        } else {
+          const int sc = slice(c - W);
+          P[(size_t)s * Lx + sc] = P[(size_t)sc * Lx + s] = v;
+        }
+      };
+      out(c0, x0, a0);
+      if (b2) out(c0 + 1, x1, d0);
+    }
+    // the chain of column s starts with the boundary column of G_ss
+    for (int r = tid; r < W; r += DY_THREADS) {
+      const cxf_ v = bc[((size_t)s * 2 + sd) * W + r];
+      V[(size_t)k * W + r] = v;
+      if (r == rb) P[(size_t)s * Lx + s] = v;
+    }
+    if (k + 1 < steps) put(gb[(k + 1) & 1]);
+    __syncthreads();
+  }
+  cl.sync();                                      // the rows of both halves are written
+  // pairs across the middle: P[s][c] = row_s . row_c, s <= m < c
+  const int na = m + 1, ncr = Lx - 1 - m;
+  cxf_* tb = reinterpret_cast<cxf_*>(smem_raw);   // [W][33] rows of 32 slices c, transposed (the chain's space)
+  for (int c0 = 0; c0 < ncr; c0 += 32) {
+    __syncthreads();
+    for (int e = tid; e < 32 * W; e += DY_THREADS) {
+      const int q = e / W, x = e - q * W;
+      tb[x * 33 + q] = c0 + q < ncr ? Rr[(size_t)(m + 1 + c0 + q) * W + x] : cxf_{0.f, 0.f};
+    }
+    __syncthreads();
+    for (int s = half * DY_WARPS + wid; s < na; s += 2 * DY_WARPS) {
+      cxf_ a = {0.f, 0.f}, d = {0.f, 0.f};
+      const cxf_* row = Rr + (size_t)s * W;
+      for (int x = 0; x < W; x += 2) {
+        a = cfma(row[x], tb[x * 33 + lane], a);
+        d = cfma(row[x + 1], tb[(x + 1) * 33 + lane], d);
+      }
+      a = a + d;
+      const int c = m + 1 + c0 + lane;
+      if (c < Lx) P[(size_t)s * Lx + c] = P[(size_t)c * Lx + s] = a;
+    }
+  }
+}
+
 // C (M x N, row stride ldc) = alpha X Y (+ D), X: M x K, Y: K x N, D: M x N, all in
 // global memory in any of binary64 / complex64 (converted to complex64 on load),
 // 32 x 32 tiles staged through shared memory and multiplied on the tensor cores
@@ -683,6 +822,12 @@ cudaError_t launch_surface(const Geo& g, const Bufs& b, int K, cudaStream_t st) 
     return launch_clustered(k_surface_3d<cxd>, dim3(grid), C, 0, st, g, b, K);
   }
   if (g.W > SURF_MAXW || g.Lx > DY_LPRE_MAXLX_G) return cudaErrorInvalidValue;
+  if (b.g64) {                             // mixed form: from the two-sided factors
+    size_t smem = (3 * (size_t)g.W * g.W + (size_t)(g.Lx / 2) * g.W) * sizeof(cxf_);
+    const size_t tb = (size_t)33 * g.W * sizeof(cxf_);
+    if (smem < tb) smem = tb;
+    return launch_clustered(g.W == 32 ? k_surface_two<32> : k_surface_two<0>, dim3(4 * g.p, K), 2, smem, st, g, b);
+  }
   if (g.Lx > DY_LPRE_MAXLX) {
     if (g.W != 32 || !b.lpv) return cudaErrorInvalidValue;
     k_surface_g<<<dim3(g.p, K), DY_THREADS, surface_g_smem(), st>>>(g, b);
