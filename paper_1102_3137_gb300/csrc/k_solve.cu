@@ -231,7 +231,7 @@ void dyson_internal_ring_plan(const Geo& g, bool mixed, int* S, int* CR, int* NT
   const RingPlan rp = mixed ? ring_plan<float>(g) : ring_plan<double>(g);
   *S = rp.S;
   *CR = rp.CR;
-  *NT = DY_THREADS;
+  *NT = g.W > DY_MAXW_SMEM ? WIDE_THREADS : DY_THREADS;
 }
 
 int dyson_internal_ring_candidates(const Geo& g, bool mixed, int* S, int* CR, int* ROWS, int max) {

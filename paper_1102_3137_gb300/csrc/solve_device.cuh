@@ -181,7 +181,8 @@ __device__ __forceinline__ void ring_wait(uint64_t* bar, uint32_t parity, bool& 
 
 // Per-CTA copy pipeline: S slots of one W x W block each, one mbarrier per slot.
 struct Pipe {
-  uint64_t* bar;   // [S] in static shared memory
+  uint64_t* bar;   // [S] in static shared memory: a slot's copy has landed
+  uint64_t* empty; // [S] a slot's block has been read (the wide form, one arrival per compute warp)
   void* ring;      // S slots in dynamic shared memory
   void* ybuf;      // forward intermediates in shared memory, or null (global scratch)
   int S;
@@ -191,10 +192,24 @@ struct Pipe {
 };
 
 constexpr int MAX_STAGES = 8;
+constexpr int WIDE_WARPS = 16;                    // compute warps of the wide sweep, one more issues the copies
+constexpr int WIDE_THREADS = 32 * (WIDE_WARPS + 1);
+template <int WF>
+constexpr int solve_threads() { return WF == 0 ? WIDE_THREADS : DY_THREADS; }
+// groups of compute threads of the wide sweep: W / V threads cover a block row
+// 16 bytes each (V entries)
+template <typename R>
+__host__ __device__ inline int wide_groups(int W) { return 32 * WIDE_WARPS / (W * (int)sizeof(cx<R>) / 16); }
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
 
 __device__ void pipe_init(Pipe& pp) {
   if (threadIdx.x == 0) {
-    for (int k = 0; k < pp.S; ++k) mbar_init(pp.bar + k, 1);
+    for (int k = 0; k < pp.S; ++k) {
+      mbar_init(pp.bar + k, 1);
+      mbar_init(pp.empty + k, WIDE_WARPS);
+    }
     *pp.err = 0;
     fence_mbar_init();
   }
@@ -428,92 +443,123 @@ __device__ void sweep(const Geo& g, int i, const SweepArgs<R>& a, cx<R>* sm, Pip
 }
 
 // Wide slices (W > 64, 3D slabs): a slice block streams as NC = W / CR chunks
-// of CR rows (NC = 1 when whole blocks leave enough ring slots); each chunk's
-// rows are finished as soon as it arrives and its slot is released after a
-// barrier.  The row buffer yb is always on chip on this path.
+// of CR rows.  The blocks are symmetric, so a chunk's rows are read as columns:
+// thread (grp, rv) owns the outputs rv V .. rv V + V - 1 (16 bytes of a row, V = 2
+// in complex64) and adds up the chunk rows grp, grp + ng, ... of every chunk of the
+// slice in registers; the ng partial sums of an output meet once a slice.  Nothing
+// synchronises the CTA between chunks: a warp waits for a chunk's copy, and its
+// arrival on the slot's second barrier lets the producer warp refill it.  (Finishing
+// a chunk's rows with shuffles and a CTA barrier each, in 256 threads, took 12.8 k
+// cycles a slice at W = 128, 16.6 k at 144, several times the copies' time.)
+// The row buffer yb is always on chip on this path.
 template <typename R>
 __device__ void sweep_chunked(const Geo& g, int i, const SweepArgs<R>& a, cx<R>* sm, Pipe& pp,
                               unsigned long long* cnt) {
+  using C = cx<R>;
+  constexpr int V = 16 / (int)sizeof(C), NTC = 32 * WIDE_WARPS;
   bool dead = *pp.err != 0;              // an earlier wait of this CTA ran out
   const int W = g.W, Lx = g.Lx;
-  const int CR = pp.CR, NC = W / CR;
-  const SweepLayout L = sweep_layout(CR, W);
-  cx<R>* zbuf = sm;
-  cx<R>* ring = reinterpret_cast<cx<R>*>(pp.ring);
-  cx<R>* yb = reinterpret_cast<cx<R>*>(pp.ybuf);
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int rr = lane / L.G, cg = lane - rr * L.G;
-  const int lrow = wid * L.RPW + rr;     // row inside a chunk
-  const bool rvalid = lrow < CR;
-  const bool owner = rvalid && cg == 0;
-  const int rot = (W % L.G == 0) ? (rr * L.G) % W : 0;
+  const int CR = pp.CR, NC = W / CR, WV = W / V, ng = wide_groups<R>(W);
+  C* zbuf = sm;                          // [2][W]
+  C* part = sm + 2 * W;                  // [ng][W]
+  C* ring = reinterpret_cast<C*>(pp.ring);
+  C* yb = reinterpret_cast<C*>(pp.ybuf);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int grp = tid / WV, rv = (tid - grp * WV) * V;
+  const bool active = tid < NTC && grp < ng;
   const R t = (R)g.t;
-  const int WW = W * W, CW = CR * W;
-  const uint32_t bytes = (uint32_t)(CW * sizeof(cx<R>));
+  const int CW = CR * W;
+  const uint32_t bytes = (uint32_t)(CW * sizeof(C));
   const int NL = 2 * Lx - 1, NQ = NL * NC;
   const int S = pp.S;
   auto slice_of = [&](int n) { return n < Lx ? n : 2 * Lx - 2 - n; };
-  auto issue = [&](int q) {
-    const unsigned qq = pp.seq + q;
-    const int slot = (int)(qq % S);
-    const int n = q / NC, c = q - n * NC;
-    bulk_load(ring + (size_t)slot * CW, a.g + (size_t)slice_of(n) * WW + (size_t)c * CW, bytes,
-              pp.bar + slot);
-  };
+  auto csync = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(NTC) : "memory"); };
 
-  __syncthreads();
-  if (tid == 0) {
+  // the producer's next chunk: q-th of the sweep, chunk pc of step pn
+  int q = 0, pn = 0, pc = 0;
+  auto issue = [&]() {
+    const unsigned qq = pp.seq + q, u = qq / S;
+    const int slot = (int)(qq - u * S);
+    if (u > 0) ring_wait(pp.empty + slot, (u - 1) & 1u, dead, pp.err);
+    bulk_load(ring + (size_t)slot * CW, a.g + ((size_t)slice_of(pn) * NC + pc) * CW, bytes, pp.bar + slot);
+    ++q;
+    if (++pc == NC) {
+      pc = 0;
+      ++pn;
+    }
+  };
+  __syncthreads();                       // previous users of zbuf and yb are done
+  if (tid == NTC) {                      // the first S chunks: their slots were read in the last sweep
     fence_proxy_async();
-    for (int q = 0; q < S && q < NQ; ++q) issue(q);
+    while (q < S && q < NQ) issue();
   }
   sweep_prepass<R>(g, i, a, yb);
   __syncthreads();
-  for (int e = tid; e < W; e += (int)blockDim.x) zbuf[e] = yb[e];
-  __syncthreads();
-  for (int n = 0; n < NL; ++n) {
-    const int s = slice_of(n);
-    const cx<R>* zc = zbuf + (n & 1) * W;
-    cx<R>* zn = zbuf + ((n + 1) & 1) * W;
-    for (int c = 0; c < NC; ++c) {
-      const int q = n * NC + c;
-      const unsigned qq = pp.seq + q;
-      const int slot = (int)(qq % S);
-      ring_wait(pp.bar + slot, (qq / S) & 1u, dead, pp.err);
-      const cx<R>* grow = ring + (size_t)slot * CW + (size_t)lrow * W;
-      cx<R> acc = {0, 0};
-      if (rvalid) {
-#pragma unroll 4
-        for (int k = 0; k < L.CPG; ++k) {
-          const int base = cg + L.G * k;
-          if (base < W) {
-            int col = base + rot;
-            if (col >= W) col -= W;
-            acc = cfma(grow[col], zc[col], acc);
+  if (tid == NTC)
+    while (q < NQ) issue();
+  if (tid < NTC) {
+    if (tid < W) zbuf[tid] = yb[tid];
+    csync();
+    unsigned qq = pp.seq, u = qq / S;
+    int slot = (int)(qq - u * S);
+    uint32_t ph = u & 1u;
+    for (int n = 0; n < NL; ++n) {
+      const int s = slice_of(n);
+      const C* zc = zbuf + (n & 1) * W;
+      C* zn = zbuf + ((n + 1) & 1) * W;
+      C acc[2][V] = {};
+      for (int c = 0; c < NC; ++c) {
+        ring_wait(pp.bar + slot, ph, dead, pp.err);
+        if (active) {
+          const C* blk = ring + (size_t)slot * CW + rv;
+          const C* zk = zc + c * CR;
+          auto term = [&](int r, int k) {
+            const C z = zk[r];
+            if constexpr (V == 2) {
+              const float4 m = *reinterpret_cast<const float4*>(blk + r * W);
+              acc[k][0] = cfma(C{m.x, m.y}, z, acc[k][0]);
+              acc[k][1] = cfma(C{m.z, m.w}, z, acc[k][1]);
+            } else {
+              acc[k][0] = cfma(blk[r * W], z, acc[k][0]);
+            }
+          };
+          int r = grp;
+          for (; r + 3 * ng < CR; r += 4 * ng) {
+            term(r, 0);
+            term(r + ng, 1);
+            term(r + 2 * ng, 0);
+            term(r + 3 * ng, 1);
           }
+          for (; r < CR; r += ng) term(r, 0);
+        }
+        __syncwarp();                    // the warp's reads of the slot are done
+        if (lane == 0) mbar_arrive(pp.empty + slot);
+        if (++slot == S) {
+          slot = 0;
+          ph ^= 1u;
         }
       }
-      for (int off = L.G >> 1; off > 0; off >>= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
+      if (active) {
+#pragma unroll
+        for (int v = 0; v < V; ++v) part[grp * W + rv + v] = acc[0][v] + acc[1][v];
       }
-      if (owner) {
-        const int row = c * CR + lrow;
+      csync();
+      if (tid < W) {
+        C y = part[tid];
+        for (int k = 1; k < ng; ++k) y = y + part[k * W + tid];
         if (n < Lx) {                    // forward: row s of yb becomes y_s
-          yb[(size_t)s * W + row] = acc;
-          zn[row] = (s + 1 < Lx) ? yb[(size_t)(s + 1) * W + row] - t * acc : acc;
+          yb[(size_t)s * W + tid] = y;
+          zn[tid] = (s + 1 < Lx) ? yb[(size_t)(s + 1) * W + tid] - t * y : y;
         } else {                         // backward: row s of yb becomes x_s
-          const cx<R> xv = yb[(size_t)s * W + row] - t * acc;
-          yb[(size_t)s * W + row] = xv;
-          zn[row] = xv;
+          const C xv = yb[(size_t)s * W + tid] - t * y;
+          yb[(size_t)s * W + tid] = xv;
+          zn[tid] = xv;
         }
       }
-      __syncthreads();                   // chunk slot released; rows of z for n+1 written
-      if (tid == 0 && q + S < NQ) {
-        fence_proxy_async();
-        issue(q + S);
-      }
+      csync();
     }
   }
+  __syncthreads();
   sweep_postpass<R>(g, i, a, yb);
   pp.seq += NQ;
   if (tid == 0 && cnt) *cnt += 1;
@@ -755,50 +801,102 @@ __device__ void cluster_sum_r(cg::cluster_group& cl, RedSmem& rs, int& phase, in
 // COCG for S y = b on the interface (S = C - E^T B^-1 E never formed), all in
 // precision R: the FP64 form solves to krylov_tol in FP64; the mixed form's
 // inner solves (refined in FP64 one level up) run entirely in complex64.
-// z = M_l^-1 r on interface line i with the exact layer block of S (2D
-// strips): a dense symmetric product, thread a owning output a; the stored
-// inverse is symmetric, so column a is read contiguously across threads.
-// r must be complete (a barrier after its writers) before the call.
-template <typename R>
-__device__ __noinline__ void lpre_apply(const Geo& g, const Bufs& b, int vs, int i, const cx<R>* r,
-                                        cx<R>* z) {
-  using C = cx<R>;
-  const int Lx = g.A;               // the layer's sites (Lx in 2D, Lx Ly in 3D)
-  const C* rsh = r;                 // every thread reads all of r: served by L1
-  const C* M = reinterpret_cast<const C*>(b.lpm) + ((size_t)slot_freq(g, vs) * (g.p - 1) + i) * (size_t)Lx * Lx;
-  // eight entries of the column in flight per thread before any is used: M is
-  // read from HBM on every application (long lines keep 2 MB per line), so the
-  // product is bound by how many loads each thread keeps outstanding
+// z = M_l^-1 r on interface line i with the exact layer block of S: a dense symmetric
+// product (the stored inverse is symmetric, so column a is read contiguously across
+// threads), its columns split over the warps: warp task (32 V outputs, one of CS column ranges), the CS
+// partials added in a fixed order.  The block (2 MB at A = 512) comes from HBM on
+// every application, so what counts is the bytes in flight: V = 2 outputs a lane
+// by 16-byte loads where a row's length keeps them aligned, eight columns at a time.
+// part: the free row buffer [Lx][W], CS x A entries of it.  r must be complete (a
+// barrier after its writers) before the call.
+template <typename R, int V>
+__device__ __forceinline__ void lpre_apply_v(const Geo& g, const Bufs& b, int vs, int i, const cx<R>* r, cx<R>* z,
+                                             cx<R>* part) {
+  const int A = g.A, nw = (int)blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nblk = (A + 32 * V - 1) / (32 * V);
+  int CS = (3 * nw + nblk - 1) / nblk;
+  if (CS > g.W / g.T) CS = g.W / g.T;    // the scratch holds W / T entries per layer site
+  const int per = (A + CS - 1) / CS;
+  const cx<R>* M = reinterpret_cast<const cx<R>*>(b.lpm) + ((size_t)slot_freq(g, vs) * (g.p - 1) + i) * (size_t)A * A;
   constexpr int U = 8;
-  for (int a = threadIdx.x; a < Lx; a += (int)blockDim.x) {
-    C acc[4] = {};
-    const C* col = M + a;
-    int c = 0;
-    for (; c + U <= Lx; c += U) {
-      C mv[U];
+  for (int task = wid; task < nblk * CS; task += nw) {
+    const int blk = task % nblk, ch = task / nblk, a = (blk * 32 + lane) * V;
+    const int c0 = ch * per, c1 = min(A, c0 + per);
+    if (a >= A) continue;
+    cx<R> acc[2][V] = {};
+    const cx<R>* col = M + a;
+    auto mul = [&](int c, int k) {
+      if constexpr (V == 2) {
+        const float4 m = *reinterpret_cast<const float4*>(col + (size_t)c * A);
+        const cxf rv = r[c];
+        acc[k][0] = cfma(cxf{m.x, m.y}, rv, acc[k][0]);
+        acc[k][1] = cfma(cxf{m.z, m.w}, rv, acc[k][1]);
+      } else {
+        acc[k][0] = cfma(col[(size_t)c * A], r[c], acc[k][0]);
+      }
+    };
+    int c = c0;
+    for (; c + U <= c1; c += U) {
+      if constexpr (V == 2) {
+        float4 m[U];
+        cxf rv[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) mv[u] = col[(size_t)(c + u) * Lx];
+        for (int u = 0; u < U; ++u) m[u] = *reinterpret_cast<const float4*>(col + (size_t)(c + u) * A);
 #pragma unroll
-      for (int u = 0; u < U; ++u) acc[u & 3] = cfma(mv[u], rsh[c + u], acc[u & 3]);
+        for (int u = 0; u < U; ++u) rv[u] = r[c + u];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          acc[u & 1][0] = cfma(cxf{m[u].x, m[u].y}, rv[u], acc[u & 1][0]);
+          acc[u & 1][1] = cfma(cxf{m[u].z, m[u].w}, rv[u], acc[u & 1][1]);
+        }
+      } else {
+        cx<R> m[U], rv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) m[u] = col[(size_t)(c + u) * A];
+#pragma unroll
+        for (int u = 0; u < U; ++u) rv[u] = r[c + u];
+#pragma unroll
+        for (int u = 0; u < U; ++u) acc[u & 1][0] = cfma(m[u], rv[u], acc[u & 1][0]);
+      }
     }
-    for (; c < Lx; ++c) acc[0] = cfma(col[(size_t)c * Lx], rsh[c], acc[0]);
-    z[a] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    for (; c < c1; ++c) mul(c, 0);
+#pragma unroll
+    for (int v = 0; v < V; ++v) part[ch * A + a + v] = acc[0][v] + acc[1][v];
   }
+  __syncthreads();
+  for (int a = threadIdx.x; a < A; a += (int)blockDim.x) {
+    cx<R> s = part[a];
+    for (int ch = 1; ch < CS; ++ch) s = s + part[ch * A + a];
+    z[a] = s;
+  }
+}
+template <typename R>
+__device__ __noinline__ void lpre_apply(const Geo& g, const Bufs& b, int vs, int i, const cx<R>* r, cx<R>* z,
+                                        cx<R>* part) {
+  if constexpr (sizeof(R) == 4) {
+    if (g.A % 2 == 0) {                  // rows start on 16-byte boundaries
+      lpre_apply_v<R, 2>(g, b, vs, i, r, z, part);
+      return;
+    }
+  }
+  lpre_apply_v<R, 1>(g, b, vs, i, r, z, part);
 }
 
 template <typename R>
 __device__ __forceinline__ void interface_precond(const Geo& g, const Bufs& b, int vs, int i, const cx<R>* r,
-                                                  cx<R>* z) {
-  if (g.lpre) lpre_apply<R>(g, b, vs, i, r, z);
+                                                  cx<R>* z, cx<R>* part) {
+  if (g.lpre) lpre_apply<R>(g, b, vs, i, r, z, part);
   else precond_apply<R>(g, b, vs, i, r, z);
 }
 
-// Right-hand side in IF_B, solution in IF_X.  Returns the iteration count;
-// *conv is set to 0 if the cap was hit.
+// Right-hand side in IF_B, solution y in IF_X.  Returns the iteration count;
+// *conv is set to 0 if the cap was hit.  xB += xs B^-1 E y (the subdomain block; "="
+// when fresh) comes along without a sweep of its own: the iteration's product
+// B^-1 E p is still in the row buffer when its step length alpha is known.
 template <typename R, int WF>
 __device__ int schur_cocg(cg::cluster_group& cl, RedSmem& rs, int& phase, const Geo& g,
                           const Bufs& b, int vs, int i, double tol, cx<R>* sm, Pipe& pp,
-                          int* conv) {
+                          cxd* xB, double xs, bool fresh, int* conv) {
   using C = cx<R>;
   const int p = g.p, A = g.A;
   const bool has = i < p - 1;
@@ -821,7 +919,9 @@ __device__ int schur_cocg(cg::cluster_group& cl, RedSmem& rs, int& phase, const 
     }
   }
   __syncthreads();
-  if (has) interface_precond<R>(g, b, vs, i, Rv + o, Z + o);
+  C* yb = pp.ybuf ? reinterpret_cast<C*>(pp.ybuf) : sweep_base<R>(g, b, vs, i).y;   // the sweeps' row buffer
+  const int W = g.W, wd = g.T * g.h[i], nsub = g.Lx * W;
+  if (has) interface_precond<R>(g, b, vs, i, Rv + o, Z + o, yb);
   __syncthreads();
   C v2[2] = {{0, 0}, {0, 0}};
   if (has) {
@@ -836,7 +936,12 @@ __device__ int schur_cocg(cg::cluster_group& cl, RedSmem& rs, int& phase, const 
   C rho = v2[0];
   const R bn = v2[1].x;
   *conv = 1;
-  if (bn == (R)0) return 0;
+  if (bn == (R)0) {
+    if (fresh)
+      for (int e = threadIdx.x; e < nsub; e += (int)blockDim.x)
+        if (e % W < wd) xB[e] = cxd{0, 0};
+    return 0;
+  }
   SweepArgs<R> sa = sweep_base<R>(g, b, vs, i);
   sa.lay_lo = (i > 0) ? P + (size_t)(i - 1) * A : nullptr;
   sa.lay_hi = has ? P + o : nullptr;
@@ -863,27 +968,34 @@ __device__ int schur_cocg(cg::cluster_group& cl, RedSmem& rs, int& phase, const 
     }
     cluster_sum_r<R, 1>(cl, rs, phase, p, v1);
     const C alpha = cdiv(rho, v1[0]);
+    v1[0] = C{0, 0};
     if (has) {
       for (int a = threadIdx.x; a < A; a += (int)blockDim.x) {
         X[o + a] = X[o + a] + alpha * P[o + a];
-        Rv[o + a] = Rv[o + a] - alpha * SP[o + a];
+        const C r = Rv[o + a] - alpha * SP[o + a];
+        Rv[o + a] = r;
+        v1[0].x += cabs2(r);
       }
     }
-    __syncthreads();
-    if (has) interface_precond<R>(g, b, vs, i, Rv + o, Z + o);
-    __syncthreads();
-    v2[0] = v2[1] = C{0, 0};
-    if (has) {
-      for (int a = threadIdx.x; a < A; a += (int)blockDim.x) {
-        C zz = Z[o + a], r = Rv[o + a];
-        v2[0] = cfma(r, zz, v2[0]);
-        v2[1].x += cabs2(r);
-      }
+    for (int e = threadIdx.x; e < nsub; e += (int)blockDim.x) {
+      if (e % W >= wd) continue;
+      const cxd d = cconv<double>(alpha * yb[e]);
+      cxd x = fresh ? cxd{0, 0} : xB[e];
+      x.x = fma(xs, d.x, x.x);
+      x.y = fma(xs, d.y, x.y);
+      xB[e] = x;
     }
-    cluster_sum_r<R, 2>(cl, rs, phase, p, v2);
-    if (v2[1].x <= tol2 * bn) break;
-    const C beta = cdiv(v2[0], rho);
-    rho = v2[0];
+    fresh = false;
+    cluster_sum_r<R, 1>(cl, rs, phase, p, v1);  // also: the row buffer is free (the preconditioner's scratch)
+    if (v1[0].x <= tol2 * bn) break;
+    if (has) interface_precond<R>(g, b, vs, i, Rv + o, Z + o, yb);
+    __syncthreads();
+    v1[0] = C{0, 0};
+    if (has)
+      for (int a = threadIdx.x; a < A; a += (int)blockDim.x) v1[0] = cfma(Rv[o + a], Z[o + a], v1[0]);
+    cluster_sum_r<R, 1>(cl, rs, phase, p, v1);
+    const C beta = cdiv(v1[0], rho);
+    rho = v1[0];
     if (has) {
       for (int a = threadIdx.x; a < A; a += (int)blockDim.x) P[o + a] = Z[o + a] + beta * P[o + a];
     }
@@ -1031,16 +1143,8 @@ __device__ int solve_H(cg::cluster_group& cl, RedSmem& rs, int& phase, const Geo
     for (int a = threadIdx.x; a < A; a += (int)blockDim.x) Bv[(size_t)i * A + a] = cconv<R>(isc * rc[a]);
   }
   __syncthreads();
-  int it = schur_cocg<R, WF>(cl, rs, phase, g, b, vs, i, tol, sm, pp, conv);
-  cl.sync();
+  int it = schur_cocg<R, WF>(cl, rs, phase, g, b, vs, i, tol, sm, pp, xout + i * nsub, -sc, zero_B, conv);
   const cx<R>* X = ifv_ptr<R>(g, b, vs, IF_X);
-  SweepArgs<R> sb = sweep_base<R>(g, b, vs, i);
-  sb.lay_lo = (i > 0) ? X + (size_t)(i - 1) * A : nullptr;
-  sb.lay_hi = has ? X + (size_t)i * A : nullptr;
-  sb.dst = xout + i * nsub;
-  sb.out_scale = sc;
-  sb.dst_op = zero_B ? 3 : 2;
-  sweep<R, WF>(g, i, sb, sm, pp, sweep_cnt(g, b, vs, i));
   if (has) {
     cxd* xc = xout + g.ifc_off + (size_t)i * A;
     for (int a = threadIdx.x; a < A; a += (int)blockDim.x) xc[a] = sc * cconv<double>(X[(size_t)i * A + a]);
@@ -1049,6 +1153,7 @@ __device__ int solve_H(cg::cluster_group& cl, RedSmem& rs, int& phase, const Geo
 }
 
 constexpr size_t YBUF_MAX = 64 * 1024;   // forward intermediates kept on chip up to this size
+constexpr size_t SMEM_LIMIT = 223 * 1024;   // dynamic shared memory per CTA, below the 227 KB cap (static: ~3 KB)
 
 // Shared-memory plan of a sweep: ring of S slots of CR x W entries (CR = W when
 // a whole slice block fits a slot, the W <= 64 strips of the FP64 form; row
@@ -1063,7 +1168,7 @@ __host__ __device__ inline RingPlan ring_plan(int W, int Lx) {
   RingPlan rp;
   const size_t cs = sizeof(cx<R>);
   const size_t yb = (size_t)Lx * W * cs;
-  rp.zw = 2 * W;
+  rp.zw = 2 * W + (W > DY_MAXW_SMEM ? wide_groups<R>(W) * W : 0);
   if (W <= DY_MAXW_SMEM) {
     rp.ybuf = yb <= YBUF_MAX ? yb : 0;
     rp.CR = W;
@@ -1073,15 +1178,15 @@ __host__ __device__ inline RingPlan ring_plan(int W, int Lx) {
     rp.S = (int)S;
   } else {
     rp.ybuf = yb;                                                       // one CTA per SM
-    const long budget = (long)200 * 1024 - (long)yb - (long)(2 * W * cs);
-    // largest divisor of W whose chunks leave >= 4 ring slots (>= 2 as a last
-    // resort); a chunk row is W entries, a multiple of 32 bytes, so any row count
-    // keeps the bulk copies 16-byte aligned
+    const long budget = (long)SMEM_LIMIT - (long)yb - (long)(rp.zw * cs);
+    // largest divisor of W whose chunks are at most 32 KB and leave >= 4 ring slots
+    // (>= 2, and any size, as a last resort); a chunk row is W entries, a multiple of
+    // 32 bytes, so any row count keeps the bulk copies 16-byte aligned
     rp.CR = 0;
     rp.S = 0;
     for (int want = 4; want >= 2 && !rp.CR; want -= 2)
       for (int cr = W; cr >= 1; --cr) {
-        if (W % cr) continue;
+        if (W % cr || (want > 2 && (size_t)cr * W * cs > 32 * 1024)) continue;
         const long S = budget / (long)((size_t)cr * W * cs);
         if (S >= want) {
           rp.CR = cr;
@@ -1095,7 +1200,6 @@ __host__ __device__ inline RingPlan ring_plan(int W, int Lx) {
 }
 // The plan of a geometry: the heuristic above, or the autotuner's choice of
 // slots (and chunk rows for W > 64) with the same row buffer and z area.
-constexpr size_t SMEM_LIMIT = 223 * 1024;   // dynamic shared memory per CTA, below the 227 KB cap (static: ~3 KB)
 template <typename R>
 __host__ __device__ inline RingPlan ring_plan(const Geo& g) {
   RingPlan rp = ring_plan<R>(g.W, g.Lx);
@@ -1131,8 +1235,9 @@ inline int ring_candidates(const Geo& g, int* S, int* CR, int max) {
   if (g.W <= DY_MAXW_SMEM) {
     for (int s = 2; s <= MAX_STAGES; ++s) add(s, g.W);
   } else {
-    for (int cr = g.W; cr >= 1; --cr) {
-      if (g.W % cr) continue;
+    for (int cr = g.W; cr >= 1; --cr) {            // chunks of 8 to 64 KB
+      const size_t bytes = (size_t)cr * g.W * cs;
+      if (g.W % cr || bytes > 64 * 1024 || bytes < 8 * 1024) continue;
       int best = 0;
       for (int s = MAX_STAGES; s >= 2; --s)
         if (fits(s, cr)) {
@@ -1155,10 +1260,10 @@ inline int ring_candidates(const Geo& g, int* S, int* CR, int max) {
 //              residuals of B, u against FP64 residuals of H, each until the
 //              relative residual is below refine_tol.
 template <typename R, int WF>
-__global__ void __launch_bounds__(DY_THREADS, 2) k_xmatvec(Geo g, Bufs b, int j, int mixed, int ncols) {
+__global__ void __launch_bounds__(solve_threads<WF>(), WF == 0 ? 1 : 2) k_xmatvec(Geo g, Bufs b, int j, int mixed, int ncols) {
   cg::cluster_group cl = cg::this_cluster();
   __shared__ RedSmem rs;
-  __shared__ __align__(8) uint64_t bars[MAX_STAGES];
+  __shared__ __align__(8) uint64_t bars[2 * MAX_STAGES];
   __shared__ int err;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   // one cluster per (frequency, block column): slot vs = f * nb + c
@@ -1169,6 +1274,7 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_xmatvec(Geo g, Bufs b, int j,
   if (st[ST_DONE]) return;
   Pipe pp;
   pp.bar = bars;
+  pp.empty = bars + MAX_STAGES;
   const RingPlan rp = ring_plan<R>(g);
   pp.S = rp.S;
   pp.CR = rp.CR;
@@ -1215,17 +1321,10 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_xmatvec(Geo g, Bufs b, int j,
         Bv[(size_t)i * A + a] = (R)g.t * (bl_i[a] + bl_n[a]) - cconv<R>(qc[a]);
     }
     __syncthreads();
-    iters += schur_cocg<R, WF>(cl, rs, phase, g, b, vs, i, g.krylov_tol, sm, pp, &conv);
+    iters += schur_cocg<R, WF>(cl, rs, phase, g, b, vs, i, g.krylov_tol, sm, pp, u + i * nsub, 1.0, true, &conv);
     conv_all &= conv;
     solves = 1;
-    cl.sync();
     const cx<R>* X = ifv_ptr<R>(g, b, vs, IF_X);
-    SweepArgs<R> sb = sweep_base<R>(g, b, vs, i);
-    sb.lay_lo = (i > 0) ? X + (size_t)(i - 1) * A : nullptr;
-    sb.lay_hi = has ? X + (size_t)i * A : nullptr;
-    sb.dst = u + i * nsub;
-    sb.dst_op = 0;
-    sweep<R, WF>(g, i, sb, sm, pp, sweep_cnt(g, b, vs, i));
     if (has) {
       cxd* uc = u + g.ifc_off + (size_t)i * A;
       for (int a = threadIdx.x; a < A; a += (int)blockDim.x) uc[a] = -cconv<double>(X[(size_t)i * A + a]);
@@ -1338,14 +1437,15 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_xmatvec(Geo g, Bufs b, int j,
 
 // w = blkdiag(B^-1, 0) q for DD-layout vectors (Eq. 7), one CTA per subdomain.
 template <typename R, int WF>
-__global__ void __launch_bounds__(DY_THREADS, 2) k_bsolve(Geo g, Bufs b, const cxd* q, cxd* w) {
-  __shared__ __align__(8) uint64_t bars[MAX_STAGES];
+__global__ void __launch_bounds__(solve_threads<WF>(), WF == 0 ? 1 : 2) k_bsolve(Geo g, Bufs b, const cxd* q, cxd* w) {
+  __shared__ __align__(8) uint64_t bars[2 * MAX_STAGES];
   __shared__ int err;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int i = blockIdx.x, kf = blockIdx.y, vs = kf * g.nb;   // scratch of the frequency's first slot
   const size_t nsub = (size_t)g.Lx * g.W;
   Pipe pp;
   pp.bar = bars;
+  pp.empty = bars + MAX_STAGES;
   const RingPlan rp = ring_plan<R>(g);
   pp.S = rp.S;
   pp.CR = rp.CR;
@@ -1413,8 +1513,8 @@ cudaError_t run_bsolve(const Geo& g, const Bufs& b, int K, const cxd* q_dd, cxd*
   template <>                                                                                     \
   cudaError_t run_xmatvec<R, WF>(const Geo& g, const Bufs& b, int K, int j, int mixed, int ncols, \
                                  cudaStream_t st) {                                               \
-    return launch_cluster(k_xmatvec<R, WF>, dim3(g.p, K * g.nb), g.p, sweep_smem<R>(g), st, g, b, j, mixed, \
-                          ncols);                                                                 \
+    return launch_cluster_nt(k_xmatvec<R, WF>, dim3(g.p, K * g.nb), g.p, solve_threads<WF>(),     \
+                             sweep_smem<R>(g), st, g, b, j, mixed, ncols);                        \
   }                                                                                               \
   template <>                                                                                     \
   cudaError_t run_bsolve<R, WF>(const Geo& g, const Bufs& b, int K, const cxd* q_dd, cxd* w_dd,   \
@@ -1422,6 +1522,6 @@ cudaError_t run_bsolve(const Geo& g, const Bufs& b, int K, const cxd* q_dd, cxd*
     const size_t smem = sweep_smem<R>(g);                                                         \
     cudaError_t e = raise_smem_limit((const void*)k_bsolve<R, WF>, smem);                         \
     if (e != cudaSuccess) return e;                                                               \
-    k_bsolve<R, WF><<<dim3(g.p, K), DY_THREADS, smem, st>>>(g, b, q_dd, w_dd);                    \
+    k_bsolve<R, WF><<<dim3(g.p, K), solve_threads<WF>(), smem, st>>>(g, b, q_dd, w_dd);           \
     return cudaGetLastError();                                                                    \
   }

@@ -567,73 +567,6 @@ __device__ __forceinline__ cxf scaled(float s, const cdfl& a) { return {s * (a.x
 __device__ __forceinline__ dfl dfl_of(double v) { return d2dfl_bits(v); }
 
 // ---------------------------------------------------------------- interface solve
-// z = M_l^-1 r with the exact layer block (see lpre_apply), its columns split
-// over the warps: warp task (32 V outputs, one of CS column ranges), the CS
-// partials added in a fixed order.  The block (2 MB at A = 512) comes from HBM on
-// every application, so what counts is the bytes in flight: V = 2 outputs a lane
-// by 16-byte loads where a row's length keeps them aligned, eight columns at a time.
-// part: CS x A entries of scratch.
-template <int V>
-__device__ __forceinline__ void mix_lpre(const Geo& g, const Bufs& b, int vs, int i, const cxf* r, cxf* z, cxf* part) {
-  const int A = g.A, nw = (int)blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nblk = (A + 32 * V - 1) / (32 * V);
-  int CS = (3 * nw + nblk - 1) / nblk;
-  if (CS > g.W) CS = g.W;                // the scratch holds W entries per line site
-  const int per = (A + CS - 1) / CS;
-  const cxf* M = reinterpret_cast<const cxf*>(b.lpm) + ((size_t)slot_freq(g, vs) * (g.p - 1) + i) * (size_t)A * A;
-  constexpr int U = 8;
-  for (int task = wid; task < nblk * CS; task += nw) {
-    const int blk = task % nblk, ch = task / nblk, a = (blk * 32 + lane) * V;
-    const int c0 = ch * per, c1 = min(A, c0 + per);
-    if (a >= A) continue;
-    cxf acc[2][V] = {};
-    const cxf* col = M + a;
-    auto mul = [&](int c, int k) {
-      if constexpr (V == 2) {
-        const float4 m = *reinterpret_cast<const float4*>(col + (size_t)c * A);
-        const cxf rv = r[c];
-        acc[k][0] = cfma(cxf{m.x, m.y}, rv, acc[k][0]);
-        acc[k][1] = cfma(cxf{m.z, m.w}, rv, acc[k][1]);
-      } else {
-        acc[k][0] = cfma(col[(size_t)c * A], r[c], acc[k][0]);
-      }
-    };
-    int c = c0;
-    for (; c + U <= c1; c += U) {
-      if constexpr (V == 2) {
-        float4 m[U];
-        cxf rv[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) m[u] = *reinterpret_cast<const float4*>(col + (size_t)(c + u) * A);
-#pragma unroll
-        for (int u = 0; u < U; ++u) rv[u] = r[c + u];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          acc[u & 1][0] = cfma(cxf{m[u].x, m[u].y}, rv[u], acc[u & 1][0]);
-          acc[u & 1][1] = cfma(cxf{m[u].z, m[u].w}, rv[u], acc[u & 1][1]);
-        }
-      } else {
-        cxf m[U], rv[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) m[u] = col[(size_t)(c + u) * A];
-#pragma unroll
-        for (int u = 0; u < U; ++u) rv[u] = r[c + u];
-#pragma unroll
-        for (int u = 0; u < U; ++u) acc[u & 1][0] = cfma(m[u], rv[u], acc[u & 1][0]);
-      }
-    }
-    for (; c < c1; ++c) mul(c, 0);
-#pragma unroll
-    for (int v = 0; v < V; ++v) part[ch * A + a + v] = acc[0][v] + acc[1][v];
-  }
-  __syncthreads();
-  for (int a = threadIdx.x; a < A; a += (int)blockDim.x) {
-    cxf s = part[a];
-    for (int ch = 1; ch < CS; ++ch) s = s + part[ch * A + a];
-    z[a] = s;
-  }
-}
-
 struct MixSolve {
   bool useB0;                            // the subdomain part is B0 - alpha B1 (else - alpha B1)
   cxf alpha;
@@ -671,8 +604,7 @@ __device__ __noinline__ MixSolve mix_cocg(const Geo& g, const Bufs& b, const Mix
   cxf* phi = P + o;
   const float t = cx.t;
   auto precond = [&](const cxf* r, cxf* z) {
-    if (g.lpre && A % 2 == 0) mix_lpre<2>(g, b, vs, i, r, z, B1);
-    else if (g.lpre) mix_lpre<1>(g, b, vs, i, r, z, B1);
+    if (g.lpre) lpre_apply<float>(g, b, vs, i, r, z, B1);
     else precond_apply<float>(g, b, vs, i, r, z);
   };
   MixSolve out = {keep0, {0.f, 0.f}, 0, 1};
