@@ -209,6 +209,123 @@ __global__ void __launch_bounds__(DY_THREADS) k_factor(Geo g, Bufs b) {
   }
 }
 
+// ---------------------------------------------------------------- triangle inversion
+// Inverse of a complex symmetric W x W block (W <= WF) by the sweep operator (see
+// gj_invert) on the upper triangle, whose entries stay in the registers of warps
+// 1..7 (thread t of them owns triangle entries t, t + 224, ...).  Warp 0 runs one pivot
+// ahead: while the others apply pivot k it brings column k + 1 up to date itself,
+// inverts pivot k + 1 and scales the column, so a pivot costs one barrier and the
+// longer of the two (~650 cycles at W = 32 in double-float) instead of their sum
+// (2250).  Every product is renormalised as it is added: sums without it, 48
+// operations a term instead of 60, made the diagonal's error 1.2 to 1.4 times as large.
+template <typename R>
+struct TriSmem {
+  cx<R>*prow, *fcol, *craw;                  // [2][W] each: the pivot's column, scaled by the inverse
+                                             // pivot, and the column after it (one pivot behind)
+};
+template <int WF>
+struct Tri {
+  static constexpr int OWN = DY_THREADS - 32;
+  static constexpr int NE = (WF * (WF + 1) / 2 + OWN - 1) / OWN;                 // triangle entries an owner holds
+  static constexpr int NP = (WF * (WF + 1) / 2 + DY_THREADS - 1) / DY_THREADS;   // and a thread of all of them
+};
+// triangle entry number e (rows of length W, W - 1, ...) as (r, c), r <= c; false, (0, 0) past the end
+__device__ __forceinline__ bool tri_entry(int e, int W, int& r, int& c) {
+  r = 0;
+  const bool on = e < W * (W + 1) / 2;
+  while (on && e >= W - r) {
+    e -= W - r;
+    ++r;
+  }
+  c = on ? r + e : 0;
+  return on;
+}
+
+// 1 / z: in double-float one Newton step from the binary32 reciprocal of |z|^2, with
+// its square term (the start is off by at most 2^-24, so the result by ~2^-70 before
+// rounding)
+template <typename R>
+__device__ __forceinline__ cx<R> inv_fast(const cx<R>& z) {
+  if constexpr (std::is_same<R, dfl>::value) {
+    dfl d = dfl(0.f, 0.f);
+    dfl_mac(d, z.x, z.x);
+    dfl_mac(d, z.y, z.y);
+    d = dfl_fast(d.hi, d.lo);
+    const float r0 = __frcp_rn(d.hi);
+    const float e = __fmaf_rn(-d.lo, r0, __fmaf_rn(-d.hi, r0, 1.f));
+    const dfl r = dfl_fast(r0, r0 * __fmaf_rn(e, e, e));
+    const dfl im = z.y * r;
+    return {z.x * r, dfl(-im.hi, -im.lo)};
+  } else {
+    return cinv(z);
+  }
+}
+
+// from(r, c) (r <= c) gives the block's entries, to(r, c, v) takes the inverse's; from
+// is not called after the first barrier, to not before the last one (the caller syncs
+// before the results are read).  er, ec, eon: this thread's entries (tri_entry of
+// tid - 32 + OWN q for warps 1..7).
+template <typename R, int WF, typename From, typename To>
+__device__ __forceinline__ void tri_invert(int W, const TriSmem<R>& ts, const int (&er)[Tri<WF>::NE],
+                                           const int (&ec)[Tri<WF>::NE], unsigned eon, From from, To to) {
+  using C = cx<R>;
+  constexpr int NE = Tri<WF>::NE;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  C v[NE];
+#pragma unroll
+  for (int q = 0; q < NE; ++q) v[q] = wid > 0 ? from(er[q], ec[q]) : C{0, 0};
+  if (wid == 0) {
+    for (int e = lane; e < W; e += 32) {
+      ts.prow[e] = from(0, e);
+      if (W > 1) ts.craw[W + e] = from(e < 1 ? e : 1, e < 1 ? 1 : e);       // column 1
+    }
+    __syncwarp();
+    const C piv = inv_fast<R>(ts.prow[0]);
+    for (int e = lane; e < W; e += 32) ts.fcol[e] = e == 0 ? -piv : ts.prow[e] * piv;
+  }
+  for (int k = 0; k < W; ++k) {
+    const C *pk = ts.prow + (k & 1) * W, *fk = ts.fcol + (k & 1) * W, *cr = ts.craw + ((k + 1) & 1) * W;
+    C *pn = ts.prow + ((k + 1) & 1) * W, *fn = ts.fcol + ((k + 1) & 1) * W, *cn = ts.craw + (k & 1) * W;
+    __syncthreads();                         // pk, fk and column k + 1 as of pivot k - 1 are complete
+    if (wid == 0) {
+      if (k + 1 < W) {
+        const C p1 = pk[k + 1], f1 = fk[k + 1];
+        for (int e = lane; e < W; e += 32) {
+          // the same product the entry's owner forms (f of the row, p of the column)
+          const bool up = e <= k + 1;
+          C x = cfma(up ? -fk[e] : -f1, up ? p1 : pk[e], cr[e]);
+          if (e == k) x = f1;
+          pn[e] = x;
+        }
+        __syncwarp();
+        const C piv = inv_fast<R>(pn[k + 1]);
+        for (int e = lane; e < W; e += 32) {
+          const C x = pn[e] * piv;
+          fn[e] = e == k + 1 ? -piv : x;
+        }
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < NE; ++q) {
+        const int r = er[q], c = ec[q];
+        const C f = fk[r], x = fk[r == k ? c : r];
+        const C u = cfma(-f, pk[c], v[q]);
+        v[q] = r == k || c == k ? x : u;
+      }
+#pragma unroll
+      for (int q = 0; q < NE; ++q) {         // column k + 2 for the pivot warp
+        if (!(eon >> q & 1)) continue;
+        if (er[q] == k + 2) cn[ec[q]] = v[q];
+        else if (ec[q] == k + 2) cn[er[q]] = v[q];
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NE; ++q)               // -(-A^-1)
+    if (eon >> q & 1) to(er[q], ec[q], -v[q]);
+}
+
 // ---------------------------------------------------------------- two-sided, double-float
 // The mixed form's recursion for W <= 64, from both ends, so that the complex64
 // sweeps can run two chains at once.  With m = Lx / 2:
@@ -223,39 +340,11 @@ __global__ void __launch_bounds__(DY_THREADS) k_factor(Geo g, Bufs b) {
 // right one, which meet at the middle block (each inverts it for itself) and go back
 // separately.  One CTA running both chains in turn took 65 us a slice at W = 28 with
 // 21 x 4 units on 152 SMs.
-//
-// Inversion: the sweep operator on the upper triangle, whose entries stay in the
-// registers of warps 1..7 (thread t of them owns triangle entries t, t + 224, ...).
-// Warp 0 runs one pivot ahead: while the others apply pivot k it brings column k + 1
-// up to date itself, inverts pivot k + 1 and scales the column, so a pivot costs one
-// barrier and the longer of the two (~650 cycles at W = 32) instead of their sum
-// (2250).  Every product is renormalised as it is added: sums without it, 48
-// operations a term instead of 60, made the diagonal's error 1.2 to 1.4 times as large.
-template <int WF>
-struct TwoCfg {
-  static constexpr int OWN = DY_THREADS - 32;
-  static constexpr int NE = (WF * (WF + 1) / 2 + OWN - 1) / OWN;                 // triangle entries an owner holds
-  static constexpr int NP = (WF * (WF + 1) / 2 + DY_THREADS - 1) / DY_THREADS;   // and a thread of the last product
-};
 using cxl = cx<dfl>;
-
-// 1 / z: one Newton step from the binary32 reciprocal of |z|^2, with its square term
-// (the start is off by at most 2^-24, so the result by ~2^-70 before rounding)
-__device__ __forceinline__ cxl inv_l(const cxl& z) {
-  dfl d = dfl(0.f, 0.f);
-  dfl_mac(d, z.x, z.x);
-  dfl_mac(d, z.y, z.y);
-  d = dfl_fast(d.hi, d.lo);
-  const float r0 = __frcp_rn(d.hi);
-  const float e = __fmaf_rn(-d.lo, r0, __fmaf_rn(-d.hi, r0, 1.f));
-  const dfl r = dfl_fast(r0, r0 * __fmaf_rn(e, e, e));
-  const dfl im = z.y * r;
-  return {z.x * r, dfl(-im.hi, -im.lo)};
-}
 
 template <int WF>
 __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo g, Bufs b) {
-  constexpr int NE = TwoCfg<WF>::NE, NP = TwoCfg<WF>::NP, OWN = TwoCfg<WF>::OWN;
+  constexpr int NE = Tri<WF>::NE, NP = Tri<WF>::NP, OWN = Tri<WF>::OWN;
   constexpr int NB = (WF * WF + DY_THREADS - 1) / DY_THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cg::cluster_group cl = cg::this_cluster();
@@ -264,10 +353,8 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
   cxl* A = reinterpret_cast<cxl*>(smem_raw);
   cxl* Bm = A + n;
   cxl* Cm = Bm + n;
-  cxl* prow = Cm + n;                        // [2][W] the pivot's column, by pivot parity
-  cxl* fcol = prow + 2 * W;                  // [2][W] the column scaled by the inverse pivot
-  cxl* craw = fcol + 2 * W;                  // [2][W] the column after it, one pivot behind
-  cxl* dg = craw + 2 * W;                    // [W] H_ii of the slice being formed
+  const TriSmem<dfl> ts = {Cm + n, Cm + n + 2 * W, Cm + n + 4 * W};
+  cxl* dg = Cm + n + 6 * W;                    // [W] H_ii of the slice being formed
   cxl* Gprev = dg + W;                       // [2][W] columns of the last off-diagonal block at the boundary rows
   cxl* Gmid = Gprev + 2 * W;                 // [2][W] rows of G_{m+1,m} at the boundary rows (left CTA's copy is used)
   const size_t uoff = ((size_t)kf * g.p + i) * (size_t)Lx * n;
@@ -281,25 +368,14 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
   const dfl t = (dfl)g.t, t2 = (dfl)(g.t * g.t);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
-  // triangle entry number e (rows of length W, W - 1, ...) as (r, c), r <= c; (0, 0) past the end
-  auto tri = [&](int e, int& r, int& c) {
-    r = 0;
-    const bool on = e < ntri;
-    while (on && e >= W - r) {
-      e -= W - r;
-      ++r;
-    }
-    c = on ? r + e : 0;
-    return on;
-  };
   int er[NE], ec[NE], pr[NP], pc[NP];
   unsigned eon = 0, pon = 0;                 // bit q: entry q exists
 #pragma unroll
   for (int q = 0; q < NE; ++q)
-    if (tri(wid > 0 ? tid - 32 + OWN * q : ntri, er[q], ec[q])) eon |= 1u << q;
+    if (tri_entry(wid > 0 ? tid - 32 + OWN * q : ntri, W, er[q], ec[q])) eon |= 1u << q;
 #pragma unroll
   for (int q = 0; q < NP; ++q)
-    if (tri(tid + DY_THREADS * q, pr[q], pc[q])) pon |= 1u << q;
+    if (tri_entry(tid + DY_THREADS * q, W, pr[q], pc[q])) pon |= 1u << q;
 
   auto load_h = [&](int s) {
     if (tid < W) {
@@ -311,79 +387,28 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
   // null) may be A itself; stored in slot s when keep.  dg holds slice s's diagonal;
   // slice sn's (if >= 0) is fetched for the next call.
   auto invert = [&](int s, const cxl* pa, const cxl* pb, bool keep, int sn) {
-    cxl v[NE];
     cdfl hn = {dfl(0.f, 0.f), dfl(0.f, 0.f)};
     if (sn >= 0 && tid < W) hn = hd[(size_t)sn * W + tid];
-    auto formed = [&](int r, int c) -> cxl {
-      const int e = r * W + c;
-      cxl x = {0, 0};
-      if (pa) x = x - t2 * pa[e];
-      if (pb) x = x - t2 * pb[e];
-      if (r < w && c < w) {
-        if (r == c) x = x + dg[r];
-        else if (slice_adjacent<dfl>(r, c, T)) x.x += t;
-      } else {
-        x = r == c ? cxl{1, 0} : cxl{0, 0};
-      }
-      return x;
-    };
-#pragma unroll
-    for (int q = 0; q < NE; ++q) v[q] = wid > 0 ? formed(er[q], ec[q]) : cxl{0, 0};
-    if (wid == 0) {
-      for (int e = lane; e < W; e += 32) {
-        prow[e] = formed(0, e);
-        craw[W + e] = formed(e < 1 ? e : 1, e < 1 ? 1 : e);       // column 1
-      }
-      __syncwarp();
-      const cxl piv = inv_l(prow[0]);
-      for (int e = lane; e < W; e += 32) fcol[e] = e == 0 ? -piv : prow[e] * piv;
-    }
-    for (int k = 0; k < W; ++k) {
-      const cxl *pk = prow + (k & 1) * W, *fk = fcol + (k & 1) * W, *cr = craw + ((k + 1) & 1) * W;
-      cxl *pn = prow + ((k + 1) & 1) * W, *fn = fcol + ((k + 1) & 1) * W, *cn = craw + (k & 1) * W;
-      __syncthreads();                       // pk, fk and column k + 1 as of pivot k - 1 are complete
-      if (wid == 0) {
-        if (k + 1 < W) {
-          const cxl p1 = pk[k + 1], f1 = fk[k + 1];
-          for (int e = lane; e < W; e += 32) {
-            // the same product the entry's owner forms (f of the row, p of the column)
-            const bool up = e <= k + 1;
-            cxl x = cfma(up ? -fk[e] : -f1, up ? p1 : pk[e], cr[e]);
-            if (e == k) x = f1;
-            pn[e] = x;
+    tri_invert<dfl, WF>(
+        W, ts, er, ec, eon,
+        [&](int r, int c) -> cxl {
+          const int e = r * W + c;
+          cxl x = {0, 0};
+          if (pa) x = x - t2 * pa[e];
+          if (pb) x = x - t2 * pb[e];
+          if (r < w && c < w) {
+            if (r == c) x = x + dg[r];
+            else if (slice_adjacent<dfl>(r, c, T)) x.x += t;
+          } else {
+            x = r == c ? cxl{1, 0} : cxl{0, 0};
           }
-          __syncwarp();
-          const cxl piv = inv_l(pn[k + 1]);
-          for (int e = lane; e < W; e += 32) {
-            const cxl x = pn[e] * piv;
-            fn[e] = e == k + 1 ? -piv : x;
-          }
-        }
-      } else {
-#pragma unroll
-        for (int q = 0; q < NE; ++q) {
-          const int r = er[q], c = ec[q];
-          const cxl f = fk[r], x = fk[r == k ? c : r];
-          const cxl u = cfma(-f, pk[c], v[q]);
-          v[q] = r == k || c == k ? x : u;
-        }
-#pragma unroll
-        for (int q = 0; q < NE; ++q) {       // column k + 2 for the pivot warp
-          if (!(eon >> q & 1)) continue;
-          if (er[q] == k + 2) cn[ec[q]] = v[q];
-          else if (ec[q] == k + 2) cn[er[q]] = v[q];
-        }
-      }
-    }
-    __syncthreads();                         // every read of A (pa) is long past; fcol free
-#pragma unroll
-    for (int q = 0; q < NE; ++q) {           // -(-A^-1), both triangles
-      if (!(eon >> q & 1)) continue;
-      const int r = er[q], c = ec[q];
-      const cxl x = c < w ? -v[q] : cxl{0, 0};
-      A[r * W + c] = x;
-      A[c * W + r] = x;
-    }
+          return x;
+        },
+        [&](int r, int c, const cxl& v) {
+          const cxl x = c < w ? v : cxl{0, 0};
+          A[r * W + c] = x;
+          A[c * W + r] = x;
+        });
     if (sn >= 0 && tid < W) dg[tid] = cxl{hn.x, hn.y};
     __syncthreads();
     if (keep)
@@ -538,9 +563,9 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
 // the backward pass as two W x W products.
 //
 // A (subdomain, frequency) unit is worked on by a cluster of C CTAs that share the
-// tiles of every phase, C the largest of 8, 4, 2, 1 that keeps the units within the
-// DY_FACTOR_CTAS CTAs of the persistent grid: 32 units of 128 x 128 blocks
-// (128 x 128 sites, p = 1) left 120 of the 152 SMs idle with one CTA each.
+// tiles of every phase (wide_cluster): 32 units of 128 x 128 blocks (128 x 128 sites,
+// p = 1) left 120 of the 152 SMs idle with one CTA each, and 128 unblocked pivots
+// with two barriers each took most of 3.9 ms a slice; now 0.44 ms.
 constexpr int TB = 32, TP = 33;          // tile edge and padded row length in shared memory
 
 template <typename R>
@@ -565,7 +590,7 @@ __device__ __forceinline__ cx<R> tile_done(cx<R> v) {
 template <typename R>
 struct TileSmem {
   cx<R> tx[TB][TP], ty[TB][TP], tp[TB][TP];
-  cx<R> prow[TB], fcol[TB];
+  cx<R> tri[6 * TB];
 };
 
 // tile (r0, c0) of the row-major ld-wide matrix M (n x n; identity outside) to t, or
@@ -600,33 +625,6 @@ __device__ __forceinline__ void tile_mac(const cx<R> (*tx)[TP], const cx<R> (*ty
   }
 }
 
-// tp <- inverse of the complex symmetric 32 x 32 tile tp (the sweep operator of
-// gj_invert, full tile)
-template <typename R>
-__device__ void tile_invert(TileSmem<R>& sm) {
-  const int lc = threadIdx.x & 31, lr = threadIdx.x >> 5;
-  for (int k = 0; k < TB; ++k) {
-    __syncthreads();
-    if (threadIdx.x < TB) {
-      const cx<R> piv = cinv(sm.tp[k][k]);
-      const cx<R> a = sm.tp[k][threadIdx.x];
-      sm.prow[threadIdx.x] = a;
-      sm.fcol[threadIdx.x] = (int)threadIdx.x == k ? -piv : a * piv;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const int r = lr + 8 * m;
-      if (r == k || lc == k) sm.tp[r][lc] = sm.fcol[r == k ? lc : r];
-      else sm.tp[r][lc] = cfma(-sm.fcol[r], sm.prow[lc], sm.tp[r][lc]);
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int m = 0; m < 4; ++m) sm.tp[lr + 8 * m][lc] = -sm.tp[lr + 8 * m][lc];
-  __syncthreads();
-}
-
 // R: the recursion's arithmetic, binary64 (FP64 form) or double-float (mixed
 // form, on the FP32 pipe), stored in b.g (FP64 form) or b.g64 (mixed: the
 // double-float factors, beside their complex64 copy in b.g for the sweeps).
@@ -649,6 +647,12 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_factor_wide(Geo g, Bufs b, in
   C* Ob = Pw + (size_t)nt * TB * TB;     // [nt][32][32] A_ik before
   const int lc = threadIdx.x & 31, lr = threadIdx.x >> 5;
   const int gt = ci * DY_THREADS + threadIdx.x, gn = CN * DY_THREADS;
+  const TriSmem<R> ts = {sm.tri, sm.tri + 2 * TB, sm.tri + 4 * TB};
+  int er[Tri<TB>::NE], ec[Tri<TB>::NE];
+  unsigned eon = 0;
+#pragma unroll
+  for (int q = 0; q < Tri<TB>::NE; ++q)
+    if (tri_entry(threadIdx.x >= 32 ? (int)threadIdx.x - 32 + Tri<TB>::OWN * q : TB * TB, TB, er[q], ec[q])) eon |= 1u << q;
   auto sync = [&]() {
     if (CN > 1) cl.sync();
     else __syncthreads();
@@ -682,7 +686,14 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_factor_wide(Geo g, Bufs b, in
       for (int k = 0; k < nt; ++k) {
         // pivot block, by every CTA for itself
         tile_in<R, false>(sm.tp, A, W, W, k * TB, k * TB);
-        tile_invert<R>(sm);
+        __syncthreads();
+        tri_invert<R, TB>(
+            TB, ts, er, ec, eon, [&](int r, int c) -> C { return sm.tp[r][c]; },
+            [&](int r, int c, const C& v) {
+              sm.tp[r][c] = v;
+              sm.tp[c][r] = v;
+            });
+        __syncthreads();
         // panel F_i = A_ik A_kk^-1 (kept beside the old A_ik for the update)
         for (int q = ci; q < nt - 1; q += CN) {
           const int ii = q < k ? q : q + 1;
@@ -912,6 +923,29 @@ __global__ void __launch_bounds__(DY_THREADS) k_hdiag(Geo g, Bufs b) {
   }
 }
 
+// CTAs per unit of k_factor_wide with nt x nt tiles: the one with the shortest
+// longest share of a slice's 32^3 tile products, two CTAs on an SM counting 1.9
+// (they share its FP32 pipe but hide each other's barriers).  Measured: 32 units, nt = 4
+// 56 ms with 4 CTAs, 68 with 8; 128 units, nt = 4 41 ms with 2, 43 with 1; 64 units,
+// nt = 5 31.9 with 2, 32.3 with 4.
+static int wide_cluster(int units, int nt) {
+  int best = 1;
+  double t_best = 0.0;
+  for (int C = 1; C <= 8 && (C == 1 || (long long)units * C <= DY_FACTOR_CTAS); C *= 2) {
+    auto share = [&](int tiles) { return (tiles + C - 1) / C; };
+    const int products = nt * (share(nt * nt) + share(nt * (nt + 1) / 2)) +
+                         nt * (share(nt - 1) + share(nt * (nt - 1) / 2));
+    const long long ctas = (long long)units * C;
+    const double per_sm = ctas <= DY_FACTOR_CTAS / 2 ? 1.0 : 1.9;
+    const double t = products * per_sm;
+    if (C == 1 || t < t_best) {
+      best = C;
+      t_best = t;
+    }
+  }
+  return best;
+}
+
 template <typename R, typename S>
 cudaError_t launch_factor(const Geo& g, const Bufs& b, int K, cudaStream_t st) {
   if (b.hdiag) {
@@ -926,7 +960,7 @@ cudaError_t launch_factor(const Geo& g, const Bufs& b, int K, cudaStream_t st) {
     if constexpr (sizeof(cx<R>) == sizeof(cxd)) {
       if (g.W > DY_MAXW || !b.fwork) return cudaErrorInvalidValue;
       const int units = g.p * K;
-      const int C = unit_cluster(units);
+      const int C = wide_cluster(units, (g.W + TB - 1) / TB);
       const int clusters = units < DY_FACTOR_CTAS / C ? units : DY_FACTOR_CTAS / C;
       return launch_clustered(k_factor_wide<R, S>, dim3(clusters * C), C, sizeof(TileSmem<R>), st, g, b, K);
     } else {
