@@ -231,7 +231,7 @@ __device__ void mix_drain(const MixCtx<WF, ROWS>& cx, MixState& st) {
 // complete and visible to the CTA on return.
 template <int WF, int NR, bool ROWS>
 __device__ __noinline__ void mix_sweep(const MixCtx<WF, ROWS>& ctx, MixState& state, int k0) {
-  constexpr int CT = Mix<WF>::CT, PF = NR == 1 ? 4 : 2, KP = Mix<WF>::KP, WARPS = Mix<WF>::WARPS;
+  constexpr int CT = Mix<WF>::CT, PF = NR == 1 && !ROWS ? 4 : 2, KP = Mix<WF>::KP, WARPS = Mix<WF>::WARPS;
   constexpr int KH = KP < 4 ? KP : 4;    // column pairs handled at a time
   MixSmem<WF>& sm = mix_sm<WF>();
   const MixCtx<WF, ROWS> cx = ctx;
