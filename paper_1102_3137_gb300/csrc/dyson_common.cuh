@@ -24,7 +24,9 @@
 #define DY_THREADS 256      // threads per CTA of every solver kernel
 #define DY_WARPS (DY_THREADS / 32)
 #define DY_MAXW 320         // widest slice the sweep kernels take (48^3 with p = 8: 288)
-#define DY_MAXW_SMEM 64     // widest slice the shared-memory factor kernel takes
+#define DY_MAXW_SMEM 64     // widest slice the shared-memory factor kernels take
+#define DY_TWO_MAXW64 32    // widest slice of the FP64 form's two-sided factors and two-chain sweeps (a
+                            // ring of two 64 x 64 binary64 blocks a chain does not fit on chip)
 #define DY_MAXNB 4          // largest Lanczos block size
 #define DY_LPRE_MAXLX 160   // widest interface line of the shared-memory layer preconditioner
 #define DY_LPRE_MAXLX_G 1024 // widest interface line of its global-memory form
@@ -242,9 +244,9 @@ struct Bufs {
   unsigned long long* sweeps;  // [K*nb][p] subdomain sweeps performed (work accounting)
   cxd* fwork;           // [DY_FACTOR_CTAS][2][W][W] wide-slice factor workspace (W > 64 only)
   cx<float>* lpt;       // [K][p][2][Lx][Lx] boundary-row surface Green's functions (lpre)
-  cx<float>* lpg;       // [K][p][Lx][W][W] complex64 slice factors of that recursion (lpre scratch)
+  cx<float>* lpg;       // [K][p][Lx][W][W] lpre in 2D: per (frequency, strip) the boundary columns of G_ss
+                        // [Lx][2][W], then the rows across the middle [2][Lx][W] (k_surface_two)
   void* lpm;            // [K][p-1][Lx][Lx] inverse layer blocks of S, precision of the form (lpre)
-  cx<float>* lpv;       // [K][p][2][Lx][W] boundary columns of the surface recursion (lpre, Lx > 160)
   cx<float>* lpw;       // [DY_FACTOR_CTAS][2][W][2 Lx T] boundary-column chains of the 3D slab
                         // surface recursion (lpre with T > 1), not per frequency
   cxd* gram;            // [K][k_max+1][k_max+1] Gram matrix q_l^T q_m of the stored basis, entry
@@ -334,7 +336,6 @@ cudaError_t launch_init_block(const Geo& g, const Bufs& b, int K, cudaStream_t s
 cudaError_t launch_surface(const Geo& g, const Bufs& b, int K, cudaStream_t st);
 template <typename R>
 cudaError_t launch_layer_inv(const Geo& g, const Bufs& b, int K, cudaStream_t st);
-size_t dyson_internal_surface_smem(const Geo& g);
 size_t dyson_internal_layer_inv_smem(const Geo& g);
 cudaError_t launch_finalize(const Geo& g, const Bufs& b, int K, cudaStream_t st);
 template <typename R>

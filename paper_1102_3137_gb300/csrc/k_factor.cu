@@ -84,8 +84,8 @@ __device__ __forceinline__ void smem_matmul(cx<R>* C, const cx<R>* X, const cx<R
   }
 }
 
-// One CTA per (subdomain, frequency), W <= 64, binary64 (the FP64 form; the mixed
-// form runs k_factor_two): g_s left-connected for every s, stored row-major for the
+// One CTA per (subdomain, frequency), binary64, DY_TWO_MAXW64 < W <= 64 (the other
+// strips run k_factor_two): g_s left-connected for every s, stored row-major for the
 // 8-warp sweeps.
 template <typename R>
 __global__ void __launch_bounds__(DY_THREADS) k_factor(Geo g, Bufs b) {
@@ -326,24 +326,26 @@ __device__ __forceinline__ void tri_invert(int W, const TriSmem<R>& ts, const in
     if (eon >> q & 1) to(er[q], ec[q], -v[q]);
 }
 
-// ---------------------------------------------------------------- two-sided, double-float
-// The mixed form's recursion for W <= 64, from both ends, so that the complex64
-// sweeps can run two chains at once.  With m = Lx / 2:
+// ---------------------------------------------------------------- two-sided
+// The recursion from both ends, so that the sweeps can run two chains at once: the
+// mixed form for W <= 64 (R = dfl), the FP64 form for W <= DY_TWO_MAXW64 (binary64).  With m = Lx / 2:
 //   left   g_s = (D_s - t^2 g_{s-1})^-1            s < m
 //   right  g_s = (D_s - t^2 g_{s+1})^-1            s > m
 //   middle G_mm = (D_m - t^2 g_{m-1} - t^2 g_{m+1})^-1
 //   G_ss = g_s + t^2 g_s G_{s+1,s+1} g_s  (s < m),  g_s + t^2 g_s G_{s-1,s-1} g_s  (s > m)
-// Slot s holds g_s, or G_mm for s = m: in double-float in b.g64, and in complex64 in
-// b.g with column pairs interleaved (entry (r, c) at ((c / 2) W + r) 2 + c % 2, so
-// that a lane reads columns 2k, 2k+1 of its row as one 16-byte word).
+// Slot s holds g_s, or G_mm for s = m.  FP64 form: in b.g.  Mixed form: in double-float
+// in b.g64, and in complex64 in b.g with column pairs interleaved (entry (r, c) at
+// ((c / 2) W + r) 2 + c % 2, so that a lane reads columns 2k, 2k+1 of its row as one
+// 16-byte word).
 // One cluster of two CTAs per (subdomain, frequency): CTA 0 the left chain, CTA 1 the
 // right one, which meet at the middle block (each inverts it for itself) and go back
 // separately.  One CTA running both chains in turn took 65 us a slice at W = 28 with
 // 21 x 4 units on 152 SMs.
-using cxl = cx<dfl>;
 
-template <int WF>
+template <typename R, int WF>
 __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo g, Bufs b) {
+  using cxl = cx<R>;                         // 16 bytes in either arithmetic
+  constexpr bool mixed = std::is_same<R, dfl>::value;
   constexpr int NE = Tri<WF>::NE, NP = Tri<WF>::NP, OWN = Tri<WF>::OWN;
   constexpr int NB = (WF * WF + DY_THREADS - 1) / DY_THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -353,19 +355,19 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
   cxl* A = reinterpret_cast<cxl*>(smem_raw);
   cxl* Bm = A + n;
   cxl* Cm = Bm + n;
-  const TriSmem<dfl> ts = {Cm + n, Cm + n + 2 * W, Cm + n + 4 * W};
+  const TriSmem<R> ts = {Cm + n, Cm + n + 2 * W, Cm + n + 4 * W};
   cxl* dg = Cm + n + 6 * W;                    // [W] H_ii of the slice being formed
   cxl* Gprev = dg + W;                       // [2][W] columns of the last off-diagonal block at the boundary rows
   cxl* Gmid = Gprev + 2 * W;                 // [2][W] rows of G_{m+1,m} at the boundary rows (left CTA's copy is used)
   const size_t uoff = ((size_t)kf * g.p + i) * (size_t)Lx * n;
-  cxl* gout = reinterpret_cast<cxl*>(b.g64) + uoff;
+  cxl* gout = reinterpret_cast<cxl*>(mixed ? (void*)b.g64 : b.g) + uoff;
   cxf* gsw = reinterpret_cast<cxf*>(b.g) + uoff;
   cxd* dB = b.diagB + (size_t)kf * g.Ndd + (size_t)i * Lx * W;
   const cdfl* hd = reinterpret_cast<const cdfl*>(b.hdiag) + (size_t)kf * g.Ndd + (size_t)i * Lx * W;
   const bool band = !g.lpre;                 // the banded preconditioner reads the off-diagonal blocks
   cxd* oB = band && b.offB ? b.offB + ((size_t)kf * g.p + i) * (size_t)Lx * W : nullptr;
   cxd* o2 = band && b.off2 && T == 1 ? b.off2 + ((size_t)kf * g.p + i) * (size_t)Lx * W : nullptr;
-  const dfl t = (dfl)g.t, t2 = (dfl)(g.t * g.t);
+  const R t = (R)g.t, t2 = (R)(g.t * g.t);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
   int er[NE], ec[NE], pr[NP], pc[NP];
@@ -377,19 +379,22 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
   for (int q = 0; q < NP; ++q)
     if (tri_entry(tid + DY_THREADS * q, W, pr[q], pc[q])) pon |= 1u << q;
 
-  auto load_h = [&](int s) {
-    if (tid < W) {
+  // H_ii of row tid of slice s (tid < W): from the DD-layout copy in the mixed form
+  auto diag_of = [&](int s) -> cxl {
+    if constexpr (mixed) {
       const cdfl d = hd[(size_t)s * W + tid];
-      dg[tid] = cxl{d.x, d.y};
+      return cxl{d.x, d.y};
+    } else {
+      return tid < w ? dyson_diag(g, b, kf, sub_nat(g, i, s, tid)) : cxl{0, 0};
     }
   };
   // A <- (D_s - t^2 (pa + pb))^-1, zero on the padding; pa, pb (full W x W, either may be
   // null) may be A itself; stored in slot s when keep.  dg holds slice s's diagonal;
   // slice sn's (if >= 0) is fetched for the next call.
   auto invert = [&](int s, const cxl* pa, const cxl* pb, bool keep, int sn) {
-    cdfl hn = {dfl(0.f, 0.f), dfl(0.f, 0.f)};
-    if (sn >= 0 && tid < W) hn = hd[(size_t)sn * W + tid];
-    tri_invert<dfl, WF>(
+    cxl hn = {0, 0};
+    if (sn >= 0 && tid < W) hn = diag_of(sn);
+    tri_invert<R, WF>(
         W, ts, er, ec, eon,
         [&](int r, int c) -> cxl {
           const int e = r * W + c;
@@ -398,7 +403,7 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
           if (pb) x = x - t2 * pb[e];
           if (r < w && c < w) {
             if (r == c) x = x + dg[r];
-            else if (slice_adjacent<dfl>(r, c, T)) x.x += t;
+            else if (slice_adjacent<R>(r, c, T)) x.x += t;
           } else {
             x = r == c ? cxl{1, 0} : cxl{0, 0};
           }
@@ -409,18 +414,18 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
           A[r * W + c] = x;
           A[c * W + r] = x;
         });
-    if (sn >= 0 && tid < W) dg[tid] = cxl{hn.x, hn.y};
+    if (sn >= 0 && tid < W) dg[tid] = hn;
     __syncthreads();
     if (keep)
       for (int e = tid; e < n; e += DY_THREADS) {
         const int r = e / W, c = e - r * W;
         const cxl x = A[e];
         gout[(size_t)s * n + e] = x;
-        gsw[(size_t)s * n + ((size_t)(c >> 1) * W + r) * 2 + (c & 1)] = cconv<float>(x);
+        if constexpr (mixed) gsw[(size_t)s * n + ((size_t)(c >> 1) * W + r) * 2 + (c & 1)] = cconv<float>(x);
       }
   };
   // the layer preconditioner's input: columns w - 1 and 0 of G_ss (k_surface_two)
-  cxf* bc = g.lpre ? b.lpg + uoff : nullptr;
+  cxf* bc = g.lpre && b.lpg ? b.lpg + uoff : nullptr;
   auto diag_out = [&](int s) {
     for (int r = tid; r < W; r += DY_THREADS) dB[(size_t)s * W + r] = (r < w) ? cconv<double>(A[r * W + r]) : cxd{0, 0};
     if (bc)
@@ -523,7 +528,7 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
     diag_out(s);
   };
 
-  load_h(side == 0 ? 0 : Lx - 1);
+  if (tid < W) dg[tid] = diag_of(side == 0 ? 0 : Lx - 1);
   __syncthreads();
   if (side == 0) {
     for (int s = 0; s < m; ++s) invert(s, s > 0 ? A : nullptr, nullptr, true, s + 1);
@@ -967,11 +972,13 @@ cudaError_t launch_factor(const Geo& g, const Bufs& b, int K, cudaStream_t st) {
       return cudaErrorInvalidValue;
     }
   }
+  const size_t smem2 = (3 * (size_t)g.W * g.W + 11 * (size_t)g.W) * sizeof(cx<R>);
   if constexpr (std::is_same<R, dfl>::value) {
-    const size_t smem = (3 * (size_t)g.W * g.W + 11 * (size_t)g.W) * sizeof(cxl);
-    auto kern = g.W <= 16 ? k_factor_two<16> : (g.W <= 32 ? k_factor_two<32> : k_factor_two<64>);
-    return launch_clustered(kern, dim3(2 * g.p, K), 2, smem, st, g, b);
+    auto kern = g.W <= 16 ? k_factor_two<R, 16> : (g.W <= 32 ? k_factor_two<R, 32> : k_factor_two<R, 64>);
+    return launch_clustered(kern, dim3(2 * g.p, K), 2, smem2, st, g, b);
   } else {
+    if (g.W <= DY_TWO_MAXW64)
+      return launch_clustered(g.W <= 16 ? k_factor_two<R, 16> : k_factor_two<R, 32>, dim3(2 * g.p, K), 2, smem2, st, g, b);
     const size_t smem = (3 * (size_t)g.W * g.W + 4 * (size_t)g.W) * sizeof(cx<R>);
     cudaError_t e = raise_smem_limit((const void*)k_factor<R>, smem);
     if (e != cudaSuccess) return e;

@@ -12,19 +12,13 @@
 // small, so COCG on S needs one or two iterations.  S itself is never formed.
 //
 // The preconditioner may be inexact, so everything here runs in complex64:
-//   k_surface    per (strip, frequency): the left-connected slice recursion
-//                along x, g_s = (D_s - t^2 g_{s-1})^-1, then backward
-//                G_ss = g_s + t^2 g_s G_{s+1,s+1} g_s and, for every s' > s,
-//                G_{s,s'} = -t g_s G_{s+1,s'} applied to the boundary columns
-//                of G_{s',s'} (kept in shared memory); P[s][s'] is their
-//                boundary entry.
+//   k_surface_two  per (strip, side, frequency): P[s][s'] from the factorization's
+//                two-sided factors and boundary columns of G_ss, by chains of
+//                products towards the two ends of the strip.
 //   k_layer_inv  per (interface line, frequency): S_ll and its inverse by the
 //                sweep operator, symmetrised so that COCG sees a complex
 //                symmetric M^-1.
-// Lines longer than DY_LPRE_MAXLX (160) do not fit shared memory; there
-//   k_surface_g  keeps the boundary columns of G_{s,s'} in global memory
-//                (one warp per column, the column broadcast through shared
-//                memory), and
+// Layers of more than DY_LPRE_MAXLX (160) sites do not fit shared memory; there
 //   k_layer_inv_g forms S_ll in place of P_top(l) and inverts it there by the
 //                block sweep operator (32 x 32 pivots, rank-32 updates of the
 //                upper 64 x 64 tiles), then writes the mirrored inverse.
@@ -36,7 +30,7 @@
 //                G_{s,c} = -t g_s G_{s+1,c} carried on the T boundary columns
 //                of each slice c, with 32 x 32 tiles through shared memory
 //                multiplied on the tensor cores (3xTF32; persistent grid, one
-//                (slab, frequency) at a time per CTA);
+//                (slab, frequency) at a time per cluster);
 //   k_layer_inv_g  inverts the A x A blocks (A <= 1024).
 #include <type_traits>
 
@@ -79,268 +73,10 @@ __device__ __forceinline__ void sweep_invert_f(cxf_* A, int n, cxf_* prow, cxf_*
   __syncthreads();
 }
 
-// C = alpha X Y + beta D for W x W shared matrices (D may alias nothing, may be null)
-__device__ __forceinline__ void small_matmul(cxf_* C, const cxf_* X, const cxf_* Y, int W, float alpha,
-                                             const cxf_* D) {
-  for (int e = threadIdx.x; e < W * W; e += DY_THREADS) {
-    const int r = e / W, c = e - r * W;
-    cxf_ acc = {0.f, 0.f};
-    for (int k = 0; k < W; ++k) acc = cfma(X[r * W + k], Y[k * W + c], acc);
-    acc = cxf_{alpha * acc.x, alpha * acc.y};
-    if (D) acc = acc + D[e];
-    C[e] = acc;
-  }
-}
-
-// The same for W = 32 with four rows per thread sharing each load of Y:
-// lane = column, warp = first row, rows warp + 8 j.
-__device__ __forceinline__ void small_matmul32(cxf_* C, const cxf_* X, const cxf_* Y, float alpha,
-                                               const cxf_* D) {
-  constexpr int W = 32;
-  const int c = threadIdx.x & 31, r0 = threadIdx.x >> 5;
-  cxf_ acc[4] = {};
-#pragma unroll 8
-  for (int k = 0; k < W; ++k) {
-    const cxf_ y = Y[k * W + c];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[j] = cfma(X[(r0 + 8 * j) * W + k], y, acc[j]);
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int e = (r0 + 8 * j) * W + c;
-    cxf_ v = cxf_{alpha * acc[j].x, alpha * acc[j].y};
-    if (D) v = v + D[e];
-    C[e] = v;
-  }
-}
-
 constexpr int SURF_MAXW = 32;
-constexpr int SURF_NG = DY_THREADS / 32;                             // column groups (one per warp)
-constexpr int SURF_NCOL = (DY_LPRE_MAXLX + SURF_NG - 1) / SURF_NG;   // columns per thread at most
-
-__host__ __device__ __forceinline__ int surf_ldv(int Lx) { return Lx | 1; }   // odd stride: no bank conflicts
-
-// WT: the slice width at compile time (32, the common 2D strip), or 0 for any
-// width up to 32 read from the geometry
-template <int WT>
-__global__ void __launch_bounds__(DY_THREADS, 2) k_surface(Geo g, Bufs b) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int i = blockIdx.x, f = blockIdx.y;
-  const int W = WT ? WT : g.W, Lx = g.Lx, w = g.h[i], n = W * W, ldv = surf_ldv(Lx);
-  const bool need_top = i < g.p - 1, need_bot = i > 0;
-  cxf_* Gs = reinterpret_cast<cxf_*>(smem_raw);   // g_s
-  cxf_* Gd = Gs + n;                              // G_ss
-  cxf_* Tm = Gd + n;
-  cxf_* prow = Tm + n;
-  cxf_* fcol = prow + W;
-  cxf_* Vt = fcol + W;                            // [W][ldv] boundary columns of G_{s,s'}, top row
-  cxf_* Vb = Vt + (size_t)W * ldv;                // same for the bottom row
-  cxf_* gsv = b.lpg + ((size_t)f * g.p + i) * (size_t)Lx * n;   // own scratch: runs beside the factorization
-  cxf_* Pt = b.lpt + (((size_t)f * g.p + i) * 2 + 0) * (size_t)Lx * Lx;
-  cxf_* Pb = b.lpt + (((size_t)f * g.p + i) * 2 + 1) * (size_t)Lx * Lx;
-  const float t = d2f_bits(g.t), t2 = t * t;
-  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-
-  // forward: g_s = (D_s - t^2 g_{s-1})^-1, padding rows/columns carry the identity
-  for (int s = 0; s < Lx; ++s) {
-    for (int e = threadIdx.x; e < n; e += DY_THREADS) {
-      const int r = e / W, c = e - r * W;
-      cxf_ v = {0.f, 0.f};
-      if (r < w && c < w) {
-        if (r == c) {
-          const cxd d = dyson_diag(g, b, f, sub_nat(g, i, s, r));
-          v = cxf_{d2f_bits(d.x), d2f_bits(d.y)};
-        } else if (r == c + 1 || c == r + 1) {
-          v = cxf_{t, 0.f};
-        }
-        if (s > 0) v = cfma(cxf_{-t2, 0.f}, Gs[e], v);
-      } else if (r == c) {
-        v = cxf_{1.f, 0.f};
-      }
-      Gs[e] = v;
-    }
-    sweep_invert_f(Gs, W, prow, fcol);
-    for (int e = threadIdx.x; e < n; e += DY_THREADS) {
-      const int r = e / W, c = e - r * W;
-      if (r >= w || c >= w) Gs[e] = cxf_{0.f, 0.f};
-      gsv[(size_t)s * n + e] = Gs[e];
-    }
-    __syncthreads();
-  }
-  // backward: G_ss, and for every s' > s the boundary columns of
-  // G_{s,s'} = -t g_s G_{s+1,s'}; lane = row, warp = column group
-  for (int s = Lx - 1; s >= 0; --s) {
-    for (int e = threadIdx.x; e < n; e += DY_THREADS) Gs[e] = gsv[(size_t)s * n + e];
-    __syncthreads();
-    if (s == Lx - 1) {
-      for (int e = threadIdx.x; e < n; e += DY_THREADS) Gd[e] = Gs[e];
-    } else {
-      if constexpr (WT == 32) {
-        small_matmul32(Tm, Gs, Gd, 1.f, nullptr);          // g_s G_{s+1,s+1}
-        __syncthreads();
-        small_matmul32(Gd, Tm, Gs, t2, Gs);                 // g_s + t^2 g_s G g_s
-      } else {
-        small_matmul(Tm, Gs, Gd, W, 1.f, nullptr);
-        __syncthreads();
-        small_matmul(Gd, Tm, Gs, W, t2, Gs);
-      }
-      cxf_ gr[SURF_MAXW];                                  // row `lane` of g_s (symmetric)
-#pragma unroll
-      for (int k = 0; k < SURF_MAXW; ++k) gr[k] = (lane < W && k < W) ? Gs[k * W + lane] : cxf_{0.f, 0.f};
-      for (int side = 0; side < 2; ++side) {
-        if (side == 0 ? !need_top : !need_bot) continue;
-        cxf_* V = side == 0 ? Vt : Vb;
-        cxf_ out[SURF_NCOL];
-#pragma unroll
-        for (int j = 0; j < SURF_NCOL; ++j) {
-          const int c = s + 1 + grp + SURF_NG * j;
-          cxf_ acc = {0.f, 0.f};
-          if (c < Lx) {
-#pragma unroll
-            for (int k = 0; k < SURF_MAXW; ++k)
-              if (k < W) acc = cfma(gr[k], V[k * ldv + c], acc);
-          }
-          out[j] = cxf_{-t * acc.x, -t * acc.y};
-        }
-        __syncthreads();                                   // every column read before any is rewritten
-        cxf_* P = side == 0 ? Pt : Pb;
-        const int rb = side == 0 ? w - 1 : 0;
-#pragma unroll
-        for (int j = 0; j < SURF_NCOL; ++j) {
-          const int c = s + 1 + grp + SURF_NG * j;
-          if (c < Lx && lane < W) {
-            V[lane * ldv + c] = out[j];
-            if (lane == rb) {
-              P[(size_t)s * Lx + c] = out[j];
-              P[(size_t)c * Lx + s] = out[j];
-            }
-          }
-        }
-      }
-    }
-    __syncthreads();
-    // start the chain of column s' = s: the boundary columns of G_ss
-    for (int r = threadIdx.x; r < W; r += DY_THREADS) {
-      Vt[r * ldv + s] = Gd[r * W + (w - 1)];
-      Vb[r * ldv + s] = Gd[r * W + 0];
-    }
-    if (threadIdx.x == 0) {
-      Pt[(size_t)s * Lx + s] = Gd[(w - 1) * W + (w - 1)];
-      Pb[(size_t)s * Lx + s] = Gd[0];
-    }
-    __syncthreads();
-  }
-}
-
-// The same surface Green's functions for lines longer than the shared-memory
-// form takes (Lx > DY_LPRE_MAXLX, slice width 32): the boundary columns
-// V[c][r] of G_{s,c}, c > s, live in global memory (b.lpv), column-major, and
-// the update V[:, c] <- -t g_s V[:, c] runs one warp per column: the warp
-// reads its column, broadcasts it through shared memory and lane r forms row
-// r of the product from its register copy of row r of g_s.  Only that warp
-// touches column c within a step, so the in-place update needs no barrier.
-__global__ void __launch_bounds__(DY_THREADS) k_surface_g(Geo g, Bufs b) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int W = 32, n = W * W;
-  const int i = blockIdx.x, f = blockIdx.y;
-  const int Lx = g.Lx, w = g.h[i];
-  const bool need_top = i < g.p - 1, need_bot = i > 0;
-  cxf_* Gs = reinterpret_cast<cxf_*>(smem_raw);   // g_s
-  cxf_* Gd = Gs + n;                              // G_ss
-  cxf_* Tm = Gd + n;
-  cxf_* prow = Tm + n;
-  cxf_* fcol = prow + W;
-  cxf_* colb = fcol + W;                          // [8 warps][W] column broadcast
-  cxf_* gsv = b.lpg + ((size_t)f * g.p + i) * (size_t)Lx * n;
-  cxf_* Pt = b.lpt + (((size_t)f * g.p + i) * 2 + 0) * (size_t)Lx * Lx;
-  cxf_* Pb = b.lpt + (((size_t)f * g.p + i) * 2 + 1) * (size_t)Lx * Lx;
-  cxf_* Vt = b.lpv + (((size_t)f * g.p + i) * 2 + 0) * (size_t)Lx * W;   // [Lx][W]
-  cxf_* Vb = b.lpv + (((size_t)f * g.p + i) * 2 + 1) * (size_t)Lx * W;
-  const float t = d2f_bits(g.t), t2 = t * t;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-
-  // forward: g_s = (D_s - t^2 g_{s-1})^-1, padding rows/columns carry the identity
-  for (int s = 0; s < Lx; ++s) {
-    for (int e = threadIdx.x; e < n; e += DY_THREADS) {
-      const int r = e / W, c = e - r * W;
-      cxf_ v = {0.f, 0.f};
-      if (r < w && c < w) {
-        if (r == c) {
-          const cxd d = dyson_diag(g, b, f, sub_nat(g, i, s, r));
-          v = cxf_{d2f_bits(d.x), d2f_bits(d.y)};
-        } else if (r == c + 1 || c == r + 1) {
-          v = cxf_{t, 0.f};
-        }
-        if (s > 0) v = cfma(cxf_{-t2, 0.f}, Gs[e], v);
-      } else if (r == c) {
-        v = cxf_{1.f, 0.f};
-      }
-      Gs[e] = v;
-    }
-    sweep_invert_f(Gs, W, prow, fcol);
-    for (int e = threadIdx.x; e < n; e += DY_THREADS) {
-      const int r = e / W, c = e - r * W;
-      if (r >= w || c >= w) Gs[e] = cxf_{0.f, 0.f};
-      gsv[(size_t)s * n + e] = Gs[e];
-    }
-    __syncthreads();
-  }
-  // backward: G_ss, and for every c > s the boundary columns of G_{s,c} = -t g_s G_{s+1,c}
-  cxf_* cb = colb + wid * W;
-  for (int s = Lx - 1; s >= 0; --s) {
-    for (int e = threadIdx.x; e < n; e += DY_THREADS) Gs[e] = gsv[(size_t)s * n + e];
-    __syncthreads();
-    if (s == Lx - 1) {
-      for (int e = threadIdx.x; e < n; e += DY_THREADS) Gd[e] = Gs[e];
-    } else {
-      small_matmul32(Tm, Gs, Gd, 1.f, nullptr);          // g_s G_{s+1,s+1}
-      __syncthreads();
-      small_matmul32(Gd, Tm, Gs, t2, Gs);                 // g_s + t^2 g_s G g_s
-      cxf_ gr[W];                                         // row `lane` of g_s (symmetric)
-#pragma unroll
-      for (int k = 0; k < W; ++k) gr[k] = Gs[k * W + lane];
-      for (int side = 0; side < 2; ++side) {
-        if (side == 0 ? !need_top : !need_bot) continue;
-        cxf_* V = side == 0 ? Vt : Vb;
-        cxf_* P = side == 0 ? Pt : Pb;
-        const int rb = side == 0 ? w - 1 : 0;
-        for (int c = s + 1 + wid; c < Lx; c += DY_WARPS) {
-          cb[lane] = V[(size_t)c * W + lane];
-          __syncwarp();
-          cxf_ acc0 = {0.f, 0.f}, acc1 = {0.f, 0.f};
-#pragma unroll
-          for (int k = 0; k < W; k += 2) {
-            acc0 = cfma(gr[k], cb[k], acc0);
-            acc1 = cfma(gr[k + 1], cb[k + 1], acc1);
-          }
-          const cxf_ acc = acc0 + acc1;
-          const cxf_ out = {-t * acc.x, -t * acc.y};
-          __syncwarp();                                   // the column is read before it is rewritten
-          V[(size_t)c * W + lane] = out;
-          if (lane == rb) {
-            P[(size_t)s * Lx + c] = out;
-            P[(size_t)c * Lx + s] = out;
-          }
-        }
-      }
-    }
-    __syncthreads();
-    // start the chain of column c = s: the boundary columns of G_ss
-    for (int r = threadIdx.x; r < W; r += DY_THREADS) {
-      Vt[(size_t)s * W + r] = Gd[r * W + (w - 1)];
-      Vb[(size_t)s * W + r] = Gd[r * W + 0];
-    }
-    if (threadIdx.x == 0) {
-      Pt[(size_t)s * Lx + s] = Gd[(w - 1) * W + (w - 1)];
-      Pb[(size_t)s * Lx + s] = Gd[0];
-    }
-    __syncthreads();
-  }
-}
-
-// The surface Green's functions of the mixed form's strips, from the two-sided
-// factors g_s and the boundary columns of G_ss that the factorization leaves (in
-// complex64, the latter in b.lpg): no recursion of its own.  With m the middle slice
+// The surface Green's functions of the 2D strips, from the two-sided factors g_s (S:
+// complex64 or binary64) and the boundary columns of G_ss that the factorization leaves
+// in b.lpg, in complex64: no recursion of its own.  With m the middle slice
 // and rb the boundary row, per side:
 //   pairs of one half:  G_{s,c} e_rb = -t g_s G_{s+-1,c} e_rb   (towards the ends, all c at once)
 //   pairs across:       G_{s,c} = G_{s,m} N_c^T,  G_{s,m} = -t g_s G_{s+1,m} (s < m),
@@ -351,7 +87,7 @@ __global__ void __launch_bounds__(DY_THREADS) k_surface_g(Geo g, Bufs b) {
 // lane = row with its row of g_s in registers, a warp's columns two at a time by 16-byte
 // broadcasts from shared memory.  The one-CTA form ran its own complex64 recursion and a
 // chain of Lx slices: 4.0 ms at 128^2 x 32 with 128 CTAs.
-template <int WT>
+template <typename S, int WT>
 __global__ void __launch_bounds__(DY_THREADS, 2) k_surface_two(Geo g, Bufs b) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cg::cluster_group cl = cg::this_cluster();
@@ -363,20 +99,28 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_surface_two(Geo g, Bufs b) {
   cxf_* M = gb[1] + n;                            // [W columns][W]: G_{s,m} or N_s
   cxf_* V = M + n;                                // [steps][W]: the boundary columns, by distance from the middle
   const size_t unit = (size_t)f * g.p + i;
-  const cxf_* gsrc = reinterpret_cast<const cxf_*>(b.g) + unit * (size_t)Lx * n;   // column pairs interleaved
+  const cx<S>* gsrc = reinterpret_cast<const cx<S>*>(b.g) + unit * (size_t)Lx * n;   // complex64: column pairs interleaved
   const cxf_* bc = b.lpg + unit * (size_t)Lx * n;
   cxf_* Rr = b.lpg + unit * (size_t)Lx * n + (size_t)2 * Lx * W + (size_t)sd * Lx * W;   // [Lx][W] rows rb of G_{s,m} / N_s
   cxf_* P = b.lpt + (unit * 2 + sd) * (size_t)Lx * Lx;
   const float t = d2f_bits(g.t);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int n4 = n / 2;                           // 16-byte words of a block
+  const int n4 = n / 2;                           // words of two entries of a block
   auto slice = [&](int k) { return half == 0 ? m - 1 - k : m + 1 + k; };     // k-th step's slice
   constexpr int NF = (SURF_MAXW * SURF_MAXW / 2 + DY_THREADS - 1) / DY_THREADS;
   float4 nx[NF];
   auto fetch = [&](int s) {
 #pragma unroll
     for (int q = 0; q < NF; ++q)
-      if (tid + DY_THREADS * q < n4) nx[q] = reinterpret_cast<const float4*>(gsrc + (size_t)s * n)[tid + DY_THREADS * q];
+      if (tid + DY_THREADS * q < n4) {
+        if constexpr (sizeof(S) == 4) {
+          nx[q] = reinterpret_cast<const float4*>(gsrc + (size_t)s * n)[tid + DY_THREADS * q];
+        } else {                                  // columns 2 k2, 2 k2 + 1 of row r (symmetric) into the same order
+          const int e = tid + DY_THREADS * q, k2 = e / W, r = e - k2 * W;
+          const cxd v0 = gsrc[(size_t)s * n + (size_t)(2 * k2) * W + r], v1 = gsrc[(size_t)s * n + (size_t)(2 * k2 + 1) * W + r];
+          nx[q] = make_float4(d2f_bits(v0.x), d2f_bits(v0.y), d2f_bits(v1.x), d2f_bits(v1.y));
+        }
+      }
   };
   auto put = [&](cxf_* d) {
 #pragma unroll
@@ -386,7 +130,14 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_surface_two(Geo g, Bufs b) {
   // M: G_mm (slot m; symmetric, so its rows are its columns) or 1
   for (int e = tid; e < n; e += DY_THREADS) {
     const int c = e / W, r = e - c * W;
-    M[e] = half == 0 ? gsrc[(size_t)m * n + ((size_t)(c >> 1) * W + r) * 2 + (c & 1)] : cxf_{r == c ? 1.f : 0.f, 0.f};
+    if (half == 1) {
+      M[e] = cxf_{r == c ? 1.f : 0.f, 0.f};
+    } else if constexpr (sizeof(S) == 4) {
+      M[e] = gsrc[(size_t)m * n + ((size_t)(c >> 1) * W + r) * 2 + (c & 1)];
+    } else {
+      const cxd v = gsrc[(size_t)m * n + e];
+      M[e] = cxf_{d2f_bits(v.x), d2f_bits(v.y)};
+    }
   }
   if (steps > 0) {
     fetch(slice(0));
@@ -800,16 +551,10 @@ __global__ void __launch_bounds__(DY_THREADS) k_layer_inv(Geo g, Bufs b) {
 
 }  // namespace
 
-size_t dyson_internal_surface_smem(const Geo& g) {
-  return (3 * (size_t)g.W * g.W + 2 * (size_t)g.W + 2 * (size_t)g.W * surf_ldv(g.Lx)) * sizeof(cxf_);
-}
-
 size_t dyson_internal_layer_inv_smem(const Geo& g) {
   if (g.A > DY_LPRE_MAXLX) return 0;                       // global-memory form
   return ((size_t)g.A * g.A + 2 * (size_t)g.A) * sizeof(cxf_);
 }
-
-static size_t surface_g_smem() { return (3 * 32 * 32 + 2 * 32 + DY_WARPS * 32) * sizeof(cxf_); }
 
 cudaError_t launch_surface(const Geo& g, const Bufs& b, int K, cudaStream_t st) {
   if (!g.lpre) return cudaSuccess;
@@ -822,28 +567,12 @@ cudaError_t launch_surface(const Geo& g, const Bufs& b, int K, cudaStream_t st) 
     return launch_clustered(k_surface_3d<cxd>, dim3(grid), C, 0, st, g, b, K);
   }
   if (g.W > SURF_MAXW || g.Lx > DY_LPRE_MAXLX_G) return cudaErrorInvalidValue;
-  if (b.g64) {                             // mixed form: from the two-sided factors
-    size_t smem = (3 * (size_t)g.W * g.W + (size_t)(g.Lx / 2) * g.W) * sizeof(cxf_);
-    const size_t tb = (size_t)33 * g.W * sizeof(cxf_);
-    if (smem < tb) smem = tb;
-    return launch_clustered(g.W == 32 ? k_surface_two<32> : k_surface_two<0>, dim3(4 * g.p, K), 2, smem, st, g, b);
-  }
-  if (g.Lx > DY_LPRE_MAXLX) {
-    if (g.W != 32 || !b.lpv) return cudaErrorInvalidValue;
-    k_surface_g<<<dim3(g.p, K), DY_THREADS, surface_g_smem(), st>>>(g, b);
-    return cudaGetLastError();
-  }
-  const size_t smem = dyson_internal_surface_smem(g);
-  if (g.W == 32) {
-    cudaError_t e = raise_smem_limit((const void*)k_surface<32>, smem);
-    if (e != cudaSuccess) return e;
-    k_surface<32><<<dim3(g.p, K), DY_THREADS, smem, st>>>(g, b);
-  } else {
-    cudaError_t e = raise_smem_limit((const void*)k_surface<0>, smem);
-    if (e != cudaSuccess) return e;
-    k_surface<0><<<dim3(g.p, K), DY_THREADS, smem, st>>>(g, b);
-  }
-  return cudaGetLastError();
+  size_t smem = (3 * (size_t)g.W * g.W + (size_t)(g.Lx / 2) * g.W) * sizeof(cxf_);
+  const size_t tb = (size_t)33 * g.W * sizeof(cxf_);
+  if (smem < tb) smem = tb;
+  const dim3 grid(4 * g.p, K);
+  if (b.g64) return launch_clustered(g.W == 32 ? k_surface_two<float, 32> : k_surface_two<float, 0>, grid, 2, smem, st, g, b);
+  return launch_clustered(g.W == 32 ? k_surface_two<double, 32> : k_surface_two<double, 0>, grid, 2, smem, st, g, b);
 }
 
 template <typename R>

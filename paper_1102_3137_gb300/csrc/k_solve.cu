@@ -216,14 +216,17 @@ cudaError_t launch_wait_selftest(unsigned long long limit_ns, int* out, cudaStre
   return cudaGetLastError();
 }
 
+// the strips whose sweeps run as two chains (xmatvec_mixed.cuh)
+static bool two_chain(const Geo& g, bool mixed) { return g.W <= (mixed ? DY_MAXW_SMEM : DY_TWO_MAXW64); }
+
 size_t dyson_internal_sweep_smem(const Geo& g, bool mixed) {
-  if (mixed && g.W <= DY_MAXW_SMEM) return mix_plan(g).smem;
+  if (two_chain(g, mixed)) return mixed ? mix_plan<float>(g).smem : mix_plan<double>(g).smem;
   return mixed ? sweep_smem<float>(g) : sweep_smem<double>(g);
 }
 
 void dyson_internal_ring_plan(const Geo& g, bool mixed, int* S, int* CR, int* NT) {
-  if (mixed && g.W <= DY_MAXW_SMEM) {
-    *S = 2 * mix_plan(g).S;
+  if (two_chain(g, mixed)) {
+    *S = 2 * (mixed ? mix_plan<float>(g).S : mix_plan<double>(g).S);
     *CR = g.W;
     *NT = mix_threads(g.W);
     return;
@@ -235,7 +238,8 @@ void dyson_internal_ring_plan(const Geo& g, bool mixed, int* S, int* CR, int* NT
 }
 
 int dyson_internal_ring_candidates(const Geo& g, bool mixed, int* S, int* CR, int* ROWS, int max) {
-  if (mixed && g.W <= DY_MAXW_SMEM) return mix_candidates(g, S, CR, ROWS, max);
+  if (two_chain(g, mixed))
+    return mixed ? mix_candidates<float>(g, S, CR, ROWS, max) : mix_candidates<double>(g, S, CR, ROWS, max);
   for (int k = 0; k < max; ++k) ROWS[k] = 0;
   return mixed ? ring_candidates<float>(g, S, CR, max) : ring_candidates<double>(g, S, CR, max);
 }

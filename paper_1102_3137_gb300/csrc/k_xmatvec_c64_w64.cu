@@ -1,4 +1,4 @@
 // Mixed form, slices of width 32 < W <= 64 (the two-chain sweep of xmatvec_mixed.cuh).
 #include "xmatvec_mixed.cuh"
 
-DY_MIXED_VARIANT(64)
+DY_CHAIN_VARIANT(float, 64, k_xmatvec_m)

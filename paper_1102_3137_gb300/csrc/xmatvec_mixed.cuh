@@ -34,66 +34,74 @@ constexpr int MIX_MAXS = 8;              // most ring slots of one chain
 constexpr size_t MIX_SMEM_2 = 112 * 1024;   // dynamic shared memory per CTA at two CTAs per SM
 constexpr size_t MIX_SMEM_1 = 226 * 1024;   // and at one
 
-template <int WF>
+template <typename R, int WF>
 struct Mix {
   static constexpr int WARPS = WF / 8;   // compute warps of one chain
   static constexpr int CT = 32 * WARPS;
-  static constexpr int KP = WF / 8;      // column pairs a lane holds
+  static constexpr int CU = 16 / (int)sizeof(cx<R>);   // columns in a 16-byte word of a block
+  static constexpr int KP = WF / (4 * CU);   // words a lane holds (it has a quarter of a row)
   static constexpr int PROD = 2 * WARPS; // first of the two producer warps
   static constexpr int NT = WF == 16 ? 256 : 32 * (2 * WARPS + 2);   // 256, 320, 576
-  static constexpr int PER_SM = WF <= 32 ? 2 : 1;
+  static constexpr int PER_SM = WF <= (sizeof(R) == 4 ? 32 : 16) ? 2 : 1;
 };
-__host__ __device__ inline int mix_threads(int W) { return W <= 16 ? Mix<16>::NT : (W <= 32 ? Mix<32>::NT : Mix<64>::NT); }
+__host__ __device__ inline int mix_threads(int W) {
+  return W <= 16 ? Mix<float, 16>::NT : (W <= 32 ? Mix<float, 32>::NT : Mix<float, 64>::NT);
+}
 
 // Everything but the ring and the rows, at the start of the dynamic shared memory.
-template <int WF>
+template <typename R, int WF>
 struct MixSmem {
-  alignas(16) cxf z[2][2][2][WF];        // [chain][right-hand side][parity]: z of the current and next slice
-  alignas(16) cxf zm[2][2][WF];          // [chain][right-hand side]: the chain's part of the middle z
-  float wred[24 * 8];                    // per-warp partial sums
-  float slot[2][DY_MAXP * 8];            // [phase][rank]: the cluster's partial sums
+  alignas(16) cx<R> z[2][2][2][WF];      // [chain][right-hand side][parity]: z of the current and next slice
+  alignas(16) cx<R> zm[2][2][WF];        // [chain][right-hand side]: the chain's part of the middle z
+  R wred[24 * 8];                        // per-warp partial sums
+  R slot[2][DY_MAXP * 8];            // [phase][rank]: the cluster's partial sums
   alignas(8) uint64_t bars[2 * MIX_MAXS];
   int err;
 };
+template <typename R>
 __host__ __device__ constexpr size_t mix_head(int W) {
-  return ((W <= 16 ? sizeof(MixSmem<16>) : (W <= 32 ? sizeof(MixSmem<32>) : sizeof(MixSmem<64>))) + 127) & ~(size_t)127;
+  return ((W <= 16 ? sizeof(MixSmem<R, 16>) : (W <= 32 ? sizeof(MixSmem<R, 32>) : sizeof(MixSmem<R, 64>))) + 127) &
+         ~(size_t)127;
 }
 
 // Shared-memory plan: S ring slots of one block for each chain, and both row
 // buffers on chip or in the plan's scratch.  g.ring_S (slots of both chains)
 // and g.xm_rows come from the autotuner; 0: the heuristic, which keeps the
-// rows on chip when four slots a chain fit beside them.
+// rows on chip when four slots a chain (two in binary64) fit beside them.
 struct MixPlan {
   int S, rows;
   size_t smem;
 };
+template <typename R>
 __host__ __device__ inline size_t mix_smem(int W, int Lx, int S, int rows) {
-  return mix_head(W) + ((size_t)2 * S * W * W + (rows ? 2 * (size_t)Lx * W : 0)) * sizeof(cxf);
+  return mix_head<R>(W) + ((size_t)2 * S * W * W + (rows ? 2 * (size_t)Lx * W : 0)) * sizeof(cx<R>);
 }
+template <typename R>
 __host__ __device__ inline MixPlan mix_plan(const Geo& g) {
   MixPlan m;
   if (g.ring_S > 0) {
     m.S = g.ring_S / 2;
     m.rows = g.xm_rows > 0 ? 1 : 0;
   } else {
-    const size_t lim = g.W <= 32 ? MIX_SMEM_2 : MIX_SMEM_1;
-    m.rows = mix_smem(g.W, g.Lx, 4, 1) <= lim ? 1 : 0;
+    const size_t lim = g.W <= 32 && sizeof(R) == 4 ? MIX_SMEM_2 : MIX_SMEM_1;
+    m.rows = mix_smem<R>(g.W, g.Lx, sizeof(R) == 4 ? 4 : 2, 1) <= lim ? 1 : 0;
     m.S = 4;
-    while (m.S > 2 && mix_smem(g.W, g.Lx, m.S, m.rows) > lim) --m.S;
+    while (m.S > 2 && mix_smem<R>(g.W, g.Lx, m.S, m.rows) > lim) --m.S;
   }
-  m.smem = mix_smem(g.W, g.Lx, m.S, m.rows);
+  m.smem = mix_smem<R>(g.W, g.Lx, m.S, m.rows);
   return m;
 }
 // Configurations the autotuner times: slots a chain, rows on chip or not.
+template <typename R>
 inline int mix_candidates(const Geo& g, int* S, int* CR, int* ROWS, int max) {
   Geo h = g;
   h.ring_S = 0;
-  const MixPlan d = mix_plan(h);
+  const MixPlan d = mix_plan<R>(h);
   int n = 0;
   auto add = [&](int s, int rows) {
     for (int k = 0; k < n; ++k)
       if (S[k] == 2 * s && ROWS[k] == rows) return;
-    if (n < max && mix_smem(g.W, g.Lx, s, rows) <= MIX_SMEM_1) {
+    if (n < max && mix_smem<R>(g.W, g.Lx, s, rows) <= MIX_SMEM_1) {
       S[n] = 2 * s;
       CR[n] = g.W;
       ROWS[n] = rows;
@@ -109,14 +117,14 @@ inline int mix_candidates(const Geo& g, int* S, int* CR, int* ROWS, int max) {
 // The dynamic shared memory, named here so that every function (inlined or
 // not) addresses it as shared memory and not through generic pointers.
 extern __shared__ __align__(128) unsigned char mix_raw[];
-template <int WF>
-__device__ __forceinline__ MixSmem<WF>& mix_sm() {
-  return *reinterpret_cast<MixSmem<WF>*>(mix_raw);
+template <typename R, int WF>
+__device__ __forceinline__ MixSmem<R, WF>& mix_sm() {
+  return *reinterpret_cast<MixSmem<R, WF>*>(mix_raw);
 }
-template <int WF>
-__device__ __forceinline__ cxf* mix_ring() {
-  constexpr size_t head = (sizeof(MixSmem<WF>) + 127) & ~(size_t)127;
-  return reinterpret_cast<cxf*>(mix_raw + head);
+template <typename R, int WF>
+__device__ __forceinline__ cx<R>* mix_ring() {
+  constexpr size_t head = (sizeof(MixSmem<R, WF>) + 127) & ~(size_t)127;
+  return reinterpret_cast<cx<R>*>(mix_raw + head);
 }
 
 __device__ __forceinline__ void named_sync(int id, int threads) {
@@ -127,36 +135,37 @@ __device__ __forceinline__ void named_sync(int id, int threads) {
 // rest).  The addresses of the next copy and of the next wait are computed when
 // the previous one is done, off the chain's critical path: after a barrier the
 // producer only issues.
+template <typename R>
 struct MixState {
   int slot;                              // compute: slot of the next block to read; producer: next slot to fill
   int pos;                               // position of the next block to copy in the sweep's sequence
-  const cxf* src;                        // its address
+  const cx<R>* src;                      // its address
   int wslot;                             // slot of the next block to wait for
   uint32_t wph;
   bool dead;
 };
 
 // One CTA's constants and buffers.
-template <int WF, bool ROWS>
+template <typename R, int WF, bool ROWS>
 struct MixCtx {
   int W, Lx, S, m;
-  const cxf* src;                        // the subdomain's factors
-  cxf *g0, *g1;                          // row buffers in the scratch (ROWS = false)
+  const cx<R>* src;                        // the subdomain's factors
+  cx<R> *g0, *g1;                          // row buffers in the scratch (ROWS = false)
   unsigned long long* cnt;
-  float t;
+  R t;
 
-  __device__ __forceinline__ cxf* row(int k) const {
-    if constexpr (ROWS) return mix_ring<WF>() + 2 * S * W * W + (k ? Lx * W : 0);
+  __device__ __forceinline__ cx<R>* row(int k) const {
+    if constexpr (ROWS) return mix_ring<R, WF>() + 2 * S * W * W + (k ? Lx * W : 0);
     else return k ? g1 : g0;
   }
   __device__ __forceinline__ int blocks(int chain) const { return chain == 0 ? 2 * m + 1 : 2 * (Lx - 1 - m); }
   // The sequence of a chain's slices over one sweep: left 0 .. m, m-1 .. 0, right
   // Lx-1 .. m+1, m+1 .. Lx-1; the next sweep starts with the last one's last slice.
-  __device__ __forceinline__ const cxf* first(int chain) const { return src + (chain == 0 ? 0 : (size_t)(Lx - 1) * W * W); }
-  __device__ __forceinline__ void issue(int chain, MixState& st) const {
-    MixSmem<WF>& sm = mix_sm<WF>();
+  __device__ __forceinline__ const cx<R>* first(int chain) const { return src + (chain == 0 ? 0 : (size_t)(Lx - 1) * W * W); }
+  __device__ __forceinline__ void issue(int chain, MixState<R>& st) const {
+    MixSmem<R, WF>& sm = mix_sm<R, WF>();
     const int n = W * W;
-    bulk_load(mix_ring<WF>() + (chain * S + st.slot) * n, st.src, (uint32_t)(n * sizeof(cxf)),
+    bulk_load(mix_ring<R, WF>() + (chain * S + st.slot) * n, st.src, (uint32_t)(n * sizeof(cx<R>)),
               sm.bars + chain * MIX_MAXS + st.slot);
     if (++st.slot == S) st.slot = 0;
     const int up = chain == 0 ? m : Lx - 2 - m, last = blocks(chain) - 1;   // the turn: left at m, right repeats m+1
@@ -165,8 +174,8 @@ struct MixCtx {
     st.src += st.pos < up ? dn : (st.pos < up + turn || st.pos == last ? 0 : -dn);
     st.pos = st.pos == last ? 0 : st.pos + 1;
   }
-  __device__ __forceinline__ void wait(int chain, MixState& st) const {
-    MixSmem<WF>& sm = mix_sm<WF>();
+  __device__ __forceinline__ void wait(int chain, MixState<R>& st) const {
+    MixSmem<R, WF>& sm = mix_sm<R, WF>();
     ring_wait(sm.bars + chain * MIX_MAXS + st.wslot, st.wph, st.dead, &sm.err);
     if (++st.wslot == S) {
       st.wslot = 0;
@@ -175,39 +184,39 @@ struct MixCtx {
   }
 };
 
-template <int WF, bool ROWS>
-__device__ void mix_init(const MixCtx<WF, ROWS>& cx, MixState& st) {
-  MixSmem<WF>& sm = mix_sm<WF>();
+template <typename R, int WF, bool ROWS>
+__device__ void mix_init(const MixCtx<R, WF, ROWS>& ctx, MixState<R>& st) {
+  MixSmem<R, WF>& sm = mix_sm<R, WF>();
   const int tid = threadIdx.x, wid = tid >> 5;
   st.slot = st.pos = st.wslot = 0;
-  st.src = cx.first(wid == Mix<WF>::PROD + 1 ? 1 : 0);
+  st.src = ctx.first(wid == Mix<R, WF>::PROD + 1 ? 1 : 0);
   st.wph = 0;
   st.dead = false;
-  for (int e = tid; e < 8 * WF; e += Mix<WF>::NT) (&sm.z[0][0][0][0])[e] = cxf{0.f, 0.f};
-  for (int e = tid; e < 4 * WF; e += Mix<WF>::NT) (&sm.zm[0][0][0])[e] = cxf{0.f, 0.f};
+  for (int e = tid; e < 8 * WF; e += Mix<R, WF>::NT) (&sm.z[0][0][0][0])[e] = cx<R>{0, 0};
+  for (int e = tid; e < 4 * WF; e += Mix<R, WF>::NT) (&sm.zm[0][0][0])[e] = cx<R>{0, 0};
   if (tid == 0) {
     for (int k = 0; k < 2 * MIX_MAXS; ++k) mbar_init(sm.bars + k, 1);
     sm.err = 0;
     fence_mbar_init();
   }
   __syncthreads();
-  const int c = wid - Mix<WF>::PROD;
-  if ((c == 0 || c == 1) && (tid & 31) == 0 && cx.blocks(c) > 0)
-    for (int k = 0; k < cx.S; ++k) cx.issue(c, st);
+  const int c = wid - Mix<R, WF>::PROD;
+  if ((c == 0 || c == 1) && (tid & 31) == 0 && ctx.blocks(c) > 0)
+    for (int k = 0; k < ctx.S; ++k) ctx.issue(c, st);
 }
 // Before the kernel ends: the S copies of each chain issued beyond its last
 // step have landed (bounded waits, also after an earlier wait ran out; the
 // first that runs out ends it).
-template <int WF, bool ROWS>
-__device__ void mix_drain(const MixCtx<WF, ROWS>& cx, MixState& st) {
-  const int c = ((int)threadIdx.x >> 5) - Mix<WF>::PROD;
-  if ((c == 0 || c == 1) && (threadIdx.x & 31) == 0 && cx.blocks(c) > 0)
-    for (int k = 0; k < cx.S; ++k) {
-      if (!mbar_wait(mix_sm<WF>().bars + c * MIX_MAXS + st.wslot, st.wph)) {
-        mix_sm<WF>().err = 1;
+template <typename R, int WF, bool ROWS>
+__device__ void mix_drain(const MixCtx<R, WF, ROWS>& ctx, MixState<R>& st) {
+  const int c = ((int)threadIdx.x >> 5) - Mix<R, WF>::PROD;
+  if ((c == 0 || c == 1) && (threadIdx.x & 31) == 0 && ctx.blocks(c) > 0)
+    for (int k = 0; k < ctx.S; ++k) {
+      if (!mbar_wait(mix_sm<R, WF>().bars + c * MIX_MAXS + st.wslot, st.wph)) {
+        mix_sm<R, WF>().err = 1;
         break;
       }
-      if (++st.wslot == cx.S) {
+      if (++st.wslot == ctx.S) {
         st.wslot = 0;
         st.wph ^= 1u;
       }
@@ -229,58 +238,69 @@ __device__ void mix_drain(const MixCtx<WF, ROWS>& cx, MixState& st) {
 // buffer in the scratch), and a step's row is stored during the next step,
 // behind that step's loads of z.  Every warp of the CTA calls it; the rows are
 // complete and visible to the CTA on return.
-template <int WF, int NR, bool ROWS>
-__device__ __noinline__ void mix_sweep(const MixCtx<WF, ROWS>& ctx, MixState& state, int k0) {
-  constexpr int CT = Mix<WF>::CT, PF = NR == 1 && !ROWS ? 4 : 2, KP = Mix<WF>::KP, WARPS = Mix<WF>::WARPS;
+template <typename R, int WF, int NR, bool ROWS>
+__device__ __noinline__ void mix_sweep(const MixCtx<R, WF, ROWS>& ctx, MixState<R>& state, int k0) {
+  constexpr int CT = Mix<R, WF>::CT, PF = NR == 1 && !ROWS ? 4 : 2, KP = Mix<R, WF>::KP, WARPS = Mix<R, WF>::WARPS;
   constexpr int KH = KP < 4 ? KP : 4;    // column pairs handled at a time
-  MixSmem<WF>& sm = mix_sm<WF>();
-  const MixCtx<WF, ROWS> cx = ctx;
-  MixState st = state;
-  const int W = cx.W, Lx = cx.Lx, m = cx.m, qR = Lx - 1 - m;
+  using C = cx<R>;
+  using U = std::conditional_t<sizeof(R) == 4, float4, double2>;   // a 16-byte word: CU columns
+  constexpr int CU = Mix<R, WF>::CU;
+  MixSmem<R, WF>& sm = mix_sm<R, WF>();
+  const MixCtx<R, WF, ROWS> cx_ = ctx;
+  MixState<R> st = state;
+  const int W = cx_.W, Lx = cx_.Lx, m = cx_.m, qR = Lx - 1 - m;
   const int wid = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
   const int role = wid < 2 * WARPS ? 0 : (wid < 2 * WARPS + 2 ? 1 : 2);
-  const int c = role == 0 ? wid / WARPS : (role == 1 ? wid - Mix<WF>::PROD : 0);
-  const int NL = cx.blocks(c), steps = c == 0 ? m : qR;
-  const float t = cx.t;
+  const int c = role == 0 ? wid / WARPS : (role == 1 ? wid - Mix<R, WF>::PROD : 0);
+  const int NL = cx_.blocks(c), steps = c == 0 ? m : qR;
+  const R t = cx_.t;
   const int cg = lane >> 3, row = (wid % WARPS) * 8 + (lane & 7);
   const bool own = role == 0 && cg == 0 && row < W;
-  const int off0 = cg * W + (row < W ? row : 0), W4 = 4 * W, WW2 = W * W / 2;
-  const int km = W / 2 > cg ? (W / 2 - cg + 3) / 4 : 0;
-  const float4* ring4 = reinterpret_cast<const float4*>(mix_ring<WF>()) + (size_t)c * cx.S * WW2 + off0;
-  cxf* yb[2] = {cx.row(NR == 1 ? k0 : 0), cx.row(1)};
-  float4 gb[KP];
+  const int off0 = cg * W + (row < W ? row : 0), W4 = 4 * W, WW2 = W * W / CU;
+  const int wu = W / CU, km = wu > cg ? (wu - cg + 3) / 4 : 0;
+  const U* ring4 = reinterpret_cast<const U*>(mix_ring<R, WF>()) + (size_t)c * cx_.S * WW2 + off0;
+  C* yb[2] = {cx_.row(NR == 1 ? k0 : 0), cx_.row(1)};
+  U gb[KP];
   auto load = [&]() {
-    const float4* p = ring4 + st.slot * WW2;
+    const U* p = ring4 + st.slot * WW2;
 #pragma unroll
-    for (int q = 0; q < KP; ++q) gb[q] = q < km ? p[q * W4] : make_float4(0.f, 0.f, 0.f, 0.f);
-    if (++st.slot == cx.S) st.slot = 0;
+    for (int q = 0; q < KP; ++q) gb[q] = q < km ? p[q * W4] : U{};
+    if (++st.slot == cx_.S) st.slot = 0;
   };
-  auto load_z = [&](const cxf* z, int h, float4 (&zv)[KH]) {
-    const float4* z4 = reinterpret_cast<const float4*>(z) + cg + 16 * h;
+  auto load_z = [&](const C* z, int h, U (&zv)[KH]) {
+    const U* z4 = reinterpret_cast<const U*>(z) + cg + 16 * h;
 #pragma unroll
     for (int q = 0; q < KH; ++q) zv[q] = z4[4 * q];
   };
   // this lane's part of (block row) . z, the first KH pairs of z already in zv
-  auto part = [&](const cxf* z, float4 (&zv)[KH]) -> cxf {
+  auto part = [&](const C* z, U (&zv)[KH]) -> C {
     constexpr int NA = KP >= 4 ? 4 : 2;
-    cxf a[NA];
+    C a[NA];
 #pragma unroll
-    for (int q = 0; q < NA; ++q) a[q] = cxf{0.f, 0.f};
+    for (int q = 0; q < NA; ++q) a[q] = C{0, 0};
 #pragma unroll
     for (int h = 0; h < KP / KH; ++h) {
       if (h > 0) load_z(z, h, zv);
 #pragma unroll
       for (int q = 0; q < KH; ++q) {
-        const float4 gv = gb[h * KH + q];
-        a[(2 * q) % NA] = cfma(cxf{gv.x, gv.y}, cxf{zv[q].x, zv[q].y}, a[(2 * q) % NA]);
-        a[(2 * q + 1) % NA] = cfma(cxf{gv.z, gv.w}, cxf{zv[q].z, zv[q].w}, a[(2 * q + 1) % NA]);
+        const U gv = gb[h * KH + q];
+        a[(CU * q) % NA] = cfma(C{gv.x, gv.y}, C{zv[q].x, zv[q].y}, a[(CU * q) % NA]);
+        if constexpr (CU == 2) a[(2 * q + 1) % NA] = cfma(C{gv.z, gv.w}, C{zv[q].z, zv[q].w}, a[(2 * q + 1) % NA]);
       }
     }
-    cxf s = a[0] + a[1];
+    C s = a[0] + a[1];
     if constexpr (NA == 4) s = s + (a[2] + a[3]);
     return s;
   };
-  auto total = [&](cxf v) -> cxf {                       // over the row's four lanes
+  auto total = [&](C v) -> C {                           // over the row's four lanes
+    if constexpr (sizeof(R) == 8) {      // one part a lane of a pair: two binary64 sums instead of four
+      const bool odd = cg & 1;
+      R a = odd ? v.y : v.x;
+      a += __shfl_xor_sync(0xffffffffu, odd ? v.x : v.y, 8);
+      a += __shfl_xor_sync(0xffffffffu, a, 16);
+      const R o = __shfl_xor_sync(0xffffffffu, a, 8);
+      return odd ? C{o, a} : C{a, o};
+    }
     v.x += __shfl_xor_sync(0xffffffffu, v.x, 8);
     v.y += __shfl_xor_sync(0xffffffffu, v.y, 8);
     v.x += __shfl_xor_sync(0xffffffffu, v.x, 16);
@@ -288,8 +308,8 @@ __device__ __noinline__ void mix_sweep(const MixCtx<WF, ROWS>& ctx, MixState& st
     return v;
   };
   if (role == 1 && lane == 0) {
-    if (NL > 0) cx.wait(c, st);          // blocks 0 and 1
-    if (NL > 1) cx.wait(c, st);
+    if (NL > 0) cx_.wait(c, st);          // blocks 0 and 1
+    if (NL > 1) cx_.wait(c, st);
   }
   __syncthreads();                       // the rows are written; earlier readers of z are done
   if (role == 0) {
@@ -297,7 +317,7 @@ __device__ __noinline__ void mix_sweep(const MixCtx<WF, ROWS>& ctx, MixState& st
 #pragma unroll
       for (int r = 0; r < NR; ++r) {
         if (steps > 0) sm.z[c][r][0][row] = yb[r][(c == 0 ? 0 : Lx - 1) * W + row];
-        else sm.zm[c][r][row] = c == 0 ? yb[r][row] : cxf{0.f, 0.f};
+        else sm.zm[c][r][row] = c == 0 ? yb[r][row] : cx<R>{0, 0};
       }
     }
     if (NL > 0) load();
@@ -306,26 +326,26 @@ __device__ __noinline__ void mix_sweep(const MixCtx<WF, ROWS>& ctx, MixState& st
     const int d = c == 0 ? W : -W;       // row step
     int o = (c == 0 ? 0 : (Lx - 1) * W) + row;           // this step's row entry
     const int nf = c == 0 ? steps : steps - 1;           // steps whose next z has a right-hand side
-    cxf f[NR][PF], yp[NR];
+    C f[NR][PF], yp[NR];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-      yp[r] = cxf{0.f, 0.f};
+      yp[r] = cx<R>{0, 0};
 #pragma unroll
-      for (int u = 0; u < PF; ++u) f[r][u] = own && u < nf ? yb[r][o + d * (u + 1)] : cxf{0.f, 0.f};
+      for (int u = 0; u < PF; ++u) f[r][u] = own && u < nf ? yb[r][o + d * (u + 1)] : cx<R>{0, 0};
     }
     for (int n0 = 0; n0 < steps; n0 += PF) {
 #pragma unroll
       for (int u = 0; u < PF; ++u) {
         const int n = n0 + u;
         if (n < steps) {
-          cxf y[NR];
-          float4 zv[KH];
+          C y[NR];
+          U zv[KH];
           load_z(sm.z[c][0][u & 1], 0, zv);
           if (own && n > 0) {            // row n - 1 out, its slot of f refilled
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
               yb[r][o - d] = yp[r];
-              f[r][(u + PF - 1) % PF] = n - 1 + PF < nf ? yb[r][o + d * PF] : cxf{0.f, 0.f};
+              f[r][(u + PF - 1) % PF] = n - 1 + PF < nf ? yb[r][o + d * PF] : cx<R>{0, 0};
             }
           }
           y[0] = part(sm.z[c][0][u & 1], zv);
@@ -338,7 +358,7 @@ __device__ __noinline__ void mix_sweep(const MixCtx<WF, ROWS>& ctx, MixState& st
           for (int r = 0; r < NR; ++r) {
             y[r] = total(y[r]);
             if (own) {
-              cxf* zn = n + 1 < steps ? sm.z[c][r][(u + 1) & 1] : sm.zm[c][r];
+              C* zn = n + 1 < steps ? sm.z[c][r][(u + 1) & 1] : sm.zm[c][r];
               zn[row] = f[r][u] - t * y[r];
             }
             yp[r] = y[r];
@@ -354,12 +374,12 @@ __device__ __noinline__ void mix_sweep(const MixCtx<WF, ROWS>& ctx, MixState& st
     }
   } else if (role == 1) {
     named_sync(3 + c, CT + 32);          // block 0 has been read
-    if (lane == 0 && NL > 0) cx.issue(c, st);
+    if (lane == 0 && NL > 0) cx_.issue(c, st);
     for (int n = 0; n < steps; ++n) {
-      if (lane == 0 && n + 2 < NL) cx.wait(c, st);
+      if (lane == 0 && n + 2 < NL) cx_.wait(c, st);
       __syncwarp();
       named_sync(1 + c, CT + 32);        // block n + 1 has been read
-      if (lane == 0 && n + 1 < NL) cx.issue(c, st);
+      if (lane == 0 && n + 1 < NL) cx_.issue(c, st);
     }
   }
   __syncthreads();                       // both parts of the middle z are written
@@ -369,10 +389,10 @@ __device__ __noinline__ void mix_sweep(const MixCtx<WF, ROWS>& ctx, MixState& st
       for (int r = 0; r < NR; ++r) sm.z[0][r][1][row] = sm.zm[0][r][row] + sm.zm[1][r][row];
     }
     named_sync(3, CT);
-    cxf x[NR];
+    C x[NR];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-      float4 zv[KH];
+      U zv[KH];
       load_z(sm.z[0][r][1], 0, zv);
       x[r] = part(sm.z[0][r][1], zv);
     }
@@ -387,35 +407,35 @@ __device__ __noinline__ void mix_sweep(const MixCtx<WF, ROWS>& ctx, MixState& st
       }
     }
   } else if (c == 0 && role == 1 && lane == 0 && m + 2 < NL) {
-    cx.wait(c, st);
+    cx_.wait(c, st);
   }
   __syncthreads();                       // x_m is visible to both chains
-  if (c == 0 && role == 1 && lane == 0 && m + 1 < NL) cx.issue(c, st);
+  if (c == 0 && role == 1 && lane == 0 && m + 1 < NL) cx_.issue(c, st);
   const int n1 = c == 0 ? m + 1 : qR;
   if (role == 0) {
     // ---- back from the middle: step k is slice m -+ (k + 1)
     const int d = c == 0 ? -W : W;
     int o = (c == 0 ? m - 1 : m + 1) * W + row;
-    cxf f[NR][PF], xp[NR];
+    C f[NR][PF], xp[NR];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-      xp[r] = cxf{0.f, 0.f};
+      xp[r] = cx<R>{0, 0};
 #pragma unroll
-      for (int u = 0; u < PF; ++u) f[r][u] = own && u < steps ? yb[r][o + d * u] : cxf{0.f, 0.f};
+      for (int u = 0; u < PF; ++u) f[r][u] = own && u < steps ? yb[r][o + d * u] : cx<R>{0, 0};
     }
     for (int kb = 0; kb < steps; kb += PF) {
 #pragma unroll
       for (int u = 0; u < PF; ++u) {
         const int k = kb + u;
         if (k < steps) {
-          cxf y[NR];
-          float4 zv[KH];
+          C y[NR];
+          U zv[KH];
           load_z(sm.z[c][0][u & 1], 0, zv);
           if (own && k > 0) {
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
               yb[r][o - d] = xp[r];
-              f[r][(u + PF - 1) % PF] = k - 1 + PF < steps ? yb[r][o + d * (PF - 1)] : cxf{0.f, 0.f};
+              f[r][(u + PF - 1) % PF] = k - 1 + PF < steps ? yb[r][o + d * (PF - 1)] : cx<R>{0, 0};
             }
           }
           y[0] = part(sm.z[c][0][u & 1], zv);
@@ -442,28 +462,28 @@ __device__ __noinline__ void mix_sweep(const MixCtx<WF, ROWS>& ctx, MixState& st
   } else if (role == 1) {
     for (int k = 0; k < steps; ++k) {
       const int n = n1 + k;
-      if (lane == 0 && n + 2 < NL) cx.wait(c, st);
+      if (lane == 0 && n + 2 < NL) cx_.wait(c, st);
       __syncwarp();
       named_sync(1 + c, CT + 32);
-      if (lane == 0 && n + 1 < NL) cx.issue(c, st);
+      if (lane == 0 && n + 1 < NL) cx_.issue(c, st);
     }
   }
   __syncthreads();
   state = st;
-  if (threadIdx.x == 0 && cx.cnt) *cx.cnt += 1;
+  if (threadIdx.x == 0 && cx_.cnt) *cx_.cnt += 1;
 }
 
 // ---------------------------------------------------------------- reductions
-// Cluster-wide sums of NV binary32 values (every thread gets them), and this
+// Cluster-wide sums of NV values of R (every thread gets them), and this
 // CTA's own totals in loc if not null.  Warp totals, their sum by warp 0, which
 // puts it into every CTA's slot for this rank; after the cluster barrier each
 // warp adds the ranks' slots by the same tree, so all threads of the cluster
 // hold the same bits.  `phase` alternates two slot sets.
-template <int WF, int NV>
-__device__ __forceinline__ void mix_sum(cg::cluster_group& cl, int& phase, int p, float (&v)[NV], float* loc = nullptr) {
-  MixSmem<WF>& sm = mix_sm<WF>();
+template <typename R, int WF, int NV>
+__device__ __forceinline__ void mix_sum(cg::cluster_group& cl, int& phase, int p, R (&v)[NV], R* loc = nullptr) {
+  MixSmem<R, WF>& sm = mix_sm<R, WF>();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  constexpr int NW = Mix<WF>::NT / 32;
+  constexpr int NW = Mix<R, WF>::NT / 32;
   const int me = (int)cl.block_rank();
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
@@ -475,22 +495,22 @@ __device__ __forceinline__ void mix_sum(cg::cluster_group& cl, int& phase, int p
   }
   __syncthreads();
   if (wid == 0) {
-    float s[NV];
+    R s[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) s[k] = lane < NW ? sm.wred[lane * 8 + k] : 0.f;
+    for (int k = 0; k < NV; ++k) s[k] = lane < NW ? sm.wred[lane * 8 + k] : R(0);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
       for (int k = 0; k < NV; ++k) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
     if (lane < p) {
-      float* rem = cl.map_shared_rank(&sm.slot[phase][me * 8], lane);
+      R* rem = cl.map_shared_rank(&sm.slot[phase][me * 8], lane);
 #pragma unroll
       for (int k = 0; k < NV; ++k) rem[k] = s[k];
     }
   }
   cl.sync();
 #pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = lane < p ? sm.slot[phase][lane * 8 + k] : 0.f;
+  for (int k = 0; k < NV; ++k) v[k] = lane < p ? sm.slot[phase][lane * 8 + k] : R(0);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -567,9 +587,10 @@ __device__ __forceinline__ cxf scaled(float s, const cdfl& a) { return {s * (a.x
 __device__ __forceinline__ dfl dfl_of(double v) { return d2dfl_bits(v); }
 
 // ---------------------------------------------------------------- interface solve
+template <typename R>
 struct MixSolve {
   bool useB0;                            // the subdomain part is B0 - alpha B1 (else - alpha B1)
-  cxf alpha;
+  cx<R> alpha;
   int iters, conv;
 };
 
@@ -578,44 +599,45 @@ struct MixSolve {
 // as B0 - alpha B1: each iteration but the last is folded into B0, the last one
 // is the caller's.  keep0: B0 holds a vector to add to (else it counts as zero).
 // IF_B is complete (a barrier after its writers) on entry.
-template <int WF, bool ROWS>
-__device__ __noinline__ MixSolve mix_cocg(const Geo& g, const Bufs& b, const MixCtx<WF, ROWS>& cx, MixState& st,
+template <typename R, int WF, bool ROWS>
+__device__ __noinline__ MixSolve<R> mix_cocg(const Geo& g, const Bufs& b, const MixCtx<R, WF, ROWS>& ctx, MixState<R>& st,
                                           int& phase_, int vs, bool keep0) {
+  using C = cx<R>;
   cg::cluster_group cl = cg::this_cluster();
   int phase = phase_;
-  constexpr int nt = Mix<WF>::NT;
-  const int i = blockIdx.x, A = g.A, p = g.p, W = cx.W, Lx = cx.Lx, T = g.T, w = T * g.h[i], nsub = Lx * W;
+  constexpr int nt = Mix<R, WF>::NT;
+  const int i = blockIdx.x, A = g.A, p = g.p, W = ctx.W, Lx = ctx.Lx, T = g.T, w = T * g.h[i], nsub = Lx * W;
   const int ds = nt / W, dj = nt % W;
   const bool has = i < p - 1;
-  cxf* B0 = cx.row(0);
-  cxf* B1 = cx.row(1);
+  C* B0 = ctx.row(0);
+  C* B1 = ctx.row(1);
   const size_t o = (size_t)i * A;
-  cxf* X = ifv_ptr<float>(g, b, vs, IF_X) + o;
-  cxf* Rv = ifv_ptr<float>(g, b, vs, IF_R) + o;
-  cxf* Z = ifv_ptr<float>(g, b, vs, IF_Z) + o;
-  cxf* P = ifv_ptr<float>(g, b, vs, IF_P);
-  cxf* SP = ifv_ptr<float>(g, b, vs, IF_SP) + o;
-  const cxf* Bv = ifv_ptr<float>(g, b, vs, IF_B) + o;
-  const cxf* dC = ifv_ptr<float>(g, b, vs, IF_D) + o;
-  cxf* blo = bnd_ptr<float>(g, b, vs, i, 0);
-  cxf* bhi = bnd_ptr<float>(g, b, vs, i, 1);
-  const cxf* bnx = has ? bnd_ptr<float>(g, b, vs, i + 1, 0) : nullptr;
-  const cxf* plo = i > 0 ? P + o - A : nullptr;
-  cxf* phi = P + o;
-  const float t = cx.t;
-  auto precond = [&](const cxf* r, cxf* z) {
-    if (g.lpre) lpre_apply<float>(g, b, vs, i, r, z, B1);
-    else precond_apply<float>(g, b, vs, i, r, z);
+  C* X = ifv_ptr<R>(g, b, vs, IF_X) + o;
+  C* Rv = ifv_ptr<R>(g, b, vs, IF_R) + o;
+  C* Z = ifv_ptr<R>(g, b, vs, IF_Z) + o;
+  C* P = ifv_ptr<R>(g, b, vs, IF_P);
+  C* SP = ifv_ptr<R>(g, b, vs, IF_SP) + o;
+  const C* Bv = ifv_ptr<R>(g, b, vs, IF_B) + o;
+  const C* dC = ifv_ptr<R>(g, b, vs, IF_D) + o;
+  C* blo = bnd_ptr<R>(g, b, vs, i, 0);
+  C* bhi = bnd_ptr<R>(g, b, vs, i, 1);
+  const C* bnx = has ? bnd_ptr<R>(g, b, vs, i + 1, 0) : nullptr;
+  const C* plo = i > 0 ? P + o - A : nullptr;
+  C* phi = P + o;
+  const R t = ctx.t;
+  auto precond = [&](const C* r, C* z) {
+    if (g.lpre) lpre_apply<R>(g, b, vs, i, r, z, B1);
+    else precond_apply<R>(g, b, vs, i, r, z);
   };
-  MixSolve out = {keep0, {0.f, 0.f}, 0, 1};
+  MixSolve<R> out = {keep0, {0, 0}, 0, 1};
   if (has) precond(Bv, Z);
   __syncthreads();
-  float v3[3] = {0.f, 0.f, 0.f};
+  R v3[3] = {0, 0, 0};
   if (has) {
-    cxf rz = {0.f, 0.f};
+    C rz = {0, 0};
     for (int a = threadIdx.x; a < A; a += nt) {
-      const cxf zz = Z[a], r = Bv[a];
-      X[a] = cxf{0.f, 0.f};
+      const C zz = Z[a], r = Bv[a];
+      X[a] = C{0, 0};
       Rv[a] = r;
       phi[a] = zz;
       rz = cfma(r, zz, rz);
@@ -624,11 +646,11 @@ __device__ __noinline__ MixSolve mix_cocg(const Geo& g, const Bufs& b, const Mix
     v3[0] = rz.x;
     v3[1] = rz.y;
   }
-  mix_sum<WF, 3>(cl, phase, p, v3);      // also: P of the neighbour layers is final
-  cxf rho = {v3[0], v3[1]};
-  const float bn = v3[2];
-  const float tol2 = (float)(g.krylov_tol * g.krylov_tol);
-  if (bn > 0.f || bn != bn) {
+  mix_sum<R, WF, 3>(cl, phase, p, v3);      // also: P of the neighbour layers is final
+  C rho = {v3[0], v3[1]};
+  const R bn = v3[2];
+  const R tol2 = (R)(g.krylov_tol * g.krylov_tol);
+  if (bn > 0 || bn != bn) {
     for (;;) {
       if (out.iters >= g.krylov_maxit) {
         out.conv = 0;
@@ -638,22 +660,22 @@ __device__ __noinline__ MixSolve mix_cocg(const Geo& g, const Bufs& b, const Mix
         // fold the last product into B0, then the next direction
         const bool z0 = !out.useB0;
         for (int e = threadIdx.x; e < nsub; e += nt) {
-          const cxf q = out.alpha * B1[e];
+          const C q = out.alpha * B1[e];
           B0[e] = z0 ? -q : B0[e] - q;
         }
         out.useB0 = true;
         __syncthreads();                 // B1 is free (the preconditioner's scratch)
         if (has) precond(Rv, Z);
         __syncthreads();
-        float v2[2] = {0.f, 0.f};
+        R v2[2] = {0, 0};
         if (has) {
-          cxf rz = {0.f, 0.f};
+          C rz = {0, 0};
           for (int a = threadIdx.x; a < A; a += nt) rz = cfma(Rv[a], Z[a], rz);
           v2[0] = rz.x;
           v2[1] = rz.y;
         }
-        mix_sum<WF, 2>(cl, phase, p, v2);
-        const cxf rn = {v2[0], v2[1]}, beta = cdiv(rn, rho);
+        mix_sum<R, WF, 2>(cl, phase, p, v2);
+        const C rn = {v2[0], v2[1]}, beta = cdiv(rn, rho);
         rho = rn;
         if (has)
           for (int a = threadIdx.x; a < A; a += nt) phi[a] = Z[a] + beta * phi[a];
@@ -662,7 +684,7 @@ __device__ __noinline__ MixSolve mix_cocg(const Geo& g, const Bufs& b, const Mix
       ++out.iters;
       // B1 = E p
       for (int e = threadIdx.x, s = e / W, j = e - s * W; e < nsub; e += nt) {
-        cxf u = {0.f, 0.f};
+        C u = {0, 0};
         if (plo && j < T) u = u + t * plo[s + Lx * j];
         if (has && j >= w - T && j < w) u = u + t * phi[s + Lx * (j - (w - T))];
         B1[e] = u;
@@ -673,36 +695,36 @@ __device__ __noinline__ MixSolve mix_cocg(const Geo& g, const Bufs& b, const Mix
           ++s;
         }
       }
-      mix_sweep<WF, 1, ROWS>(cx, st, 1);
+      mix_sweep<R, WF, 1, ROWS>(ctx, st, 1);
       for (int e = threadIdx.x; e < A; e += nt) {
         const int j = T == 1 ? 0 : e / Lx, s = e - j * Lx;
         blo[e] = B1[s * W + j];
         bhi[e] = B1[s * W + (w - T) + j];
       }
       cl.sync();                         // boundary rows of every subdomain written
-      float v2[2] = {0.f, 0.f};
+      R v2[2] = {0, 0};
       if (has) {
-        cxf ps = {0.f, 0.f};
+        C ps = {0, 0};
         for (int a = threadIdx.x; a < A; a += nt) {
-          const cxf sp = layer_C_apply<float>(g, dC, phi, a) - t * (bhi[a] + bnx[a]);
+          const C sp = layer_C_apply<R>(g, dC, phi, a) - t * (bhi[a] + bnx[a]);
           SP[a] = sp;
           ps = cfma(phi[a], sp, ps);
         }
         v2[0] = ps.x;
         v2[1] = ps.y;
       }
-      mix_sum<WF, 2>(cl, phase, p, v2);
-      out.alpha = cdiv(rho, cxf{v2[0], v2[1]});
-      float v1[1] = {0.f};
+      mix_sum<R, WF, 2>(cl, phase, p, v2);
+      out.alpha = cdiv(rho, C{v2[0], v2[1]});
+      R v1[1] = {0};
       if (has) {
         for (int a = threadIdx.x; a < A; a += nt) {
           X[a] = X[a] + out.alpha * phi[a];
-          const cxf r = Rv[a] - out.alpha * SP[a];
+          const C r = Rv[a] - out.alpha * SP[a];
           Rv[a] = r;
           v1[0] += cabs2(r);
         }
       }
-      mix_sum<WF, 1>(cl, phase, p, v1);
+      mix_sum<R, WF, 1>(cl, phase, p, v1);
       if (v1[0] <= tol2 * bn) break;
     }
   }
@@ -724,10 +746,10 @@ __device__ __noinline__ MixSolve mix_cocg(const Geo& g, const Bufs& b, const Mix
 // what a complex64 correction leaves); the scale only keeps the values inside
 // the binary32 range, and the norms are measured on the scaled rows.
 template <int WF, bool ROWS>
-__global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
+__global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
     k_xmatvec_m(const __grid_constant__ Geo g, const __grid_constant__ Bufs b, int j, int ncols) {
   cg::cluster_group cl = cg::this_cluster();
-  constexpr int nt = Mix<WF>::NT;
+  constexpr int nt = Mix<float, WF>::NT;
   const int i = blockIdx.x, vs = blockIdx.y, p = g.p, A = g.A, W = g.W, Lx = g.Lx, T = g.T;
   const int f = slot_freq(g, vs), c = vs - f * g.nb;
   if (c >= ncols) return;                  // same values in every CTA of the cluster
@@ -736,18 +758,18 @@ __global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
   const size_t Ndd = g.Ndd;
   const int nsub = Lx * W, w = T * g.h[i], hh = g.h[i], tid = threadIdx.x;
   const int ds = nt / W, dj = nt % W, s_0 = tid / W, j_0 = tid - s_0 * W;
-  MixCtx<WF, ROWS> cx;
+  MixCtx<float, WF, ROWS> cx;
   cx.W = W;
   cx.Lx = Lx;
-  cx.S = mix_plan(g).S;
+  cx.S = mix_plan<float>(g).S;
   cx.m = Lx / 2;
   cx.src = reinterpret_cast<const cxf*>(b.g) + ((size_t)f * p + i) * (size_t)nsub * W;
   cx.g0 = reinterpret_cast<cxf*>(b.yscr) + ((size_t)vs * p + i) * nsub;
   cx.g1 = reinterpret_cast<cxf*>(b.v2 + (size_t)vs * Ndd + (size_t)i * nsub);
   cx.cnt = sweep_cnt(g, b, vs, i);
   cx.t = (float)g.t;
-  MixState ms;
-  mix_init<WF, ROWS>(cx, ms);
+  MixState<float> ms;
+  mix_init<float, WF, ROWS>(cx, ms);
   int phase = 0;
   cxf* B0 = cx.row(0);
   cxf* B1 = cx.row(1);
@@ -790,7 +812,7 @@ __global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
       const cdfl d = hd[lo + a];
       dC[a] = cxf{d.x.hi, d.y.hi};
     }
-  mix_sweep<WF, 1, ROWS>(cx, ms, 0);
+  mix_sweep<float, WF, 1, ROWS>(cx, ms, 0);
   for (int e = tid; e < nsub; e += nt) ws[e] = from_f(B0[e]);      // zero on the padding
   for (int e = tid; e < A; e += nt) {
     const int jj = T == 1 ? 0 : e / Lx, s = e - jj * Lx;
@@ -811,7 +833,7 @@ __global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
         h3.add(cxf{h.x.hi, h.y.hi});
       }
     float v[6] = {h3.m, h3.s, h3.b, qn.m, qn.s, qn.b}, own[6];
-    mix_sum<WF, 6>(cl, phase, p, v, own);
+    mix_sum<float, WF, 6>(cl, phase, p, v, own);
     hn2 = Norm3::value(v[0], v[1], v[2]);
     qn2 = Norm3::value(own[3], own[4], own[5]);
   }
@@ -823,7 +845,7 @@ __global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
     if (has)
       for (int a = tid; a < A; a += nt) Bv[a] = scaled(ihf, rc[a]);
     __syncthreads();
-    const MixSolve sv = mix_cocg<WF, ROWS>(g, b, cx, ms, phase, vs, false);
+    const MixSolve<float> sv = mix_cocg<float, WF, ROWS>(g, b, cx, ms, phase, vs, false);
     iters += sv.iters;
     conv_all &= sv.conv;
     ++solves;
@@ -928,7 +950,7 @@ __global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
         v[1] += cabs2(hsc);
       }
     }
-    mix_sum<WF, 3>(cl, phase, p, v, own);
+    mix_sum<float, WF, 3>(cl, phase, p, v, own);
     const double wn = (double)own[2] / (sw * sw);   // this subdomain's, which decides for its w alone
     if (!wdone && (wn <= tol2 * qn2 || wn > REFINE_STALL * prev_w)) wdone = true;
     if (!wdone) prev_w = wn;
@@ -937,15 +959,15 @@ __global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
     if (udone) {
       // u is done: go on only if some w of the cluster is not
       float go[1] = {!wdone && tid == 0 ? 1.f : 0.f};
-      mix_sum<WF, 1>(cl, phase, p, go);
+      mix_sum<float, WF, 1>(cl, phase, p, go);
       if (go[0] == 0.f) break;
     }
     prev_u = rn;
     ++refines;
     // ---- z = B^-1 r_u in B0, d_w = B^-1 r_w in B1
     const bool wgo = !wdone;
-    if (wgo) mix_sweep<WF, 2, ROWS>(cx, ms, 0);
-    else mix_sweep<WF, 1, ROWS>(cx, ms, 0);
+    if (wgo) mix_sweep<float, WF, 2, ROWS>(cx, ms, 0);
+    else mix_sweep<float, WF, 1, ROWS>(cx, ms, 0);
     const double isu = 1.0 / su;
     const float isuf = (float)isu, iswf = (float)(1.0 / sw), ratio = (float)(su / sw);
     if (wgo)
@@ -960,7 +982,7 @@ __global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
     if (has)
       for (int a = tid; a < A; a += nt) Bv[a] = scaled(suf, rc[a]) - tf * (bhi[a] + bnx[a]);
     __syncthreads();
-    const MixSolve sv = mix_cocg<WF, ROWS>(g, b, cx, ms, phase, vs, true);
+    const MixSolve<float> sv = mix_cocg<float, WF, ROWS>(g, b, cx, ms, phase, vs, true);
     iters += sv.iters;
     conv_all &= sv.conv;
     ++solves;
@@ -982,9 +1004,9 @@ __global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
     if (has)
       for (int a = tid; a < A; a += nt) ud[lo + a] = cwiden(u[lo + a]);
   }
-  mix_drain<WF, ROWS>(cx, ms);
+  mix_drain<float, WF, ROWS>(cx, ms);
   __syncthreads();
-  if (tid == 0 && mix_sm<WF>().err) atomicOr(st + ST_STATUS, ST_WAIT_TIMEOUT);
+  if (tid == 0 && mix_sm<float, WF>().err) atomicOr(st + ST_STATUS, ST_WAIT_TIMEOUT);
   if (i == 0 && tid == 0) {               // the nb clusters of a frequency share its counters
     atomicAdd(st + ST_ITERS, iters);
     atomicAdd(st + ST_SOLVES, solves);
@@ -994,62 +1016,148 @@ __global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
   cl.sync();          // no CTA exits while a peer may still read its shared memory
 }
 
-// w = blkdiag(B^-1, 0) q for DD-layout vectors (Eq. 7), one CTA per subdomain.
+// The FP64 form of the strips (W <= 32): the same sweeps and interface solve in binary64,
+//   w = B^-1 q_B (boundary rows only), y = S^-1 (E^T w - q_C) to krylov_tol,
+//   u_B = B^-1 E y (from the interface solve's own products), u_C = -y.
+// The one-chain sweep of eight warps took 255 steps of 2.5 us a sweep at 128^2; the two
+// chains share the SM's binary64 pipe (2 multiply-adds a clock: 1 us a 32 x 32 product)
+// and hide each other's latency.
 template <int WF, bool ROWS>
-__global__ void __launch_bounds__(Mix<WF>::NT, Mix<WF>::PER_SM)
+__global__ void __launch_bounds__(Mix<double, WF>::NT, Mix<double, WF>::PER_SM)
+    k_xmatvec_d(const __grid_constant__ Geo g, const __grid_constant__ Bufs b, int j, int ncols) {
+  cg::cluster_group cl = cg::this_cluster();
+  constexpr int nt = Mix<double, WF>::NT;
+  const int i = blockIdx.x, vs = blockIdx.y, A = g.A, W = g.W, Lx = g.Lx, T = g.T;
+  const int f = slot_freq(g, vs), c = vs - f * g.nb;
+  if (c >= ncols) return;                  // same values in every CTA of the cluster
+  int* st = b.st + (size_t)f * ST_N;
+  if (st[ST_DONE]) return;
+  const size_t Ndd = g.Ndd;
+  const int nsub = Lx * W, w = T * g.h[i], tid = threadIdx.x;
+  const bool has = i < g.p - 1;
+  cxd* u = b.u + (size_t)vs * Ndd;
+  cxd* us = u + (size_t)i * nsub;
+  const cxd* q = b.Q + ((size_t)f * (g.k_max + g.nb) + (size_t)j * g.nb + c) * Ndd;
+  MixCtx<double, WF, ROWS> ctx;
+  ctx.W = W;
+  ctx.Lx = Lx;
+  ctx.S = mix_plan<double>(g).S;
+  ctx.m = Lx / 2;
+  ctx.src = reinterpret_cast<const cxd*>(b.g) + ((size_t)f * g.p + i) * (size_t)nsub * W;
+  ctx.g0 = reinterpret_cast<cxd*>(b.yscr) + ((size_t)vs * g.p + i) * nsub;
+  ctx.g1 = us;                             // the result's own place: an entry is read before it is written
+  ctx.cnt = sweep_cnt(g, b, vs, i);
+  ctx.t = g.t;
+  MixState<double> ms;
+  mix_init<double, WF, ROWS>(ctx, ms);
+  int phase = 0;
+  layer_diag<double>(g, b, vs, i);
+  cxd* B0 = ctx.row(0);
+  cxd* B1 = ctx.row(1);
+  for (int e = tid; e < nsub; e += nt) B0[e] = e % W < w ? q[(size_t)i * nsub + e] : cxd{0, 0};
+  mix_sweep<double, WF, 1, ROWS>(ctx, ms, 0);
+  cxd* blo = bnd_ptr<double>(g, b, vs, i, 0);
+  cxd* bhi = bnd_ptr<double>(g, b, vs, i, 1);
+  for (int e = tid; e < A; e += nt) {
+    const int jj = T == 1 ? 0 : e / Lx, s = e - jj * Lx;
+    blo[e] = B0[s * W + jj];
+    bhi[e] = B0[s * W + (w - T) + jj];
+  }
+  cl.sync();                               // boundary rows of the neighbours
+  const size_t lo = (size_t)g.ifc_off + (size_t)i * A;
+  if (has) {
+    cxd* Bv = ifv_ptr<double>(g, b, vs, IF_B) + (size_t)i * A;
+    const cxd* bnx = bnd_ptr<double>(g, b, vs, i + 1, 0);
+    for (int a = tid; a < A; a += nt) Bv[a] = g.t * (bhi[a] + bnx[a]) - q[lo + a];
+  }
+  __syncthreads();
+  const MixSolve<double> sv = mix_cocg<double, WF, ROWS>(g, b, ctx, ms, phase, vs, false);
+  for (int e = tid; e < nsub; e += nt) {   // zero on the padding, which the Lanczos step reads too
+    cxd v = sv.iters > 0 ? sv.alpha * B1[e] : cxd{0, 0};
+    if (sv.useB0) v = v - B0[e];
+    us[e] = v;
+  }
+  if (has) {
+    const cxd* X = ifv_ptr<double>(g, b, vs, IF_X) + (size_t)i * A;
+    for (int a = tid; a < A; a += nt) u[lo + a] = sv.iters > 0 ? -X[a] : cxd{0, 0};
+  }
+  mix_drain<double, WF, ROWS>(ctx, ms);
+  __syncthreads();
+  if (tid == 0 && mix_sm<double, WF>().err) atomicOr(st + ST_STATUS, ST_WAIT_TIMEOUT);
+  if (i == 0 && tid == 0) {               // the nb clusters of a frequency share its counters
+    atomicAdd(st + ST_ITERS, sv.iters);
+    atomicAdd(st + ST_SOLVES, 1);
+    if (!sv.conv) atomicOr(st + ST_STATUS, 4);
+  }
+  cl.sync();          // no CTA exits while a peer may still read its shared memory
+}
+
+// w = blkdiag(B^-1, 0) q for DD-layout vectors (Eq. 7), one CTA per subdomain.
+template <typename R, int WF, bool ROWS>
+__global__ void __launch_bounds__(Mix<R, WF>::NT, Mix<R, WF>::PER_SM)
     k_bsolve_m(const __grid_constant__ Geo g, const __grid_constant__ Bufs b, const cxd* q, cxd* w) {
-  constexpr int nt = Mix<WF>::NT;
+  constexpr int nt = Mix<R, WF>::NT;
   const int i = blockIdx.x, kf = blockIdx.y, vs = kf * g.nb, W = g.W, nsub = g.Lx * W, wd = g.T * g.h[i];
-  MixCtx<WF, ROWS> cx;
-  cx.W = W;
-  cx.Lx = g.Lx;
-  cx.S = mix_plan(g).S;
-  cx.m = g.Lx / 2;
-  cx.src = reinterpret_cast<const cxf*>(b.g) + ((size_t)kf * g.p + i) * (size_t)nsub * W;
-  cx.g0 = cx.g1 = reinterpret_cast<cxf*>(b.yscr) + ((size_t)vs * g.p + i) * nsub;
-  cx.cnt = sweep_cnt(g, b, vs, i);
-  cx.t = (float)g.t;
-  MixState ms;
-  mix_init<WF, ROWS>(cx, ms);
-  cxf* B0 = cx.row(0);
+  MixCtx<R, WF, ROWS> ctx;
+  ctx.W = W;
+  ctx.Lx = g.Lx;
+  ctx.S = mix_plan<R>(g).S;
+  ctx.m = g.Lx / 2;
+  ctx.src = reinterpret_cast<const cx<R>*>(b.g) + ((size_t)kf * g.p + i) * (size_t)nsub * W;
+  ctx.g0 = ctx.g1 = reinterpret_cast<cx<R>*>(b.yscr) + ((size_t)vs * g.p + i) * nsub;
+  ctx.cnt = sweep_cnt(g, b, vs, i);
+  ctx.t = (R)g.t;
+  MixState<R> ms;
+  mix_init<R, WF, ROWS>(ctx, ms);
+  cx<R>* B0 = ctx.row(0);
   const cxd* qs = q + (size_t)kf * g.Ndd + (size_t)i * nsub;
   cxd* ws = w + (size_t)kf * g.Ndd + (size_t)i * nsub;
-  for (int e = threadIdx.x; e < nsub; e += nt) B0[e] = e % W < wd ? c2f_bits(qs[e]) : cxf{0.f, 0.f};
-  mix_sweep<WF, 1, ROWS>(cx, ms, 0);
+  for (int e = threadIdx.x; e < nsub; e += nt) {
+    cx<R> v = {0, 0};
+    if (e % W < wd) {
+      if constexpr (sizeof(R) == 4) v = c2f_bits(qs[e]);
+      else v = qs[e];
+    }
+    B0[e] = v;
+  }
+  mix_sweep<R, WF, 1, ROWS>(ctx, ms, 0);
   for (int e = threadIdx.x; e < nsub; e += nt)
-    if (e % W < wd) ws[e] = c2d_bits(B0[e]);
+    if (e % W < wd) {
+      if constexpr (sizeof(R) == 4) ws[e] = c2d_bits(B0[e]);
+      else ws[e] = B0[e];
+    }
   if (i < g.p - 1)
     for (int a = threadIdx.x; a < g.A; a += nt)
       w[(size_t)kf * g.Ndd + g.ifc_off + (size_t)i * g.A + a] = cxd{0, 0};
-  mix_drain<WF, ROWS>(cx, ms);
+  mix_drain<R, WF, ROWS>(ctx, ms);
   __syncthreads();
-  if (threadIdx.x == 0 && mix_sm<WF>().err) atomicOr(b.st + (size_t)kf * ST_N + ST_STATUS, ST_WAIT_TIMEOUT);
+  if (threadIdx.x == 0 && mix_sm<R, WF>().err) atomicOr(b.st + (size_t)kf * ST_N + ST_STATUS, ST_WAIT_TIMEOUT);
 }
 
 }  // namespace
 
-template <int WF>
+template <typename R, int WF>
 cudaError_t run_xmatvec_m(const Geo& g, const Bufs& b, int K, int j, int ncols, cudaStream_t st);
-template <int WF>
+template <typename R, int WF>
 cudaError_t run_bsolve_m(const Geo& g, const Bufs& b, int K, const cxd* q_dd, cxd* w_dd, cudaStream_t st);
 
-#define DY_MIXED_VARIANT(WF)                                                                               \
+#define DY_CHAIN_VARIANT(R, WF, KERN)                                                                      \
   template <>                                                                                              \
-  cudaError_t run_xmatvec_m<WF>(const Geo& g, const Bufs& b, int K, int j, int ncols, cudaStream_t st) {   \
-    const MixPlan mp = mix_plan(g);                                                                        \
+  cudaError_t run_xmatvec_m<R, WF>(const Geo& g, const Bufs& b, int K, int j, int ncols, cudaStream_t st) { \
+    const MixPlan mp = mix_plan<R>(g);                                                                     \
     if (mp.rows)                                                                                           \
-      return launch_cluster_nt(k_xmatvec_m<WF, true>, dim3(g.p, K * g.nb), g.p, Mix<WF>::NT, mp.smem, st,  \
-                               g, b, j, ncols);                                                            \
-    return launch_cluster_nt(k_xmatvec_m<WF, false>, dim3(g.p, K * g.nb), g.p, Mix<WF>::NT, mp.smem, st,   \
-                             g, b, j, ncols);                                                              \
+      return launch_cluster_nt(KERN<WF, true>, dim3(g.p, K * g.nb), g.p, Mix<R, WF>::NT, mp.smem, st, g,   \
+                               b, j, ncols);                                                               \
+    return launch_cluster_nt(KERN<WF, false>, dim3(g.p, K * g.nb), g.p, Mix<R, WF>::NT, mp.smem, st, g, b, \
+                             j, ncols);                                                                    \
   }                                                                                                        \
   template <>                                                                                              \
-  cudaError_t run_bsolve_m<WF>(const Geo& g, const Bufs& b, int K, const cxd* q_dd, cxd* w_dd,             \
-                               cudaStream_t st) {                                                          \
-    const MixPlan mp = mix_plan(g);                                                                        \
-    auto kern = mp.rows ? k_bsolve_m<WF, true> : k_bsolve_m<WF, false>;                                    \
+  cudaError_t run_bsolve_m<R, WF>(const Geo& g, const Bufs& b, int K, const cxd* q_dd, cxd* w_dd,          \
+                                  cudaStream_t st) {                                                       \
+    const MixPlan mp = mix_plan<R>(g);                                                                     \
+    auto kern = mp.rows ? k_bsolve_m<R, WF, true> : k_bsolve_m<R, WF, false>;                              \
     cudaError_t e = raise_smem_limit((const void*)kern, mp.smem);                                          \
     if (e != cudaSuccess) return e;                                                                        \
-    kern<<<dim3(g.p, K), Mix<WF>::NT, mp.smem, st>>>(g, b, q_dd, w_dd);                                    \
+    kern<<<dim3(g.p, K), Mix<R, WF>::NT, mp.smem, st>>>(g, b, q_dd, w_dd);                                 \
     return cudaGetLastError();                                                                             \
   }
