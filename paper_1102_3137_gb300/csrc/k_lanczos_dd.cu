@@ -14,37 +14,49 @@
 // Classical Gram-Schmidt twice, with the three-term part folded in and the
 // second pass's coefficients taken from the Gram matrix of the stored basis:
 //   pass A:  g  = Q_j^T u                     (alpha_j = g_j)
+//            M's column j: Q_j^T q_j
 //            h  = g - M g,  M = Q_j^T Q_j     (M kept per frequency, binary64)
 //   pass B:  r  = u - Q_j (g + h)             (formed in binary64, stored split)
-//            M's next column: Q_j^T r / beta_{j+1}
 // In exact arithmetic h = Q_j^T (u - Q_j g) is the second pass's coefficient
 // vector, so r is the classical Gram-Schmidt residual orthogonalised twice;
 // reading Q_j^T Q_j from M instead of re-projecting u - Q_j g saves a sweep
-// over the basis (two reads of Q per step instead of three, three multiply-
-// accumulates per basis entry instead of four).  With the unit diagonal of M
+// over the basis: two reads of Q per step, the new column of M coming from the
+// entries that pass A has in registers anyway.  With the unit diagonal of M
 // exact, M - I holds the basis's measured loss of orthogonality, which h
 // removes to second order (one-reduce CGS2 in the Gram-matrix form); the
 // remaining error is the rounding of g, ~2^-47 ||u|| / |beta_{j+1}|.
-// Thread layout.  The CTA's part of the DD layout is walked in groups of
-// TG = 128 consecutive entries.  The per-site sum over the basis (r) runs two
-// threads per site along l (even and odd l), reading each vector's entries
-// coalesced across the warp.  Per-vector sums (g and the Gram column) run one
-// warp per eight vectors l = w + 8m, the lanes over the
-// group's sites, with the group's u (pass A) or r (pass B) staged in shared
-// memory; pass B re-reads the group's basis entries right after its per-site
-// half, from L2.  Per-vector totals are warp-shuffled, then summed over the
-// cluster's CTAs in rank order in binary64, so every CTA of a frequency holds
-// bit-identical coefficients.  Rank caps up to 64 (eight vectors per warp);
-// larger caps take the binary64 kernel.  The running sums are double-floats
-// updated by TwoProduct and TwoSum without renormalising the low word.
+//
+// What bounds it: the double-float multiply-accumulates (48 instructions per
+// complex one, three per basis entry) and the reads of Q (32 bytes per entry)
+// cost about the same, so neither may be spent on anything else.  Thread
+// layout: a thread has its own sites in both passes.  Pass A takes BV = 4
+// vectors at a time over T sites of every lane, the sums g and M in registers,
+// then folds the eight sums of the 32 lanes by a halving butterfly (nine
+// complex adds a lane instead of forty) into the warp's own row of shared
+// memory; no barrier until all vectors are done.  u and q_j of the T sites are
+// read again for each four vectors, from L1 (the basis itself bypasses it).
+// Pass B sums a site's basis entries in its thread.  Per-CTA sums are added
+// over the cluster in a fixed order in binary64, so every CTA of a frequency
+// holds bit-identical coefficients.  Rank caps up to 64; larger caps take the
+// binary64 kernel.  The running sums are double-floats updated by TwoProduct
+// and TwoSum without renormalising the low word.
+// Measured (average of the 16 steps at k = 16, cold L2): 256^2 x 16 frequencies
+// 0.77 -> 0.22 ms, 512^2 x 16 2.85 -> 0.79 ms, 101^2 x 21 0.16 -> 0.11 ms, against a
+// kernel that gave each warp whole vectors (its index work and barriers were most of
+// its instructions; 1.6x the instructions and half the SMs idle at 256^2).
 #include "solve_device.cuh"
 
 namespace {
 
-constexpr int LPW = 8;                   // basis vectors per warp in the per-vector passes
-constexpr int LDD_MAX = DY_WARPS * LPW;  // 64: largest j + 1 this kernel takes
-constexpr int TG = 128;                  // sites per group
-static_assert(DY_THREADS == 2 * TG, "two threads per site of a group");
+constexpr int LDD_MAX = 64;              // largest j + 1 this kernel takes
+constexpr int BV = 4;                    // basis vectors at a time in pass A (g and M sums: eight values)
+constexpr int T = 8;                     // sites of a thread between two folds
+// A strip is shared by 2 or 4 CTAs where each keeps this many sites: below, the folds
+// and the wider cluster's barriers cost what the split saves (64^2 x 16 solve, strips of
+// 1024: 5.7 ms unsplit, 5.9 in two, 6.1 in four; 101^2 x 63, 2525: 18.4 / 19.5 / 22.7);
+// above, one CTA a strip leaves SMs idle (256^2 x 16, 8192: 0.31 ms a step, 0.22 in two).
+constexpr int SPLIT_MIN = 2048;
+constexpr int MAX_RANKS = 16;            // CTAs of a cluster
 // The Lanczos thresholds scaled to double-float arithmetic: the same multiples of the
 // unit roundoff as TERM_TOL and BRK_TOL are of binary64's (2^-47 / 2^-53 = 64).
 constexpr double TERM_TOL_DD = 64.0 * TERM_TOL;
@@ -66,90 +78,143 @@ __device__ __forceinline__ cdfl cadd(const cdfl& a, const cdfl& b) { return {a.x
 __device__ __forceinline__ cdfl csub(const cdfl& a, const cdfl& b) { return {a.x - b.x, a.y - b.y}; }
 __device__ __forceinline__ cdfl cnorm(const cdfl& a) { return {dfl_fast(a.x.hi, a.x.lo), dfl_fast(a.y.hi, a.y.lo)}; }
 
-__device__ __forceinline__ cdfl warp_sum_dd(cdfl v) {
-  v = cnorm(v);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    v.x = v.x + shfl_xor_any(v.x, off);
-    v.y = v.y + shfl_xor_any(v.y, off);
-  }
-  return v;
-}
-
 struct LanDDSmem {
-  cxd vpart[2][LDD_MAX];               // this CTA's per-vector partial sums (phase double-buffered)
-  cxd vres[LDD_MAX];                   // the cluster totals
-  cxd gv[LDD_MAX];                     // g = Q^T u (pass A totals)
-  cdfl coef[LDD_MAX];                  // coefficients of the current pass, double-float
-  cdfl st[2][TG];                      // staged per-site values of one group (u; r1 halves)
+  cdfl wred[DY_WARPS][2 * LDD_MAX];      // per warp: Q^T u, then Q^T v, of its sites
+  cxd vpart[2 * LDD_MAX];                // this CTA's sums (read by its peers)
+  cxd vres[2 * LDD_MAX];                 // the cluster totals
+  cdfl coef[LDD_MAX];                    // g + h, double-float
 };
 
-// Cluster total of the per-vector partials vpart[phase][0..n): every CTA adds
-// the P CTAs' partials in rank order (binary64), so all hold the same bits.
-__device__ void cluster_vec_sum(cg::cluster_group& cl, LanDDSmem& sm, int& vphase, int P, int n) {
-  __syncthreads();
-  cl.sync();
-  for (int l = threadIdx.x; l < n; l += DY_THREADS) {
-    cxd s = {0, 0};
-    for (int r = 0; r < P; ++r) {
-      const LanDDSmem* rem = cl.map_shared_rank(&sm, r);
-      s = s + rem->vpart[vphase][l];
-    }
-    sm.vres[l] = s;
-  }
-  __syncthreads();
-  vphase ^= 1;
-}
-
-// this warp's accumulated per-vector sums -> vpart (binary64), vectors l = w + 8m <= j
-__device__ __forceinline__ void put_partials(LanDDSmem& sm, int vphase, int j, const cdfl (&acc)[LPW]) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+// v[0..7] summed over the warp; lane 4 i holds the sum of v[i] on return.  The first
+// three steps halve the values as they add (a lane keeps the half its bit selects).
+__device__ __forceinline__ cdfl warp_fold8(cdfl (&v)[8]) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int m = 0; m < LPW; ++m) {
-    const int l = w + DY_WARPS * m;
-    if (l <= j) {
-      const cdfl s = warp_sum_dd(acc[m]);
-      if (lane == 0) sm.vpart[vphase][l] = cwiden(s);
+  for (int i = 0; i < 8; ++i) v[i] = cnorm(v[i]);
+#pragma unroll
+  for (int h = 4, off = 16; h > 0; h >>= 1, off >>= 1) {
+    const bool up = lane & off;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (i >= h) break;
+      const cdfl give = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+      v[i] = {keep.x + shfl_xor_any(give.x, off), keep.y + shfl_xor_any(give.y, off)};
     }
   }
+#pragma unroll
+  for (int off = 2; off > 0; off >>= 1)
+    v[0] = {v[0].x + shfl_xor_any(v[0].x, off), v[0].y + shfl_xor_any(v[0].y, off)};
+  return v[0];
 }
 
-// sum over l = l0, l0 + dl, ... <= j of Q_l[k] c_l (double-float): the entries of
-// eight vectors are loaded before any is used (eight loads in flight per
-// thread), then summed in two interleaved chains
-__device__ __forceinline__ cdfl basis_sum(const cdfl* Q, size_t Ndd, size_t k, int j, int l0, int dl,
-                                          const cdfl* coef) {
+// The basis is read once per pass: past L1, which keeps u and q_j.
+__device__ __forceinline__ cdfl ld_basis(const cdfl* p) {
+  const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
+  return {dfl(v.x, v.y), dfl(v.z, v.w)};
+}
+
+// Totals over the cluster's CTAs of this CTA's sites e in [e0, e1) of Q_l^T u and
+// Q_l^T v, l <= j (v a double-float vector): sm.vres[l] and sm.vres[LDD_MAX + l].
+__device__ __noinline__ void basis_dots(cg::cluster_group& cl, LanDDSmem& sm, const Geo& g, int i, int P, int e0,
+                                        int e1, const cdfl* Q, const cxd* u, const cdfl* v, int j) {
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nsub = g.Lx * g.W;
+  const size_t Ndd = g.Ndd;
+  cdfl* row = sm.wred[w];
+  for (int l = lane; l < 2 * LDD_MAX; l += 32) row[l] = czero();
+  __syncwarp();
+  // a warp's sites: 32 consecutive ones every DY_THREADS
+  for (int eb = e0 + 32 * w; eb < e1; eb += DY_THREADS * T) {
+    for (int lb = 0; lb <= j; lb += BV) {
+      cdfl a[2 * BV];
+#pragma unroll
+      for (int m = 0; m < 2 * BV; ++m) a[m] = czero();
+      const cdfl* Qb = Q + (size_t)lb * Ndd;
+      for (int t = 0; t < T; ++t) {
+        const int e = eb + t * DY_THREADS + lane;
+        if (e >= e1) break;
+        const size_t k = own_idx(g, i, e, nsub);
+        cdfl qv[BV];
+#pragma unroll
+        for (int m = 0; m < BV; ++m) qv[m] = lb + m <= j ? ld_basis(Qb + (size_t)m * Ndd + k) : czero();
+        const cdfl ud = csplit(u[k]), vd = v[k];
+#pragma unroll
+        for (int m = 0; m < BV; ++m)
+          if (lb + m <= j) {
+            cmac(a[m], qv[m], ud);
+            cmac(a[BV + m], qv[m], vd);
+          }
+      }
+      __syncwarp();
+      const cdfl s = warp_fold8(a);
+      if ((lane & 3) == 0) {
+        const int m = lane >> 2, l = lb + (m & (BV - 1)) + (m / BV) * LDD_MAX;
+        row[l] = cadd(row[l], s);
+      }
+    }
+  }
+  __syncthreads();
+  // two threads a value, each half the warps, then half the cluster's CTAs
+  const int x = tid >> 1, hf = tid & 1;
+  const bool act = (x & (LDD_MAX - 1)) <= j;
+  {
+    cxd s = {0, 0};
+#pragma unroll
+    for (int k = 0; k < DY_WARPS / 2; ++k) s = s + cwiden(sm.wred[2 * k + hf][x]);
+    s = {s.x + __shfl_xor_sync(0xffffffffu, s.x, 1), s.y + __shfl_xor_sync(0xffffffffu, s.y, 1)};
+    if (hf == 0) sm.vpart[x] = s;
+  }
+  cl.sync();
+  cxd rv[MAX_RANKS / 2];
+#pragma unroll
+  for (int k = 0; k < MAX_RANKS / 2; ++k) {
+    const int r = 2 * k + hf;
+    rv[k] = cxd{0, 0};
+    if (act && r < P) rv[k] = cl.map_shared_rank(sm.vpart, r)[x];
+  }
+  cxd s = {0, 0};
+#pragma unroll
+  for (int k = 0; k < MAX_RANKS / 2; ++k) s = s + rv[k];
+  s = {s.x + __shfl_xor_sync(0xffffffffu, s.x, 1), s.y + __shfl_xor_sync(0xffffffffu, s.y, 1)};
+  if (hf == 0) sm.vres[x] = s;
+  __syncthreads();
+}
+static_assert(DY_THREADS == 4 * LDD_MAX && DY_WARPS % 2 == 0 && BV == 4, "basis_dots' sums");
+
+// sum over l < n of Q_l[k] c_l (double-float): the entries of eight vectors are
+// loaded before any is used (eight loads in flight per thread), then summed in two
+// interleaved chains
+__device__ __forceinline__ cdfl basis_sum(const cdfl* Q, size_t Ndd, size_t k, int n, const cdfl* coef) {
   cdfl s0 = czero(), s1 = czero();
-  for (int lb = l0; lb <= j; lb += 8 * dl) {
+  for (int lb = 0; lb < n; lb += 8) {
     cdfl qv[8];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const int l = lb + m * dl;
-      qv[m] = l <= j ? Q[(size_t)l * Ndd + k] : czero();
-    }
+    for (int m = 0; m < 8; ++m) qv[m] = lb + m < n ? ld_basis(Q + (size_t)(lb + m) * Ndd + k) : czero();
 #pragma unroll
     for (int m = 0; m < 8; m += 2) {
-      const int l = lb + m * dl;
-      if (l <= j) cmac(s0, qv[m], coef[l]);
-      if (l + dl <= j) cmac(s1, qv[m + 1], coef[l + dl]);
+      if (lb + m < n) cmac(s0, qv[m], coef[lb + m]);
+      if (lb + m + 1 < n) cmac(s1, qv[m + 1], coef[lb + m + 1]);
     }
   }
   return cadd(cnorm(s0), cnorm(s1));
 }
 
-template <int SPLIT>
-__global__ void __launch_bounds__(DY_THREADS, 2) k_lanczos_dd(Geo g, Bufs b, int j) {
+// Three CTAs an SM: with two, 14 clusters of 16 fit the chip and the 16 of a 512^2 group
+// ran in two waves (1.02 ms a step, 0.79 with three; 256^2 0.29 and 0.22).
+__global__ void __launch_bounds__(DY_THREADS, 3) k_lanczos_dd(Geo g, Bufs b, int j) {
   cg::cluster_group cl = cg::this_cluster();
   __shared__ RedSmem rs;
   __shared__ LanDDSmem sm;
-  const int i = blockIdx.x / SPLIT, part = blockIdx.x - i * SPLIT, kf = blockIdx.y, P = g.p * SPLIT;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  // a strip's entries in `split` runs of whole 32s, one a CTA
+  const int P = gridDim.x, split = P / g.p;
+  const int i = blockIdx.x / split, part = blockIdx.x - i * split, kf = blockIdx.y;
+  const int tid = threadIdx.x;
   int* stt = b.st + (size_t)kf * ST_N;
   if (stt[ST_DONE]) return;
-  int phase = 0, vphase = 0;
+  int phase = 0;
   const size_t Ndd = g.Ndd;
   const int nsub = g.Lx * g.W, n = own_count(g, i);
-  const int ngrp = (n + TG - 1) / TG;
+  const int n32 = (n + 31) / 32;
+  const int e0 = n32 * part / split * 32, e1 = min(n, n32 * (part + 1) / split * 32);
   // the basis is stored as double-floats (Geo::qsplit)
   cdfl* Q = reinterpret_cast<cdfl*>(b.Q + (size_t)kf * (g.k_max + g.nb) * Ndd);
   const cdfl* qj = Q + (size_t)j * Ndd;
@@ -164,123 +229,62 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_lanczos_dd(Geo g, Bufs b, int
   // read before the first cluster barrier: CTA 0 updates it once all CTAs passed the last one
   const double maxT_prev = b.maxT[kf];
 
-  // ---- pass A: g = Q^T u (warp w: vectors w + 8m; lanes over the group's sites)
-  {
-    cdfl a[LPW];
-#pragma unroll
-    for (int m = 0; m < LPW; ++m) a[m] = czero();
-    for (int gr = part; gr < ngrp; gr += SPLIT) {
-      const int e0 = gr * TG;
-      if (tid < TG) {
-        const int e = e0 + tid;
-        sm.st[0][tid] = e < n ? csplit(u[own_idx(g, i, e, nsub)]) : czero();
-      }
-      __syncthreads();
-      for (int c = lane; c < TG; c += 32) {
-        const int e = e0 + c;
-        if (e >= n) break;
-        const size_t k = own_idx(g, i, e, nsub);
-        const cdfl ud = sm.st[0][c];
-        cdfl qv[LPW];
-#pragma unroll
-        for (int m = 0; m < LPW; ++m) {
-          const int l = w + DY_WARPS * m;
-          qv[m] = l <= j ? Q[(size_t)l * Ndd + k] : czero();
-        }
-#pragma unroll
-        for (int m = 0; m < LPW; ++m)
-          if (w + DY_WARPS * m <= j) cmac(a[m], qv[m], ud);
-      }
-      __syncthreads();
-    }
-    put_partials(sm, vphase, j, a);
-  }
-  cluster_vec_sum(cl, sm, vphase, P, j + 1);
-  const cxd alpha = sm.vres[j];
-  for (int l = tid; l <= j; l += DY_THREADS) sm.gv[l] = sm.vres[l];
-  __syncthreads();
+  // ---- pass A: g = Q^T u, M's column j = Q^T q_j
+  basis_dots(cl, sm, g, i, P, e0, e1, Q, u, qj, j);
+  const cxd* gv = sm.vres;
+  const cxd* mj = sm.vres + LDD_MAX;
+  const cxd alpha = gv[j];
   // ---- second Gram-Schmidt coefficients from the Gram matrix M = Q_j^T Q_j of the
   // stored basis: h = Q_j^T (u - Q_j g) = g - M g, so g + h = g - (M - I) g (the unit
-  // diagonal of M taken as exact; binary64)
-  for (int l = tid; l <= j; l += DY_THREADS) {
+  // diagonal of M taken as exact; binary64); four threads a row
+  {
+    const int l = tid >> 2;
     cxd s = {0, 0};
-    for (int m = 0; m <= j; ++m) {
-      if (m == l) continue;
-      const cxd e = l < m ? gram[(size_t)m * K1 + l] : gram[(size_t)l * K1 + m];
-      s = cfma(e, sm.gv[m], s);
-    }
-    sm.coef[l] = csplit(sm.gv[l] - s);
+    if (l <= j)
+      for (int m = tid & 3; m <= j; m += 4) {
+        if (m == l) continue;
+        const int lo = min(l, m), hi = max(l, m);
+        s = cfma(hi == j ? mj[lo] : gram[(size_t)hi * K1 + lo], gv[m], s);
+      }
+#pragma unroll
+    for (int off = 1; off < 4; off <<= 1)
+      s = {s.x + __shfl_xor_sync(0xffffffffu, s.x, off), s.y + __shfl_xor_sync(0xffffffffu, s.y, off)};
+    if (l <= j && (tid & 3) == 0) sm.coef[l] = csplit(gv[l] - s);
   }
+  if (blockIdx.x == 0 && tid < j) gram[(size_t)j * K1 + tid] = mj[tid];
   __syncthreads();
 
-  // ---- pass B: r = u - Q (g + h) per site (two threads per site, even and odd l),
-  // finished in binary64 and stored split, with r^T r, ||r||^2 and the Eq. 9
-  // three-vector update; then h' = Q^T r (warp w: vectors w + 8m, lanes over the
-  // group's sites, r staged in shared memory), the Gram column of the next vector
+  // ---- pass B: r = u - Q (g + h) per site, finished in binary64 and stored split,
+  // with r^T r, ||r||^2 and the Eq. 9 three-vector update
   cxd v2[3] = {{0, 0}, {0, 0}, {0, 0}};   // r^T r, ||r||^2, ||u||^2
-  const cdfl ad = csplit(alpha), bd = csplit(2.0 * beta_j);
-  const int c0 = tid & (TG - 1), half = tid / TG;
   {
-    cdfl a[LPW];
-#pragma unroll
-    for (int m = 0; m < LPW; ++m) a[m] = czero();
-    for (int gr = part; gr < ngrp; gr += SPLIT) {
-      const int e0 = gr * TG;
-      {
-        const int e = e0 + c0;
-        cdfl s = czero();
-        if (e < n) s = basis_sum(Q, Ndd, own_idx(g, i, e, nsub), j, half, 2, sm.coef);
-        sm.st[half][c0] = s;
+    const cdfl ad = csplit(alpha), bd = csplit(2.0 * beta_j);
+    for (int e = e0 + tid; e < e1; e += DY_THREADS) {
+      const size_t k = own_idx(g, i, e, nsub);
+      const cxd uv = u[k], av = acc[k];
+      const cdfl qjd = qj[k], qmd = qm ? ld_basis(qm + k) : czero();
+      cdfl tot = basis_sum(Q, Ndd, k, j - 1, sm.coef), last = czero();
+      cmac(last, qjd, sm.coef[j]);
+      if (qm) cmac(last, qmd, sm.coef[j - 1]);
+      tot = cadd(tot, cnorm(last));
+      const cxd rv = {(uv.x - f2d_bits(tot.x.hi)) - f2d_bits(tot.x.lo),
+                      (uv.y - f2d_bits(tot.y.hi)) - f2d_bits(tot.y.lo)};
+      r[k] = csplit(rv);
+      v2[0] = cfma(rv, rv, v2[0]);
+      v2[1].x += cabs2(rv);
+      v2[2].x += cabs2(uv);
+      cdfl sq = czero(), d = czero();
+      cmac(sq, qjd, qjd);
+      cmac(d, ad, cnorm(sq));
+      if (qm) {
+        cdfl pr = czero();
+        cmac(pr, qmd, qjd);
+        cmac(d, bd, cnorm(pr));
       }
-      __syncthreads();
-      cdfl rd = czero();
-      if (half == 0 && e0 + c0 < n) {
-        const size_t k = own_idx(g, i, e0 + c0, nsub);
-        const cdfl tot = cadd(sm.st[0][c0], sm.st[1][c0]);
-        const cxd uv = u[k];
-        const cxd rv = {(uv.x - f2d_bits(tot.x.hi)) - f2d_bits(tot.x.lo),
-                        (uv.y - f2d_bits(tot.y.hi)) - f2d_bits(tot.y.lo)};
-        rd = csplit(rv);
-        r[k] = rd;
-        v2[0] = cfma(rv, rv, v2[0]);
-        v2[1].x += cabs2(rv);
-        v2[2].x += cabs2(uv);
-        const cdfl qjd = qj[k];
-        cdfl sq = czero(), d = czero();
-        cmac(sq, qjd, qjd);
-        cmac(d, ad, cnorm(sq));
-        if (qm) {
-          cdfl pr = czero();
-          cmac(pr, qm[k], qjd);
-          cmac(d, bd, cnorm(pr));
-        }
-        d = cnorm(d);
-        const cxd av = acc[k];
-        acc[k] = cxd{(av.x + f2d_bits(d.x.hi)) + f2d_bits(d.x.lo), (av.y + f2d_bits(d.y.hi)) + f2d_bits(d.y.lo)};
-      }
-      __syncthreads();                     // both halves have read st before it is overwritten
-      if (half == 0) sm.st[0][c0] = rd;
-      __syncthreads();
-      for (int c = lane; c < TG; c += 32) {
-        const int e = e0 + c;
-        if (e >= n) break;
-        const size_t k = own_idx(g, i, e, nsub);
-        cdfl qv[LPW];
-#pragma unroll
-        for (int m = 0; m < LPW; ++m) {
-          const int l = w + DY_WARPS * m;
-          qv[m] = l <= j ? Q[(size_t)l * Ndd + k] : czero();
-        }
-        const cdfl rc = sm.st[0][c];
-#pragma unroll
-        for (int m = 0; m < LPW; ++m)
-          if (w + DY_WARPS * m <= j) cmac(a[m], qv[m], rc);
-      }
-      __syncthreads();
+      d = cnorm(d);
+      acc[k] = cxd{(av.x + f2d_bits(d.x.hi)) + f2d_bits(d.x.lo), (av.y + f2d_bits(d.y.hi)) + f2d_bits(d.y.lo)};
     }
-    put_partials(sm, vphase, j, a);
   }
-  cluster_vec_sum(cl, sm, vphase, P, j + 1);   // sm.vres[l] = q_l^T r
   cluster_sum<3>(cl, rs, phase, P, v2);
   cxd rr = v2[0];
   double rn2 = v2[1].x;
@@ -288,18 +292,15 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_lanczos_dd(Geo g, Bufs b, int
   // invariant subspace): the Gram form leaves r's rounding error ~2^-47 ||u|| in
   // place, so project r once more onto the complement, r -= Q (Q^T r), as the
   // classical second pass would (the selective test of Daniel, Gragg, Kaufman and
-  // Stewart, 1976); the next vector's Gram column is then zero to working accuracy
-  const bool reorth = rn2 < REORTH_ETA * REORTH_ETA * v2[2].x;
-  if (reorth) {
-    for (int l = tid; l <= j; l += DY_THREADS) sm.coef[l] = csplit(sm.vres[l]);
+  // Stewart, 1976)
+  if (rn2 < REORTH_ETA * REORTH_ETA * v2[2].x) {
+    basis_dots(cl, sm, g, i, P, e0, e1, Q, u, r, j);
+    if (tid <= j) sm.coef[tid] = csplit(mj[tid]);
     __syncthreads();
     cxd w2[2] = {{0, 0}, {0, 0}};
-    for (int gr = part + half * SPLIT; gr < ngrp; gr += 2 * SPLIT) {
-      const int e = gr * TG + c0;
-      if (e >= n) continue;
+    for (int e = e0 + tid; e < e1; e += DY_THREADS) {
       const size_t k = own_idx(g, i, e, nsub);
-      const cdfl tot = basis_sum(Q, Ndd, k, j, 0, 1, sm.coef);
-      const cdfl rn = csub(r[k], tot);
+      const cdfl rn = csub(r[k], basis_sum(Q, Ndd, k, j + 1, sm.coef));
       r[k] = rn;
       const cxd rv = cwiden(rn);
       w2[0] = cfma(rv, rv, w2[0]);
@@ -323,22 +324,13 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_lanczos_dd(Geo g, Bufs b, int
     flag = 2;
   }
   if (!done) {
-    // Gram column of q_{j+1} = r / beta: q_l^T q_{j+1} = (q_l^T r) / beta, l <= j
-    if (blockIdx.x == 0) {
-      const cxd ibd = cinv(beta);
-      for (int l = tid; l <= j; l += DY_THREADS)
-        gram[(size_t)(j + 1) * K1 + l] = reorth ? cxd{0, 0} : sm.vres[l] * ibd;
-    }
     // q_{j+1} = r / beta in double-float
     const cdfl ib = csplit(cinv(beta));
-    for (int gr = part + half * SPLIT; gr < ngrp; gr += 2 * SPLIT) {
-      const int e = gr * TG + c0;
-      if (e < n) {
-        const size_t k = own_idx(g, i, e, nsub);
-        cdfl q = czero();
-        cmac(q, r[k], ib);
-        r[k] = cnorm(q);
-      }
+    for (int e = e0 + tid; e < e1; e += DY_THREADS) {
+      const size_t k = own_idx(g, i, e, nsub);
+      cdfl q = czero();
+      cmac(q, r[k], ib);
+      r[k] = cnorm(q);
     }
   }
   if (blockIdx.x == 0 && tid == 0) {
@@ -359,7 +351,8 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_lanczos_dd(Geo g, Bufs b, int
 
 // The mixed form's Lanczos step (rank caps up to 64; the binary64 kernel otherwise).
 cudaError_t launch_lanczos_dd(const Geo& g, const Bufs& b, int K, int j, cudaStream_t st) {
-  if (g.k_max > LDD_MAX || g.nb != 1) return cudaErrorInvalidValue;
-  if (2 * g.p <= 8) return launch_cluster(k_lanczos_dd<2>, dim3(2 * g.p, K), 2 * g.p, 0, st, g, b, j);
-  return launch_cluster(k_lanczos_dd<1>, dim3(g.p, K), g.p, 0, st, g, b, j);
+  if (g.k_max > LDD_MAX || g.nb != 1 || g.p > MAX_RANKS) return cudaErrorInvalidValue;
+  int split = 1;
+  while (2 * split * g.p <= MAX_RANKS && g.Lx * g.W / (2 * split) >= SPLIT_MIN) split *= 2;
+  return launch_cluster(k_lanczos_dd, dim3(split * g.p, K), split * g.p, 0, st, g, b, j);
 }
