@@ -647,9 +647,11 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_factor_wide(Geo g, Bufs b, in
   const size_t n = (size_t)W * W;
   const R t = (R)g.t, t2 = (R)(g.t * g.t);
   C* Gw = reinterpret_cast<C*>(b.fwork) + (size_t)clu * CN * 2 * n;     // G_{s+1,s+1}
-  C* Pw = Gw + n;                        // g_s G_{s+1,s+1}; during the inversion the panels F and O
-  C* Fb = Pw;                            // [nt][32][32] F_i = A_ik A_kk^-1
-  C* Ob = Pw + (size_t)nt * TB * TB;     // [nt][32][32] A_ik before
+  C* Pw = Gw + n;                        // g_s G_{s+1,s+1}
+  // During the forward pass the space of Gw and Pw holds the panels (2 nt 32^2 <= 2 W^2
+  // entries from W = 65 on; more than the W^2 of Pw alone up to W = 76).
+  C* Fb = Gw;                            // [nt][32][32] F_i = A_ik A_kk^-1
+  C* Ob = Gw + (size_t)nt * TB * TB;     // [nt][32][32] A_ik before
   const int lc = threadIdx.x & 31, lr = threadIdx.x >> 5;
   const int gt = ci * DY_THREADS + threadIdx.x, gn = CN * DY_THREADS;
   const TriSmem<R> ts = {sm.tri, sm.tri + 2 * TB, sm.tri + 4 * TB};
