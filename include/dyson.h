@@ -72,7 +72,8 @@ extern "C" {
 /* precision forms */
 #define DYSON_FP64 0   /* every step in complex128 */
 #define DYSON_MIXED 1  /* sweeps, inner interface solves and the preconditioner in complex64
-                          with FP32 accumulation, every solve refined against FP64 residuals;
+                          with FP32 accumulation, every solve refined against residuals in
+                          double-float (slice width <= 64) or FP64;
                           diag(B^-1) from a double-float (two binary32, ~47-bit) recursion;
                           the Lanczos step's re-orthogonalisation in double-float arithmetic
                           on a double-float basis (k_max <= 64, scalar Lanczos; binary64
@@ -83,7 +84,9 @@ extern "C" {
 /* interface preconditioner of the H solves (dyson_geometry.precond) */
 #define DYSON_PRECOND_AUTO 0    /* exact layer blocks where they apply, else banded */
 #define DYSON_PRECOND_BANDED 1  /* banded approximation of each layer block of S */
-#define DYSON_PRECOND_LAYER 2   /* exact layer blocks S_ll (2D strips, Lx <= 160, slice width <= 32) */
+#define DYSON_PRECOND_LAYER 2   /* exact layer blocks S_ll: 2D strips with Lx <= 160 and slice width
+                                   <= 32 or Lx <= 1024 and slice width 32, 3D slabs with Lx Ly <=
+                                   1024 and slice width > 64 */
 
 #define DYSON_MEM_HOST 0
 #define DYSON_MEM_DEVICE 1
@@ -102,10 +105,10 @@ typedef struct {
   double krylov_tol;  /* relative residual of each interface solve; 0 = default
                          (1e-13 FP64, 1e-5 mixed inner solves) */
   int krylov_maxit;   /* iteration cap of each interface solve; 0 = default (1000) */
-  double refine_tol;  /* mixed form: relative FP64 residual after refinement; 0 = 1e-13,
+  double refine_tol;  /* mixed form: relative residual after refinement; 0 = 1e-13,
                          the FP64 form's own interface tolerance (refinement also stops
-                         once a pass no longer shrinks the residual 4-fold: the FP64
-                         rounding floor) */
+                         once a pass no longer shrinks the residual 4-fold: the rounding
+                         floor) */
   int refine_max;     /* mixed form: most refinement passes per solve; 0 = default (6) */
   int max_freqs;      /* most frequencies one dyson_solve call may carry (>= 1) */
   double eta;         /* frequency axis.  0: Matsubara, H_ii = i w_k + mu - V_i - Sigma_i
@@ -177,13 +180,13 @@ int dyson_plan_destroy(dyson_plan plan);
  * Autotuner result (batched kernels' tile choice).  At a plan's first
  * dyson_solve with p > 1, before its graph is captured, the library times one
  * X-matvec launch for each configuration the geometry admits -- copy-ring
- * slots, rows per streamed chunk when W > 64, and for the mixed form's
- * complex64 two-chain sweeps (W <= 64) the CTA size, 256 threads at two CTAs
- * per SM or 128 threads at four -- on the caller's inputs and keeps the
- * fastest.  Reports the configuration in use (*ring_slots, *chunk_rows,
- * *threads), how many were timed (*candidates, 0 before the first solve) and
- * the launch times of the heuristic's choice and of the kept one (ms).  Any
- * output pointer may be NULL.  The paper has no counterpart.
+ * slots, rows per streamed chunk when W > 64, and for the two-chain sweeps
+ * (W <= 64 mixed, W <= 32 FP64) whether the row buffers stay on chip -- on the
+ * caller's inputs and keeps the fastest.  Reports the configuration in use
+ * (*ring_slots, *chunk_rows, and *threads, the X-matvec CTA's size, which
+ * follows from the slice width), how many were timed (*candidates, 0 before
+ * the first solve) and the launch times of the heuristic's choice and of the
+ * kept one (ms).  Any output pointer may be NULL.  The paper has no counterpart.
  */
 int dyson_plan_tuning(dyson_plan plan, int* ring_slots, int* chunk_rows, int* candidates,
                       float* ms_heuristic, float* ms_best, int* threads);
@@ -260,8 +263,9 @@ int dyson_subdomain_solve(dyson_plan plan, int K, const double* omega, const dou
  * u = X q = H^-1 q - blkdiag(B^-1, 0) q, the modified Lanczos "matvec" of
  * Eqs. 6-8, for complex[K][N] q and u.  FP64 form: u from the elimination
  * y = S^-1 (E^T B^-1 q_B - q_C), u_B = B^-1 E y, u_C = -y, with S applied
- * implicitly (never formed).  Mixed form: v = H^-1 q and w refined in FP64,
- * u = v - w.
+ * implicitly (never formed).  Mixed form: w = blkdiag(B^-1, 0) q and the
+ * solution u of H u = [0; q_C - E^T w_B], refined together (the same u = v - w
+ * without its cancellation).
  */
 int dyson_xmatvec(dyson_plan plan, int K, const double* omega, const double* V,
                   const double* sigma, const double* q, double* u, int mem_kind, void* stream);

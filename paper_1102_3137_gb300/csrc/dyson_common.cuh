@@ -200,9 +200,9 @@ struct Geo {
   int ring_S;          // copy-ring slots chosen by the autotuner (0: shared-memory heuristic)
   int ring_CR;         // rows per streamed chunk chosen by the autotuner (W > 64; 0: heuristic)
   int nb;              // Lanczos block size (1: the scalar recurrence of Sec. 2.1)
-  int lpre;            // interface preconditioner: 1 exact layer blocks of S (2D strips), 0 banded
-  int xm_rows;         // mixed form, W <= 64, ring_S > 0: sweep row buffers on chip (1) or in the
-                       // plan's scratch (0), chosen by the autotuner
+  int lpre;            // interface preconditioner: 1 exact layer blocks of S, 0 banded
+  int xm_rows;         // two-chain sweep, ring_S > 0: row buffers on chip (1) or in the plan's
+                       // scratch (0), chosen by the autotuner
   int qsplit;          // the Lanczos basis is stored as double-floats (cdfl; mixed form, nb = 1,
                        // k_max <= 64, where the double-float Lanczos step runs)
 };
@@ -220,7 +220,7 @@ struct Bufs {
   const double* q1;     // [nb][N] real Lanczos start vector(s)
   const int* dd2nat;    // [Ndd] natural index of each DD slot, -1 on padding
   void* g;              // [K][p][Lx][W][W] slice factors g_s read by the sweeps (precision of the form)
-  cxd* g64;             // [K][p][Lx][W][W] FP64 g_s kept for the mixed form's FP64 recursion
+  cxd* g64;             // [K][p][Lx][W][W] double-float g_s kept for the mixed form's recursion
   cxd* diagB;           // [K][Ndd] diag(B^-1), zero on the interface
   cxd* hdiag;           // [K][Ndd] H_ii (Eq. 1) in DD layout, zero on padding (mixed form; double-floats
                         // for W <= 64), or null
@@ -229,7 +229,7 @@ struct Bufs {
   cxd* Q;               // [K][k_max+nb][Ndd] Lanczos vectors (column j*nb + c of block j)
   cxd* acc;             // [K][Ndd] running diag(Q T Q^T)
   cxd* u;               // [K*nb][Ndd] X q, per slot
-  cxd* v1;              // [K*nb][Ndd] work vectors of the mixed form, per slot
+  cxd* v1;              // [K*nb][Ndd] work vectors of the mixed form's refinement, per slot
   cxd* v2;
   cxd* v3;
   void* yscr;           // [K*nb][p][Lx][W] forward-sweep intermediates (precision of the form)
