@@ -5,22 +5,51 @@
 
 namespace {
 
+// v[0..7] summed over the warp; lane 4 i holds the sum of v[i] on return.  The first
+// three steps halve the values as they add (a lane keeps the half its bit selects):
+// 18 binary64 adds a lane instead of 80.
+__device__ __forceinline__ cxd warp_fold8(cxd (&v)[8]) {
+  const int lane = threadIdx.x & 31;
+  auto add = [](cxd a, cxd b, int off) -> cxd {
+    return {a.x + __shfl_xor_sync(0xffffffffu, b.x, off), a.y + __shfl_xor_sync(0xffffffffu, b.y, off)};
+  };
+#pragma unroll
+  for (int h = 4, off = 16; h > 0; h >>= 1, off >>= 1) {
+    const bool up = lane & off;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (i >= h) break;
+      const cxd give = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+      v[i] = add(keep, give, off);
+    }
+  }
+  v[0] = add(v[0], v[0], 2);
+  return add(v[0], v[0], 1);
+}
+
 // One step of complex-symmetric Lanczos on X with the bilinear form
 // (Sec. 2.1, Freund et al.), full CGS2 re-orthogonalisation in the same form,
 // and the three-vector update of diag(Q T Q^T) (Sec. 2.3 after Eq. 9).
-// One cluster per frequency; SPLIT CTAs share each subdomain's entries
-// (interleaved), so the FP64 work of a frequency spreads over SPLIT * p SMs.
-template <int SPLIT>
+// One cluster per frequency; gridDim.x / p CTAs share each subdomain's entries
+// (interleaved), so the FP64 work of a frequency spreads over as many SMs.
+// The coefficients of a pass are exchanged once: each warp folds eight vectors'
+// sums at a time (warp_fold8) into its row, and the cluster adds all of them after
+// the last; summed and exchanged eight vectors at a time, the sums took the FP64
+// pipe as long as a quarter of the products (128^2 x 8, k = 32: 0.276 ms a step on
+// average, 0.236 with one exchange, two CTAs a strip in both).
 __global__ void __launch_bounds__(DY_THREADS) k_lanczos(Geo g, Bufs b, int j) {
   cg::cluster_group cl = cg::this_cluster();
   __shared__ RedSmem rs;
   __shared__ cxd hs[KMAX_SMEM];
-  const int i = blockIdx.x / SPLIT, part = blockIdx.x - i * SPLIT, kf = blockIdx.y, p = g.p * SPLIT;
-  const int e0 = threadIdx.x + part * DY_THREADS;
-  constexpr int ES = SPLIT * DY_THREADS;
+  __shared__ cxd wred[DY_WARPS][KMAX_SMEM];   // per warp: Q^T r of its entries
+  __shared__ cxd vpart[2][KMAX_SMEM];         // this CTA's sums, per pass (read by its peers)
+  const int p = gridDim.x, split = p / g.p, kf = blockIdx.y;
+  const int i = blockIdx.x / split, part = blockIdx.x - i * split;
+  const int e0 = threadIdx.x + part * DY_THREADS, ES = split * DY_THREADS;
   int* st = b.st + (size_t)kf * ST_N;
   if (st[ST_DONE]) return;
   int phase = 0;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const size_t Ndd = g.Ndd;
   const int nsub = g.Lx * g.W, n = own_count(g, i);
   cxd* Q = b.Q + (size_t)kf * (g.k_max + g.nb) * Ndd;
@@ -59,13 +88,28 @@ __global__ void __launch_bounds__(DY_THREADS) k_lanczos(Geo g, Bufs b, int j) {
         for (int m = 0; m < 8; ++m)
           if (c0 + m <= j) h8[m] = cfma(Q[(size_t)(c0 + m) * Ndd + k], rv, h8[m]);
       }
-      cluster_sum<8>(cl, rs, phase, p, h8);
-      if (threadIdx.x < 8 && c0 + threadIdx.x <= j) hs[c0 + threadIdx.x] = h8[threadIdx.x];
+      const cxd s = warp_fold8(h8);
+      if ((lane & 3) == 0) wred[wid][c0 + (lane >> 2)] = s;
+    }
+    __syncthreads();
+    for (int l = threadIdx.x; l <= j; l += DY_THREADS) {
+      cxd s = wred[0][l];
+#pragma unroll
+      for (int w = 1; w < DY_WARPS; ++w) s = s + wred[w][l];
+      vpart[pass][l] = s;
+    }
+    cl.sync();                           // one exchange for all vectors
+    for (int l = threadIdx.x; l <= j; l += DY_THREADS) {
+      cxd s = {0, 0};
+#pragma unroll 8
+      for (int r = 0; r < p; ++r) s = s + cl.map_shared_rank(vpart[pass], r)[l];
+      hs[l] = s;
     }
     __syncthreads();
     for (int e = e0; e < n; e += ES) {
       size_t k = own_idx(g, i, e, nsub);
       cxd rv = r[k];
+#pragma unroll 8
       for (int m = 0; m <= j; ++m) rv = cfma(-hs[m], Q[(size_t)m * Ndd + k], rv);   // fused: 4 FP64 ops
       r[k] = rv;
     }
@@ -246,8 +290,11 @@ int dyson_internal_ring_candidates(const Geo& g, bool mixed, int* S, int* CR, in
 
 cudaError_t launch_lanczos(const Geo& g, const Bufs& b, int K, int j, cudaStream_t st) {
   if (g.k_max > KMAX_SMEM) return cudaErrorInvalidValue;
-  if (2 * g.p <= 8) return launch_cluster(k_lanczos<2>, dim3(2 * g.p, K), 2 * g.p, 0, st, g, b, j);
-  return launch_cluster(k_lanczos<1>, dim3(g.p, K), g.p, 0, st, g, b, j);
+  // four CTAs a strip where each keeps 1024 entries or more (128^2 x 16, p = 4: solve 70.0
+  // ms with two, 69.2 with four), two where the cluster then has at most 8
+  int split = 2 * g.p <= 8 ? 2 : 1;
+  while (2 * split * g.p <= 16 && g.Lx * g.W / (2 * split) >= 1024) split *= 2;
+  return launch_cluster(k_lanczos, dim3(split * g.p, K), split * g.p, 0, st, g, b, j);
 }
 
 cudaError_t launch_init(const Geo& g, const Bufs& b, int K, cudaStream_t st) {

@@ -1,14 +1,14 @@
 """The strip, slab and Lanczos kernels at the edges of their tiles, rules and splits,
 against the oracle through the C ABI.  Tolerances are those of the same quantities in the
 other parity tests (FP64 / mixed): diag(B^-1) 1e-12 / 1e-10, B^-1 q 1e-12 / 1e-5, X q
-1e-11 / 1e-9, a truncated run step by step 1e-6."""
+1e-11 / 1e-9, a truncated run step by step 1e-10 / 1e-6."""
 import numpy as np
 import pytest
 
 from oracle import dyson_oracle as O
 from paper_1102_3137_gb300 import dyson as D
 from paper_1102_3137_gb300 import inputs as I
-from parity_util import OPEN, TOL_MIXED, oracle_parts, plan_for, relerr, stepwise_check, wl
+from parity_util import OPEN, TOL_FP64, TOL_MIXED, oracle_parts, plan_for, relerr, stepwise_check, wl
 
 pytestmark = pytest.mark.gpu
 
@@ -67,15 +67,16 @@ def test_wide_factor_cluster_sizes(L, p, precision, tol):
         assert relerr(out[100][k][mask], subs.diagB[mask]) < tol
 
 
-# strips of one (20 sites: fewer than a warp each), two and four CTAs; k = 9 and 4 end inside
-# and at the end of four basis vectors
+# mixed: strips of one (20 sites: fewer than a warp each), two and four CTAs; FP64: two, four
+# and eight; k = 9 and 4 end inside and at the end of a group of basis vectors
 @pytest.mark.parametrize("L,p,k", [((5, 9), 2, 4), ((256, 33), 2, 9), ((300, 65), 2, 4)])
-def test_lanczos_step_splits(L, p, k):
+@pytest.mark.parametrize("precision,tol", [(D.DYSON_FP64, TOL_FP64), (D.DYSON_MIXED, TOL_MIXED)])
+def test_lanczos_step_splits(L, p, k, precision, tol):
     w = wl(L, p, k, K=2, seed=7)
     omega, V, sigma, q1 = I.make_inputs(w)
-    pl = plan_for(w, D.DYSON_MIXED)
+    pl = plan_for(w, precision)
     out = pl.solve(omega, V, sigma, q1)
     info = pl.info(w.K)
     for f in range(w.K):
         subs, X = oracle_parts(w, omega[f], V, sigma[f])
-        assert stepwise_check(w, pl, f, subs, X, q1, out[f], info, TOL_MIXED) == k
+        assert stepwise_check(w, pl, f, subs, X, q1, out[f], info, tol) == k
