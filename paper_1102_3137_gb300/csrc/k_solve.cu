@@ -290,10 +290,10 @@ int dyson_internal_ring_candidates(const Geo& g, bool mixed, int* S, int* CR, in
 
 cudaError_t launch_lanczos(const Geo& g, const Bufs& b, int K, int j, cudaStream_t st) {
   if (g.k_max > KMAX_SMEM) return cudaErrorInvalidValue;
-  // four CTAs a strip where each keeps 1024 entries or more (128^2 x 16, p = 4: solve 70.0
-  // ms with two, 69.2 with four), two where the cluster then has at most 8
-  int split = 2 * g.p <= 8 ? 2 : 1;
-  while (2 * split * g.p <= 16 && g.Lx * g.W / (2 * split) >= 1024) split *= 2;
+  // Two CTAs a strip where the cluster then has at most 8.  Clusters of 16 are no gain: alone
+  // on the chip a solve is 1 % faster (128^2 x 16, p = 4: 70.0 -> 69.2 ms), with more groups
+  // in flight slower (128^2 x 64 135 -> 143, 256^2 x 32, p = 8: 169 -> 173, 200^2 x 32 492 -> 497).
+  const int split = 2 * g.p <= 8 ? 2 : 1;
   return launch_cluster(k_lanczos, dim3(split * g.p, K), split * g.p, 0, st, g, b, j);
 }
 

@@ -67,8 +67,8 @@ def test_wide_factor_cluster_sizes(L, p, precision, tol):
         assert relerr(out[100][k][mask], subs.diagB[mask]) < tol
 
 
-# mixed: strips of one (20 sites: fewer than a warp each), two and four CTAs; FP64: two, four
-# and eight; k = 9 and 4 end inside and at the end of a group of basis vectors
+# mixed: strips of one (20 sites: fewer than a warp each), two and four CTAs; FP64: two; k = 9
+# and 4 end inside and at the end of a group of basis vectors
 @pytest.mark.parametrize("L,p,k", [((5, 9), 2, 4), ((256, 33), 2, 9), ((300, 65), 2, 4)])
 @pytest.mark.parametrize("precision,tol", [(D.DYSON_FP64, TOL_FP64), (D.DYSON_MIXED, TOL_MIXED)])
 def test_lanczos_step_splits(L, p, k, precision, tol):
