@@ -72,8 +72,7 @@ extern "C" {
 /* precision forms */
 #define DYSON_FP64 0   /* every step in complex128 */
 #define DYSON_MIXED 1  /* sweeps, inner interface solves and the preconditioner in complex64
-                          with FP32 accumulation, every solve refined against residuals in
-                          double-float (slice width <= 64) or FP64;
+                          with FP32 accumulation, every solve refined against FP64 residuals;
                           diag(B^-1) from a double-float (two binary32, ~47-bit) recursion;
                           the Lanczos step's re-orthogonalisation in double-float arithmetic
                           on a double-float basis (k_max <= 64, scalar Lanczos; binary64
@@ -105,10 +104,10 @@ typedef struct {
   double krylov_tol;  /* relative residual of each interface solve; 0 = default
                          (1e-13 FP64, 1e-5 mixed inner solves) */
   int krylov_maxit;   /* iteration cap of each interface solve; 0 = default (1000) */
-  double refine_tol;  /* mixed form: relative residual after refinement; 0 = 1e-13,
+  double refine_tol;  /* mixed form: relative FP64 residual after refinement; 0 = 1e-13,
                          the FP64 form's own interface tolerance (refinement also stops
-                         once a pass no longer shrinks the residual 4-fold: the rounding
-                         floor) */
+                         once a pass no longer shrinks the residual 4-fold: the FP64
+                         rounding floor) */
   int refine_max;     /* mixed form: most refinement passes per solve; 0 = default (6) */
   int max_freqs;      /* most frequencies one dyson_solve call may carry (>= 1) */
   double eta;         /* frequency axis.  0: Matsubara, H_ii = i w_k + mu - V_i - Sigma_i

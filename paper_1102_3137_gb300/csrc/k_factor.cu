@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
   cxl* gout = reinterpret_cast<cxl*>(mixed ? (void*)b.g64 : b.g) + uoff;
   cxf* gsw = reinterpret_cast<cxf*>(b.g) + uoff;
   cxd* dB = b.diagB + (size_t)kf * g.Ndd + (size_t)i * Lx * W;
-  const cdfl* hd = reinterpret_cast<const cdfl*>(b.hdiag) + (size_t)kf * g.Ndd + (size_t)i * Lx * W;
+  const cxd* hd = b.hdiag + (size_t)kf * g.Ndd + (size_t)i * Lx * W;
   const bool band = !g.lpre;                 // the banded preconditioner reads the off-diagonal blocks
   cxd* oB = band && b.offB ? b.offB + ((size_t)kf * g.p + i) * (size_t)Lx * W : nullptr;
   cxd* o2 = band && b.off2 && T == 1 ? b.off2 + ((size_t)kf * g.p + i) * (size_t)Lx * W : nullptr;
@@ -382,8 +382,7 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
   // H_ii of row tid of slice s (tid < W): from the DD-layout copy in the mixed form
   auto diag_of = [&](int s) -> cxl {
     if constexpr (mixed) {
-      const cdfl d = hd[(size_t)s * W + tid];
-      return cxl{d.x, d.y};
+      return cconv<R>(hd[(size_t)s * W + tid]);
     } else {
       return tid < w ? dyson_diag(g, b, kf, sub_nat(g, i, s, tid)) : cxl{0, 0};
     }
@@ -916,17 +915,13 @@ __global__ void __launch_bounds__(DY_THREADS) k_precond(Geo g, Bufs b) {
 }  // namespace
 
 // H_ii (Eq. 1) of every DD slot, zero on padding: the mixed form's residuals
-// read it coalesced instead of gathering V and Sigma in natural order.  For
-// slices of up to 64 sites, whose residuals run in double-float arithmetic, an
-// entry is stored as a cdfl, else in binary64 (16 bytes either way).
+// read it coalesced instead of gathering V and Sigma in natural order.
 __global__ void __launch_bounds__(DY_THREADS) k_hdiag(Geo g, Bufs b) {
   const int kf = blockIdx.y;
   for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < (size_t)g.Ndd;
        k += (size_t)gridDim.x * blockDim.x) {
     const int nat = b.dd2nat[k];
-    const cxd d = nat >= 0 ? dyson_diag(g, b, kf, nat) : cxd{0, 0};
-    if (g.W <= DY_MAXW_SMEM) reinterpret_cast<cdfl*>(b.hdiag)[(size_t)kf * g.Ndd + k] = cdfl{dfl(d.x), dfl(d.y)};   // 48 bits
-    else b.hdiag[(size_t)kf * g.Ndd + k] = d;
+    b.hdiag[(size_t)kf * g.Ndd + k] = nat >= 0 ? dyson_diag(g, b, kf, nat) : cxd{0, 0};
   }
 }
 

@@ -20,11 +20,9 @@
 // 3. No closing sweep: the interface solve's last product B^-1 E p is still in
 //    the row buffer when its step length alpha is known, and u_B is the sum of
 //    alpha B^-1 E p over the iterations, so B^-1 E y needs no sweep of its own.
-// 4. Residuals in double-float arithmetic: w and u are held as double-floats
-//    (47 bits; 16 bytes a complex entry like binary64) until the last pass
-//    widens u.  The part issues 2 binary64 operations per clock and SM, so the
-//    ~28 of a site's two binary64 residuals took ~14 clocks; ~280 binary32 ones
-//    take ~2.
+// w, u, H_ii and the residuals are binary64, as are the sums over warps and
+// CTAs: what the refinement ends at is the rounding floor of the binary64
+// residual, whatever H is.
 #pragma once
 #include "solve_device.cuh"
 
@@ -53,8 +51,9 @@ template <typename R, int WF>
 struct MixSmem {
   alignas(16) cx<R> z[2][2][2][WF];      // [chain][right-hand side][parity]: z of the current and next slice
   alignas(16) cx<R> zm[2][2][WF];        // [chain][right-hand side]: the chain's part of the middle z
-  R wred[24 * 8];                        // per-warp partial sums
-  R slot[2][DY_MAXP * 8];            // [phase][rank]: the cluster's partial sums
+  double wred[24 * 8];                   // per-warp partial sums
+  double slot[2][DY_MAXP * 8];           // [phase][rank]: the CTAs' partial sums
+  double res[8];                         // the cluster's sums
   alignas(8) uint64_t bars[2 * MIX_MAXS];
   int err;
 };
@@ -474,117 +473,69 @@ __device__ __noinline__ void mix_sweep(const MixCtx<R, WF, ROWS>& ctx, MixState<
 }
 
 // ---------------------------------------------------------------- reductions
-// Cluster-wide sums of NV values of R (every thread gets them), and this
-// CTA's own totals in loc if not null.  Warp totals, their sum by warp 0, which
-// puts it into every CTA's slot for this rank; after the cluster barrier each
-// warp adds the ranks' slots by the same tree, so all threads of the cluster
-// hold the same bits.  `phase` alternates two slot sets.
-template <typename R, int WF, int NV>
-__device__ __forceinline__ void mix_sum(cg::cluster_group& cl, int& phase, int p, R (&v)[NV], R* loc = nullptr) {
+// Cluster-wide sums of NV values of V (every thread gets them), and this CTA's
+// own totals in loc if not null.  A warp's total is formed in V, the sums over
+// warps and CTAs in binary64: warp 0 adds the warps and puts the total into every
+// CTA's slot for this rank; after the cluster barrier it adds the ranks' slots by
+// the same tree in every CTA, so all threads of the cluster hold the same bits.
+// active (the same in a warp): this warp has something to add.  `phase` alternates
+// two slot sets.
+template <typename R, int WF, int NV, typename V>
+__device__ __forceinline__ void mix_sum(cg::cluster_group& cl, int& phase, int p, V (&v)[NV], double (&out)[NV],
+                                        bool active = true, double* loc = nullptr) {
   MixSmem<R, WF>& sm = mix_sm<R, WF>();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   constexpr int NW = Mix<R, WF>::NT / 32;
   const int me = (int)cl.block_rank();
+  if (active) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
+    for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+      for (int k = 0; k < NV; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+  }
   if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) sm.wred[wid * 8 + k] = v[k];
+    for (int k = 0; k < NV; ++k) sm.wred[wid * 8 + k] = active ? (double)v[k] : 0.0;
   }
   __syncthreads();
   if (wid == 0) {
-    R s[NV];
+    double s[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) s[k] = lane < NW ? sm.wred[lane * 8 + k] : R(0);
+    for (int k = 0; k < NV; ++k) s[k] = lane < NW ? sm.wred[lane * 8 + k] : 0.0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
       for (int k = 0; k < NV; ++k) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
     if (lane < p) {
-      R* rem = cl.map_shared_rank(&sm.slot[phase][me * 8], lane);
+      double* rem = cl.map_shared_rank(&sm.slot[phase][me * 8], lane);
 #pragma unroll
       for (int k = 0; k < NV; ++k) rem[k] = s[k];
     }
   }
   cl.sync();
+  if (wid == 0) {
+    double s[NV];
 #pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = lane < p ? sm.slot[phase][lane * 8 + k] : R(0);
+    for (int k = 0; k < NV; ++k) s[k] = lane < p ? sm.slot[phase][lane * 8 + k] : 0.0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
+    for (int o = DY_MAXP / 2; o > 0; o >>= 1)
 #pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+      for (int k = 0; k < NV; ++k) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+    if (lane == 0) {
+#pragma unroll
+      for (int k = 0; k < NV; ++k) sm.res[k] = s[k];
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NV; ++k) out[k] = sm.res[k];
   if (loc) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) loc[k] = sm.slot[phase][me * 8 + k];
   }
   phase ^= 1;
 }
-
-// A sum of squares in binary32 without a known scale: three accumulators, of
-// which value() takes the one that neither under- nor overflowed.
-struct Norm3 {
-  float m = 0.f, s = 0.f, b = 0.f;
-  __device__ __forceinline__ void add(cxf v) {
-    constexpr float UP = 18446744073709551616.f, DN = 1.f / 18446744073709551616.f;   // 2^64, 2^-64
-    m += cabs2(v);
-    s += cabs2(UP * v);
-    b += cabs2(DN * v);
-  }
-  __device__ static __forceinline__ double value(float m, float s, float b) {
-    constexpr double UP2 = 340282366920938463463374607431768211456.0;                 // 2^128
-    if (m > 1e-28f && m < 1e28f) return (double)m;
-    return m >= 1e28f ? (double)b * UP2 : (double)s / UP2;
-  }
-};
-
-// ---------------------------------------------------------------- double-float pieces
-// a + b: the high words by TwoSum, the low words and the error added up (not renormalised)
-__device__ __forceinline__ void acc_add(dfl& a, dfl b) {
-  float s, e;
-  dfl_two_sum(a.hi, b.hi, s, e);
-  a.hi = s;
-  a.lo = __fadd_rn(__fadd_rn(a.lo, b.lo), e);
-}
-// a - b c
-__device__ __forceinline__ void acc_sub_mul(dfl& a, dfl b, dfl c) {
-  float p, e, s, t;
-  dfl_two_prod(-b.hi, c.hi, p, e);
-  e = __fmaf_rn(-b.hi, c.lo, e);
-  e = __fmaf_rn(-b.lo, c.hi, e);
-  dfl_two_sum(a.hi, p, s, t);
-  a.hi = s;
-  a.lo = __fadd_rn(a.lo, __fadd_rn(t, e));
-}
-__device__ __forceinline__ void acc_add(cdfl& a, const cdfl& b) {
-  acc_add(a.x, b.x);
-  acc_add(a.y, b.y);
-}
-// a - s b, s real
-__device__ __forceinline__ void acc_sub_scaled(cdfl& a, dfl s, const cdfl& b) {
-  acc_sub_mul(a.x, s, b.x);
-  acc_sub_mul(a.y, s, b.y);
-}
-// a - b c
-__device__ __forceinline__ void acc_sub_cmul(cdfl& a, const cdfl& b, const cdfl& c) {
-  acc_sub_mul(a.x, b.x, c.x);
-  acc_sub_mul(a.x, dfl(-b.y.hi, -b.y.lo), c.y);
-  acc_sub_mul(a.y, b.x, c.y);
-  acc_sub_mul(a.y, b.y, c.x);
-}
-__device__ __forceinline__ dfl renorm(dfl a) { return dfl_fast(a.hi, a.lo); }
-__device__ __forceinline__ cdfl renorm(const cdfl& a) { return {renorm(a.x), renorm(a.y)}; }
-// a + s c with a binary32 correction
-__device__ __forceinline__ dfl add_f(dfl a, float c) {
-  float s, e;
-  dfl_two_sum(a.hi, c, s, e);
-  return dfl_fast(s, __fadd_rn(a.lo, e));
-}
-__device__ __forceinline__ cdfl add_f(const cdfl& a, cxf c) { return {add_f(a.x, c.x), add_f(a.y, c.y)}; }
-__device__ __forceinline__ cdfl from_f(cxf v) { return {dfl(v.x, 0.f), dfl(v.y, 0.f)}; }
-__device__ __forceinline__ cxf scaled(float s, const cdfl& a) { return {s * (a.x.hi + a.x.lo), s * (a.y.hi + a.y.lo)}; }
-__device__ __forceinline__ dfl dfl_of(double v) { return d2dfl_bits(v); }
+static_assert(DY_MAXP == 16, "mix_sum adds the ranks over 16 lanes");
 
 // ---------------------------------------------------------------- interface solve
 template <typename R>
@@ -625,6 +576,7 @@ __device__ __noinline__ MixSolve<R> mix_cocg(const Geo& g, const Bufs& b, const 
   const C* plo = i > 0 ? P + o - A : nullptr;
   C* phi = P + o;
   const R t = ctx.t;
+  const bool act = has && ((int)threadIdx.x & ~31) < A;   // this warp has interface sites
   auto precond = [&](const C* r, C* z) {
     if (g.lpre) lpre_apply<R>(g, b, vs, i, r, z, B1);
     else precond_apply<R>(g, b, vs, i, r, z);
@@ -646,9 +598,10 @@ __device__ __noinline__ MixSolve<R> mix_cocg(const Geo& g, const Bufs& b, const 
     v3[0] = rz.x;
     v3[1] = rz.y;
   }
-  mix_sum<R, WF, 3>(cl, phase, p, v3);      // also: P of the neighbour layers is final
-  C rho = {v3[0], v3[1]};
-  const R bn = v3[2];
+  double s3[3];
+  mix_sum<R, WF>(cl, phase, p, v3, s3, act);   // also: P of the neighbour layers is final
+  C rho = {(R)s3[0], (R)s3[1]};
+  const R bn = (R)s3[2];
   const R tol2 = (R)(g.krylov_tol * g.krylov_tol);
   if (bn > 0 || bn != bn) {
     for (;;) {
@@ -674,8 +627,9 @@ __device__ __noinline__ MixSolve<R> mix_cocg(const Geo& g, const Bufs& b, const 
           v2[0] = rz.x;
           v2[1] = rz.y;
         }
-        mix_sum<R, WF, 2>(cl, phase, p, v2);
-        const C rn = {v2[0], v2[1]}, beta = cdiv(rn, rho);
+        double s2[2];
+        mix_sum<R, WF>(cl, phase, p, v2, s2, act);
+        const C rn = {(R)s2[0], (R)s2[1]}, beta = cdiv(rn, rho);
         rho = rn;
         if (has)
           for (int a = threadIdx.x; a < A; a += nt) phi[a] = Z[a] + beta * phi[a];
@@ -713,8 +667,9 @@ __device__ __noinline__ MixSolve<R> mix_cocg(const Geo& g, const Bufs& b, const 
         v2[0] = ps.x;
         v2[1] = ps.y;
       }
-      mix_sum<R, WF, 2>(cl, phase, p, v2);
-      out.alpha = cdiv(rho, C{v2[0], v2[1]});
+      double s2[2], s1[1];
+      mix_sum<R, WF>(cl, phase, p, v2, s2, act);
+      out.alpha = cdiv(rho, C{(R)s2[0], (R)s2[1]});
       R v1[1] = {0};
       if (has) {
         for (int a = threadIdx.x; a < A; a += nt) {
@@ -724,8 +679,8 @@ __device__ __noinline__ MixSolve<R> mix_cocg(const Geo& g, const Bufs& b, const 
           v1[0] += cabs2(r);
         }
       }
-      mix_sum<R, WF, 1>(cl, phase, p, v1);
-      if (v1[0] <= tol2 * bn) break;
+      mix_sum<R, WF>(cl, phase, p, v1, s1, act);
+      if ((R)s1[0] <= tol2 * bn) break;
     }
   }
   phase_ = phase;
@@ -733,18 +688,25 @@ __device__ __noinline__ MixSolve<R> mix_cocg(const Geo& g, const Bufs& b, const 
 }
 
 // ---------------------------------------------------------------- the X-matvec
+// r + mt x, mt = -t
+__device__ __forceinline__ void sub_scaled(cxd& r, double mt, cxd x) {
+  r.x = fma(mt, x.x, r.x);
+  r.y = fma(mt, x.y, r.y);
+}
+__device__ __forceinline__ void add_norm(double& n, cxd r) { n = fma(r.x, r.x, fma(r.y, r.y, n)); }
+
 // w = blkdiag(B^-1, 0) q and u = X q = H^-1 [0; q_C - E^T w_B] (Eqs. 6-8, no
 // cancellation) are found together:
 //   w  from one sweep on q_B, u from one interface solve on q_C - E^T w_B;
 //   then, until both relative residuals are below refine_tol, the residuals
-//     r_w = q_B - B w,   r_u = [0; q_C - E^T w] - H u       (double-float)
+//     r_w = q_B - B w,   r_u = [0; q_C - E^T w] - H u       (binary64)
 //   and one correction: a sweep on both subdomain residuals gives d_w and
 //   z = B^-1 r_u, an interface solve on r_u,C - E^T (d_w + z) gives d_y, and
 //   w += d_w,  u_B += z - B^-1 E d_y,  u_C += d_y.
 // The residual pass writes its rows straight into the row buffers in complex64,
 // scaled by an estimate of their size (1e6 over the last residual's norm: about
 // what a complex64 correction leaves); the scale only keeps the values inside
-// the binary32 range, and the norms are measured on the scaled rows.
+// the binary32 range.
 template <int WF, bool ROWS>
 __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
     k_xmatvec_m(const __grid_constant__ Geo g, const __grid_constant__ Bufs b, int j, int ncols) {
@@ -778,13 +740,13 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
   const cdfl* qs = reinterpret_cast<const cdfl*>(qd);
   const bool split = g.qsplit != 0;
   const size_t qo = (size_t)i * nsub, lo = (size_t)g.ifc_off + (size_t)i * A, o = (size_t)i * A;
-  cdfl* u = reinterpret_cast<cdfl*>(b.u + (size_t)vs * Ndd);       // double-floats until the last pass
-  cdfl* wv = reinterpret_cast<cdfl*>(b.v1 + (size_t)vs * Ndd);     // w_B
-  cdfl* rc = reinterpret_cast<cdfl*>(b.v2 + (size_t)vs * Ndd) + lo;   // interface residual
-  cdfl *us = u + qo, *ws = wv + qo;
-  const cdfl* hd = reinterpret_cast<const cdfl*>(b.hdiag + (size_t)f * Ndd);
-  const cdfl* hs = hd + qo;
-  const dfl td = dfl_of(g.t);
+  cxd* u = b.u + (size_t)vs * Ndd;
+  cxd* wv = b.v1 + (size_t)vs * Ndd;                               // w_B
+  cxd* rc = b.v2 + (size_t)vs * Ndd + lo;                          // interface residual
+  cxd *us = u + qo, *ws = wv + qo;
+  const cxd* hd = b.hdiag + (size_t)f * Ndd;
+  const cxd* hs = hd + qo;
+  const double mt = -g.t;
   const float tf = cx.t;
   cxf* Bv = ifv_ptr<float>(g, b, vs, IF_B) + o;
   cxf* X = ifv_ptr<float>(g, b, vs, IF_X) + o;
@@ -792,28 +754,25 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
   cxf* blo = bnd_ptr<float>(g, b, vs, i, 0);
   cxf* bhi = bnd_ptr<float>(g, b, vs, i, 1);
   const cxf* bnx = has ? bnd_ptr<float>(g, b, vs, i + 1, 0) : nullptr;
-  auto ldq = [&](size_t k) -> cdfl { return split ? qs[k] : csplit(qd[k]); };
+  auto ldq = [&](size_t k) -> cxd { return split ? cwiden(qs[k]) : qd[k]; };
 
   // ---- w_0 = B^-1 q_B
-  Norm3 qn;                                // ||q_B||^2 of this subdomain
+  double qn = 0.0;                         // ||q_B||^2 of this subdomain
   for (int e = tid, jj = j_0; e < nsub; e += nt) {
     cxf v = {0.f, 0.f};
     if (jj < w) {
-      const cdfl q = ldq(qo + e);
-      v = cxf{q.x.hi, q.y.hi};
-      qn.add(v);
+      const cxd q = ldq(qo + e);
+      v = c2f_bits(q);
+      add_norm(qn, q);
     }
     B0[e] = v;
     jj += dj;
     if (jj >= W) jj -= W;
   }
   if (has)
-    for (int a = tid; a < A; a += nt) {
-      const cdfl d = hd[lo + a];
-      dC[a] = cxf{d.x.hi, d.y.hi};
-    }
+    for (int a = tid; a < A; a += nt) dC[a] = c2f_bits(hd[lo + a]);
   mix_sweep<float, WF, 1, ROWS>(cx, ms, 0);
-  for (int e = tid; e < nsub; e += nt) ws[e] = from_f(B0[e]);      // zero on the padding
+  for (int e = tid; e < nsub; e += nt) ws[e] = c2d_bits(B0[e]);    // zero on the padding
   for (int e = tid; e < A; e += nt) {
     const int jj = T == 1 ? 0 : e / Lx, s = e - jj * Lx;
     blo[e] = B0[s * W + jj];
@@ -822,28 +781,25 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
   cl.sync();                               // boundary rows (and w) of the neighbour subdomains are final
   double hn2, qn2;
   {
-    Norm3 h3;
+    double v[2] = {0.0, qn}, tot[2], own[2];
     if (has)
       for (int a = tid; a < A; a += nt) {
-        cdfl h = ldq(lo + a);
-        acc_sub_scaled(h, td, from_f(bhi[a]));
-        acc_sub_scaled(h, td, from_f(bnx[a]));
-        h = renorm(h);
+        cxd h = ldq(lo + a);
+        sub_scaled(h, mt, c2d_bits(bhi[a]));
+        sub_scaled(h, mt, c2d_bits(bnx[a]));
         rc[a] = h;
-        h3.add(cxf{h.x.hi, h.y.hi});
+        add_norm(v[0], h);
       }
-    float v[6] = {h3.m, h3.s, h3.b, qn.m, qn.s, qn.b}, own[6];
-    mix_sum<float, WF, 6>(cl, phase, p, v, own);
-    hn2 = Norm3::value(v[0], v[1], v[2]);
-    qn2 = Norm3::value(own[3], own[4], own[5]);
+    mix_sum<float, WF>(cl, phase, p, v, tot, true, own);
+    hn2 = tot[0];
+    qn2 = own[1];
   }
   int iters = 0, solves = 0, refines = 0, conv_all = 1;
   const double hn = sqrt(hn2), ihn = hn2 > 0.0 ? 1.0 / hn : 1.0;
-  const float ihf = (float)ihn;
   // ---- u_0 = H^-1 [0; hr]
   if (hn2 > 0.0) {
     if (has)
-      for (int a = tid; a < A; a += nt) Bv[a] = scaled(ihf, rc[a]);
+      for (int a = tid; a < A; a += nt) Bv[a] = c2f_bits(ihn * rc[a]);
     __syncthreads();
     const MixSolve<float> sv = mix_cocg<float, WF, ROWS>(g, b, cx, ms, phase, vs, false);
     iters += sv.iters;
@@ -853,67 +809,61 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
     for (int e = tid; e < nsub; e += nt) {   // zero on the padding, which the Lanczos step reads too
       cxf v = sv.iters > 0 ? sv.alpha * B1[e] : cxf{0.f, 0.f};
       if (sv.useB0) v = v - B0[e];
-      us[e] = from_f(-(hf * v));
+      us[e] = c2d_bits(-(hf * v));
     }
     if (has)
-      for (int a = tid; a < A; a += nt) u[lo + a] = from_f(hf * X[a]);
+      for (int a = tid; a < A; a += nt) u[lo + a] = c2d_bits(hf * X[a]);
   } else {
-    for (int e = tid; e < nsub; e += nt) us[e] = from_f(cxf{0.f, 0.f});
+    for (int e = tid; e < nsub; e += nt) us[e] = cxd{0, 0};
     if (has)
-      for (int a = tid; a < A; a += nt) u[lo + a] = from_f(cxf{0.f, 0.f});
+      for (int a = tid; a < A; a += nt) u[lo + a] = cxd{0, 0};
   }
   // ---- refinement of w and u together
-  const cdfl* xlo = i > 0 ? u + g.ifc_off + (size_t)(i - 1) * A : nullptr;
-  const cdfl* xhi = u + lo;
+  const cxd* xlo = i > 0 ? u + g.ifc_off + (size_t)(i - 1) * A : nullptr;
+  const cxd* xhi = u + lo;
   const double tol2 = g.refine_tol * g.refine_tol;
   double su = 1e6 * ihn, sw = qn2 > 0.0 ? 1e6 / sqrt(qn2) : 1.0;   // row scales
   double prev_u = INFINITY, prev_w = INFINITY;
   bool wdone = qn2 == 0.0;
   for (int pass = 0; pass < g.refine_max; ++pass) {
     cl.sync();                             // u and w of the neighbours are final
-    const float suf = (float)su, swf = (float)sw;
-    float nu = 0.f, nw = 0.f;
+    double v[3] = {0.0, 0.0, 0.0}, tot[3], own[3];   // ||r_u||^2, ||hr||^2, ||r_w||^2
     for (int e = tid, s = s_0, jj = j_0; e < nsub; e += nt) {
       cxf ru = {0.f, 0.f}, rw = {0.f, 0.f};
       if (jj < w) {
         const int tr = T == 1 ? 0 : jj % T, sl = T == 1 ? jj : jj / T;
-        const cdfl dv = hs[e];
+        const cxd dv = hs[e];
         const bool pl = s > 0, pr = s < Lx - 1, dl = sl > 0, dr = sl < hh - 1;
-        const cdfl zero = from_f(cxf{0.f, 0.f});
-        // the sum of x over the neighbours inside the subdomain; every load is issued
-        // before the first sum
-        auto neighbours = [&](const cdfl* x, const cdfl& lo_, const cdfl& hi_) -> cdfl {
-          cdfl n = pl ? x[e - W] : zero;
-          const cdfl n1 = pr ? x[e + W] : zero, n2 = dl ? x[e - T] : lo_, n3 = dr ? x[e + T] : hi_;
-          cdfl n4 = zero, n5 = zero;
+        const cxd zero = {0, 0};
+        // r - t (sum of x over the neighbours) - H_ii x, one fused multiply-add a term;
+        // every load is issued before the first of them
+        auto residual = [&](cxd r, const cxd* x, const cxd& lo_, const cxd& hi_) -> cxd {
+          const cxd xc = x[e], n0 = pl ? x[e - W] : zero, n1 = pr ? x[e + W] : zero;
+          const cxd n2 = dl ? x[e - T] : lo_, n3 = dr ? x[e + T] : hi_;
+          cxd n4 = zero, n5 = zero;
           if (T > 1) {
             n4 = tr > 0 ? x[e - 1] : zero;
             n5 = tr < T - 1 ? x[e + 1] : zero;
           }
-          acc_add(n, n1);
-          acc_add(n, n2);
-          acc_add(n, n3);
+          sub_scaled(r, mt, n0);
+          sub_scaled(r, mt, n1);
+          sub_scaled(r, mt, n2);
+          sub_scaled(r, mt, n3);
           if (T > 1) {
-            acc_add(n, n4);
-            acc_add(n, n5);
+            sub_scaled(r, mt, n4);
+            sub_scaled(r, mt, n5);
           }
-          return n;
+          return cfma(-dv, xc, r);
         };
         // the interface layers' u stands in for the neighbour outside the subdomain
-        const cdfl ul = !dl && xlo ? xlo[s + Lx * tr] : zero, uh = !dr && has ? xhi[s + Lx * tr] : zero;
-        const cdfl uc = us[e];
-        cdfl r = zero;
-        acc_sub_scaled(r, td, neighbours(us, ul, uh));
-        acc_sub_cmul(r, dv, uc);
-        ru = scaled(suf, r);
-        nu += cabs2(ru);
+        const cxd ul = !dl && xlo ? xlo[s + Lx * tr] : zero, uh = !dr && has ? xhi[s + Lx * tr] : zero;
+        cxd r = residual(zero, us, ul, uh);
+        ru = c2f_bits(su * r);
+        add_norm(v[0], r);
         if (!wdone) {
-          const cdfl wc = ws[e];
-          r = ldq(qo + e);
-          acc_sub_scaled(r, td, neighbours(ws, zero, zero));
-          acc_sub_cmul(r, dv, wc);
-          rw = scaled(swf, r);
-          nw += cabs2(rw);
+          r = residual(ldq(qo + e), ws, zero, zero);
+          rw = c2f_bits(sw * r);
+          add_norm(v[2], r);
         }
       }
       B0[e] = ru;
@@ -925,42 +875,39 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
         ++s;
       }
     }
-    float v[3] = {nu, 0.f, nw}, own[3];      // ||su r_u||^2, ||hr / hn||^2, ||sw r_w||^2
     if (has) {
-      const cdfl* xa = u + (size_t)(i + 1) * nsub;   // subdomain i + 1: its bottom row touches layer i
-      const cdfl* wa = wv + (size_t)(i + 1) * nsub;
+      const cxd* xa = u + (size_t)(i + 1) * nsub;    // subdomain i + 1: its bottom row touches layer i
+      const cxd* wa = wv + (size_t)(i + 1) * nsub;
       const int hi = T * (hh - 1);
       for (int a = tid; a < A; a += nt) {
         const int tr = T == 1 ? 0 : a / Lx, xx = a - tr * Lx;
         const int kb = xx * W + hi + tr, ka = xx * W + tr;
-        cdfl r = ldq(lo + a), n = ws[kb];
-        acc_add(n, wa[ka]);
-        acc_sub_scaled(r, td, n);              // hr = q_C - E^T w
-        const cxf hsc = scaled(ihf, r);
-        n = us[kb];
-        acc_add(n, xa[ka]);
-        if (xx > 0) acc_add(n, xhi[a - 1]);
-        if (xx < Lx - 1) acc_add(n, xhi[a + 1]);
-        if (tr > 0) acc_add(n, xhi[a - Lx]);
-        if (tr < T - 1) acc_add(n, xhi[a + Lx]);
-        acc_sub_scaled(r, td, n);
-        acc_sub_cmul(r, hd[lo + a], xhi[a]);
-        rc[a] = renorm(r);
-        v[0] += cabs2(scaled(suf, r));
-        v[1] += cabs2(hsc);
+        cxd r = ldq(lo + a);
+        sub_scaled(r, mt, ws[kb]);
+        sub_scaled(r, mt, wa[ka]);             // hr = q_C - E^T w
+        add_norm(v[1], r);
+        sub_scaled(r, mt, us[kb]);
+        sub_scaled(r, mt, xa[ka]);
+        if (xx > 0) sub_scaled(r, mt, xhi[a - 1]);
+        if (xx < Lx - 1) sub_scaled(r, mt, xhi[a + 1]);
+        if (tr > 0) sub_scaled(r, mt, xhi[a - Lx]);
+        if (tr < T - 1) sub_scaled(r, mt, xhi[a + Lx]);
+        r = cfma(-hd[lo + a], xhi[a], r);
+        rc[a] = r;
+        add_norm(v[0], r);
       }
     }
-    mix_sum<float, WF, 3>(cl, phase, p, v, own);
-    const double wn = (double)own[2] / (sw * sw);   // this subdomain's, which decides for its w alone
+    mix_sum<float, WF>(cl, phase, p, v, tot, true, own);
+    const double rn = tot[0], wn = own[2];   // w: this subdomain's, which decides for its w alone
     if (!wdone && (wn <= tol2 * qn2 || wn > REFINE_STALL * prev_w)) wdone = true;
     if (!wdone) prev_w = wn;
-    const double rn = (double)v[0] / (su * su);
-    const bool udone = rn <= tol2 * ((double)v[1] * hn2) || rn > REFINE_STALL * prev_u;
+    const bool udone = rn <= tol2 * tot[1] || rn > REFINE_STALL * prev_u;
     if (udone) {
       // u is done: go on only if some w of the cluster is not
       float go[1] = {!wdone && tid == 0 ? 1.f : 0.f};
-      mix_sum<float, WF, 1>(cl, phase, p, go);
-      if (go[0] == 0.f) break;
+      double any[1];
+      mix_sum<float, WF>(cl, phase, p, go, any, tid < 32);
+      if (any[0] == 0.0) break;
     }
     prev_u = rn;
     ++refines;
@@ -971,7 +918,7 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
     const double isu = 1.0 / su;
     const float isuf = (float)isu, iswf = (float)(1.0 / sw), ratio = (float)(su / sw);
     if (wgo)
-      for (int e = tid; e < nsub; e += nt) ws[e] = add_f(ws[e], iswf * B1[e]);
+      for (int e = tid; e < nsub; e += nt) ws[e] = ws[e] + c2d_bits(iswf * B1[e]);
     for (int e = tid; e < A; e += nt) {
       const int jj = T == 1 ? 0 : e / Lx, s = e - jj * Lx;
       const int k0 = s * W + jj, k1 = s * W + (w - T) + jj;
@@ -980,7 +927,7 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
     }
     cl.sync();                             // boundary rows of the neighbours
     if (has)
-      for (int a = tid; a < A; a += nt) Bv[a] = scaled(suf, rc[a]) - tf * (bhi[a] + bnx[a]);
+      for (int a = tid; a < A; a += nt) Bv[a] = c2f_bits(su * rc[a]) - tf * (bhi[a] + bnx[a]);
     __syncthreads();
     const MixSolve<float> sv = mix_cocg<float, WF, ROWS>(g, b, cx, ms, phase, vs, true);
     iters += sv.iters;
@@ -989,20 +936,12 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
     for (int e = tid; e < nsub; e += nt) {
       cxf v2 = B0[e];
       if (sv.iters > 0) v2 = v2 - sv.alpha * B1[e];
-      us[e] = add_f(us[e], isuf * v2);
+      us[e] = us[e] + c2d_bits(isuf * v2);
     }
     if (has)
-      for (int a = tid; a < A; a += nt) u[lo + a] = add_f(u[lo + a], isuf * X[a]);
+      for (int a = tid; a < A; a += nt) u[lo + a] = u[lo + a] + c2d_bits(isuf * X[a]);
     if (rn > 0.0) su = 1e6 / sqrt(rn);
     if (wgo && prev_w > 0.0) sw = 1e6 / sqrt(prev_w);
-  }
-  // ---- u to binary64 (in place: an entry is 16 bytes in both forms; the residuals that
-  // read this u were followed by a cluster barrier)
-  {
-    cxd* ud = b.u + (size_t)vs * Ndd;
-    for (int e = tid; e < nsub; e += nt) ud[qo + e] = cwiden(us[e]);
-    if (has)
-      for (int a = tid; a < A; a += nt) ud[lo + a] = cwiden(u[lo + a]);
   }
   mix_drain<float, WF, ROWS>(cx, ms);
   __syncthreads();
