@@ -136,6 +136,41 @@ __device__ __forceinline__ double f2d_bits(float f) {
   if (ef == 0xffu) hi = sign | 0x7ff00000u | (m >> 3), lo = m << 29;
   return __longlong_as_double((long long)(((unsigned long long)hi << 32) | lo));
 }
+// The same with a factor of 2^k (|k| up to some thousands), rounded once and with no
+// intermediate value that could leave the range: d 2^k in binary32, f 2^k in binary64.
+// Results beyond either end become a signed zero or infinity, as above.
+__device__ __forceinline__ float d2f_scaled(double d, int k) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+  const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
+  const unsigned sign = hi & 0x80000000u;
+  const int ed = (int)((hi >> 20) & 0x7ffu);
+  const int e = ed - 1023 + 127 + k;
+  const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const unsigned rest = lo & 0x1fffffffu;
+  unsigned out = ((unsigned)e << 23) | m;
+  out += (rest > 0x10000000u || (rest == 0x10000000u && (m & 1u))) ? 1u : 0u;
+  if (e >= 255) out = 0x7f800000u;
+  if (e <= 0 || ed == 0) out = 0u;
+  if (ed == 0x7ff) out = 0x7f800000u | (((hi & 0xfffffu) | lo) ? 0x400000u : 0u);
+  return __uint_as_float(sign | out);
+}
+__device__ __forceinline__ double f2d_scaled(float f, int k) {
+  const unsigned u = __float_as_uint(f);
+  const unsigned sign = u & 0x80000000u;
+  const unsigned ef = (u >> 23) & 0xffu, m = u & 0x7fffffu;
+  const int e = (int)ef + 1023 - 127 + k;
+  unsigned hi = sign | ((unsigned)e << 20) | (m >> 3), lo = m << 29;
+  if (e <= 0 || ef == 0u) hi = sign, lo = 0u;
+  if (e >= 0x7ff) hi = sign | 0x7ff00000u, lo = 0u;
+  if (ef == 0xffu) hi = sign | 0x7ff00000u | (m >> 3), lo = m << 29;
+  return __longlong_as_double((long long)(((unsigned long long)hi << 32) | lo));
+}
+// e with 2^e <= sqrt(n2) < 2^(e+1), n2 >= 0; -512 for zero and subnormals, 512 for inf and NaN
+__device__ __forceinline__ int norm_exp(double n2) {
+  return ((int)(((unsigned)__double2hiint(n2) >> 20) & 0x7ffu) - 1023) >> 1;
+}
+// 2^e, -126 <= e <= 127
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 // binary64 -> double-float by integer operations (no binary64 instruction):
 // hi takes the leading 24 significant bits (truncated: the exponent rebiased in
 // place, then sign, exponent and the top 23 mantissa bits funnel-shifted into
@@ -172,6 +207,8 @@ __device__ __forceinline__ cxd cwiden(const cdfl& a) { return {dfl2d_bits(a.x), 
 
 __device__ __forceinline__ cxf c2f_bits(cxd a) { return {d2f_bits(a.x), d2f_bits(a.y)}; }
 __device__ __forceinline__ cxd c2d_bits(cxf a) { return {f2d_bits(a.x), f2d_bits(a.y)}; }
+__device__ __forceinline__ cxf c2f_scaled(cxd a, int k) { return {d2f_scaled(a.x, k), d2f_scaled(a.y, k)}; }
+__device__ __forceinline__ cxd c2d_scaled(cxf a, int k) { return {f2d_scaled(a.x, k), f2d_scaled(a.y, k)}; }
 
 // ---------------------------------------------------------------- geometry
 struct Geo {

@@ -537,6 +537,26 @@ __device__ __forceinline__ void mix_sum(cg::cluster_group& cl, int& phase, int p
 }
 static_assert(DY_MAXP == 16, "mix_sum adds the ranks over 16 lanes");
 
+// Sum of v over the CTA in binary64 (every thread gets it).
+template <typename R, int WF>
+__device__ __forceinline__ double cta_sum(double v) {
+  MixSmem<R, WF>& sm = mix_sm<R, WF>();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  constexpr int NW = Mix<R, WF>::NT / 32;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) sm.wred[wid] = v;
+  __syncthreads();
+  if (wid == 0) {
+    double s = lane < NW ? sm.wred[lane] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) sm.res[0] = s;
+  }
+  __syncthreads();
+  return sm.res[0];
+}
+
 // ---------------------------------------------------------------- interface solve
 template <typename R>
 struct MixSolve {
@@ -550,6 +570,10 @@ struct MixSolve {
 // as B0 - alpha B1: each iteration but the last is folded into B0, the last one
 // is the caller's.  keep0: B0 holds a vector to add to (else it counts as zero).
 // IF_B is complete (a barrier after its writers) on entry.
+// In binary32 IF_B may have any size: its first dot products are binary64, and from
+// there the iteration runs on IF_B 2^kc with a norm of about 1 (the squares of its
+// dot products would leave the range at 1e-23 and 1e19); alpha carries the factor
+// 2^-kc back, so y and B^-1 E y have IF_B's own scale.
 template <typename R, int WF, bool ROWS>
 __device__ __noinline__ MixSolve<R> mix_cocg(const Geo& g, const Bufs& b, const MixCtx<R, WF, ROWS>& ctx, MixState<R>& st,
                                           int& phase_, int vs, bool keep0) {
@@ -584,24 +608,46 @@ __device__ __noinline__ MixSolve<R> mix_cocg(const Geo& g, const Bufs& b, const 
   MixSolve<R> out = {keep0, {0, 0}, 0, 1};
   if (has) precond(Bv, Z);
   __syncthreads();
-  R v3[3] = {0, 0, 0};
+  constexpr bool f32 = sizeof(R) == 4;
+  auto wide = [](C v) -> cxd {
+    if constexpr (f32) return c2d_bits(v);
+    else return v;
+  };
+  double v3[3] = {0, 0, 0};
   if (has) {
-    C rz = {0, 0};
+    cxd rz = {0, 0};
     for (int a = threadIdx.x; a < A; a += nt) {
       const C zz = Z[a], r = Bv[a];
       X[a] = C{0, 0};
-      Rv[a] = r;
+      if (!f32) Rv[a] = r;
       phi[a] = zz;
-      rz = cfma(r, zz, rz);
-      v3[2] += cabs2(r);
+      rz = cfma(wide(r), wide(zz), rz);
+      v3[2] += cabs2(wide(r));
     }
     v3[0] = rz.x;
     v3[1] = rz.y;
   }
   double s3[3];
   mix_sum<R, WF>(cl, phase, p, v3, s3, act);   // also: P of the neighbour layers is final
-  C rho = {(R)s3[0], (R)s3[1]};
-  const R bn = (R)s3[2];
+  C rho;
+  R bn, fs = 1, back = 1;                // 2^kc, 2^-kc
+  if constexpr (f32) {
+    const int kc = min(126, max(-126, -norm_exp(s3[2])));
+    fs = pow2f(kc);
+    back = pow2f(-kc);
+    rho = C{d2f_scaled(s3[0], 2 * kc), d2f_scaled(s3[1], 2 * kc)};
+    bn = d2f_scaled(s3[2], 2 * kc);
+    if (has)
+      for (int a = threadIdx.x; a < A; a += nt) Rv[a] = fs * Bv[a];
+  } else {
+    rho = C{s3[0], s3[1]};
+    bn = s3[2];
+  }
+  R pf = fs;                             // P's factor: the first direction is stored unscaled
+  auto scaled = [](R c, C v) -> C {
+    if constexpr (f32) return c * v;
+    else return v;
+  };
   const R tol2 = (R)(g.krylov_tol * g.krylov_tol);
   if (bn > 0 || bn != bn) {
     for (;;) {
@@ -632,15 +678,17 @@ __device__ __noinline__ MixSolve<R> mix_cocg(const Geo& g, const Bufs& b, const 
         const C rn = {(R)s2[0], (R)s2[1]}, beta = cdiv(rn, rho);
         rho = rn;
         if (has)
-          for (int a = threadIdx.x; a < A; a += nt) phi[a] = Z[a] + beta * phi[a];
+          for (int a = threadIdx.x; a < A; a += nt) phi[a] = Z[a] + beta * scaled(pf, phi[a]);
+        pf = 1;
         cl.sync();                       // P of the neighbour layers is final
       }
       ++out.iters;
       // B1 = E p
+      const R tp = t * pf;
       for (int e = threadIdx.x, s = e / W, j = e - s * W; e < nsub; e += nt) {
         C u = {0, 0};
-        if (plo && j < T) u = u + t * plo[s + Lx * j];
-        if (has && j >= w - T && j < w) u = u + t * phi[s + Lx * (j - (w - T))];
+        if (plo && j < T) u = u + tp * plo[s + Lx * j];
+        if (has && j >= w - T && j < w) u = u + tp * phi[s + Lx * (j - (w - T))];
         B1[e] = u;
         s += ds;
         j += dj;
@@ -660,21 +708,22 @@ __device__ __noinline__ MixSolve<R> mix_cocg(const Geo& g, const Bufs& b, const 
       if (has) {
         C ps = {0, 0};
         for (int a = threadIdx.x; a < A; a += nt) {
-          const C sp = layer_C_apply<R>(g, dC, phi, a) - t * (bhi[a] + bnx[a]);
+          const C sp = scaled(pf, layer_C_apply<R>(g, dC, phi, a)) - t * (bhi[a] + bnx[a]);
           SP[a] = sp;
-          ps = cfma(phi[a], sp, ps);
+          ps = cfma(scaled(pf, phi[a]), sp, ps);
         }
         v2[0] = ps.x;
         v2[1] = ps.y;
       }
       double s2[2], s1[1];
       mix_sum<R, WF>(cl, phase, p, v2, s2, act);
-      out.alpha = cdiv(rho, C{(R)s2[0], (R)s2[1]});
+      const C alpha = cdiv(rho, C{(R)s2[0], (R)s2[1]});
+      out.alpha = scaled(back, alpha);
       R v1[1] = {0};
       if (has) {
         for (int a = threadIdx.x; a < A; a += nt) {
-          X[a] = X[a] + out.alpha * phi[a];
-          const C r = Rv[a] - out.alpha * SP[a];
+          X[a] = X[a] + out.alpha * scaled(pf, phi[a]);
+          const C r = Rv[a] - alpha * SP[a];
           Rv[a] = r;
           v1[0] += cabs2(r);
         }
@@ -704,9 +753,17 @@ __device__ __forceinline__ void add_norm(double& n, cxd r) { n = fma(r.x, r.x, f
 //   z = B^-1 r_u, an interface solve on r_u,C - E^T (d_w + z) gives d_y, and
 //   w += d_w,  u_B += z - B^-1 E d_y,  u_C += d_y.
 // The residual pass writes its rows straight into the row buffers in complex64,
-// scaled by an estimate of their size (1e6 over the last residual's norm: about
-// what a complex64 correction leaves); the scale only keeps the values inside
-// the binary32 range.
+// scaled by an estimate of their size (2^20 over the last residual's norm: about
+// what a complex64 correction leaves).  The scale only keeps the values inside the
+// binary32 range, and must do so for any q: a vector local to one strip reaches the
+// others and the interface 30 and more decades down, and a scale held as a binary32
+// number overflows there (at a norm of 3e-26 in the second pass).  So every scale is an
+// exponent, applied in the conversions between binary64 and binary32: kq for q_B and kw
+// for r_w, this subdomain's own, ku for r_u.  Where the subdomain and the interface
+// differ in size, kw is kept within 2^60 below ku, so that the two corrections add up on
+// the boundary rows in binary32; ku stays within 2^120 of q's own scale, which makes
+// that possible.  An interface right-hand side below 2^-120 ||q|| counts as zero: a
+// Lanczos vector's entries, and 1 / beta, end at the binary32 range.
 template <int WF, bool ROWS>
 __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
     k_xmatvec_m(const __grid_constant__ Geo g, const __grid_constant__ Bufs b, int j, int ncols) {
@@ -756,14 +813,23 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
   const cxf* bnx = has ? bnd_ptr<float>(g, b, vs, i + 1, 0) : nullptr;
   auto ldq = [&](size_t k) -> cxd { return split ? cwiden(qs[k]) : qd[k]; };
 
+  // the neighbour subdomain's w at layer i, and the two rows next to it
+  const cxd* wa = wv + (size_t)(i + 1) * nsub;
+  const int top = T * (hh - 1);
+  auto layer_rows = [&](int a, int& kb, int& ka) {
+    const int tr = T == 1 ? 0 : a / Lx, xx = a - tr * Lx;
+    kb = xx * W + top + tr;
+    ka = xx * W + tr;
+  };
+
   // ---- w_0 = B^-1 q_B
-  double qn = 0.0;                         // ||q_B||^2 of this subdomain
+  double qn2 = 0.0;                        // ||q_B||^2 of this subdomain
   for (int e = tid, jj = j_0; e < nsub; e += nt) {
     cxf v = {0.f, 0.f};
     if (jj < w) {
       const cxd q = ldq(qo + e);
       v = c2f_bits(q);
-      add_norm(qn, q);
+      add_norm(qn2, q);
     }
     B0[e] = v;
     jj += dj;
@@ -771,48 +837,60 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
   }
   if (has)
     for (int a = tid; a < A; a += nt) dC[a] = c2f_bits(hd[lo + a]);
-  mix_sweep<float, WF, 1, ROWS>(cx, ms, 0);
-  for (int e = tid; e < nsub; e += nt) ws[e] = c2d_bits(B0[e]);    // zero on the padding
-  for (int e = tid; e < A; e += nt) {
-    const int jj = T == 1 ? 0 : e / Lx, s = e - jj * Lx;
-    blo[e] = B0[s * W + jj];
-    bhi[e] = B0[s * W + (w - T) + jj];
+  qn2 = cta_sum<float, WF>(qn2);
+  int kq = -norm_exp(qn2);
+  if (kq >= -8 && kq <= 8) {               // the usual size of a Lanczos vector: as it is
+    kq = 0;
+  } else {
+    for (int e = tid, jj = j_0; e < nsub; e += nt) {
+      if (jj < w) B0[e] = c2f_scaled(ldq(qo + e), kq);
+      jj += dj;
+      if (jj >= W) jj -= W;
+    }
   }
-  cl.sync();                               // boundary rows (and w) of the neighbour subdomains are final
-  double hn2, qn2;
+  mix_sweep<float, WF, 1, ROWS>(cx, ms, 0);
+  for (int e = tid; e < nsub; e += nt) ws[e] = c2d_scaled(B0[e], -kq);   // zero on the padding
+  cl.sync();                               // w of the neighbour subdomains is final
+  double hn2, qa2;                         // ||hr||^2, ||q||^2 (the whole vector)
   {
-    double v[2] = {0.0, qn}, tot[2], own[2];
+    double v[2] = {0.0, tid == 0 ? qn2 : 0.0}, tot[2];
     if (has)
       for (int a = tid; a < A; a += nt) {
+        int kb, ka;
+        layer_rows(a, kb, ka);
         cxd h = ldq(lo + a);
-        sub_scaled(h, mt, c2d_bits(bhi[a]));
-        sub_scaled(h, mt, c2d_bits(bnx[a]));
+        add_norm(v[1], h);
+        sub_scaled(h, mt, ws[kb]);
+        sub_scaled(h, mt, wa[ka]);
         rc[a] = h;
         add_norm(v[0], h);
       }
-    mix_sum<float, WF>(cl, phase, p, v, tot, true, own);
+    mix_sum<float, WF>(cl, phase, p, v, tot);
     hn2 = tot[0];
-    qn2 = own[1];
+    qa2 = tot[1];
   }
   int iters = 0, solves = 0, refines = 0, conv_all = 1;
-  const double hn = sqrt(hn2), ihn = hn2 > 0.0 ? 1.0 / hn : 1.0;
+  constexpr int K0 = 20, KB = 120;
+  constexpr double TINY2 = 0x1p-240;       // (2^-KB)^2
+  const int ktop = K0 - norm_exp(qa2) + KB;
+  const bool live = !(hn2 <= TINY2 * qa2);
   // ---- u_0 = H^-1 [0; hr]
-  if (hn2 > 0.0) {
+  if (live) {
+    const int kh = -norm_exp(hn2);
     if (has)
-      for (int a = tid; a < A; a += nt) Bv[a] = c2f_bits(ihn * rc[a]);
+      for (int a = tid; a < A; a += nt) Bv[a] = c2f_scaled(rc[a], kh);
     __syncthreads();
     const MixSolve<float> sv = mix_cocg<float, WF, ROWS>(g, b, cx, ms, phase, vs, false);
     iters += sv.iters;
     conv_all &= sv.conv;
     ++solves;
-    const float hf = (float)hn;
     for (int e = tid; e < nsub; e += nt) {   // zero on the padding, which the Lanczos step reads too
       cxf v = sv.iters > 0 ? sv.alpha * B1[e] : cxf{0.f, 0.f};
       if (sv.useB0) v = v - B0[e];
-      us[e] = c2d_bits(-(hf * v));
+      us[e] = c2d_scaled(-v, -kh);
     }
     if (has)
-      for (int a = tid; a < A; a += nt) u[lo + a] = c2d_bits(hf * X[a]);
+      for (int a = tid; a < A; a += nt) u[lo + a] = c2d_scaled(X[a], -kh);
   } else {
     for (int e = tid; e < nsub; e += nt) us[e] = cxd{0, 0};
     if (has)
@@ -822,10 +900,10 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
   const cxd* xlo = i > 0 ? u + g.ifc_off + (size_t)(i - 1) * A : nullptr;
   const cxd* xhi = u + lo;
   const double tol2 = g.refine_tol * g.refine_tol;
-  double su = 1e6 * ihn, sw = qn2 > 0.0 ? 1e6 / sqrt(qn2) : 1.0;   // row scales
+  int ku = min(K0 - norm_exp(hn2), ktop), kw = max(K0 - norm_exp(qn2), ku - KB / 2);   // row scales
   double prev_u = INFINITY, prev_w = INFINITY;
   bool wdone = qn2 == 0.0;
-  for (int pass = 0; pass < g.refine_max; ++pass) {
+  for (int pass = 0; live && pass < g.refine_max; ++pass) {
     cl.sync();                             // u and w of the neighbours are final
     double v[3] = {0.0, 0.0, 0.0}, tot[3], own[3];   // ||r_u||^2, ||hr||^2, ||r_w||^2
     for (int e = tid, s = s_0, jj = j_0; e < nsub; e += nt) {
@@ -858,11 +936,11 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
         // the interface layers' u stands in for the neighbour outside the subdomain
         const cxd ul = !dl && xlo ? xlo[s + Lx * tr] : zero, uh = !dr && has ? xhi[s + Lx * tr] : zero;
         cxd r = residual(zero, us, ul, uh);
-        ru = c2f_bits(su * r);
+        ru = c2f_scaled(r, ku);
         add_norm(v[0], r);
         if (!wdone) {
           r = residual(ldq(qo + e), ws, zero, zero);
-          rw = c2f_bits(sw * r);
+          rw = c2f_scaled(r, kw);
           add_norm(v[2], r);
         }
       }
@@ -877,11 +955,10 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
     }
     if (has) {
       const cxd* xa = u + (size_t)(i + 1) * nsub;    // subdomain i + 1: its bottom row touches layer i
-      const cxd* wa = wv + (size_t)(i + 1) * nsub;
-      const int hi = T * (hh - 1);
       for (int a = tid; a < A; a += nt) {
         const int tr = T == 1 ? 0 : a / Lx, xx = a - tr * Lx;
-        const int kb = xx * W + hi + tr, ka = xx * W + tr;
+        int kb, ka;
+        layer_rows(a, kb, ka);
         cxd r = ldq(lo + a);
         sub_scaled(r, mt, ws[kb]);
         sub_scaled(r, mt, wa[ka]);             // hr = q_C - E^T w
@@ -915,10 +992,9 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
     const bool wgo = !wdone;
     if (wgo) mix_sweep<float, WF, 2, ROWS>(cx, ms, 0);
     else mix_sweep<float, WF, 1, ROWS>(cx, ms, 0);
-    const double isu = 1.0 / su;
-    const float isuf = (float)isu, iswf = (float)(1.0 / sw), ratio = (float)(su / sw);
+    const float ratio = pow2f(max(ku - kw, -126));   // at most 2^60; below 2^-126 it adds nothing
     if (wgo)
-      for (int e = tid; e < nsub; e += nt) ws[e] = ws[e] + c2d_bits(iswf * B1[e]);
+      for (int e = tid; e < nsub; e += nt) ws[e] = ws[e] + c2d_scaled(B1[e], -kw);
     for (int e = tid; e < A; e += nt) {
       const int jj = T == 1 ? 0 : e / Lx, s = e - jj * Lx;
       const int k0 = s * W + jj, k1 = s * W + (w - T) + jj;
@@ -927,7 +1003,7 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
     }
     cl.sync();                             // boundary rows of the neighbours
     if (has)
-      for (int a = tid; a < A; a += nt) Bv[a] = c2f_bits(su * rc[a]) - tf * (bhi[a] + bnx[a]);
+      for (int a = tid; a < A; a += nt) Bv[a] = c2f_scaled(rc[a], ku) - tf * (bhi[a] + bnx[a]);
     __syncthreads();
     const MixSolve<float> sv = mix_cocg<float, WF, ROWS>(g, b, cx, ms, phase, vs, true);
     iters += sv.iters;
@@ -936,12 +1012,12 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
     for (int e = tid; e < nsub; e += nt) {
       cxf v2 = B0[e];
       if (sv.iters > 0) v2 = v2 - sv.alpha * B1[e];
-      us[e] = us[e] + c2d_bits(isuf * v2);
+      us[e] = us[e] + c2d_scaled(v2, -ku);
     }
     if (has)
-      for (int a = tid; a < A; a += nt) u[lo + a] = u[lo + a] + c2d_bits(isuf * X[a]);
-    if (rn > 0.0) su = 1e6 / sqrt(rn);
-    if (wgo && prev_w > 0.0) sw = 1e6 / sqrt(prev_w);
+      for (int a = tid; a < A; a += nt) u[lo + a] = u[lo + a] + c2d_scaled(X[a], -ku);
+    ku = min(K0 - norm_exp(rn), ktop);
+    kw = max(K0 - norm_exp(wgo ? prev_w : qn2), ku - KB / 2);
   }
   mix_drain<float, WF, ROWS>(cx, ms);
   __syncthreads();

@@ -5,7 +5,7 @@ import pytest
 from oracle import dyson_oracle as O
 from paper_1102_3137_gb300 import dyson as D
 from paper_1102_3137_gb300 import inputs as I
-from parity_util import OPEN, plan_for, wl
+from parity_util import OPEN, TOL_FP64, TOL_MIXED, plan_for, wl
 
 pytestmark = pytest.mark.gpu
 
@@ -59,4 +59,84 @@ def test_refinement_reaches_binary64_rounding(L, p, eta):
     for k in range(2):
         y, s = stencil(w.L, w.t, O.axis_diagonal(omega[k], w.mu, V, sigma[k], eta), u[k])
         assert np.max(np.abs(y[sub])) <= 10 * 2.0 ** -53 * np.max(s[sub])
+    pl.close()
+
+
+def local_X(w, omega_k, V, sigma_k):
+    """q -> X q = H^-1 [0; q_C - E^T w_B] with w = B^-1 q, without the cancellation of
+    Eq. 8: accurate relative to max |u| also where u lies 30 decades below q."""
+    z = O.dyson_diagonal(omega_k, w.mu, V, sigma_k)
+    subs, full = O.Subdomains(w.L, OPEN, w.t, z, w.p), O.FullLattice(w.L, OPEN, w.t, z)
+    mask = interface_mask(w.L, w.p)
+
+    def X(q):
+        r = q - O.apply_H(w.L, OPEN, w.t, w.mu, V, sigma_k, omega_k, subs.solve(q))
+        return full.solve(np.where(mask, r, 0))
+
+    return subs, X
+
+
+def vector(kind, w, rng):
+    x, y = np.arange(w.N) % w.L[0], np.arange(w.N) // w.L[0]
+    if kind[0] == "site":                      # a point source; its interface right-hand side is ~1e-29
+        return ((x == kind[1]) & (y == kind[2])).astype(complex)
+    if kind[0] == "gauss":                     # tails of 1e-30 and less in the far strips
+        return np.exp(-((x - kind[1]) ** 2 + (y - kind[2]) ** 2) / 18.0).astype(complex)
+    return kind[1] * (rng.normal(size=w.N) + 1j * rng.normal(size=w.N))
+
+
+@pytest.mark.parametrize("precision,tol", [(D.DYSON_FP64, 1e-11), (D.DYSON_MIXED, 1e-9)])
+@pytest.mark.parametrize("kind", [("site", 64, 8), ("site", 4, 15), ("gauss", 40, 50), ("dense", 1e-20), ("dense", 1e20)])
+def test_xmatvec_of_small_and_local_vectors(kind, precision, tol):
+    """The trap workload's lowest frequencies on 128^2, p = 4; the bounds are those of
+    dense vectors of norm ~1 in the other parity tests."""
+    w = wl((128, 128), 4, 4, K=2, beta=20.0)
+    omega, V, sigma, _ = I.make_inputs(w)
+    q = vector(kind, w, np.random.default_rng(5))
+    pl = plan_for(w, precision)
+    qs = np.stack([q, q])
+    u = np.zeros_like(qs)
+    D.dyson_xmatvec(pl.handle, 2, omega, V, sigma, qs, u)
+    for k in range(2):
+        ref = local_X(w, omega[k], V, sigma[k])[1](q)
+        assert np.all(np.isfinite(u[k]))
+        assert np.max(np.abs(u[k] - ref)) <= tol * np.max(np.abs(ref))
+    pl.close()
+
+
+@pytest.mark.parametrize("L,p", [((40, 33), 2), ((64, 129), 2)])     # W = 16 and 64
+def test_xmatvec_of_a_vector_on_one_strip(L, p):
+    """q is zero, or 1e-25 and 1e-35 of the rest, on the second strip."""
+    w = wl(L, p, 4, K=3)
+    omega, V, sigma, _ = I.make_inputs(w)
+    rng = np.random.default_rng(6)
+    q = rng.normal(size=w.N) + 1j * rng.normal(size=w.N)
+    y = np.arange(w.N) // w.L[0]
+    qs = np.stack([np.where(y > w.L[1] // 2, f, 1.0) * q for f in (0.0, 1e-25, 1e-35)])
+    pl = plan_for(w, D.DYSON_MIXED)
+    u = np.zeros_like(qs)
+    D.dyson_xmatvec(pl.handle, 3, omega, V, sigma, qs, u)
+    for k in range(3):
+        ref = local_X(w, omega[k], V, sigma[k])[1](qs[k])
+        assert np.max(np.abs(u[k] - ref)) <= 1e-9 * np.max(np.abs(ref))
+    pl.close()
+
+
+@pytest.mark.parametrize("precision,tol", [(D.DYSON_FP64, TOL_FP64), (D.DYSON_MIXED, TOL_MIXED)])
+@pytest.mark.parametrize("site", [(64, 8), (64, 28)])
+def test_solve_from_a_unit_start_vector(site, precision, tol):
+    """The rank-4 sum is nearly zero on interface sites away from the start vector, so the
+    error is taken relative to the largest diagonal entry."""
+    w = wl((128, 128), 4, 4, K=2, beta=20.0)
+    omega, V, sigma, _ = I.make_inputs(w)
+    q1 = np.zeros(w.N)
+    q1[site[0] + w.L[0] * site[1]] = 1.0
+    pl = plan_for(w, precision)
+    out = pl.solve(omega, V, sigma, q1)
+    for k in range(2):
+        subs, X = local_X(w, omega[k], V, sigma[k])
+        acc, al = O.cs_lanczos(X, q1, w.k)[:2]
+        assert pl.info(2)["steps"][k] == len(al) == w.k
+        ref = subs.diagB + acc
+        assert np.max(np.abs(out[k] - ref)) <= tol * np.max(np.abs(ref))
     pl.close()
