@@ -1081,14 +1081,18 @@ int dyson_xmatvec(dyson_plan p, int K, const double* omega, const double* V, con
   else LK(launch_precond<double>(g, p->b, K, s));
   // one vector per frequency: column 0 of block 0, result in the frequency's first slot
   LK(launch_gather(g, p->b, K, qn, p->b.Q, (size_t)(g.k_max + g.nb) * g.Ndd, s));
-  LK(launch_qsplit(g, p->b, K, s));
   CK(cudaMemsetAsync(p->b.st, 0, (size_t)K * ST_N * sizeof(int), s));
   if (g.p > 1) {
-    if (p->mixed) LK(launch_xmatvec<float>(g, p->b, K, 0, 1, 1, s));
-    else LK(launch_xmatvec<double>(g, p->b, K, 0, 0, 1, s));
+    // the caller's q is read in binary64: as double-floats (the plan's basis) entries below
+    // 2^-103 would keep 24 bits
+    Geo gx = g;
+    gx.qsplit = 0;
+    if (p->mixed) LK(launch_xmatvec<float>(gx, p->b, K, 0, 1, 1, s));
+    else LK(launch_xmatvec<double>(gx, p->b, K, 0, 0, 1, s));
   } else {
     CK(cudaMemsetAsync(p->b.u, 0, (size_t)K * g.nb * g.Ndd * sizeof(cxd), s));
   }
+  LK(launch_qsplit(g, p->b, K, s));        // the plan's basis form again, as dyson_lanczos_basis reads it
   cxd* dst = mem_kind == DYSON_MEM_HOST ? p->b.out : reinterpret_cast<cxd*>(u);
   LK(launch_scatter(g, p->b, K, p->b.u, dst, (size_t)g.nb * g.Ndd, s));
   if (mem_kind == DYSON_MEM_HOST) CK(cudaMemcpyAsync(u, dst, bytes, cudaMemcpyDeviceToHost, s));

@@ -325,7 +325,8 @@ cudaError_t launch_scatter(const Geo& g, const Bufs& b, int K, const cxd* dd, cx
 }
 
 // Vector 0 of each frequency's basis, written in binary64 (dyson_xmatvec's
-// caller vector), rewritten in place as double-floats when the basis is split.
+// caller vector, after its X-matvec), rewritten in place as double-floats when the
+// basis is split.
 __global__ void k_qsplit(Geo g, Bufs b) {
   const int kf = blockIdx.y;
   cxd* q = b.Q + (size_t)kf * (g.k_max + g.nb) * g.Ndd;

@@ -140,3 +140,20 @@ def test_solve_from_a_unit_start_vector(site, precision, tol):
         ref = subs.diagB + acc
         assert np.max(np.abs(out[k] - ref)) <= tol * np.max(np.abs(ref))
     pl.close()
+
+
+@pytest.mark.parametrize("L,p", [((64, 65), 2), ((4, 16, 17), 2)])   # strips; slabs with slices of 128 sites
+def test_xmatvec_reads_small_vectors_in_binary64(L, p):
+    """q and 2^-100 q (exact, ~1e-30): the same X q times 2^-100 to the stopping tolerance of
+    the refinement, 1e-13, in both, times the lattice's condition (|H^-1| <= 1 / w_0 = 3.2,
+    |H| < 12) with room for two of them."""
+    w = wl(L, p, 4, K=2)
+    omega, V, sigma, _ = I.make_inputs(w)
+    rng = np.random.default_rng(8)
+    q = rng.normal(size=(2, w.N)) + 1j * rng.normal(size=(2, w.N))
+    pl = plan_for(w, D.DYSON_MIXED)
+    u, us = np.zeros_like(q), np.zeros_like(q)
+    D.dyson_xmatvec(pl.handle, 2, omega, V, sigma, q, u)
+    D.dyson_xmatvec(pl.handle, 2, omega, V, sigma, q * 2.0 ** -100, us)
+    assert np.max(np.abs(us * 2.0 ** 100 - u)) <= 2 * 40 * 1e-13 * np.max(np.abs(u))
+    pl.close()
