@@ -873,7 +873,7 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
   constexpr int K0 = 20, KB = 120;
   constexpr double TINY2 = 0x1p-240;       // (2^-KB)^2
   const int ktop = K0 - norm_exp(qa2) + KB;
-  const bool live = !(hn2 <= TINY2 * qa2);
+  const bool live = hn2 > TINY2 * qa2;     // not for a NaN in H or q either: X q counts as zero then
   // ---- u_0 = H^-1 [0; hr]
   if (live) {
     const int kh = -norm_exp(hn2);
@@ -976,8 +976,12 @@ __global__ void __launch_bounds__(Mix<float, WF>::NT, Mix<float, WF>::PER_SM)
     }
     mix_sum<float, WF>(cl, phase, p, v, tot, true, own);
     const double rn = tot[0], wn = own[2];   // w: this subdomain's, which decides for its w alone
-    if (!wdone && (wn <= tol2 * qn2 || wn > REFINE_STALL * prev_w)) wdone = true;
+    if (!wdone && (wn <= tol2 * qn2 || !(wn <= REFINE_STALL * prev_w))) wdone = true;
     if (!wdone) prev_w = wn;
+    if (rn != rn) {                          // the interface solve broke down: nothing left to refine
+      conv_all = 0;
+      break;
+    }
     const bool udone = rn <= tol2 * tot[1] || rn > REFINE_STALL * prev_u;
     if (udone) {
       // u is done: go on only if some w of the cluster is not

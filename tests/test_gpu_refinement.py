@@ -157,3 +157,21 @@ def test_xmatvec_reads_small_vectors_in_binary64(L, p):
     D.dyson_xmatvec(pl.handle, 2, omega, V, sigma, q * 2.0 ** -100, us)
     assert np.max(np.abs(us * 2.0 ** 100 - u)) <= 2 * 40 * 1e-13 * np.max(np.abs(u))
     pl.close()
+
+
+def test_nan_frequency_costs_no_iterations():
+    """A NaN in Sigma makes the interface right-hand side of its frequency NaN: X q counts as
+    zero there, without interface iterations, and the other frequencies keep their bits."""
+    w = wl((40, 33), 2, 4, K=3)
+    omega, V, sigma, q1 = I.make_inputs(w)
+    pl = plan_for(w, D.DYSON_MIXED)
+    clean = pl.solve(omega, V, sigma, q1)
+    bad = sigma.copy()
+    bad[1, 500] = np.nan
+    out = pl.solve(omega, V, bad, q1)
+    info = pl.info(3)
+    assert info["iters"][1] == 0 and info["steps"][1] == 1
+    for k in (0, 2):
+        assert np.array_equal(out[k], clean[k])
+    assert np.isnan(out[1, 500])
+    pl.close()
