@@ -166,11 +166,12 @@ size_t layout(const Geo& g, int K, bool mixed, size_t off[B_COUNT]) {
   sz[B_U] = Ks * Ndd * sizeof(cxd);
   sz[B_V1] = mixed ? Ks * Ndd * sizeof(cxd) : 0;
   sz[B_V2] = sz[B_V1];
-  sz[B_V3] = sz[B_V1];
+  sz[B_V3] = g.W > DY_MAXW_SMEM ? sz[B_V1] : 0;   // the wide X-matvec's
   sz[B_YSCR] = Ks * g.p * nsub * cs;
   sz[B_BND] = Ks * g.p * 2 * g.A * sizeof(cxd);
   sz[B_IFV] = Ks * IF_N * nifc(g) * sizeof(cxd);
-  sz[B_PRE] = Kz * nifc(g) * 3 * sizeof(cxd);
+  const bool band = banded(g);
+  sz[B_PRE] = band ? Kz * nifc(g) * 3 * sizeof(cxd) : 0;
   sz[B_LAN] = Kz * (g.k_max + g.nb) * 2 * g.nb * sizeof(cxd);
   sz[B_MAXT] = Kz * sizeof(double);
   sz[B_ST] = Kz * ST_N * sizeof(int);
@@ -178,12 +179,12 @@ size_t layout(const Geo& g, int K, bool mixed, size_t off[B_COUNT]) {
   sz[B_STATUS] = Kz * sizeof(int);
   sz[B_SWEEPS] = Ks * g.p * sizeof(unsigned long long);
   sz[B_FWORK] = g.W > DY_MAXW_SMEM ? (size_t)DY_FACTOR_CTAS * 2 * g.W * g.W * sizeof(cxd) : 0;
-  sz[B_OFFB] = Kz * g.p * nsub * sizeof(cxd);
-  sz[B_OFF2] = g.penta ? Kz * g.p * nsub * sizeof(cxd) : 0;
+  sz[B_OFFB] = band ? Kz * g.p * nsub * sizeof(cxd) : 0;
+  sz[B_OFF2] = band && g.penta ? Kz * g.p * nsub * sizeof(cxd) : 0;
   const size_t A2 = (size_t)g.A * g.A;   // layer blocks (A = Lx in 2D)
   sz[B_LPT] = g.lpre ? Kz * g.p * 2 * A2 * sizeof(cxf) : 0;
   sz[B_LPM] = g.lpre ? Kz * (g.p - 1) * A2 * cs : 0;
-  sz[B_LPG] = (g.lpre && g.T == 1) ? Kz * g.p * nsub * g.W * sizeof(cxf) : 0;
+  sz[B_LPG] = (g.lpre && g.T == 1) ? Kz * g.p * lpg_entries(g) * sizeof(cxf) : 0;
   sz[B_LPW] = (g.lpre && g.T > 1) ? (size_t)DY_FACTOR_CTAS * 2 * g.W * 2 * (size_t)g.Lx * g.T * sizeof(cxf) : 0;
   sz[B_HDIAG] = mixed ? Kz * Ndd * sizeof(cxd) : 0;
   sz[B_GRAM] = g.qsplit ? Kz * (size_t)(g.k_max + 1) * (g.k_max + 1) * sizeof(cxd) : 0;
@@ -381,7 +382,7 @@ Bufs sub_bufs(const Geo& g, const Bufs& b, bool mixed, int k0) {
   const size_t A2 = (size_t)g.A * g.A;
   s.lpt = b.lpt ? b.lpt + K0 * g.p * 2 * A2 : nullptr;
   s.lpm = adv(reinterpret_cast<char*>(b.lpm), K0 * (g.p > 1 ? g.p - 1 : 0) * A2 * cs);
-  s.lpg = b.lpg ? b.lpg + K0 * g.p * nsub * g.W : nullptr;
+  s.lpg = b.lpg ? b.lpg + K0 * g.p * lpg_entries(g) : nullptr;
   s.gram = b.gram ? b.gram + K0 * (size_t)(g.k_max + 1) * (g.k_max + 1) : nullptr;
   return s;
 }
@@ -603,22 +604,23 @@ int dyson_plan_create(const dyson_geometry* geom, dyson_plan* out) {
   b.u = at<cxd>(p, B_U);
   b.v1 = p->mixed ? at<cxd>(p, B_V1) : nullptr;
   b.v2 = p->mixed ? at<cxd>(p, B_V2) : nullptr;
-  b.v3 = p->mixed ? at<cxd>(p, B_V3) : nullptr;
+  b.v3 = p->mixed && p->g.W > DY_MAXW_SMEM ? at<cxd>(p, B_V3) : nullptr;
   b.yscr = at<void>(p, B_YSCR);
   b.bnd = at<cxd>(p, B_BND);
   b.ifv = at<cxd>(p, B_IFV);
-  b.pre = at<cxd>(p, B_PRE);
+  const bool band = banded(p->g);
+  b.pre = band ? at<cxd>(p, B_PRE) : nullptr;
   b.lan = at<cxd>(p, B_LAN);
   b.maxT = at<double>(p, B_MAXT);
   b.st = at<int>(p, B_ST);
   b.out = at<cxd>(p, B_OUT);
   b.sweeps = at<unsigned long long>(p, B_SWEEPS);
   b.fwork = p->g.W > DY_MAXW_SMEM ? at<cxd>(p, B_FWORK) : nullptr;
-  b.offB = at<cxd>(p, B_OFFB);
-  b.off2 = p->g.penta ? at<cxd>(p, B_OFF2) : nullptr;
+  b.offB = band ? at<cxd>(p, B_OFFB) : nullptr;
+  b.off2 = band && p->g.penta ? at<cxd>(p, B_OFF2) : nullptr;
   b.lpt = p->g.lpre ? at<cxf>(p, B_LPT) : nullptr;
   b.lpm = p->g.lpre ? (void*)at<char>(p, B_LPM) : nullptr;
-  b.lpg = p->g.lpre ? at<cxf>(p, B_LPG) : nullptr;
+  b.lpg = (p->g.lpre && p->g.T == 1) ? at<cxf>(p, B_LPG) : nullptr;
   b.lpw = (p->g.lpre && p->g.T > 1) ? at<cxf>(p, B_LPW) : nullptr;
   b.gram = p->g.qsplit ? at<cxd>(p, B_GRAM) : nullptr;
   p->status_d = at<int>(p, B_STATUS);

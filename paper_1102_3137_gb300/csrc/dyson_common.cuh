@@ -280,7 +280,7 @@ struct Bufs {
   unsigned long long* sweeps;  // [K*nb][p] subdomain sweeps performed (work accounting)
   cxd* fwork;           // [DY_FACTOR_CTAS][2][W][W] wide-slice factor workspace (W > 64 only)
   cx<float>* lpt;       // [K][p][2][Lx][Lx] boundary-row surface Green's functions (lpre)
-  cx<float>* lpg;       // [K][p][Lx][W][W] lpre in 2D: per (frequency, strip) the boundary columns of G_ss
+  cx<float>* lpg;       // [K][p][4 Lx W] lpre in 2D: per (frequency, strip) the boundary columns of G_ss
                         // [Lx][2][W], then the rows across the middle [2][Lx][W] (k_surface_two)
   void* lpm;            // [K][p-1][Lx][Lx] inverse layer blocks of S, precision of the form (lpre)
   cx<float>* lpw;       // [DY_FACTOR_CTAS][2][W][2 Lx T] boundary-column chains of the 3D slab
@@ -314,6 +314,11 @@ __device__ __forceinline__ int sub_nat(const Geo& g, int i, int s, int j) {
 // `bytes`.  Plans of different sizes share the kernels, and a graph captured
 // for a large plan may be replayed after a small plan ran, so the limit only grows.
 cudaError_t raise_smem_limit(const void* func, size_t bytes);
+
+// Entries of Bufs::lpg per (frequency, strip).
+__host__ __device__ inline size_t lpg_entries(const Geo& g) { return (size_t)4 * g.Lx * g.W; }
+// The plan runs the banded preconditioner (which reads the off-diagonal blocks of B^-1).
+inline bool banded(const Geo& g) { return g.p > 1 && !g.lpre; }
 
 // CTAs that share one unit of a tiled factorization kernel: the largest of 8, 4, 2,
 // 1 that keeps the units within the DY_FACTOR_CTAS CTAs of one wave.

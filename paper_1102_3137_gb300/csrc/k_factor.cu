@@ -364,9 +364,9 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
   cxf* gsw = reinterpret_cast<cxf*>(b.g) + uoff;
   cxd* dB = b.diagB + (size_t)kf * g.Ndd + (size_t)i * Lx * W;
   const cxd* hd = b.hdiag + (size_t)kf * g.Ndd + (size_t)i * Lx * W;
-  const bool band = !g.lpre;                 // the banded preconditioner reads the off-diagonal blocks
-  cxd* oB = band && b.offB ? b.offB + ((size_t)kf * g.p + i) * (size_t)Lx * W : nullptr;
-  cxd* o2 = band && b.off2 && T == 1 ? b.off2 + ((size_t)kf * g.p + i) * (size_t)Lx * W : nullptr;
+  // off-diagonal blocks: for the banded preconditioner only
+  cxd* oB = b.offB ? b.offB + ((size_t)kf * g.p + i) * (size_t)Lx * W : nullptr;
+  cxd* o2 = b.off2 && T == 1 ? b.off2 + ((size_t)kf * g.p + i) * (size_t)Lx * W : nullptr;
   const R t = (R)g.t, t2 = (R)(g.t * g.t);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(DY_THREADS, WF <= 32 ? 2 : 1) k_factor_two(Geo
       }
   };
   // the layer preconditioner's input: columns w - 1 and 0 of G_ss (k_surface_two)
-  cxf* bc = g.lpre && b.lpg ? b.lpg + uoff : nullptr;
+  cxf* bc = b.lpg ? b.lpg + ((size_t)kf * g.p + i) * lpg_entries(g) : nullptr;
   auto diag_out = [&](int s) {
     for (int r = tid; r < W; r += DY_THREADS) dB[(size_t)s * W + r] = (r < w) ? cconv<double>(A[r * W + r]) : cxd{0, 0};
     if (bc)

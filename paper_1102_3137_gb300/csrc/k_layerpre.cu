@@ -100,8 +100,8 @@ __global__ void __launch_bounds__(DY_THREADS, 2) k_surface_two(Geo g, Bufs b) {
   cxf_* V = M + n;                                // [steps][W]: the boundary columns, by distance from the middle
   const size_t unit = (size_t)f * g.p + i;
   const cx<S>* gsrc = reinterpret_cast<const cx<S>*>(b.g) + unit * (size_t)Lx * n;   // complex64: column pairs interleaved
-  const cxf_* bc = b.lpg + unit * (size_t)Lx * n;
-  cxf_* Rr = b.lpg + unit * (size_t)Lx * n + (size_t)2 * Lx * W + (size_t)sd * Lx * W;   // [Lx][W] rows rb of G_{s,m} / N_s
+  const cxf_* bc = b.lpg + unit * lpg_entries(g);
+  cxf_* Rr = b.lpg + unit * lpg_entries(g) + (size_t)(2 + sd) * Lx * W;   // [Lx][W] rows rb of G_{s,m} / N_s
   cxf_* P = b.lpt + (unit * 2 + sd) * (size_t)Lx * Lx;
   const float t = d2f_bits(g.t);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
