@@ -264,7 +264,9 @@ int dyson_subdomain_solve(dyson_plan plan, int K, const double* omega, const dou
  * y = S^-1 (E^T B^-1 q_B - q_C), u_B = B^-1 E y, u_C = -y, with S applied
  * implicitly (never formed).  Mixed form: w = blkdiag(B^-1, 0) q and the
  * solution u of H u = [0; q_C - E^T w_B], refined together (the same u = v - w
- * without its cancellation).
+ * without its cancellation).  With slices of up to 64 sites q may have any size
+ * whose squared norm binary64 holds, also differing between strips, and an interface
+ * part q_C - E^T w_B below 2^-120 ||q|| counts as zero (u = 0).
  */
 int dyson_xmatvec(dyson_plan plan, int K, const double* omega, const double* V,
                   const double* sigma, const double* q, double* u, int mem_kind, void* stream);

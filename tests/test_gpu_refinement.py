@@ -104,6 +104,19 @@ def test_xmatvec_of_small_and_local_vectors(kind, precision, tol):
     pl.close()
 
 
+@pytest.mark.parametrize("size", [1e-100, 1e100])
+def test_mixed_xmatvec_of_any_size(size):
+    w = wl((64, 65), 2, 4, K=1)
+    omega, V, sigma, _ = I.make_inputs(w)
+    q = vector(("dense", size), w, np.random.default_rng(7))[None]
+    pl = plan_for(w, D.DYSON_MIXED)
+    u = np.zeros_like(q)
+    D.dyson_xmatvec(pl.handle, 1, omega, V, sigma, q, u)
+    ref = local_X(w, omega[0], V, sigma[0])[1](q[0])
+    assert np.max(np.abs(u[0] - ref)) <= 1e-9 * np.max(np.abs(ref))
+    pl.close()
+
+
 @pytest.mark.parametrize("L,p", [((40, 33), 2), ((64, 129), 2)])     # W = 16 and 64
 def test_xmatvec_of_a_vector_on_one_strip(L, p):
     """q is zero, or 1e-25 and 1e-35 of the rest, on the second strip."""
@@ -174,4 +187,33 @@ def test_nan_frequency_costs_no_iterations():
     for k in (0, 2):
         assert np.array_equal(out[k], clean[k])
     assert np.isnan(out[1, 500])
+    pl.close()
+
+
+@pytest.mark.parametrize("L,p", [((6, 527), 16), ((6, 1039), 16)])   # W = 32, 64
+@pytest.mark.parametrize("precision,tol", [(D.DYSON_FP64, 1e-11), (D.DYSON_MIXED, 1e-9)])
+def test_sixteen_strips(L, p, precision, tol):
+    """The largest cluster, 16 CTAs with up to an SM's shared memory each."""
+    w = wl(L, p, 4, K=2, trap=1e-5)
+    omega, V, sigma, _ = I.make_inputs(w)
+    rng = np.random.default_rng(9)
+    q = rng.normal(size=(2, w.N)) + 1j * rng.normal(size=(2, w.N))
+    pl = plan_for(w, precision)
+    u = np.zeros_like(q)
+    D.dyson_xmatvec(pl.handle, 2, omega, V, sigma, q, u)
+    for k in range(2):
+        ref = local_X(w, omega[k], V, sigma[k])[1](q[k])
+        assert np.max(np.abs(u[k] - ref)) <= tol * np.max(np.abs(ref))
+    pl.close()
+
+
+def test_infinite_interface_entry_is_not_answered_with_zero():
+    w = wl((40, 33), 2, 4, K=1)              # the interface line is y = 16
+    omega, V, sigma, _ = I.make_inputs(w)
+    q = np.ones((1, w.N), complex)
+    q[0, 5 + 40 * 16] = np.inf
+    pl = plan_for(w, D.DYSON_MIXED, krylov_maxit=50)
+    u = np.zeros_like(q)
+    D.dyson_xmatvec(pl.handle, 1, omega, V, sigma, q, u)
+    assert not np.any(np.isfinite(u))
     pl.close()
