@@ -82,6 +82,13 @@ def union_ms(starts, ends):
     return float(tot)
 
 
+def xmatvec_kernel(W, mixed):
+    """The X-matvec kernel of slices of width W (padded to a multiple of 4)."""
+    if W > 64:
+        return "k_xmatvec<float>" if mixed else "k_xmatvec<double>"
+    return "k_xmatvec_m" if mixed else ("k_xmatvec_d" if W <= 32 else "k_xmatvec<double>")
+
+
 def recorded_traffic(kernel, workload):
     """DRAM bytes per step (all launches of the kernel) from the last ncu capture, if the
     kernel has not changed since."""
@@ -430,6 +437,7 @@ def run_ours(a, rank, world, local_rank):
     n_xm = max(1, len(xm))
     hbm_peak, peak_src = peaks()
     xm_avg_ms = float(xm.mean()) if len(xm) else float("nan")
+    xm_kernel = xmatvec_kernel(4 * -(-int(wi.max()) // 4), prec == D.DYSON_MIXED)
     # the frequency groups' X-matvec launches overlap in time: the kernel's time
     # in the step is the union of its launch intervals (CUDA events on each
     # launch's own stream, inside the replayed graph)
@@ -438,8 +446,8 @@ def run_ours(a, rank, world, local_rank):
     if prec == D.DYSON_MIXED:
         ach = sw_bytes / (xm_union_ms / 1e3) / 1e9
         roof = dict(bound="hbm", achieved=ach, peak=hbm_peak, unit="GB/s", frac=ach / hbm_peak,
-                    traffic=recorded_traffic("k_xmatvec<float>", a.workload),
-                    kernel="k_xmatvec<float>", peak_source=peak_src,
+                    traffic=recorded_traffic(xm_kernel, a.workload),
+                    kernel=xm_kernel, peak_source=peak_src,
                     per_step_algorithmic_bytes=sw_bytes,
                     per_launch_algorithmic_bytes=sw_bytes / n_xm,
                     per_launch_achieved=sw_bytes / n_xm / (xm_avg_ms / 1e3) / 1e9)
@@ -447,8 +455,8 @@ def run_ours(a, rank, world, local_rank):
         ach = sw_flops / (xm_union_ms / 1e3) / 1e12
         roof = dict(bound="alu", achieved=ach, peak=FP64_PEAK_TFLOPS, unit="TFLOP/s",
                     frac=ach / FP64_PEAK_TFLOPS,
-                    traffic=recorded_traffic("k_xmatvec<double>", a.workload),
-                    kernel="k_xmatvec<double>",
+                    traffic=recorded_traffic(xm_kernel, a.workload),
+                    kernel=xm_kernel,
                     peak_source="derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz",
                     per_step_algorithmic_flops=sw_flops,
                     per_launch_algorithmic_flops=sw_flops / n_xm,
@@ -461,8 +469,8 @@ def run_ours(a, rank, world, local_rank):
     # the Lanczos step (row a7/a8), complex128-sized entries of 16 B per site.  The
     # FP64 form's CGS2 reads the basis three times per step (g = Q^T u; r1 = u - Q g
     # with h = Q^T r1 in the same pass; r = r1 - Q h); the mixed form's takes h from
-    # the Gram matrix of the basis and reads it twice (g = Q^T u; r = u - Q (g + h)
-    # with the next Gram column Q^T r in the same pass).  Plus ~6 vectors (u, q_j,
+    # the Gram matrix of the basis and reads it twice (g = Q^T u with the Gram column
+    # Q^T q_j in the same pass; r = u - Q (g + h)).  Plus ~6 vectors (u, q_j,
     # q_{j-1}, r written, the running diagonal read and written).  A frequency that
     # ran n steps moves sum_{j=1..n} (reads j + 6) N 16 B.
     lz = kms[kinds == 4]

@@ -449,7 +449,8 @@ int enqueue_solve(dyson_plan p, int K, cudaStream_t s, bool cap) {
 // an interface, on the caller's staged inputs, run init, factorization and
 // preconditioner once, then time one X-matvec launch (after one untimed) for
 // each copy-ring configuration the geometry admits (ring slots; chunk height
-// for W > 64; rows on chip or in scratch for the mixed form's strips) and keep the fastest for every later launch and captured graph.
+// for W > 64; rows on chip or in scratch for the two-chain strips) and keep the
+// fastest for every later launch and captured graph.
 int autotune(dyson_plan p, int K, cudaStream_t s) {
   p->tuned = true;
   if (p->g.p < 2) return DYSON_OK;

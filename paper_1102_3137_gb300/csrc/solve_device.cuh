@@ -798,13 +798,10 @@ __device__ void cluster_sum_r(cg::cluster_group& cl, RedSmem& rs, int& phase, in
   phase ^= 1;
 }
 
-// COCG for S y = b on the interface (S = C - E^T B^-1 E never formed), all in
-// precision R: the FP64 form solves to krylov_tol in FP64; the mixed form's
-// inner solves (refined in FP64 one level up) run entirely in complex64.
 // z = M_l^-1 r on interface line i with the exact layer block of S: a dense symmetric
 // product (the stored inverse is symmetric, so column a is read contiguously across
-// threads), its columns split over the warps: warp task (32 V outputs, one of CS column ranges), the CS
-// partials added in a fixed order.  The block (2 MB at A = 512) comes from HBM on
+// threads), its columns split over the warps: warp task (32 V outputs, one of CS
+// column ranges), the CS partials added in a fixed order.  The block (2 MB at A = 512) comes from HBM on
 // every application, so what counts is the bytes in flight: V = 2 outputs a lane
 // by 16-byte loads where a row's length keeps them aligned, eight columns at a time.
 // part: the free row buffer [Lx][W], CS x A entries of it.  r must be complete (a
@@ -889,6 +886,9 @@ __device__ __forceinline__ void interface_precond(const Geo& g, const Bufs& b, i
   else precond_apply<R>(g, b, vs, i, r, z);
 }
 
+// COCG for S y = b on the interface (S = C - E^T B^-1 E never formed), all in
+// precision R: the FP64 form solves to krylov_tol in FP64; the mixed form's
+// inner solves (refined against FP64 residuals one level up) run in complex64.
 // Right-hand side in IF_B, solution y in IF_X.  Returns the iteration count;
 // *conv is set to 0 if the cap was hit.  xB += xs B^-1 E y (the subdomain block; "="
 // when fresh) comes along without a sweep of its own: the iteration's product
