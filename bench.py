@@ -480,7 +480,7 @@ def run_ours(a, rank, world, local_rank):
     lz_union = union_ms(t0[kinds == 4], t1[kinds == 4])
     lz_ach = lz_bytes / (lz_union / 1e3) / 1e9 if lz_union > 0 else float("nan")
     roof_lz = dict(bound="hbm", achieved=lz_ach, peak=hbm_peak, unit="GB/s", frac=lz_ach / hbm_peak,
-                   traffic=recorded_traffic("k_lanczos", a.workload),
+                   traffic=recorded_traffic("k_lanczos_dd" if prec == D.DYSON_MIXED else "k_lanczos", a.workload),
                    kernel="k_lanczos_dd" if prec == D.DYSON_MIXED else "k_lanczos", peak_source=peak_src,
                    per_step_algorithmic_bytes=lz_bytes, launches_per_step=int(len(lz)),
                    union_ms_per_step=lz_union, mean_launch_ms=float(lz.mean()) if len(lz) else None,
